@@ -30,7 +30,7 @@ def _stale(out: str, deps: list[str]) -> bool:
 
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
-    headers = [os.path.join(CSRC, "qw_internal.h"), os.path.join(CSRC, "qw_device.cuh"),
+    headers = [os.path.join(CSRC, "qw_internal.h"), os.path.join(CSRC, "qw_device.cuh"), os.path.join(CSRC, "qw_amp.cuh"),
                os.path.join(os.path.dirname(HERE), "include", "qwalk.h")]
     objs, procs = [], []
     for src in SOURCES:

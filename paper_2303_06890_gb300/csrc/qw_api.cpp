@@ -380,6 +380,7 @@ extern "C" int qw_sim_create(const qw_csc *mats, int32_t ninst, const qw_sim_opt
         std::memcpy(&d.tau_hi_bits, &hi, 8);
         std::memcpy(&d.tau_lo_bits, &lo, 8);
         d.tau2f = (float)(tau * tau);
+        d.thr32 = (float)(std::max(tau, std::ldexp(1.0, sim->fp32 ? -60 : -100)) * (1.0 + std::ldexp(1.0, -20)));
     }
     d.rot_calc = o.rot_bits == 0;
     d.inv_sqrt_s = 1.0 / std::sqrt((double)s);

@@ -82,6 +82,7 @@ struct QwSimDev {
     uint64_t tau_hi_bits;     /* bits of tau (1 + 2^-30): |x| above it => kept */
     uint64_t tau_lo_bits;     /* bits of tau sqrt(1/2) (1 - 2^-30): |x|,|y| at most it => pruned */
     float tau2f;              /* tau^2 as float (complex64 path) */
+    float thr32;              /* at least tau and 2^-100 (2^-60 for complex64, whose squares it keeps normal): above it (plus the approximation's error) => kept */
     int rot_calc;             /* rot_bits == 0: the FP32 rotation pairs follow from the code alone */
     double inv_sqrt_s;        /* 1 / sqrt(s) */
     double two_over_s;        /* 2 / s */

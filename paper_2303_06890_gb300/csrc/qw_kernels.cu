@@ -34,6 +34,7 @@
 
 #include "../../include/qwalk.h"
 #include "qw_internal.h"
+#include "qw_amp.cuh"
 #include "qw_device.cuh"
 
 /* Rotation controls carried in the key between a map and its rotation: the
@@ -420,10 +421,15 @@ template <> struct KeyB1<uint32_t> { static constexpr int bit = 31; };
 __host__ __device__ inline bool key32_fits(const QwSimDev &d) { return 1 + 2 * d.nb <= 29; }
 
 /* per-warp shared memory of the fused kernels (byte offsets, 16-byte aligned):
- * keys x2, amplitudes x3 (a pair list holds two per key), the zero-type group (b2 = 0 values, b2 = 1 values,
- * presence), the staged QRAM row, pair-head indices, the row's rotation values */
+ * keys x2, amplitudes x2, the zero-type group (each slot's pair and kept flags), the staged QRAM row, pair-head indices, the row's
+ * rotation values */
+struct ZeroFlags { /* a zero-type slot's PairState and its magnitude bound */
+    float m;
+    uint8_t c0, c1, lossy, pad;
+};
+
 struct WalkLayout {
-    size_t kP, kQ, aP, aQ, aX, zbuf, z1buf, simg, pbuf, hidx, sfg, per_warp;
+    size_t kP, kQ, aP, aQ, zp, simg, zf, hidx, sfg, per_warp;
 };
 
 template <typename AmpT, typename KeyT>
@@ -439,11 +445,9 @@ __host__ __device__ inline WalkLayout walk_layout(const QwSimDev &d)
     QW_TAKE(kQ, C * sizeof(KeyT));
     QW_TAKE(aP, C * sizeof(AmpT));
     QW_TAKE(aQ, C * sizeof(AmpT));
-    QW_TAKE(aX, C * sizeof(AmpT));
-    QW_TAKE(zbuf, s * sizeof(AmpT));
-    QW_TAKE(z1buf, s * sizeof(AmpT));
+    QW_TAKE(zp, 2 * s * sizeof(AmpT));
     QW_TAKE(simg, s * sizeof(uint32_t));
-    QW_TAKE(pbuf, s * sizeof(int16_t));
+    QW_TAKE(zf, s * sizeof(ZeroFlags));
     QW_TAKE(hidx, 64 * sizeof(int16_t));
     QW_TAKE(sfg, s * 16);
 #undef QW_TAKE
@@ -461,392 +465,6 @@ __host__ __device__ inline WalkLayout walk_layout(const QwSimDev &d)
  * H P H needs no grouping at all: a branch outside the zero-type groups is
  * only negated, and the zero-type groups are found by a predicate on the key.
  */
-
-/* sign flips as integer operations on the sign bit (keeps FP64 negations
- * and selects off GB300's slow FP64 pipe) */
-/* sign flip of an FP64 value as an integer XOR on its high word, kept opaque
-   (inline PTX) so that it stays on the integer pipe: an FP64 negation would
-   take a slot of GB300's 1/64-rate FP64 pipe */
-__device__ __forceinline__ double flip_if(double x, bool neg)
-{
-    const int m = (int)((unsigned)neg << 31);
-    int hi = __double2hiint(x);
-    asm("xor.b32 %0, %0, %1;" : "+r"(hi) : "r"(m));
-    return __hiloint2double(hi, __double2loint(x));
-}
-__device__ __forceinline__ float flip_if(float x, bool neg)
-{
-    return __int_as_float(__float_as_int(x) ^ ((int)neg << 31));
-}
-
-template <typename AmpT> struct Amp;
-
-/* complex128 path: FP64 arithmetic throughout */
-__device__ __noinline__ double2 scale_c128(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
-
-/* the pruning decision inside the band around tau (rarely reached) */
-__device__ __noinline__ bool keep_band(double x, double y, double tau2)
-{
-    return __dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)) > tau2;
-}
-
-template <> struct Amp<double2> {
-    typedef double2 T;
-    static constexpr bool kHeadLanes = true; /* rotate with one lane per pair head */
-    struct Norm {
-        double v = 0.0;
-        __device__ void add(T a) { v = fma(a.x, a.x, fma(a.y, a.y, v)); }
-        __device__ double get() const { return v; }
-        __device__ double warp_total() const
-        {
-            double t = v;
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
-            return t;
-        }
-    };
-    /* sum of a zero-type Hadamard group (FP64) */
-    struct Sum {
-        double x = 0.0, y = 0.0;
-        __device__ void add(T a) { x += a.x; y += a.y; }
-        __device__ void set(T a) { x = a.x; y = a.y; } /* add() to an empty sum */
-        /* lane t < min(s, 32) holds the partial sums of the values t, t + 32, ...
-           (s a power of two); with width < 32 each aligned group of width
-           lanes reduces its own values.  Butterfly over the w = min(s, 32) lanes, x on
-           lanes t < w/2 and y on lanes t >= w/2 after the first level, so one
-           FP64 add serves both components; the same pairs and order as a
-           butterfly over each component alone (FP64 addition commutes). */
-        __device__ void reduce(int s, int width = 32)
-        {
-            const int w = s < 32 ? s : 32, h = w >> 1;
-            if (h > 0) {
-                const bool hy = (lane_id() & h) != 0;
-                const double recv = __shfl_xor_sync(FULL, hy ? x : y, h);
-                double v = (hy ? y : x) + recv;
-                for (int o = h >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-                x = v;
-                y = v;
-            }
-            x = __shfl_sync(FULL, x, 0, width);
-            y = __shfl_sync(FULL, y, h, width);
-        }
-        __device__ void scale_pow2(double f) { x *= f; y *= f; }
-        __device__ T minus(T a) const { return make_double2(x - a.x, y - a.y); }
-        /* scale_pow2(f) then minus(a) in one FMA per component: f is a power of
-           two, so f x is exact and the result is the same rounding */
-        __device__ T scaled_minus(double f, T a) const { return make_double2(fma(f, x, -a.x), fma(f, y, -a.y)); }
-        __device__ double2 value() const { return make_double2(x, y); }
-    };
-    __device__ static T zero() { return make_double2(0.0, 0.0); }
-    __device__ static T neg(T a) { return make_double2(flip_if(a.x, true), flip_if(a.y, true)); }
-    __device__ static double2 to_d(T a) { return a; }
-    __device__ static T from_d(double2 a) { return a; }
-    /* |a|^2 > tau^2 exactly as the un-fused FP64 formula, decided from the
-       exponent bits except in a narrow band around tau; the band's FP64
-       arithmetic sits in a call of its own, so that it is not if-converted
-       into every call (a predicated-off FP64 instruction still takes its
-       slot of the 1/64-rate FP64 pipe) */
-    __device__ static bool keep(const QwSimDev &d, T a)
-    {
-        const uint64_t ux = (uint64_t)__double_as_longlong(a.x) & 0x7fffffffffffffffull;
-        const uint64_t uy = (uint64_t)__double_as_longlong(a.y) & 0x7fffffffffffffffull;
-        const uint64_t um = ux > uy ? ux : uy;
-        if (um > d.tau_hi_bits) return true;
-        if (um <= d.tau_lo_bits) return false;
-        return keep_band(a.x, a.y, d.tau2);
-    }
-    struct Scale { /* the renormalisation (off by default for complex128): out of
-                      line, so its FP64 products are not if-converted into the
-                      loads that do not rescale */
-        double s;
-        __device__ explicit Scale(double v) : s(v) {}
-        __device__ T apply(T a) const { return scale_c128(a, s); }
-        /* staged once per block (the factor in 8 bytes of shared memory) */
-        __device__ static void to_shared(double v, double *buf) { buf[0] = v; }
-        __device__ static Scale from_shared(const double *buf) { return Scale(buf[0]); }
-    };
-    typedef double2 RotVal; /* (sqrt|a|, sqrt(1-|a|)) */
-    __device__ static RotVal rot_table(const QwSimDev &d, uint32_t A) { return __ldg(d.fg + A); }
-    __device__ static RotVal rot_zero() { return make_double2(0.0, 1.0); }
-    static constexpr bool kRotCode = false; /* FP64 square roots: read the table */
-    __device__ static RotVal rot_code(uint32_t) { return rot_zero(); }
-    __device__ static void rot(RotVal t, uint32_t A, bool dag, bool sneg, T a0, T a1, T &o0, T &o1);
-    /* rot(t, A, true, sneg, a0, 0): R^dag of a pair whose b2 = 1 member is 0 */
-    __device__ static void rot_dag_b2zero(RotVal t, uint32_t A, bool sneg, T a0, T &o0, T &o1);
-    static constexpr bool kB2ZeroPath = true;
-};
-
-/* complex64 path: amplitudes are float; each rotation output f a0 +- g a1 is
-   formed from error-free products and an error-free sum on the FP32 pipe
-   (f, g held as float pairs with ~48 significant bits) and rounded once. */
-template <> struct Amp<float2> {
-    typedef float2 T;
-    static constexpr bool kHeadLanes = false;
-    struct Norm { /* |a|^2 rounded to FP32 once per branch (relative 2^-24), then
-                     summed by TwoSum into a float pair, so the sum adds no
-                     rounding error of note beyond those per-term roundings */
-        float hi = 0.f, lo = 0.f;
-        __device__ void add(T a)
-        {
-            const float v = __fadd_rn(__fmul_rn(a.x, a.x), __fmul_rn(a.y, a.y));
-            const float s = __fadd_rn(hi, v);
-            const float bp = __fsub_rn(s, hi);
-            lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(v, bp)));
-            hi = s;
-        }
-        __device__ double get() const { return (double)hi + (double)lo; }
-        /* the warp's sum: a butterfly of float-pair additions, one conversion
-           to FP64 on the lane that returns it (lane 0; the others return 0) */
-        __device__ double warp_total() const;
-    };
-    /* float-pair (hi + lo) accumulator built from Knuth's TwoSum (the sum and
-       its exact rounding error), ~48 significant bits */
-    struct DF {
-        float h = 0.f, l = 0.f;
-        __device__ void add(float v)
-        {
-            const float s = __fadd_rn(h, v);
-            const float bp = __fsub_rn(s, h);
-            const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bp)), __fsub_rn(v, bp));
-            h = s;
-            l = __fadd_rn(l, e);
-        }
-        __device__ void add(float vh, float vl)
-        {
-            add(vh);
-            l = __fadd_rn(l, vl);
-            const float s = __fadd_rn(h, l); /* renormalise: |l| small */
-            l = __fsub_rn(l, __fsub_rn(s, h));
-            h = s;
-        }
-
-        /* round(h + l - v) */
-        __device__ float minus(float v) const
-        {
-            const float s = __fsub_rn(h, v);
-            const float bp = __fsub_rn(s, h);
-            const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bp)), __fsub_rn(-v, bp));
-            return __fadd_rn(s, __fadd_rn(e, l));
-        }
-    };
-    /* sum of a zero-type Hadamard group of FP32 terms in a float pair: its
-       error is of order 2^-46 times the sum of the terms' magnitudes */
-    struct Sum {
-        DF x, y;
-        __device__ void add(T a) { x.add(a.x); y.add(a.y); }
-        __device__ void set(T a) /* add() to an empty sum: the value, no error term */
-        {
-            x.h = a.x;
-            x.l = 0.f;
-            y.h = a.y;
-            y.l = 0.f;
-        }
-        /* lane t < min(s, 32) holds the partial sums of the values t, t + 32, ...
-           (s a power of two); with width < 32 each aligned group of width
-           lanes reduces its own values.  Butterfly over the w = min(s, 32) lanes, x on
-           lanes t < w/2 and y on lanes t >= w/2 after the first level (where a
-           y lane adds its own pair to its partner's, the order the partner
-           would use), so one float-pair add serves both components. */
-        __device__ void reduce(int s, int width = 32)
-        {
-            const int w = s < 32 ? s : 32, h = w >> 1;
-            if (h > 0) {
-                const bool hy = (lane_id() & h) != 0;
-                const float rh = __shfl_xor_sync(FULL, hy ? x.h : y.h, h);
-                const float rl = __shfl_xor_sync(FULL, hy ? x.l : y.l, h);
-                DF v;
-                if (hy) { /* partner's y, then own y */
-                    v.h = rh;
-                    v.l = rl;
-                    v.add(y.h, y.l);
-                } else {
-                    v = x;
-                    v.add(rh, rl);
-                }
-                for (int o = h >> 1; o > 0; o >>= 1) {
-                    const float oh = __shfl_xor_sync(FULL, v.h, o), ol = __shfl_xor_sync(FULL, v.l, o);
-                    v.add(oh, ol);
-                }
-                x = v;
-                y = v;
-            }
-            x.h = __shfl_sync(FULL, x.h, 0, width);
-            x.l = __shfl_sync(FULL, x.l, 0, width);
-            y.h = __shfl_sync(FULL, y.h, h, width);
-            y.l = __shfl_sync(FULL, y.l, h, width);
-        }
-        __device__ void scale_pow2(double f)
-        {
-            const float g = (float)f; /* 2/s: a power of two, exact */
-            x.h *= g; x.l *= g; y.h *= g; y.l *= g;
-        }
-        __device__ T minus(T a) const { return make_float2(x.minus(a.x), y.minus(a.y)); }
-        __device__ T scaled_minus(double f, T a) const
-        {
-            Sum c = *this;
-            c.scale_pow2(f);
-            return c.minus(a);
-        }
-        __device__ double2 value() const
-        {
-            return make_double2((double)x.h + (double)x.l, (double)y.h + (double)y.l);
-        }
-    };
-    __device__ static T zero() { return make_float2(0.f, 0.f); }
-    __device__ static T neg(T a) { return make_float2(-a.x, -a.y); }
-    __device__ static double2 to_d(T a) { return make_double2((double)a.x, (double)a.y); }
-    __device__ static T from_d(double2 a) { return make_float2((float)a.x, (float)a.y); }
-    __device__ static bool keep(const QwSimDev &d, T a)
-    {
-        return __fadd_rn(__fmul_rn(a.x, a.x), __fmul_rn(a.y, a.y)) > d.tau2f;
-    }
-    /* a * s with s = sh + sl, rounded once */
-    __device__ static float mul_split(float a, float sh, float sl)
-    {
-        const float p = __fmul_rn(sh, a);
-        float e = __fmaf_rn(sh, a, -p);
-        e = __fmaf_rn(sl, a, e);
-        return __fadd_rn(p, e);
-    }
-    struct Scale { /* the FP64 factor as a float pair, applied with one rounding */
-        float sh, sl;
-        __device__ explicit Scale(double v) : sh((float)v), sl((float)(v - (double)(float)v)) {}
-        __device__ Scale(float h, float l) : sh(h), sl(l) {}
-        __device__ T apply(T a) const { return make_float2(mul_split(a.x, sh, sl), mul_split(a.y, sh, sl)); }
-        /* the split computed once per block (its FP64 conversions would
-           otherwise take a slot of the 1/64-rate FP64 pipe in every thread) */
-        __device__ static void to_shared(double v, double *buf)
-        {
-            float *f = reinterpret_cast<float *>(buf);
-            f[0] = (float)v;
-            f[1] = (float)(v - (double)(float)v);
-        }
-        __device__ static Scale from_shared(const double *buf)
-        {
-            const float *f = reinterpret_cast<const float *>(buf);
-            return Scale(f[0], f[1]);
-        }
-    };
-    /* round(A x + B y), A = ah + al, B = bh + bl: the products by the FMA-based
-       TwoProduct (p = fl(a b), e = fma(a, b, -p) exact), their sum by Knuth's
-       TwoSum, the low parts added to the error term, one final rounding */
-    __device__ static float dot2(float ah, float al, float x, float bh, float bl, float y)
-    {
-        const float p1 = __fmul_rn(ah, x);
-        float e1 = __fmaf_rn(ah, x, -p1);
-        e1 = __fmaf_rn(al, x, e1);
-        const float p2 = __fmul_rn(bh, y);
-        float e2 = __fmaf_rn(bh, y, -p2);
-        e2 = __fmaf_rn(bl, y, e2);
-        const float s = __fadd_rn(p1, p2);
-        const float bp = __fsub_rn(s, p1);
-        const float t = __fadd_rn(__fsub_rn(p1, __fsub_rn(s, bp)), __fsub_rn(p2, bp));
-        return __fadd_rn(s, __fadd_rn(t, __fadd_rn(e1, e2)));
-    }
-    typedef float4 RotVal; /* (sqrt|a|, sqrt(1-|a|)) as float pairs */
-    __device__ static RotVal rot_table(const QwSimDev &d, uint32_t A) { return __ldg(d.fg32 + A); }
-    /* the table entry of code A (rot_bits = 0) computed in place: hi the
-       correctly rounded square root, lo the Newton correction (x - hi^2) /
-       (2 hi) with the residual exact by FMA -- the host builds the table the
-       same way, so the bits agree */
-    static constexpr bool kRotCode = true;
-    __device__ static RotVal rot_code(uint32_t A)
-    {
-        const int q = (int)(int16_t)(uint16_t)A;
-        const float x = (float)(q < 0 ? -q : q) * (1.0f / 32768.0f), y = 1.0f - x;
-        const float fh = __fsqrt_rn(x), gh = __fsqrt_rn(y);
-        const float fl = fh > 0.0f ? __fdiv_rn(__fmaf_rn(-fh, fh, x), 2.0f * fh) : 0.0f;
-        const float gl = gh > 0.0f ? __fdiv_rn(__fmaf_rn(-gh, gh, y), 2.0f * gh) : 0.0f;
-        return make_float4(fh, fl, gh, gl);
-    }
-    __device__ static RotVal rot_zero() { return make_float4(0.f, 0.f, 1.f, 0.f); }
-    __device__ static void rot(RotVal t, uint32_t A, bool dag, bool sneg, T a0, T a1, T &o0, T &o1);
-    __device__ static void rot_dag_b2zero(RotVal t, uint32_t A, bool sneg, T a0, T &o0, T &o1);
-    static constexpr bool kB2ZeroPath = false;
-    /* dot2 with y = 0: round(A x) -- the same bits (p1 + e1 rounded once) */
-    __device__ static float dot1(float ah, float al, float x)
-    {
-        const float p1 = __fmul_rn(ah, x);
-        float e1 = __fmaf_rn(ah, x, -p1);
-        e1 = __fmaf_rn(al, x, e1);
-        return __fadd_rn(p1, e1);
-    }
-};
-
-__device__ double Amp<float2>::Norm::warp_total() const
-{
-    DF v;
-    v.h = hi;
-    v.l = lo;
-    for (int o = 16; o > 0; o >>= 1) {
-        const float oh = __shfl_xor_sync(FULL, v.h, o), ol = __shfl_xor_sync(FULL, v.l, o);
-        v.add(oh, ol);
-    }
-    return lane_id() == 0 ? (double)v.h + (double)v.l : 0.0;
-}
-
-/* multiply by 1 (real f) or by i*sigma (imaginary f), sigma = sneg ? -1 : 1:
- * i sigma (x + i y) = -sigma y + i sigma x */
-template <typename T>
-__device__ __forceinline__ T rho(T a, bool imag, bool sneg)
-{
-    T r;
-    r.x = imag ? flip_if(a.y, !sneg) : a.x;
-    r.y = imag ? flip_if(a.x, sneg) : a.y;
-    return r;
-}
-
-/* R:    o0 = f a0 - g a1,        o1 = g a0 + conj(f) a1
- * R^dag: o0 = conj(f) a0 + g a1, o1 = f a1 - g a0
- * with f = fm (a >= 0) or i sigma fm (a < 0): f x = fm rho(x, sigma),
- * conj(f) x = fm rho(x, -sigma). */
-__device__ void Amp<double2>::rot(RotVal t, uint32_t A, bool dag, bool sneg, T a0, T a1, T &o0, T &o1)
-{
-    const double fm = t.x, g = t.y;
-    const bool imag = (int16_t)(uint16_t)A < 0;
-    const double2 x0 = rho(a0, imag, dag ? !sneg : sneg);
-    const double2 x1 = rho(a1, imag, dag ? sneg : !sneg);
-    if (!dag) {
-        o0 = make_double2(fma(fm, x0.x, -g * a1.x), fma(fm, x0.y, -g * a1.y));
-        o1 = make_double2(fma(g, a0.x, fm * x1.x), fma(g, a0.y, fm * x1.y));
-    } else {
-        o0 = make_double2(fma(fm, x0.x, g * a1.x), fma(fm, x0.y, g * a1.y));
-        o1 = make_double2(fma(fm, x1.x, -g * a0.x), fma(fm, x1.y, -g * a0.y));
-    }
-}
-
-/* R^dag (a0, 0): o0 = conj(f) a0, o1 = -g a0 -- the general formulas with
-   a1 = 0, whose products by 0 change no rounding */
-__device__ void Amp<double2>::rot_dag_b2zero(RotVal t, uint32_t A, bool sneg, T a0, T &o0, T &o1)
-{
-    const double fm = t.x, g = t.y;
-    const bool imag = (int16_t)(uint16_t)A < 0;
-    const double2 x0 = rho(a0, imag, !sneg);
-    o0 = make_double2(fm * x0.x, fm * x0.y);
-    o1 = make_double2(-g * a0.x, -g * a0.y);
-}
-
-__device__ void Amp<float2>::rot_dag_b2zero(RotVal t, uint32_t A, bool sneg, T a0, T &o0, T &o1)
-{
-    const bool imag = (int16_t)(uint16_t)A < 0;
-    const float2 x0 = rho(a0, imag, !sneg);
-    o0 = make_float2(dot1(t.x, t.y, x0.x), dot1(t.x, t.y, x0.y));
-    o1 = make_float2(dot1(-t.z, -t.w, a0.x), dot1(-t.z, -t.w, a0.y));
-}
-
-__device__ void Amp<float2>::rot(RotVal t, uint32_t A, bool dag, bool sneg, T a0, T a1, T &o0, T &o1)
-{
-    /* t = (fh, fl, gh, gl) */
-    const bool imag = (int16_t)(uint16_t)A < 0;
-    const float2 x0 = rho(a0, imag, dag ? !sneg : sneg);
-    const float2 x1 = rho(a1, imag, dag ? sneg : !sneg);
-    if (!dag) {
-        o0 = make_float2(dot2(t.x, t.y, x0.x, -t.z, -t.w, a1.x), dot2(t.x, t.y, x0.y, -t.z, -t.w, a1.y));
-        o1 = make_float2(dot2(t.z, t.w, a0.x, t.x, t.y, x1.x), dot2(t.z, t.w, a0.y, t.x, t.y, x1.y));
-    } else {
-        o0 = make_float2(dot2(t.x, t.y, x0.x, t.z, t.w, a1.x), dot2(t.x, t.y, x0.y, t.z, t.w, a1.y));
-        o1 = make_float2(dot2(t.x, t.y, x1.x, -t.z, -t.w, a0.x), dot2(t.x, t.y, x1.y, -t.z, -t.w, a0.y));
-    }
-}
 
 /* Pair up to 32 branches held one per lane (valid lanes carry distinct keys):
  * b2-partners (keys equal but for bit 0) become adjacent, b2 = 0 first, in
@@ -1034,14 +652,23 @@ template <typename KeyT>
 __device__ __forceinline__ KeyT map_t(const QwSimDev &d, const Row &r, KeyT key, uint32_t &slot, uint32_t &A,
                                       bool &sneg);
 
-/* The pair headed by key k (b2 = 0 member amplitude a0, b2 = 1 member a1,
- * zero where absent): the register maps of one half-step on the key, then
- * R^dag (WHICH = 0, T~^dag) or R (WHICH = 1, T~).  The maps never read b2,
- * so the head maps the key once for both members; the rotation is controlled
- * by A and sigma, which the maps return beside the key.  Outputs o0 (b2 = 0)
- * and o1 (b2 = 1) under kb (b2 = 0, the b1 tag kept), and whether each is
- * kept by the pruning rule. */
-template <int WHICH, typename AmpT, typename KeyT>
+/* A is 0 or the value of slot `slot` of row j: staged rotation values for a
+ * slot of this row, the per-code table otherwise */
+template <typename AmpT>
+__device__ __forceinline__ typename Amp<AmpT>::RotVal rot_of(const QwSimDev &d, const Row &r, uint32_t slot, uint32_t A)
+{
+    if (A == 0) return Amp<AmpT>::rot_zero();
+    if (slot < (uint32_t)d.s && r.sfg) return static_cast<const typename Amp<AmpT>::RotVal *>(r.sfg)[slot];
+    return Amp<AmpT>::rot_table(d, A);
+}
+
+/* T~ after H on the pair headed by key k (b2 = 0 member amplitude a0, b2 = 1
+ * member a1, zero where absent): the register maps on the key, then R.  The
+ * maps never read b2, so the head maps the key once for both members; the
+ * rotation is controlled by A and sigma, which the maps return beside the
+ * key.  Outputs o0 (b2 = 0) and o1 (b2 = 1) under kb (b2 = 0, the b1 tag
+ * kept), and whether each is kept by the pruning rule. */
+template <typename AmpT, typename KeyT>
 __device__ __forceinline__ void rot_head(const QwSimDev &d, const Row &r, KeyT k, AmpT a0, AmpT a1, AmpT &o0,
                                          AmpT &o1, bool &c0, bool &c1, KeyT &kb)
 {
@@ -1049,60 +676,23 @@ __device__ __forceinline__ void rot_head(const QwSimDev &d, const Row &r, KeyT k
     const KeyT key = k & ~((KeyT)1 | b1bit);
     uint32_t slot, A;
     bool sneg;
-    const KeyT mk = (WHICH == 0) ? map_tdag<KeyT>(d, r, key, slot, A, sneg) : map_t<KeyT>(d, r, key, slot, A, sneg);
-    /* A is 0 or the value of slot `slot` of row j: staged rotation values for
-       a slot of this row, the per-code table otherwise */
-    typename Amp<AmpT>::RotVal t;
-    if (A == 0) t = Amp<AmpT>::rot_zero();
-    else if (slot < (uint32_t)d.s && r.sfg) t = static_cast<const typename Amp<AmpT>::RotVal *>(r.sfg)[slot];
-    else t = Amp<AmpT>::rot_table(d, A);
-    Amp<AmpT>::rot(t, A, WHICH == 0, sneg, a0, a1, o0, o1);
+    const KeyT mk = map_t<KeyT>(d, r, key, slot, A, sneg);
+    Amp<AmpT>::rot(rot_of<AmpT>(d, r, slot, A), A, false, sneg, a0, a1, o0, o1);
     c0 = Amp<AmpT>::keep(d, o0);
     c1 = Amp<AmpT>::keep(d, o1);
     kb = mk | b1bit;
 }
 
-/* Appends rotated pairs to a warp buffer, pair-adjacent (b2 = 0 first), kept
- * outputs only.  REFL: H P H folded in -- k_high | kc | b1 all zero in a row
- * with jc = 0 marks the zero-type Hadamard group (b2 = 0: set aside in zbuf
- * for the reflection; b2 = 1: negated, set aside beside it); every other
- * output is negated here.  Called by all lanes of the warp together. */
-template <typename AmpT, typename KeyT, bool REFL>
+/* Appends pairs to a warp buffer, pair-adjacent (b2 = 0 first), kept outputs
+ * only.  Called by all lanes of the warp together. */
+template <typename AmpT, typename KeyT>
 struct PairSink {
     KeyT *kd;
     AmpT *ad;
-    int cap, out, div;
-    KeyT zm;
-    bool rowzero;
-    int smask;
-    AmpT *zbuf, *z1buf;
-    int16_t *pbuf;
-    __device__ PairSink(const QwSimDev &d, const Row &r, KeyT *kd_, AmpT *ad_, int cap_, AmpT *zb, AmpT *z1b,
-                        int16_t *pb)
-        : kd(kd_), ad(ad_), cap(cap_), out(0), div(0), smask(d.s - 1), zbuf(zb), z1buf(z1b), pbuf(pb)
+    int cap, out;
+    __device__ PairSink(KeyT *kd_, AmpT *ad_, int cap_) : kd(kd_), ad(ad_), cap(cap_), out(0) {}
+    __device__ __forceinline__ void put(KeyT kb, AmpT o0, AmpT o1, bool c0, bool c1)
     {
-        const int ash = 1 + 2 * d.nb;
-        zm = ((((KeyT)1 << ash) - 1) & ~(((KeyT)1 << (d.L + 1)) - 1)) | ((KeyT)1 << KeyB1<KeyT>::bit);
-        rowzero = REFL && r.jc == 0;
-    }
-    __device__ __forceinline__ void put(bool head, KeyT kb, AmpT o0, AmpT o1, bool c0, bool c1)
-    {
-        if (REFL) {
-            const bool zt = head && rowzero && (kb & zm) == 0;
-            div += __popc(__ballot_sync(FULL, zt && c0)) + __popc(__ballot_sync(FULL, zt && c1));
-            if (zt) {
-                const int u = (int)((kb >> 1) & (KeyT)smask);
-                if (c0) zbuf[u] = o0;
-                if (c1) {
-                    z1buf[u] = Amp<AmpT>::neg(o1);
-                    pbuf[u] = 1;
-                }
-                c0 = c1 = false;
-            } else {
-                o0 = Amp<AmpT>::neg(o0);
-                o1 = Amp<AmpT>::neg(o1);
-            }
-        }
         int total;
         int pos = out + warp_compact2(c0, c1, total);
         if (c0) {
@@ -1116,110 +706,89 @@ struct PairSink {
     }
 };
 
-/* The same outputs as PairSink, as a pair list: one entry per pair with a
- * kept member -- key kb (b2 = 0), the b2 = 0 and b2 = 1 amplitudes, zero for a
- * member that is absent (a kept amplitude is never zero: it exceeds tau).
- * elems counts the kept branches. */
-template <typename AmpT, typename KeyT, bool REFL>
-struct PairListSink {
-    KeyT *kd;
-    AmpT *a0d, *a1d;
-    int cap, out, div, elems;
+/* One pair of a row through T~^dag, P, T~ (the walk operator on a pair,
+ * above): a pair outside the zero-type groups comes back under its own key as
+ * -(a0, a1) and goes to the output list; a pair of slot l of a zero-type group
+ * (k_high | kc | b1 all zero after O_s'^dag, in a row with jc = 0) is set
+ * aside for the reflection.  Called by all lanes of the warp together. */
+template <typename AmpT, typename KeyT>
+struct WalkSink {
+    PairSink<AmpT, KeyT> out;
+    AmpT *zp;
+    ZeroFlags *zf;
     KeyT zm;
     bool rowzero;
-    int smask;
-    AmpT *zbuf, *z1buf;
-    int16_t *pbuf;
-    __device__ PairListSink(const QwSimDev &d, const Row &r, KeyT *kd_, AmpT *a0_, AmpT *a1_, int cap_, AmpT *zb,
-                            AmpT *z1b, int16_t *pb)
-        : kd(kd_), a0d(a0_), a1d(a1_), cap(cap_), out(0), div(0), elems(0), smask(d.s - 1), zbuf(zb), z1buf(z1b),
-          pbuf(pb)
+    unsigned rdag, hph; /* branches kept after R^dag, and after H P H outside the zero-type groups */
+    __device__ WalkSink(const QwSimDev &d, const Row &r, KeyT *kd, AmpT *ad, int cap, AmpT *zp_, ZeroFlags *zf_)
+        : out(kd, ad, cap), zp(zp_), zf(zf_), rdag(0), hph(0)
     {
         const int ash = 1 + 2 * d.nb;
         zm = ((((KeyT)1 << ash) - 1) & ~(((KeyT)1 << (d.L + 1)) - 1)) | ((KeyT)1 << KeyB1<KeyT>::bit);
-        rowzero = REFL && r.jc == 0;
+        rowzero = r.jc == 0;
     }
-    __device__ __forceinline__ void put(bool head, KeyT kb, AmpT o0, AmpT o1, bool c0, bool c1)
+    __device__ __forceinline__ void put(const QwSimDev &d, const Row &r, bool head, KeyT k, AmpT a0, AmpT a1)
     {
-        if (REFL) {
-            const bool zt = head && rowzero && (kb & zm) == 0;
-            div += __popc(__ballot_sync(FULL, zt && c0)) + __popc(__ballot_sync(FULL, zt && c1));
+        AmpT r0 = Amp<AmpT>::zero(), r1 = Amp<AmpT>::zero();
+        bool c0 = false, c1 = false;
+        const KeyT kb = k & ~(KeyT)1;
+        unsigned kept = 0;
+        bool zt = false;
+        if (head) {
+            const KeyT b1bit = k & ((KeyT)1 << KeyB1<KeyT>::bit);
+            uint32_t slot, A;
+            bool sneg;
+            const KeyT mk = map_tdag<KeyT>(d, r, kb & ~b1bit, slot, A, sneg) | b1bit;
+            const typename Amp<AmpT>::RotVal t = rot_of<AmpT>(d, r, slot, A);
+            zt = rowzero && (mk & zm) == 0;
             if (zt) {
-                const int u = (int)((kb >> 1) & (KeyT)smask);
-                if (c0) zbuf[u] = o0;
-                if (c1) {
-                    z1buf[u] = Amp<AmpT>::neg(o1);
-                    pbuf[u] = 1;
-                }
-                c0 = c1 = false;
+                const int u = (int)((mk >> 1) & (KeyT)(d.s - 1));
+                float m;
+                const PairState<AmpT> p = pair_state<AmpT>(d, t, A, sneg, a0, a1, Amp<AmpT>::approx2(a0),
+                                                           Amp<AmpT>::approx2(a1), m);
+                zp[2 * u] = a0;
+                zp[2 * u + 1] = a1;
+                zf[u] = ZeroFlags{m, (uint8_t)p.c0, (uint8_t)p.c1, (uint8_t)p.lossy, 0};
+                kept = (p.c0 ? 1u : 0u) + (p.c1 ? 1u : 0u);
             } else {
-                o0 = Amp<AmpT>::neg(o0);
-                o1 = Amp<AmpT>::neg(o1);
+                kept = pair_negate<AmpT>(d, t, A, sneg, a0, a1, r0, r1);
+                c0 = Amp<AmpT>::keep(d, r0);
+                c1 = Amp<AmpT>::keep(d, r1);
             }
         }
-        const bool any = c0 || c1;
-        const unsigned m = __ballot_sync(FULL, any);
-        elems += __popc(__ballot_sync(FULL, c0)) + __popc(__ballot_sync(FULL, c1));
-        if (any) {
-            const int pos = out + __popc(m & ((1u << lane_id()) - 1u));
-            if (pos < cap) {
-                kd[pos] = kb;
-                a0d[pos] = c0 ? o0 : Amp<AmpT>::zero();
-                a1d[pos] = c1 ? o1 : Amp<AmpT>::zero();
-            }
-        }
-        out += __popc(m);
+        const unsigned all = __reduce_add_sync(FULL, kept), rest = __reduce_add_sync(FULL, zt ? 0u : kept);
+        rdag += all;
+        hph += rest;
+        out.put(kb, r0, r1, c0, c1);
     }
 };
 
-/* One half-step over a pair list of np entries: one lane per pair. */
-template <int WHICH, typename AmpT, typename KeyT, typename Sink>
-__device__ void map_rot_list(const QwSimDev &d, const Row &r, const KeyT *ks, const AmpT *a0s, const AmpT *a1s,
-                             int np, Sink &sink)
-{
-    for (int base = 0; base < np; base += 32) {
-        const int p = base + lane_id();
-        const bool head = p < np;
-        AmpT o0 = Amp<AmpT>::zero(), o1 = Amp<AmpT>::zero();
-        bool c0 = false, c1 = false;
-        KeyT kb = 0;
-        if (head) rot_head<WHICH, AmpT, KeyT>(d, r, ks[p], a0s[p], a1s[p], o0, o1, c0, c1, kb);
-        sink.put(head, kb, o0, o1, c0, c1);
-    }
-    __syncwarp();
-}
-
-/* One half-step (maps + rotation) over a warp buffer of n branches with
- * b2-pairs adjacent: each pair head (a b2 = 0 branch, or a b2 = 1 one
- * without its partner) rotates both members; the outputs go to the sink. */
-template <int WHICH, typename AmpT, typename KeyT, typename Sink>
-__device__ void map_rot_pairs(const QwSimDev &d, const Row &r, const KeyT *ks, const AmpT *as, int n, Sink &sink,
-                              int16_t *hidx)
+/* A pass over a warp buffer of n branches with b2-pairs adjacent: pair(head,
+ * key, a0, a1) for each pair head (a b2 = 0 branch, or a b2 = 1 one without
+ * its partner), all lanes of the warp together. */
+template <typename AmpT, typename KeyT, typename Pair>
+__device__ void for_pairs(const KeyT *ks, const AmpT *as, int n, int16_t *hidx, Pair &&pair)
 {
     const int lane = lane_id();
     auto pair_at = [&](int i, bool head) {
-        AmpT o0 = Amp<AmpT>::zero(), o1 = Amp<AmpT>::zero();
-        bool c0 = false, c1 = false;
-        KeyT kb = 0;
+        KeyT k = 0;
+        AmpT a0 = Amp<AmpT>::zero(), a1 = Amp<AmpT>::zero();
         if (head) {
-            const KeyT k = ks[i];
-            AmpT a0 = Amp<AmpT>::zero(), a1 = Amp<AmpT>::zero();
+            k = ks[i];
             if ((k & (KeyT)1) == 0) {
                 a0 = as[i];
                 if (i + 1 < n && ks[i + 1] == (k | (KeyT)1)) a1 = as[i + 1];
             } else {
                 a1 = as[i];
             }
-            rot_head<WHICH, AmpT, KeyT>(d, r, k, a0, a1, o0, o1, c0, c1, kb);
         }
-        sink.put(head, kb, o0, o1, c0, c1);
+        pair(head, k, a0, a1);
     };
     auto is_head = [&](int i) {
         return i < n && !(i > 0 && ks[i - 1] == (ks[i] ^ (KeyT)1));
     };
     if (Amp<AmpT>::kHeadLanes) {
         /* blocks of 64 branches: list the heads, then one lane per head, so no
-           lane idles through the (FP64) rotation for a pair's second member */
+           lane idles through the FP64 work for a pair's second member */
         const unsigned lt = (1u << lane) - 1u;
         for (int base = 0; base < n; base += 64) {
             int nh = 0;
@@ -1243,9 +812,23 @@ __device__ void map_rot_pairs(const QwSimDev &d, const Row &r, const KeyT *ks, c
     }
 }
 
-/* T~^dag on up to 32 loaded branches held one per lane (valid lanes carry
- * distinct keys): b2-partners found by a warp match on key >> 1, the head of
- * each pair takes its partner's amplitude by a shuffle and rotates both. */
+/* T~ after H over a warp buffer of n branches (k_tinit) */
+template <typename AmpT, typename KeyT>
+__device__ void map_rot_pairs(const QwSimDev &d, const Row &r, const KeyT *ks, const AmpT *as, int n,
+                              PairSink<AmpT, KeyT> &sink, int16_t *hidx)
+{
+    for_pairs<AmpT, KeyT>(ks, as, n, hidx, [&](bool head, KeyT k, AmpT a0, AmpT a1) {
+        AmpT o0 = Amp<AmpT>::zero(), o1 = Amp<AmpT>::zero();
+        bool c0 = false, c1 = false;
+        KeyT kb = 0;
+        if (head) rot_head<AmpT, KeyT>(d, r, k, a0, a1, o0, o1, c0, c1, kb);
+        sink.put(kb, o0, o1, c0, c1);
+    });
+}
+
+/* Up to 32 loaded branches held one per lane (valid lanes carry distinct
+ * keys): b2-partners found by a warp match on key >> 1, the head of each pair
+ * takes its partner's amplitude by a shuffle and puts the pair. */
 template <typename AmpT, typename KeyT, typename Sink>
 __device__ __forceinline__ void rot0_chunk(const QwSimDev &d, const Row &r, KeyT k, AmpT a, bool valid, Sink &sink)
 {
@@ -1259,15 +842,9 @@ __device__ __forceinline__ void rot0_chunk(const QwSimDev &d, const Row &r, KeyT
     AmpT pa;
     pa.x = __shfl_sync(FULL, a.x, src);
     pa.y = __shfl_sync(FULL, a.y, src);
-    AmpT o0 = Amp<AmpT>::zero(), o1 = Amp<AmpT>::zero();
-    bool c0 = false, c1 = false;
-    KeyT kb = 0;
-    if (head) {
-        const AmpT a0 = b2one ? Amp<AmpT>::zero() : a;
-        const AmpT a1 = b2one ? a : (other ? pa : Amp<AmpT>::zero());
-        rot_head<0, AmpT, KeyT>(d, r, k, a0, a1, o0, o1, c0, c1, kb);
-    }
-    sink.put(head, kb, o0, o1, c0, c1);
+    const AmpT a0 = b2one ? Amp<AmpT>::zero() : a;
+    const AmpT a1 = b2one ? a : (other ? pa : Amp<AmpT>::zero());
+    sink.put(d, r, head, k, a0, a1);
 }
 
 /* Close a sink: its branch count, capped at the buffer (overflow flagged). */
@@ -1283,27 +860,46 @@ __device__ int sink_count(Sink &sink, int32_t *status)
 }
 
 
-/* The zero-type Hadamard group of H P H, after T~^dag's rotation has negated
- * every other branch and set the group aside (PairListSink with REFL): in a
- * row with jc = b1 = 0, the group (kc = k_high = b2 = 0) maps a_u ->
- * (2/s) sum_v a_v - a_u for all s values of u (H P H = 2|+><+| - 1 there).
- * Appends the s pairs (u: the reflected b2 = 0 value, and the set-aside
- * negated b2 = 1 partner) to the np entries of the pair list; elems receives
- * the number of branches appended.  The sum is taken by u in a fixed order
- * (FP64 for complex128, a float pair for complex64); with readout,
- * (1/sqrt s) sum_v a_v -- the flag-0 amplitude of T~^dag's output -- goes into
- * the QLS accumulator. */
+/* The zero-type Hadamard group of a row with jc = b1 = 0, whose pairs
+ * WalkSink has set aside: r = (2/s) sum_u over its s slots (by u in a fixed
+ * order; FP64 for complex128, a float pair for complex64), every slot's pair
+ * (f r - a0, g r - a1) -- absent members are 0 -- appended to the output list
+ * under T~'s key of the slot.  elems receives the branches kept after H P H.
+ * With readout, (1/sqrt s) sum_u -- the flag-0 amplitude of T~^dag's output --
+ * goes into the QLS accumulator. */
 template <typename AmpT, typename KeyT>
-__device__ int reflect_zero_list(const QwSimDev &d, const Row &r, KeyT *kd, AmpT *a0d, AmpT *a1d, int np, int cap,
-                                 int32_t *status, const QwStepArgs &a, const AmpT *zbuf, const AmpT *z1buf,
-                                 const int16_t *pbuf, int &elems)
+__device__ void reflect_zero_list(const QwSimDev &d, const Row &r, WalkSink<AmpT, KeyT> &sink, const QwStepArgs &a,
+                                  unsigned &elems)
 {
     elems = 0;
-    if (r.jc != 0) return np;
+    if (r.jc != 0) return;
     const int lane = lane_id();
     const int s = d.s;
+    /* slot u's rotation and its term of the sum (0 where R^dag's output was
+       dropped) */
+    struct Slot {
+        KeyT key;
+        uint32_t A;
+        bool sneg;
+        typename Amp<AmpT>::RotVal t;
+        typename Amp<AmpT>::Wide u;
+    };
+    auto slot_at = [&](int u) {
+        Slot x;
+        uint32_t slot;
+        x.key = map_t<KeyT>(d, r, (KeyT)u << 1, slot, x.A, x.sneg);
+        x.t = rot_of<AmpT>(d, r, slot, x.A);
+        x.u = sink.zf[u].c0 ? Amp<AmpT>::rdag0(x.t, x.A, x.sneg, sink.zp[2 * u], sink.zp[2 * u + 1])
+                            : Amp<AmpT>::wide_zero();
+        return x;
+    };
+    Slot x0{};
     typename Amp<AmpT>::Sum sum;
-    for (int t = lane; t < s; t += 32) sum.add(zbuf[t]);
+    if (lane < s) {
+        x0 = slot_at(lane);
+        sum.set(x0.u);
+    }
+    for (int t = lane + 32; t < s; t += 32) sum.add(slot_at(t).u);
     sum.reduce(s);
     if (a.qls_readout && r.valid && lane == 0) {
         const double2 sv = sum.value();
@@ -1314,36 +910,30 @@ __device__ int reflect_zero_list(const QwSimDev &d, const Row &r, KeyT *kd, AmpT
         a.qls_y[r.j] = acc;
     }
     sum.scale_pow2(d.two_over_s);
-    int out = np;
     for (int ub = 0; ub < s; ub += 32) {
         const int u = ub + lane;
-        const bool vu = u < s;
-        AmpT o0 = Amp<AmpT>::zero();
-        bool c1 = false;
-        if (vu) {
-            o0 = sum.minus(zbuf[u]);
-            c1 = pbuf[u] > 0;
+        AmpT r0 = Amp<AmpT>::zero(), r1 = Amp<AmpT>::zero();
+        bool e0 = false, e1 = false;
+        KeyT key = 0;
+        unsigned kept = 0;
+        if (u < s) {
+            const ZeroFlags z = sink.zf[u];
+            const Slot x = ub == 0 ? x0 : slot_at(u);
+            PairState<AmpT> p;
+            p.c0 = z.c0 != 0;
+            p.c1 = z.c1 != 0;
+            p.lossy = z.lossy != 0;
+            bool d0;
+            key = x.key;
+            pair_reflect<AmpT>(d, sum, x.t, x.A, x.sneg, sink.zp[2 * u], sink.zp[2 * u + 1], x.u, z.m, p, r0, r1, d0);
+            kept = (d0 ? 1u : 0u) + (p.c1 ? 1u : 0u);
+            e0 = Amp<AmpT>::keep(d, r0);
+            e1 = Amp<AmpT>::keep(d, r1);
         }
-        const bool c0 = vu && Amp<AmpT>::keep(d, o0);
-        const bool any = c0 || c1;
-        const unsigned m = __ballot_sync(FULL, any);
-        elems += __popc(__ballot_sync(FULL, c0)) + __popc(__ballot_sync(FULL, c1));
-        if (any) {
-            const int pos = out + __popc(m & ((1u << lane) - 1u));
-            if (pos < cap) {
-                kd[pos] = (KeyT)u << 1;
-                a0d[pos] = c0 ? o0 : Amp<AmpT>::zero();
-                a1d[pos] = c1 ? z1buf[u] : Amp<AmpT>::zero();
-            }
-        }
-        out += __popc(m);
+        elems += __reduce_add_sync(FULL, kept);
+        sink.out.put(key, r0, r1, e0, e1);
     }
     __syncwarp();
-    if (out > cap) {
-        if (lane == 0) atomicOr(status, QW_ST_WARP_OVERFLOW);
-        out = cap;
-    }
-    return out;
 }
 
 /* Register maps of T~^dag before R^dag.  T~^dag applies O_s'^dag, O_A', O_s',
@@ -1453,16 +1043,17 @@ __device__ void emit_pairs(const QwSimDev &d, const Row &r, const KeyT *ks, cons
 /* Per-warp shared buffers of the row pipeline (offsets from walk_layout). */
 template <typename AmpT, typename KeyT> struct WalkBufs {
     KeyT *kP, *kQ;
-    AmpT *aP, *aQ, *aX, *zbuf, *z1buf;
+    AmpT *aP, *aQ, *zp;
     uint32_t *simg;
-    int16_t *pbuf, *hidx;
+    ZeroFlags *zf;
+    int16_t *hidx;
     typename Amp<AmpT>::RotVal *sfg;
     __device__ WalkBufs(unsigned char *b, const WalkLayout &lay)
         : kP(reinterpret_cast<KeyT *>(b + lay.kP)), kQ(reinterpret_cast<KeyT *>(b + lay.kQ)),
           aP(reinterpret_cast<AmpT *>(b + lay.aP)), aQ(reinterpret_cast<AmpT *>(b + lay.aQ)),
-          aX(reinterpret_cast<AmpT *>(b + lay.aX)), zbuf(reinterpret_cast<AmpT *>(b + lay.zbuf)),
-          z1buf(reinterpret_cast<AmpT *>(b + lay.z1buf)), simg(reinterpret_cast<uint32_t *>(b + lay.simg)),
-          pbuf(reinterpret_cast<int16_t *>(b + lay.pbuf)), hidx(reinterpret_cast<int16_t *>(b + lay.hidx)),
+          zp(reinterpret_cast<AmpT *>(b + lay.zp)),
+          simg(reinterpret_cast<uint32_t *>(b + lay.simg)), zf(reinterpret_cast<ZeroFlags *>(b + lay.zf)),
+          hidx(reinterpret_cast<int16_t *>(b + lay.hidx)),
           sfg(reinterpret_cast<typename Amp<AmpT>::RotVal *>(b + lay.sfg))
     {
     }
@@ -1532,15 +1123,15 @@ __device__ __forceinline__ void walk_item(const QwSimDev &d, const QwBufDev &in,
     st.in += n;
     if (r.jc == 0) { /* the zero-type group's slots, filled by T~^dag */
         for (int t = lane; t < d.s; t += 32) {
-            B.zbuf[t] = Amp<AmpT>::zero();
-            B.pbuf[t] = -1;
+            B.zp[2 * t] = B.zp[2 * t + 1] = Amp<AmpT>::zero();
+            B.zf[t] = ZeroFlags{0.f, 0, 0, 0, 0};
         }
         __syncwarp();
     }
-    PairListSink<AmpT, KeyT, true> s0(d, r, B.kQ, B.aQ, B.aX, C, B.zbuf, B.z1buf, B.pbuf);
+    WalkSink<AmpT, KeyT> s0(d, r, B.kQ, B.aQ, C, B.zp, B.zf);
     if (!Amp<AmpT>::kHeadLanes && it.n0 <= 32 && it.n1 <= 32) {
-        /* rows of <= 32: T~^dag straight from the loaded registers, the
-           pairs found by one warp match per chunk of <= 32 */
+        /* rows of <= 32: straight from the loaded registers, the pairs found by
+           one warp match per chunk of <= 32 */
         const int ash = 1 + 2 * d.nb;
         const KeyT tagB = (KeyT)1 << B1;
         uint64_t anc = 0;
@@ -1577,20 +1168,18 @@ __device__ __forceinline__ void walk_item(const QwSimDev &d, const QwBufDev &in,
     } else {
         load_seg<AmpT, KeyT>(d, in, it.bA, it.n0, it.tagA, it.bB, it.n1, rescale, scale, B.kP, B.aP, B.kQ, B.aQ, C,
                              have_cur, hk, ha, a.status);
-        map_rot_pairs<0, AmpT, KeyT>(d, r, B.kP, B.aP, n, s0, B.hidx);
+        for_pairs<AmpT, KeyT>(B.kP, B.aP, n, B.hidx,
+                              [&](bool head, KeyT k, AmpT a0, AmpT a1) { s0.put(d, r, head, k, a0, a1); });
     }
     prefetch();
-    int np = sink_count(s0, a.status); /* T~^dag, H P H signs */
-    st.rdag += s0.elems + s0.div;
-    int ez = 0;
-    np = reflect_zero_list<AmpT, KeyT>(d, r, B.kQ, B.aQ, B.aX, np, C, a.status, a, B.zbuf, B.z1buf, B.pbuf,
-                                       ez); /* H P H */
-    st.hph += s0.elems + ez;
-    PairSink<AmpT, KeyT, false> s1(d, r, B.kP, B.aP, C, nullptr, nullptr, nullptr);
-    map_rot_list<1, AmpT, KeyT>(d, r, B.kQ, B.aQ, B.aX, np, s1);
-    n = sink_count(s1, a.status); /* T~ */
+    __syncwarp();
+    unsigned ez = 0;
+    reflect_zero_list<AmpT, KeyT>(d, r, s0, a, ez);
+    st.rdag += s0.rdag;
+    st.hph += s0.hph + ez;
+    n = sink_count(s0.out, a.status);
     st.out += n;
-    emit_pairs<AmpT, KeyT>(d, r, B.kP, B.aP, n, out, a.status, nrm); /* S */
+    emit_pairs<AmpT, KeyT>(d, r, B.kQ, B.aQ, n, out, a.status, nrm); /* S */
     __syncwarp();
 }
 
@@ -2190,15 +1779,15 @@ __global__ void __launch_bounds__(WARPS * 32, 4) k_walk_slot(QwSimDev d, QwBufDe
             const uint32_t w = ws[lane], col = w >> 16, val = w & 0xffffu;
             const RotVal rv = rotv[lane];
             const bool sneg = U.j > col;
-            AmpT o0, o1;
-            Amp<AmpT>::rot(rv, val, true, sneg, ta[2 * lane], ta[2 * lane + 1], o0, o1); /* R^dag */
-            const bool c0 = Amp<AmpT>::keep(d, o0), c1 = Amp<AmpT>::keep(d, o1);
-            st.rdag += __popc(__ballot_sync(FULL, c0)) + __popc(__ballot_sync(FULL, c1));
-            /* H P H on the zero-type group: a_l -> (2/s) sum_v a_v - a_l; the
-               b2 = 1 member, outside every zero-type group, is negated */
-            const AmpT z0 = c0 ? o0 : zero;
+            const AmpT p0 = ta[2 * lane], p1 = ta[2 * lane + 1];
+            typename Amp<AmpT>::Wide u;
+            float m;
+            const PairState<AmpT> ps = pair_tdag<AmpT>(d, rv, val, sneg, p0, p1, u, m); /* R^dag */
+            __syncwarp();
+            st.rdag += __popc(__ballot_sync(FULL, ps.c0)) + __popc(__ballot_sync(FULL, ps.c1));
+            /* H P H on the zero-type group and R: the unit's slots reflected */
             typename Amp<AmpT>::Sum sum;
-            sum.set(z0);
+            sum.set(u);
             sum.reduce(S, S);
             if (a.qls_readout && U.valid && (lane % S) == 0) {
                 const double2 sv = sum.value();
@@ -2208,13 +1797,12 @@ __global__ void __launch_bounds__(WARPS * 32, 4) k_walk_slot(QwSimDev d, QwBufDe
                 acc.y += coef * (d.inv_sqrt_s * sv.y);
                 a.qls_y[U.j] = acc;
             }
-            const AmpT h0 = sum.scaled_minus(d.two_over_s, z0);
-            const bool d0 = Amp<AmpT>::keep(d, h0);
-            st.hph += __popc(__ballot_sync(FULL, d0)) + __popc(__ballot_sync(FULL, c1));
-            /* T~: O_A' reads slot l (A = a_{j,l}), O_s' takes (l, 0) to (K(j, l), 0);
-               R; the rest of T~ returns A to 0 */
+            sum.scale_pow2(d.two_over_s);
             AmpT r0, r1;
-            Amp<AmpT>::rot(rv, val, false, sneg, d0 ? h0 : zero, c1 ? Amp<AmpT>::neg(o1) : zero, r0, r1);
+            bool d0;
+            pair_reflect<AmpT>(d, sum, rv, val, sneg, p0, p1, u, m, ps, r0, r1, d0);
+            __syncwarp();
+            st.hph += __popc(__ballot_sync(FULL, d0)) + __popc(__ballot_sync(FULL, ps.c1));
             const bool e0 = Amp<AmpT>::keep(d, r0), e1 = Amp<AmpT>::keep(d, r1);
             st.out += __popc(__ballot_sync(FULL, e0)) + __popc(__ballot_sync(FULL, e1));
             SlotOut<AmpT> outA, none; /* S */
@@ -2268,49 +1856,36 @@ __global__ void __launch_bounds__(WARPS * 32, 4) k_walk_slot(QwSimDev d, QwBufDe
             const bool isext = (meta & 0x8000u) != 0;
             const AmpT a0 = act ? ia[2 * q] : zero, a1 = act ? ia[2 * q + 1] : zero;
             int ut;
-            uint32_t b1, Adag, At, k_out = 0, kc_out = 0;
-            bool sdag, st_neg;
-            RotVal rdag, rt;
-            KeyT key = 0;
+            uint32_t b1, A, k_out = 0, kc_out = 0;
+            bool sneg;
+            RotVal rv;
             if (!isext) { /* slot t of a b1 = 1 row: (l, 0) both ways */
                 const int t = (int)(meta & 63u);
                 ut = t / S;
                 b1 = 1;
                 const uint32_t w = ws[t];
                 k_out = w >> 16;
-                Adag = At = w & 0xffffu;
-                rdag = rt = rotv[t];
-                sdag = st_neg = units[ut].j > k_out;
-            } else { /* an extra: the general maps of rot_head */
+                A = w & 0xffffu;
+                rv = rotv[t];
+                sneg = units[ut].j > k_out;
+            } else { /* an extra: the general map of T~^dag; T~'s leads back to its own key */
                 const uint64_t e = ek[meta & 0x7fffu];
                 ut = (int)(e >> 56);
-                key = (KeyT)(e & ~(0xffull << 56));
+                KeyT key = (KeyT)(e & ~(0xffull << 56));
                 b1 = (uint32_t)((key >> B1) & (KeyT)1);
                 key &= ~(((KeyT)1) | ((KeyT)1 << B1));
                 const Row r = slot_row(units[ut], ws + ut * S, rotv + ut * S);
                 uint32_t slot;
-                key = map_tdag<KeyT>(d, r, key, slot, Adag, sdag);
-                rdag = Adag == 0 ? Amp<AmpT>::rot_zero()
-                                 : (slot < (uint32_t)S ? rotv[ut * S + slot] : Amp<AmpT>::rot_table(d, Adag));
+                map_tdag<KeyT>(d, r, key, slot, A, sneg);
+                rv = A == 0 ? Amp<AmpT>::rot_zero() : (slot < (uint32_t)S ? rotv[ut * S + slot] : Amp<AmpT>::rot_table(d, A));
+                k_out = (uint32_t)(key >> 1) & msk;
+                kc_out = (uint32_t)(key >> (1 + d.nb)) & msk;
             }
-            AmpT o0, o1;
-            Amp<AmpT>::rot(rdag, Adag, true, sdag, a0, a1, o0, o1); /* R^dag */
-            const bool c0 = act && Amp<AmpT>::keep(d, o0), c1 = act && Amp<AmpT>::keep(d, o1);
-            const int kept = __popc(__ballot_sync(FULL, c0)) + __popc(__ballot_sync(FULL, c1));
+            AmpT r0, r1; /* R^dag, -1, R */
+            unsigned kept = pair_negate<AmpT>(d, rv, A, sneg, a0, a1, r0, r1);
+            kept = __reduce_add_sync(FULL, act ? kept : 0u);
             st.rdag += kept;
-            st.hph += kept; /* H P H: -1 here */
-            if (isext && act) {
-                const Row r = slot_row(units[ut], ws + ut * S, rotv + ut * S);
-                uint32_t slot;
-                const KeyT kt = map_t<KeyT>(d, r, key, slot, At, st_neg);
-                k_out = (uint32_t)(kt >> 1) & msk;
-                kc_out = (uint32_t)(kt >> (1 + d.nb)) & msk;
-                rt = At == 0 ? Amp<AmpT>::rot_zero()
-                             : (slot < (uint32_t)S ? rotv[ut * S + slot] : Amp<AmpT>::rot_table(d, At));
-            }
-            AmpT r0, r1;
-            Amp<AmpT>::rot(rt, At, false, st_neg, c0 ? Amp<AmpT>::neg(o0) : zero, c1 ? Amp<AmpT>::neg(o1) : zero,
-                           r0, r1); /* R */
+            st.hph += kept;
             const bool e0 = act && Amp<AmpT>::keep(d, r0), e1 = act && Amp<AmpT>::keep(d, r1);
             st.out += __popc(__ballot_sync(FULL, e0)) + __popc(__ballot_sync(FULL, e1));
             SlotOut<AmpT> outB, none;
@@ -2479,17 +2054,6 @@ struct PosStats {
     }
 };
 
-/* 1 for a non-zero amplitude (+-0 is zero), tested on the bits: an FP64
-   comparison would take a slot of the FP64 pipe */
-__device__ __forceinline__ unsigned int nz(float2 a)
-{
-    return ((__float_as_uint(a.x) | __float_as_uint(a.y)) << 1) != 0u ? 1u : 0u;
-}
-__device__ __forceinline__ unsigned int nz(double2 a)
-{
-    return (((uint64_t)__double_as_longlong(a.x) | (uint64_t)__double_as_longlong(a.y)) << 1) != 0ull ? 1u : 0u;
-}
-
 template <typename AmpT, int S, int PW>
 __global__ void __launch_bounds__(PW * 32, PosCfg<AmpT>::blocks / (S > 32 ? 2 : 1))
     k_walk_pos(QwSimDev d, const AmpT *__restrict__ pin, AmpT *__restrict__ pout, QwStepArgs a)
@@ -2621,21 +2185,19 @@ __global__ void __launch_bounds__(PW * 32, PosCfg<AmpT>::blocks / (S > 32 ? 2 : 
         AmpT rA0[SPL], rA1[SPL];
         bool eA0[SPL], eA1[SPL];
         {
-            AmpT o1[SPL], z0[SPL];
-            bool c1[SPL];
+            typename Amp<AmpT>::Wide u[SPL];
+            PairState<AmpT> ps[SPL];
+            float m[SPL];
 #pragma unroll
             for (int k = 0; k < SPL; ++k) {
-                AmpT o0;
-                Amp<AmpT>::rot(rv[k], val[k], true, sneg[k], a0[k], a1[k], o0, o1[k]);
-                const bool c0 = Amp<AmpT>::keep(d, o0);
-                c1[k] = Amp<AmpT>::keep(d, o1[k]);
-                st.rdag += (c0 ? 1u : 0u) + (c1[k] ? 1u : 0u);
-                z0[k] = c0 ? o0 : zero;
+                ps[k] = pair_tdag<AmpT>(d, rv[k], val[k], sneg[k], a0[k], a1[k], u[k], m[k]);
+                st.rdag += (ps[k].c0 ? 1u : 0u) + (ps[k].c1 ? 1u : 0u);
             }
+            __syncwarp();
             typename Amp<AmpT>::Sum sum;
-            sum.set(z0[0]);
+            sum.set(u[0]);
 #pragma unroll
-            for (int k = 1; k < SPL; ++k) sum.add(z0[k]);
+            for (int k = 1; k < SPL; ++k) sum.add(u[k]);
             sum.reduce(SW, SW);
             if (a.qls_readout && valid && lb == 0) {
                 const double2 sv = sum.value();
@@ -2645,13 +2207,12 @@ __global__ void __launch_bounds__(PW * 32, PosCfg<AmpT>::blocks / (S > 32 ? 2 : 
                 acc.y += coef * (d.inv_sqrt_s * sv.y);
                 a.qls_y[j] = acc;
             }
+            sum.scale_pow2(d.two_over_s);
 #pragma unroll
             for (int k = 0; k < SPL; ++k) {
-                const AmpT h0 = sum.scaled_minus(d.two_over_s, z0[k]);
-                const bool d0 = Amp<AmpT>::keep(d, h0);
-                st.hph += (d0 ? 1u : 0u) + (c1[k] ? 1u : 0u);
-                Amp<AmpT>::rot(rv[k], val[k], false, sneg[k], d0 ? h0 : zero, c1[k] ? Amp<AmpT>::neg(o1[k]) : zero,
-                               rA0[k], rA1[k]);
+                bool d0;
+                pair_reflect<AmpT>(d, sum, rv[k], val[k], sneg[k], a0[k], a1[k], u[k], m[k], ps[k], rA0[k], rA1[k], d0);
+                st.hph += (d0 ? 1u : 0u) + (ps[k].c1 ? 1u : 0u);
                 eA0[k] = Amp<AmpT>::keep(d, rA0[k]);
                 eA1[k] = Amp<AmpT>::keep(d, rA1[k]);
             }
@@ -2661,21 +2222,9 @@ __global__ void __launch_bounds__(PW * 32, PosCfg<AmpT>::blocks / (S > 32 ? 2 : 
 #pragma unroll
         for (int k = 0; k < SPL; ++k) {
             AmpT rB0, rB1;
-            AmpT o0, o1;
-            /* in the walk's reachable states the b2 = 1 member of a b1 = 1 pair
-               is 0: then R^dag takes half the products (same results).  Taken
-               on the FP64-pipe-bound complex128 path only: on complex64 the
-               vote and the second code path cost more than the products */
-            if (Amp<AmpT>::kB2ZeroPath && __all_sync(FULL, nz(q1[k]) == 0u))
-                Amp<AmpT>::rot_dag_b2zero(rv[k], val[k], sneg[k], q0[k], o0, o1);
-            else
-                Amp<AmpT>::rot(rv[k], val[k], true, sneg[k], q0[k], q1[k], o0, o1);
-            const bool c0 = Amp<AmpT>::keep(d, o0), c1 = Amp<AmpT>::keep(d, o1);
-            const unsigned int kept = (c0 ? 1u : 0u) + (c1 ? 1u : 0u);
+            const unsigned int kept = pair_negate<AmpT>(d, rv[k], val[k], sneg[k], q0[k], q1[k], rB0, rB1);
             st.rdag += kept;
             st.hph += kept;
-            Amp<AmpT>::rot(rv[k], val[k], false, sneg[k], c0 ? Amp<AmpT>::neg(o0) : zero,
-                           c1 ? Amp<AmpT>::neg(o1) : zero, rB0, rB1);
             const bool eB0 = Amp<AmpT>::keep(d, rB0), eB1 = Amp<AmpT>::keep(d, rB1);
             if (valid) {
                 const AmpT s0 = eA0[k] ? rA0[k] : zero, s1 = eB0 ? rB0 : zero;
@@ -3003,8 +2552,8 @@ __global__ void __launch_bounds__(WARPS * 32) k_tinit(QwSimDev d, QwBufDev buf, 
             m = d.s;
         }
         __syncwarp();
-        PairSink<AmpT, KeyT, false> s1(d, r, kQ, aQ, C, nullptr, nullptr, nullptr);
-        map_rot_pairs<1, AmpT, KeyT>(d, r, kP, aP, m, s1, hidx);
+        PairSink<AmpT, KeyT> s1(kQ, aQ, C);
+        map_rot_pairs<AmpT, KeyT>(d, r, kP, aP, m, s1, hidx);
         m = sink_count(s1, status);
         /* write back in place: the row keeps its registers (jc, j, b1) */
         for (int i = lane; i < m && i < d.cap_row; i += 32) {
