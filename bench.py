@@ -38,7 +38,7 @@ UNIT = "walk steps/s"
 PROFILE = os.path.join(ROOT, "profiles", "k_walk_n16384_s16.md")
 PROFILE_SLOT = os.path.join(ROOT, "profiles", "k_walk_slot_n16384_s16.md")
 PROFILE_POS = os.path.join(ROOT, "profiles", "k_walk_pos_n16384_s16.md")
-KERNEL_SRC = [os.path.join(ROOT, "paper_2303_06890_gb300", "csrc", f) for f in ("qw_kernels.cu", "qw_amp.cuh", "qw_device.cuh")]
+KERNEL_SRC = [os.path.join(ROOT, "paper_2303_06890_gb300", "csrc", f) for f in ("qw_kernels.cu", "qw_pos.cuh", "qw_amp.cuh", "qw_device.cuh")]
 L2_FLUSH_BYTES = 256 << 20
 
 

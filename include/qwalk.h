@@ -123,8 +123,11 @@ typedef struct {
                                 qw_state_export, qw_state_import or a register-faithful
                                 session; row_capacity grows to 2 s + 2 E (E: the most
                                 unpaired padded columns pointing at one row) */
-    int32_t graphs;          /* 1 (default): runs of >= 6 walk steps are issued as replays
-                                of a captured 6-step CUDA graph; 0: one launch per step */
+    int32_t graphs;          /* 1 (default): runs of walk steps are issued together -- in the
+                                positional layout as one cooperative launch of up to 1024
+                                steps whose blocks wait for one another between steps,
+                                otherwise as replays of a captured 6-step CUDA graph
+                                (runs of >= 6); 0: one launch per step */
     int32_t spill_rows;      /* slots of the table holding rows with jc != 0 (reached only
                                 from states outside the walk's physical subspace, e.g. by
                                 qw_state_import); a power of two, 0 = auto (2N/8 over all
@@ -189,8 +192,8 @@ int qw_state_init(qw_sim *sim, int32_t inst, const double *b_re, const double *b
 
 /*
  * Apply nsteps walk steps W = S T~ P T~^dag (Alg. "Quantum walk operator")
- * to every instance.  Each step is one launch over all rows; no host
- * synchronisation happens between steps.  The call synchronises once at the
+ * to every instance.  Each step runs over all rows at once, one launch a step
+ * or several (opts.graphs); no host synchronisation happens between steps.  The call synchronises once at the
  * end to read the device status word.  With overflow_fallback, steps that
  * outgrew the row buckets or the on-chip buffers are run again on the flat
  * path (then the call synchronises between those steps).
@@ -218,7 +221,9 @@ int qw_enqueue_walk_steps(qw_sim *sim, int64_t nsteps);
  * Synchronise the stream and read the device status word.  On a device
  * error the state is the output of the last step that completed cleanly
  * (later steps did nothing) and the error code is returned:
- * QW_ERR_CAPACITY, QW_ERR_DEVICE_STATUS or QW_ERR_CUDA.  With
+ * QW_ERR_CAPACITY, QW_ERR_DEVICE_STATUS or QW_ERR_CUDA.  (The positional layout
+ * has one error of its own, a launch whose blocks waited for one another too
+ * long: QW_ERR_DEVICE_STATUS, and the state is lost.)  With
  * overflow_fallback, steps enqueued since the last synchronising call that
  * outgrew the buckets are first run again on the flat path.
  */
@@ -264,8 +269,9 @@ int qw_cks_coefficients(double kappa, double eps, double *coeffs, int64_t cap, i
  * Y += coeffs[j] * Pi_0 tau_j for j = 0..j0.  Outputs: y_out (2 N doubles,
  * interleaved re/im) = Y; psucc_out (j0+1 doubles, nullable) =
  * || Pi_0 sum_{k<=j} coeffs[k] tau_k ||^2 for each j.  Three launches per
- * term (two walk steps, one norm); with opts.graphs, runs of 3 terms replay a
- * captured CUDA graph (the coefficient index lives on the device).
+ * term (two walk steps, one norm); with opts.graphs, the positional layout runs
+ * up to 512 terms in one launch, p_j included, and the other kernels replay a
+ * captured CUDA graph of 3 terms (the coefficient index lives on the device).
  * Errors: QW_ERR_ARG, QW_ERR_STATE, QW_ERR_CAPACITY, QW_ERR_CUDA.
  */
 int qw_apply_qls(qw_sim *sim, int32_t inst, const double *coeffs, int64_t j0, double *y_out,

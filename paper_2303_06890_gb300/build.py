@@ -13,7 +13,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libqwalk.so")
-SOURCES = ["qw_kernels.cu", "qw_flat.cu", "qw_api.cpp"]
+SOURCES = ["qw_kernels.cu", "qw_pos32.cu", "qw_pos64.cu", "qw_flat.cu", "qw_api.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -30,8 +30,8 @@ def _stale(out: str, deps: list[str]) -> bool:
 
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
-    headers = [os.path.join(CSRC, "qw_internal.h"), os.path.join(CSRC, "qw_device.cuh"), os.path.join(CSRC, "qw_amp.cuh"),
-               os.path.join(os.path.dirname(HERE), "include", "qwalk.h")]
+    headers = [os.path.join(CSRC, f) for f in ("qw_internal.h", "qw_device.cuh", "qw_amp.cuh", "qw_pos.cuh")]
+    headers.append(os.path.join(os.path.dirname(HERE), "include", "qwalk.h"))
     objs, procs = [], []
     for src in SOURCES:
         path = os.path.join(CSRC, src)

@@ -122,6 +122,14 @@ template <> struct Amp<double2> {
     __device__ static Wide rdag0(RotVal t, uint32_t A, bool sneg, T a0, T a1);
     __device__ static T narrow(Wide w) { return w; }
     __device__ static T sum_amp(const Sum &r) { return make_double2(r.x, r.y); }
+    /* t times 2^-e, exactly, by integer operations (f and g are 0 or far
+       above the subnormal range) */
+    __device__ static RotVal prescale(RotVal t, int e)
+    {
+        const int fh = __double2hiint(t.x), gh = __double2hiint(t.y);
+        return make_double2(__hiloint2double(fh ? fh - (e << 20) : 0, __double2loint(t.x)),
+                            __hiloint2double(gh ? gh - (e << 20) : 0, __double2loint(t.y)));
+    }
     __device__ static Wide wide_zero() { return make_double2(0.0, 0.0); }
     /* f r - a0 and g r - a1 (reflect_pair below) */
     __device__ static void reflect(const Sum &r, RotVal t, uint32_t A, bool sneg, T a0, T a1, T &o0, T &o1);
@@ -135,14 +143,36 @@ template <> struct Amp<double2> {
         return __uint_as_float((e << 3) | (hi & 0x80000000u));
     }
     __device__ static float2 approx2(T a) { return make_float2(approx(a.x), approx(a.y)); }
+    /* the larger of |x|, |y| in FP32: cut by at most 2^-20 relative, raised to
+       2^-126 where it is smaller, 0 for 0 */
+    __device__ static float inf_norm(T a)
+    {
+        const uint32_t m = max((uint32_t)__double2hiint(a.x) & 0x7fffffffu, (uint32_t)__double2hiint(a.y) & 0x7fffffffu);
+        const uint32_t e = min(max(m, 897u << 20) - (896u << 20), 0x0fefffffu);
+        return m ? __uint_as_float(e << 3) : 0.0f;
+    }
     __device__ static float rot_f(RotVal t) { return approx(t.x); }
     __device__ static float rot_g(RotVal t) { return approx(t.y); }
+    __device__ static void scale_one_plus(float c, double *buf) { buf[0] = 1.0 + (double)c; }
     static constexpr float kApproxErr = 1.0f / 131072.0f; /* 2^-17 of the terms' magnitudes */
 };
 
 /* complex64 path: amplitudes are float; each rotation output f a0 +- g a1 is
    formed from error-free products and an error-free sum on the FP32 pipe
    (f, g held as float pairs with ~48 significant bits) and rounded once. */
+/* a * s with s = sh + sl, rounded once (a call of its own: rarely taken) */
+__device__ __forceinline__ float mul_split(float a, float sh, float sl)
+{
+    const float p = __fmul_rn(sh, a);
+    float e = __fmaf_rn(sh, a, -p);
+    e = __fmaf_rn(sl, a, e);
+    return __fadd_rn(p, e);
+}
+__device__ __noinline__ float2 scale_c64(float2 a, float sh, float sl)
+{
+    return make_float2(mul_split(a.x, sh, sl), mul_split(a.y, sh, sl));
+}
+
 /* a complex value as float pairs hi + lo, hi = the value rounded to FP32 */
 struct WideF {
     float xh, xl, yh, yl;
@@ -263,26 +293,34 @@ template <> struct Amp<float2> {
     {
         return __fadd_rn(__fmul_rn(a.x, a.x), __fmul_rn(a.y, a.y)) > d.tau2f;
     }
-    /* a * s with s = sh + sl, rounded once */
-    __device__ static float mul_split(float a, float sh, float sl)
-    {
-        const float p = __fmul_rn(sh, a);
-        float e = __fmaf_rn(sh, a, -p);
-        e = __fmaf_rn(sl, a, e);
-        return __fadd_rn(p, e);
-    }
-    struct Scale { /* the FP64 factor as a float pair, applied with one rounding */
+    struct Scale { /* the FP64 factor as a float pair, applied with one rounding;
+                      within 2^-12 of 1 (always, but after an unusual pruning) as
+                      1 + sl, which takes one FMA */
         float sh, sl;
-        __device__ explicit Scale(double v) : sh((float)v), sl((float)(v - (double)(float)v)) {}
+        __device__ explicit Scale(double v) { split(v, sh, sl); }
         __device__ Scale(float h, float l) : sh(h), sl(l) {}
-        __device__ T apply(T a) const { return make_float2(mul_split(a.x, sh, sl), mul_split(a.y, sh, sl)); }
+        __device__ static void split(double v, float &h, float &l)
+        {
+            const double c = v - 1.0;
+            if (fabs(c) < 1.0 / 4096.0) {
+                h = 1.0f;
+                l = (float)c;
+            } else {
+                h = (float)v;
+                l = (float)(v - (double)h);
+            }
+        }
+        __device__ T apply(T a) const
+        {
+            if (sh == 1.0f) return make_float2(__fmaf_rn(a.x, sl, a.x), __fmaf_rn(a.y, sl, a.y));
+            return scale_c64(a, sh, sl);
+        }
         /* the split computed once per block (its FP64 conversions would
            otherwise take a slot of the 1/64-rate FP64 pipe in every thread) */
         __device__ static void to_shared(double v, double *buf)
         {
             float *f = reinterpret_cast<float *>(buf);
-            f[0] = (float)v;
-            f[1] = (float)(v - (double)(float)v);
+            split(v, f[0], f[1]);
         }
         __device__ static Scale from_shared(const double *buf)
         {
@@ -338,6 +376,11 @@ template <> struct Amp<float2> {
     __device__ static Wide rdag0(RotVal t, uint32_t A, bool sneg, T a0, T a1);
     __device__ static T narrow(Wide w) { return make_float2(w.xh, w.yh); }
     __device__ static T sum_amp(const Sum &r) { return make_float2(r.x.h, r.y.h); }
+    __device__ static RotVal prescale(RotVal t, int e)
+    {
+        const float c = __int_as_float((127 - e) << 23);
+        return make_float4(t.x * c, t.y * c, t.z * c, t.w * c);
+    }
     __device__ static Wide wide_zero() { return Wide{0.f, 0.f, 0.f, 0.f}; }
     __device__ static void reflect(const Sum &r, RotVal t, uint32_t A, bool sneg, T a0, T a1, T &o0, T &o1);
     /* round(F R - a), F = fh + fl, R = rh + rl */
@@ -353,8 +396,15 @@ template <> struct Amp<float2> {
         return __fadd_rn(s, __fadd_rn(t, e));
     }
     __device__ static float2 approx2(T a) { return a; }
+    __device__ static float inf_norm(T a) { return fmaxf(fabsf(a.x), fabsf(a.y)); }
     __device__ static float rot_f(RotVal t) { return t.x; }
     __device__ static float rot_g(RotVal t) { return t.z; }
+    __device__ static void scale_one_plus(float c, double *buf)
+    {
+        float *f = reinterpret_cast<float *>(buf);
+        f[0] = 1.0f;
+        f[1] = c;
+    }
     static constexpr float kApproxErr = 1.0f / 524288.0f; /* 2^-19 of the terms' magnitudes */
 };
 
@@ -568,26 +618,37 @@ __device__ __forceinline__ PairState<AmpT> pair_tdag(const QwSimDev &d, typename
     return p;
 }
 
-/* the pair after H P H and R, r: (2 / s) times the group's sum; d0: the
-   reflected b2 = 0 member is kept */
+/* the pair after H P H and R where the FP32 decision left the reflected b2 = 0
+   member open, or an intermediate was lost; returns whether it is kept */
+template <typename AmpT>
+__device__ __noinline__ bool pair_reflect_exact(const QwSimDev &d, typename Amp<AmpT>::Sum r,
+                                                typename Amp<AmpT>::RotVal t, uint32_t A, bool sneg, AmpT a0, AmpT a1,
+                                                PairState<AmpT> p, AmpT &r0, AmpT &r1)
+{
+    const AmpT u = p.c0 ? Amp<AmpT>::narrow(Amp<AmpT>::rdag0(t, A, sneg, a0, a1)) : Amp<AmpT>::zero();
+    AmpT h0 = r.minus(u);
+    const bool d0 = Amp<AmpT>::keep(d, h0);
+    if (p.lossy || (!d0 && nz(h0)))
+        pair_literal<AmpT>(d, t, A, sneg, a0, a1, p.c0, p.c1, true, d0 ? h0 : Amp<AmpT>::zero(), r0, r1);
+    else
+        Amp<AmpT>::reflect(r, t, A, sneg, a0, a1, r0, r1);
+    return d0;
+}
+
+/* the pair after H P H and R, r: (2 / s) times the group's sum, ux: the
+   pair's term of the sum, approximately; d0: the reflected b2 = 0 member is
+   kept */
 template <typename AmpT>
 __device__ __forceinline__ void pair_reflect(const QwSimDev &d, const typename Amp<AmpT>::Sum &r,
                                              typename Amp<AmpT>::RotVal t, uint32_t A, bool sneg, AmpT a0, AmpT a1,
-                                             typename Amp<AmpT>::Wide u, float m, const PairState<AmpT> &p, AmpT &r0,
-                                             AmpT &r1, bool &d0)
+                                             float2 ux, float m, const PairState<AmpT> &p, AmpT &r0, AmpT &r1,
+                                             bool &d0)
 {
-    const float2 rx = Amp<AmpT>::approx2(Amp<AmpT>::sum_amp(r)), ux = Amp<AmpT>::approx2(Amp<AmpT>::narrow(u));
+    const float2 rx = Amp<AmpT>::approx2(Amp<AmpT>::sum_amp(r));
     const float lim = fmaf(Amp<AmpT>::kApproxErr, m + sum_abs(rx), d.thr32);
     d0 = max_abs(rx.x - ux.x, rx.y - ux.y) > lim;
     Amp<AmpT>::reflect(r, t, A, sneg, a0, a1, r0, r1);
-    if (!d0 || p.lossy) {
-        AmpT h0 = r.minus(Amp<AmpT>::narrow(u));
-        d0 = Amp<AmpT>::keep(d, h0);
-        if (p.lossy || (!d0 && nz(h0))) {
-            if (!d0) h0 = Amp<AmpT>::zero();
-            pair_literal<AmpT>(d, t, A, sneg, a0, a1, p.c0, p.c1, true, h0, r0, r1);
-        }
-    }
+    if (!d0 || p.lossy) d0 = pair_reflect_exact<AmpT>(d, r, t, A, sneg, a0, a1, p, r0, r1);
 }
 
 } // namespace

@@ -140,22 +140,24 @@ struct qw_sim {
     FlatList fq;
     FaithCounts fq_counts;
     bool fq_open = false;
-    /* positional layout (walk_variant 7): tables, the three row arrays that
-       rotate like buf, and whether the state lives there */
-    uint16_t *pos_tp = nullptr;
-    uint32_t *pos_xin = nullptr;
-    uint16_t *pos_xcnt = nullptr;
-    uint32_t *pos_rowbase = nullptr;
+    /* positional layout (walk_variant 7): tables, the three state arrays, the
+       barrier words of its launches, and whether the state lives there */
+    uint32_t *pos_dst = nullptr;
+    uint32_t *pos_xptr = nullptr;
+    uint32_t *pos_xdst = nullptr;
+    std::vector<uint32_t> pos_xrow; /* extras before each instance's first row, and their number */
     uint16_t *pos_rowinst = nullptr;
     void *pbuf[3] = {nullptr, nullptr, nullptr};
     size_t pbuf_bytes = 0;
+    QwPosPlan pos_plan{};
+    unsigned long long *pos_words = nullptr; /* 4 barrier words, the poison flag, the p_j shares [2][grid] */
+    unsigned long long pos_epoch = 1; /* of the next step's barrier */
+    bool pos_issued = false; /* positional steps issued since the last synchronising call */
     bool pos_built = false;
     bool pos_live = false; /* the state is pbuf[cur], not buf[cur] */
+    bool pos_full = false; /* it has branches with b1 = b2 = 1 (imported states only) */
     bool pos_try = true;   /* the bucket state may have positions (unknown or yes) */
-    int grid_pos = 1;
     int mode_alt = QW_MODE_WALK_FUSED, grid_alt = 1; /* the bucket kernel for a state without positions */
-    cudaGraphExec_t pexec[3][2] = {{nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}};
-    cudaGraphExec_t pqexec[3][2] = {{nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}};
     std::string err;
 };
 
@@ -168,10 +170,11 @@ static bool host_staged(const qw_sim *sim)
 
 static const int kGraphSteps = 6; /* a multiple of the 3-buffer and 2-slot periods */
 static const int kGraphTerms = 3;  /* QLS terms per graph: 2 walk steps each */
+static const int64_t kPosSteps = 1024; /* walk steps of one positional launch: a few milliseconds */
 
 static void drop_graphs(qw_sim *sim)
 {
-    for (auto *set : {&sim->gexec, &sim->qexec, &sim->pexec, &sim->pqexec})
+    for (auto *set : {&sim->gexec, &sim->qexec})
         for (auto &row : *set)
             for (auto &g : row)
                 if (g) {
@@ -570,7 +573,7 @@ extern "C" int qw_sim_create(const qw_csc *mats, int32_t ninst, const qw_sim_opt
         for (int m : {QW_MODE_WALK_FUSED, QW_MODE_WALK_FUSED_PF, QW_MODE_WALK_SEG, QW_MODE_WALK_SEG_PF})
             gmax = std::max(gmax, qw_step_grid(d, sim->fp32, m));
         if (qw_slot_supported(d)) gmax = std::max(gmax, qw_step_grid(d, sim->fp32, QW_MODE_WALK_SLOT));
-        if (qw_pos_supported(d) && ninst == 1) gmax = std::max(gmax, qw_pos_grid(d, sim->fp32));
+        gmax = std::max(gmax, qw_sm_count()); /* the positional kernel: one block per SM */
     }
     QW_TRY(dalloc(sim, &sim->partials, (size_t)gmax));
     sim->partials_cap = gmax;
@@ -618,11 +621,11 @@ extern "C" int qw_sim_destroy(qw_sim *sim)
     if (sim->stream) cudaStreamSynchronize(sim->stream);
     else cudaDeviceSynchronize();
     if (sim->fpool) cudaMemPoolDestroy(sim->fpool);
-    cudaFree(sim->pos_tp);
-    cudaFree(sim->pos_xin);
-    cudaFree(sim->pos_xcnt);
-    cudaFree(sim->pos_rowbase);
+    cudaFree(sim->pos_dst);
+    cudaFree(sim->pos_xdst);
     cudaFree(sim->pos_rowinst);
+    cudaFree(sim->pos_xptr);
+    cudaFree(sim->pos_words);
     for (void *p : sim->pbuf) cudaFree(p);
     cudaFree(sim->img);
     cudaFree(sim->fg);
@@ -695,6 +698,8 @@ static int check_status(qw_sim *sim, const char *where)
     const int64_t good = h.done - sim->sync_done;
     sim->last_good = good;
     sim->issued = 0;
+    const bool pos_issued = sim->pos_issued;
+    sim->pos_issued = false;
     if (h.status != 0) {
         sim->cur = (int)((sim->sync_cur + good) % 3);
         sim->scale_slot = sim->sync_slot ^ (int)(good & 1);
@@ -715,6 +720,13 @@ static int check_status(qw_sim *sim, const char *where)
     if (st & QW_ST_NOT_BTILDE) m += " [a row was not |b~> before T~]";
     if (st & QW_ST_OUTBOX_FULL) m += " [an outbox toward another partition is full: raise outbox_capacity]";
     if (st & QW_ST_SORT_WAIT) m += " [the flat path's radix sort gave up waiting for a tile's count]";
+    if (st & QW_ST_GRID_WAIT) m += " [a positional step gave up waiting for the other blocks]";
+    if (pos_issued) { /* several steps share the arrays: no clean one to go back to */
+        sim->has_state = sim->pos_live = false;
+        cudaMemsetAsync(sim->pos_words, 0, 5 * sizeof(unsigned long long), sim->stream);
+        cudaStreamSynchronize(sim->stream);
+        return fail(sim, QW_ERR_DEVICE_STATUS, m + "; the state is lost: initialise it again");
+    }
     m += "; state kept after " + std::to_string(good) + " clean steps since the last sync";
     const int code = (st & (QW_ST_ROW_OVERFLOW | QW_ST_WARP_OVERFLOW | QW_ST_SPILL_FULL | QW_ST_OUTBOX_FULL))
                          ? QW_ERR_CAPACITY
@@ -739,6 +751,7 @@ static QwStepArgs step_args(qw_sim *sim, int mode)
     a.qls_y = sim->qls_y;
     a.qls_coefs = sim->qls_c;
     a.qls_j = &sim->sc->qls_j;
+    a.qls_p = sim->qls_p;
     a.deferred = sim->deferred;
     a.deferred_ctr = &sim->sc->deferred_ctr;
     a.work_ctr = &sim->sc->work_ctr;
@@ -750,6 +763,44 @@ static int faithful_walk_step(qw_sim *sim, int readout);
 static int pos_unpack(qw_sim *sim);
 static int sync_walk(qw_sim *sim, const char *where);
 
+/* nsteps positional steps in one launch (several: a cooperative launch whose
+ * blocks wait for one another); qls_term >= 0: they are QLS terms of two steps
+ * from that one on, otherwise readout applies to the (one) step */
+static int launch_pos(qw_sim *sim, int64_t nsteps, int64_t qls_term, int readout)
+{
+    QwStepArgs a = step_args(sim, QW_MODE_WALK_POS);
+    a.qls_readout = readout;
+    QwPosArgs p{};
+    p.in = sim->pbuf[sim->cur];
+    p.out0 = sim->pbuf[(sim->cur + 1) % 3];
+    p.out1 = sim->pbuf[(sim->cur + 2) % 3];
+    p.nsteps = (int)nsteps;
+    p.qls = qls_term >= 0;
+    p.qls_term = qls_term;
+    if (nsteps > 1) {
+        p.epoch = sim->pos_epoch;
+        p.words = sim->pos_words;
+        p.poison = reinterpret_cast<unsigned int *>(sim->pos_words + 4);
+        p.pshare = reinterpret_cast<double *>(sim->pos_words + 5);
+        sim->pos_epoch += (unsigned long long)nsteps;
+    }
+    const cudaError_t e = qw_launch_walk_pos(sim->d, sim->pos_plan, p, a, sim->fp32, sim->pos_full, sim->stream);
+    sim->launches++;
+    sim->issued += nsteps;
+    sim->pos_issued = true;
+    if (e != cudaSuccess) return cuda_fail(sim, e, "walk step launch");
+    sim->cur = (sim->cur + (nsteps & 1 ? 1 : 2)) % 3;
+    sim->scale_slot ^= 1;
+    return QW_OK;
+}
+
+/* whether runs of positional steps go out as one launch */
+static bool pos_runs(const qw_sim *sim, bool capturing)
+{
+    return sim->mode == QW_MODE_WALK_POS && sim->pos_live && sim->opts.graphs && sim->pos_plan.coop &&
+           !sim->pos_full && !capturing;
+}
+
 /* one walk step: X_cur -> X_cur+1, clearing X_cur+2 */
 static int launch_walk(qw_sim *sim, int readout)
 {
@@ -757,15 +808,11 @@ static int launch_walk(qw_sim *sim, int readout)
     if (sim->mode == QW_MODE_WALK_FAITHFUL) return faithful_walk_step(sim, readout);
     if (sim->d.nparts > 1) /* the outboxes hold this step's sends only */
         QW_CUDA(sim, cudaMemsetAsync(sim->outbox_count, 0, (size_t)sim->d.nparts * 8, sim->stream));
+    if (sim->mode == QW_MODE_WALK_POS && sim->pos_live) return launch_pos(sim, 1, -1, readout);
     sim->issued++;
     const int nxt = (sim->cur + 1) % 3, clr = (sim->cur + 2) % 3;
     cudaError_t e;
-    if (sim->mode == QW_MODE_WALK_POS && sim->pos_live) {
-        QwStepArgs a = step_args(sim, QW_MODE_WALK_POS);
-        a.qls_readout = readout;
-        e = qw_launch_walk_pos(sim->d, sim->pbuf[sim->cur], sim->pbuf[nxt], a, sim->fp32, sim->grid_pos,
-                               sim->stream);
-    } else { /* a positional walk whose state has no positions runs the bucket kernel */
+    { /* a positional walk whose state has no positions runs the bucket kernel */
         const int mode = sim->mode == QW_MODE_WALK_POS ? sim->mode_alt : sim->mode;
         QwStepArgs a = step_args(sim, mode);
         a.qls_readout = readout;
@@ -1088,11 +1135,11 @@ static int flat_walk_step(qw_sim *sim, int readout)
 
 /* ---- positional layout (walk_variant 7, k_walk_pos) ------------------------ */
 
-/* The tables of the positional layout from the QRAM image: for slot (j, l)
- * with column c, the position of the branch k = j in row c -- 2 l' when row
- * c holds column j in slot l', else 2 s + 2 e for the e-th such row x of c
- * (listed in pos_xin) -- and the three row arrays.  The row buckets grow to
- * hold a whole positional row (2 s + 2 E branches). */
+/* The tables of the positional layout (qw_pos.cuh) from the QRAM image --
+ * pos_dst: for slot (j, l) with column c, the entry of the branch k = j in row
+ * c, slot l' where row c holds column j there, else an extra of row c -- the
+ * three state arrays and the barrier words.  The row buckets grow to hold a whole positional row (2 s +
+ * 2 E branches). */
 static int pos_build(qw_sim *sim)
 {
     if (sim->pos_built) return QW_OK;
@@ -1110,19 +1157,16 @@ static int pos_build(qw_sim *sim)
     }
     std::vector<uint32_t> img((size_t)nrows * s);
     QW_CUDA(sim, cudaMemcpy(img.data(), sim->img, img.size() * 4, cudaMemcpyDeviceToHost));
-    std::vector<uint16_t> tp((size_t)nrows * s);
-    std::vector<std::vector<uint32_t>> xin((size_t)nrows);
-    std::vector<uint32_t> rowbase(ninst > 1 ? (size_t)nrows : 0);
+    std::vector<uint32_t> dst((size_t)nrows * s);
+    std::vector<std::vector<uint32_t>> xin((size_t)nrows); /* the slots (x, l_x) of each row's extras */
     std::vector<uint16_t> rowinst(ninst > 1 ? (size_t)nrows : 0);
     for (int i = 0; i < ninst; ++i) {
         const int64_t g0 = row0[(size_t)i], n = sim->n_of[(size_t)i];
         for (int64_t j = 0; j < n; ++j) {
-            if (ninst > 1) {
-                rowbase[(size_t)(g0 + j)] = (uint32_t)g0;
-                rowinst[(size_t)(g0 + j)] = (uint16_t)i;
-            }
+            if (ninst > 1) rowinst[(size_t)(g0 + j)] = (uint16_t)i;
             for (int l = 0; l < s; ++l) {
-                const uint32_t c = img[(size_t)((g0 + j) * s + l)] >> 16;
+                const size_t at = (size_t)((g0 + j) * s + l);
+                const uint32_t c = img[at] >> 16;
                 const uint32_t *row = img.data() + (size_t)(g0 + c) * s;
                 int lo = 0, hi = s;
                 while (lo < hi) {
@@ -1130,67 +1174,64 @@ static int pos_build(qw_sim *sim)
                     if ((row[m] >> 16) < (uint32_t)j) lo = m + 1;
                     else hi = m;
                 }
-                auto &xc = xin[(size_t)(g0 + c)];
-                if (lo < s && (row[lo] >> 16) == (uint32_t)j) {
-                    tp[(size_t)((g0 + j) * s + l)] = (uint16_t)(2 * lo);
-                } else {
-                    tp[(size_t)((g0 + j) * s + l)] = (uint16_t)(2 * s + 2 * xc.size());
-                    xc.push_back((uint32_t)(g0 + j) << 8 | (uint32_t)l);
-                }
+                if (lo < s && (row[lo] >> 16) == (uint32_t)j)
+                    dst[at] = (uint32_t)((g0 + c) * s + lo) | (j > (int64_t)c ? 0x80000000u : 0u);
+                else
+                    xin[(size_t)(g0 + c)].push_back((uint32_t)at);
             }
         }
     }
-    size_t E = 0;
-    for (const auto &v : xin) E = std::max(E, v.size());
-    const int64_t R = 2 * s + 2 * (int64_t)E;
+    size_t E = 0, X = 0;
+    for (const auto &v : xin) {
+        E = std::max(E, v.size());
+        X += v.size();
+    }
+    const int64_t R = 2 * s + 2 * (int64_t)E, T = nrows * s + (int64_t)X;
     if (R >= 65535 || nrows >= (1 << 24) || 2 * nrows * R >= ((int64_t)1 << 31))
         return fail(sim, QW_ERR_ARG, "positional layout: too many unpaired padded columns in a row, or rows");
-    std::vector<uint32_t> hx((size_t)nrows * std::max<size_t>(E, 1), 0u);
-    std::vector<uint16_t> hc((size_t)nrows);
-    for (int64_t c = 0; c < nrows; ++c) {
-        hc[(size_t)c] = (uint16_t)xin[(size_t)c].size();
-        for (size_t e = 0; e < xin[(size_t)c].size(); ++e) hx[(size_t)c * E + e] = xin[(size_t)c][e];
+    std::vector<uint32_t> xptr((size_t)nrows + 1, 0u), xdst(std::max<size_t>(X, 1), 0u);
+    for (int64_t c = 0, e = 0; c < nrows; ++c) {
+        xptr[(size_t)c] = (uint32_t)e;
+        for (uint32_t at : xin[(size_t)c]) {
+            const int64_t x = at / (uint32_t)s; /* slot `at` of row x sends its outputs to the extra */
+            dst[at] = (uint32_t)(nrows * s + e) | (x > c ? 0x80000000u : 0u);
+            xdst[(size_t)e++] = at;
+        }
     }
+    xptr[(size_t)nrows] = (uint32_t)X;
+    sim->pos_xrow.assign((size_t)ninst + 1, (uint32_t)X);
+    for (int i = 0; i < ninst; ++i) sim->pos_xrow[(size_t)i] = xptr[(size_t)row0[(size_t)i]];
     if (d.cap_row < R) {
         const int rc = grow_rows(sim, R);
         if (rc != QW_OK) return rc;
     }
-    QW_CUDA(sim, dalloc(sim, &sim->pos_tp, tp.size()));
-    QW_CUDA(sim, dalloc(sim, &sim->pos_xin, hx.size()));
-    QW_CUDA(sim, dalloc(sim, &sim->pos_xcnt, hc.size()));
-    QW_CUDA(sim, cudaMemcpy(sim->pos_tp, tp.data(), tp.size() * 2, cudaMemcpyHostToDevice));
-    QW_CUDA(sim, cudaMemcpy(sim->pos_xin, hx.data(), hx.size() * 4, cudaMemcpyHostToDevice));
-    QW_CUDA(sim, cudaMemcpy(sim->pos_xcnt, hc.data(), hc.size() * 2, cudaMemcpyHostToDevice));
+    QW_CUDA(sim, dalloc(sim, &sim->pos_dst, dst.size()));
+    QW_CUDA(sim, dalloc(sim, &sim->pos_xptr, xptr.size()));
+    QW_CUDA(sim, dalloc(sim, &sim->pos_xdst, xdst.size()));
+    QW_CUDA(sim, cudaMemcpy(sim->pos_dst, dst.data(), dst.size() * 4, cudaMemcpyHostToDevice));
+    QW_CUDA(sim, cudaMemcpy(sim->pos_xptr, xptr.data(), xptr.size() * 4, cudaMemcpyHostToDevice));
+    QW_CUDA(sim, cudaMemcpy(sim->pos_xdst, xdst.data(), xdst.size() * 4, cudaMemcpyHostToDevice));
     if (ninst > 1) {
-        QW_CUDA(sim, dalloc(sim, &sim->pos_rowbase, rowbase.size()));
         QW_CUDA(sim, dalloc(sim, &sim->pos_rowinst, rowinst.size()));
-        QW_CUDA(sim, cudaMemcpy(sim->pos_rowbase, rowbase.data(), rowbase.size() * 4, cudaMemcpyHostToDevice));
         QW_CUDA(sim, cudaMemcpy(sim->pos_rowinst, rowinst.data(), rowinst.size() * 2, cudaMemcpyHostToDevice));
     }
-    sim->pbuf_bytes = (size_t)2 * (size_t)nrows * (size_t)R * (sim->fp32 ? sizeof(float2) : sizeof(double2));
+    sim->pbuf_bytes = 4 * (size_t)T * (sim->fp32 ? sizeof(float2) : sizeof(double2));
     for (auto &p : sim->pbuf) {
         unsigned char *b = nullptr;
         QW_CUDA(sim, dalloc(sim, &b, sim->pbuf_bytes));
         QW_CUDA(sim, cudaMemset(b, 0, sim->pbuf_bytes));
         p = b;
     }
-    d.pos_R = (int)R;
-    d.pos_E = (int)E;
     d.pos_rows = nrows;
-    d.pos_tp = sim->pos_tp;
-    d.pos_xin = sim->pos_xin;
-    d.pos_xcnt = sim->pos_xcnt;
-    d.pos_rowbase = sim->pos_rowbase;
+    d.pos_T = T;
+    d.pos_dst = sim->pos_dst;
+    d.pos_xptr = sim->pos_xptr;
+    d.pos_xdst = sim->pos_xdst;
     d.pos_rowinst = sim->pos_rowinst;
-    sim->grid_pos = qw_pos_grid(d, sim->fp32);
-    if (sim->grid_pos > sim->partials_cap) { /* one norm partial per block */
-        drop_graphs(sim); /* they hold the old array */
-        cudaFree(sim->partials);
-        sim->partials = nullptr;
-        sim->partials_cap = 0;
-        QW_CUDA(sim, dalloc(sim, &sim->partials, (size_t)sim->grid_pos));
-        sim->partials_cap = sim->grid_pos;
-    }
+    sim->pos_plan = qw_pos_plan(d, sim->fp32);
+    const size_t words = 5 + 2 * (size_t)sim->pos_plan.grid;
+    QW_CUDA(sim, dalloc(sim, &sim->pos_words, words));
+    QW_CUDA(sim, cudaMemset(sim->pos_words, 0, words * sizeof(unsigned long long)));
     sim->mode_alt = d.warp_cap < 2 * d.cap_row ? QW_MODE_WALK_FUSED
                     : (qw_slot_supported(d) ? QW_MODE_WALK_SLOT : QW_MODE_WALK_SEG);
     sim->grid_alt = qw_step_grid(d, sim->fp32, sim->mode_alt);
@@ -1209,13 +1250,18 @@ static int pos_pack(qw_sim *sim)
     sim->launches++;
     QW_CUDA(sim, cudaMemcpyAsync(sim->h_st, &sim->sc->status, sizeof(StatusView), cudaMemcpyDeviceToHost, st));
     QW_CUDA(sim, cudaStreamSynchronize(st));
-    if (sim->h_st->status == QW_ST_POS_UNREP) {
+    if (sim->h_st->status & QW_ST_POS_UNREP) {
         const int32_t zero = 0;
         QW_CUDA(sim, cudaMemcpy(&sim->sc->status, &zero, 4, cudaMemcpyHostToDevice));
         sim->pos_try = false;
         return QW_OK;
     }
-    if (sim->h_st->status != 0) return check_status(sim, "positional layout");
+    sim->pos_full = (sim->h_st->status & QW_ST_POS_FULL) != 0;
+    if (sim->h_st->status & ~QW_ST_POS_FULL) return check_status(sim, "positional layout");
+    if (sim->pos_full) {
+        const int32_t zero = 0;
+        QW_CUDA(sim, cudaMemcpy(&sim->sc->status, &zero, 4, cudaMemcpyHostToDevice));
+    }
     sim->pos_live = true;
     return QW_OK;
 }
@@ -1229,7 +1275,7 @@ static int pos_unpack(qw_sim *sim)
     if (!sim->pos_live) return QW_OK;
     for (const QwBufDev &b : sim->buf)
         QW_CUDA(sim, qw_launch_clear(sim->d, b, 0, sim->d.total_buckets, 1, sim->stream));
-    QW_CUDA(sim, qw_launch_pos_unpack(sim->d, sim->pbuf[sim->cur], sim->buf[sim->cur], sim->fp32, &sim->sc->status,
+    QW_CUDA(sim, qw_launch_pos_unpack(sim->d, sim->pbuf[sim->cur], sim->pos_full, sim->buf[sim->cur], sim->fp32, &sim->sc->status,
                                       sim->stream));
     sim->launches += 4;
     sim->pos_live = false;
@@ -1504,7 +1550,16 @@ extern "C" int qw_state_init(qw_sim *sim, int32_t inst, const double *b_re, cons
     if (pos_init) {
         int64_t g0 = 0;
         for (int i = 0; i < inst; ++i) g0 += sim->n_of[(size_t)i];
-        QW_CUDA(sim, qw_launch_tinit_pos(sim->d, sim->pbuf[sim->cur], g0, n, dre, dim,
+        const int64_t x0 = sim->pos_xrow[(size_t)inst], nx = sim->pos_xrow[(size_t)inst + 1] - x0;
+        if (all) {
+            sim->pos_full = false;
+        } else if (sim->pos_full) { /* the instance has no b1 = b2 = 1 branches now */
+            const size_t amp = sim->fp32 ? sizeof(float2) : sizeof(double2), s = (size_t)sim->d.s;
+            unsigned char *B1 = static_cast<unsigned char *>(sim->pbuf[sim->cur]) + 3 * (size_t)sim->d.pos_T * amp;
+            QW_CUDA(sim, cudaMemsetAsync(B1 + (size_t)g0 * s * amp, 0, (size_t)n * s * amp, sim->stream));
+            QW_CUDA(sim, cudaMemsetAsync(B1 + ((size_t)sim->d.pos_rows * s + x0) * amp, 0, (size_t)nx * amp, sim->stream));
+        }
+        QW_CUDA(sim, qw_launch_tinit_pos(sim->d, sim->pbuf[sim->cur], g0, n, x0, nx, dre, dim,
                                          all ? nullptr : pending_scale(sim), sim->fp32, sim->stream));
         sim->launches++;
         sim->pos_live = true;
@@ -1602,8 +1657,16 @@ extern "C" int qw_enqueue_walk_steps(qw_sim *sim, int64_t nsteps)
         const int rc = pos_prepare(sim);
         if (rc != QW_OK) return rc;
     }
-    if (sim->opts.graphs && !host_staged(sim) && sim->d.nparts == 1 && nsteps >= kGraphSteps && !capturing) {
-        cudaGraphExec_t &g = (sim->pos_live ? sim->pexec : sim->gexec)[sim->cur][sim->scale_slot];
+    if (pos_runs(sim, capturing)) {
+        while (t < nsteps) {
+            const int64_t m = std::min(nsteps - t, kPosSteps);
+            const int rc = launch_pos(sim, m, -1, 0);
+            if (rc != QW_OK) return rc;
+            t += m;
+        }
+    } else if (sim->opts.graphs && !sim->pos_live && !host_staged(sim) && sim->d.nparts == 1 &&
+               nsteps >= kGraphSteps && !capturing) {
+        cudaGraphExec_t &g = sim->gexec[sim->cur][sim->scale_slot];
         if (!g) {
             int rc = capture_graph(sim, &g, false);
             if (rc != QW_OK) return rc;
@@ -1685,12 +1748,13 @@ extern "C" int qw_autotune(qw_sim *sim, int32_t steps, int32_t *choice, double *
     QW_CUDA(sim, cudaEventCreate(&e1));
     int rc = QW_OK;
     const int graphs = sim->opts.graphs;
-    sim->opts.graphs = 0; /* time the kernels themselves */
+    /* time the kernels themselves; the positional layout as it will run */
     for (size_t c = 0; c < cand.size() && rc == QW_OK; ++c) {
         const int v = cand[c].first, mode = cand[c].second;
         if (mode != QW_MODE_WALK_POS) rc = pos_unpack(sim);
         if (rc != QW_OK) break;
         sim->mode = mode;
+        sim->opts.graphs = mode == QW_MODE_WALK_POS ? graphs : 0;
         sim->grid_walk = mode == QW_MODE_WALK_POS ? sim->grid_alt : qw_step_grid(sim->d, sim->fp32, mode);
         if (mode == QW_MODE_WALK_POS) { /* the move into the layout is not timed */
             rc = pos_prepare(sim);
@@ -1801,11 +1865,16 @@ extern "C" int qw_apply_qls(qw_sim *sim, int32_t inst, const double *coeffs, int
         const int rc = pos_prepare(sim);
         if (rc != QW_OK) return rc;
     }
-    const bool graphs = sim->opts.graphs && !host_staged(sim) && !capturing;
+    const bool graphs = sim->opts.graphs && !sim->pos_live && !host_staged(sim) && !capturing;
     int64_t j = 0, next_check = 1024;
     while (j <= j0) {
-        if (graphs && j0 + 1 - j >= kGraphTerms) {
-            cudaGraphExec_t &g = (sim->pos_live ? sim->pqexec : sim->qexec)[sim->cur][sim->scale_slot];
+        if (pos_runs(sim, capturing)) {
+            const int64_t m = std::min(j0 + 1 - j, kPosSteps / 2);
+            const int rc = launch_pos(sim, 2 * m, j, 0);
+            if (rc != QW_OK) return rc;
+            j += m;
+        } else if (graphs && j0 + 1 - j >= kGraphTerms) {
+            cudaGraphExec_t &g = sim->qexec[sim->cur][sim->scale_slot];
             if (!g) {
                 int rc = capture_graph(sim, &g, true);
                 if (rc != QW_OK) return rc;
@@ -1858,7 +1927,7 @@ extern "C" int qw_measure_register(qw_sim *sim, int32_t inst, int32_t reg, doubl
     double *dp = sim->meas_dev;
     QW_CUDA(sim, cudaMemsetAsync(dp, 0, (size_t)len * sizeof(double), sim->stream));
     if (sim->pos_live) /* read the positional layout in place */
-        QW_CUDA(sim, qw_launch_measure_pos(sim->d, sim->pbuf[sim->cur], pos_row0(sim, inst), sim->n_of[(size_t)inst],
+        QW_CUDA(sim, qw_launch_measure_pos(sim->d, sim->pbuf[sim->cur], sim->pos_full, pos_row0(sim, inst), sim->n_of[(size_t)inst],
                                            sim->fp32, pending_scale(sim), reg, dp, len, sim->stream));
     else
         QW_CUDA(sim, qw_launch_measure(sim->d, sim->buf[sim->cur], inst, sim->fp32, pending_scale(sim), reg,
@@ -1887,7 +1956,7 @@ extern "C" int qw_measure_register_noalloc(qw_sim *sim, int32_t inst, int32_t re
     if (!sim->has_state) return fail(sim, QW_ERR_STATE, "no state");
     QW_CUDA(sim, qw_launch_measure_noalloc(sim->d, sim->buf[sim->cur], inst, sim->fp32, pending_scale(sim),
                                            reg, probs, len, sim->device, sim->stream,
-                                           sim->pos_live ? sim->pbuf[sim->cur] : nullptr, pos_row0(sim, inst),
+                                           sim->pos_live ? sim->pbuf[sim->cur] : nullptr, sim->pos_full, pos_row0(sim, inst),
                                            sim->n_of[(size_t)inst]));
     sim->launches++;
     return check_status(sim, "qw_measure_register_noalloc");

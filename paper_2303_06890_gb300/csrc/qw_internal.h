@@ -40,6 +40,8 @@
 #define QW_ST_OUTBOX_FULL 32   /* a partition's outbox toward another overflowed */
 #define QW_ST_POS_UNREP 64     /* a branch the positional layout has no position for */
 #define QW_ST_SORT_WAIT 128    /* the flat path's radix sort gave up waiting for a tile's count */
+#define QW_ST_POS_FULL 256     /* a packed state has branches with b1 = b2 = 1 (pos_pack) */
+#define QW_ST_GRID_WAIT 512    /* a positional step gave up waiting for the other blocks */
 
 /* A branch sent by S to a row another partition owns: its row key
    (qw_rowkey), its local registers (R layout) and its amplitude in FP64. */
@@ -103,20 +105,18 @@ struct QwSimDev {
     QwPartEntry *outbox;
     unsigned long long *outbox_count;
     int64_t outbox_cap;
-    /* positional layout: the rows j < N of all instances in order, row g
-       (instance i, g = inst_img[i] / s + j) of pos_rows; row (g, b1) is
-       pos_R = 2 s + 2 pos_E amplitudes at (2 g + b1) pos_R.  pos_tp[g s + l]:
-       the position of the branch k = j in row col(j, l) of the instance;
-       pos_xin[g pos_E + e] = x << 8 | l for the e-th row x (global) < pos_xcnt[g]
-       whose slot l holds column j while row j holds no column x;
-       pos_rowbase[g] / pos_rowinst[g]: the first row and the instance of
-       row g's instance (null with one instance) */
-    int pos_R, pos_E;
-    int64_t pos_rows;
-    const uint16_t *pos_tp;
-    const uint32_t *pos_xin;
-    const uint16_t *pos_xcnt;
-    const uint32_t *pos_rowbase;
+    /* positional layout (qw_pos.cuh): the rows j < N of all instances in order,
+       row g (instance i, g = inst_img[i] / s + j) of pos_rows; entries g s + l
+       (slot l of row g), then the extras of row g at pos_rows s + pos_xptr[g] ..
+       pos_xptr[g + 1], pos_T entries in all; pos_dst[g s + l]: the entry of the
+       branch k = j in row col(j, l) of the instance, bit 31: j > col(j, l);
+       pos_xdst[e]: the slot (x, l_x) of extra e of row j, whose column is j
+       while row j holds no column x; pos_rowinst[g]: the instance of row g
+       (null with one) */
+    int64_t pos_rows, pos_T;
+    const uint32_t *pos_dst;
+    const uint32_t *pos_xptr;
+    const uint32_t *pos_xdst;
     const uint16_t *pos_rowinst;
 };
 
@@ -143,12 +143,34 @@ struct QwStepArgs {
     double2 *qls_y;          /* flag-0 accumulator (nullable) */
     const double *qls_coefs; /* Y += qls_coefs[*qls_j] * Pi_0 tau at this step's midpoint */
     const int64_t *qls_j;    /* index of the current QLS term (advanced by k_qls_norm) */
+    double *qls_p;           /* p_j (written by the positional kernel's own terms) */
     int qls_readout;
     int32_t *deferred;          /* slot kernel: units left to the row pipeline (dense unit u,
                                    or 0x80000000 | garbage-row slot), run by the last block */
     unsigned int *deferred_ctr; /* entries in deferred (reset by the last block) */
     unsigned int *work_ctr;     /* slot kernel: groups claimed beyond each warp's first
                                    (reset by the last block) */
+};
+
+/* positional steps: one launch runs nsteps of them, in -> out0 -> out1 -> out0
+   ...; with words, blocks wait for one another between steps (a cooperative
+   launch), otherwise nsteps is 1 */
+struct QwPosArgs {
+    const void *in;
+    void *out0, *out1;
+    int nsteps;
+    int qls;                  /* QLS terms of two steps, read out on the second */
+    int64_t qls_term;         /* index of the first */
+    unsigned long long epoch; /* of the first step: its barrier word is words[epoch & 3] */
+    unsigned long long *words; /* the barrier's 4 words, or null */
+    unsigned int *poison;     /* set when a block's norm share is not finite */
+    double *pshare;           /* [2][grid]: the blocks' shares of p_j */
+};
+struct QwPosPlan {
+    int grid, warps; /* blocks, warps a block */
+    int tab;         /* the matrix's tables fit shared memory */
+    int coop;        /* the device takes cooperative launches */
+    size_t smem;
 };
 
 /* launchers (qw_kernels.cu); all return cudaGetLastError() of the launch */
@@ -162,24 +184,61 @@ int qw_slot_supported(const QwSimDev &d);
 int qw_pos_supported(const QwSimDev &d);
 /* dynamic shared memory per block of the step kernel of `mode` */
 size_t qw_step_smem_bytes(const QwSimDev &d, int fp32, int mode);
-/* positional layout: one walk step pin -> pout (both pos_R-strided row
-   arrays), the grid of its launch, and the conversions from and to the row
-   buckets (pack: pout zeroed by the caller; a branch without a position sets
-   QW_ST_POS_UNREP; unpack: the buckets cleared by the caller) */
-cudaError_t qw_launch_walk_pos(const QwSimDev &d, const void *pin, void *pout, const QwStepArgs &a, int fp32,
-                               int grid, cudaStream_t st);
-int qw_pos_grid(const QwSimDev &d, int fp32);
-cudaError_t qw_launch_pos_pack(const QwSimDev &d, const QwBufDev &buf, void *pbuf, int fp32, int32_t *status,
-                               cudaStream_t st);
-cudaError_t qw_launch_pos_unpack(const QwSimDev &d, const void *pbuf, const QwBufDev &buf, int fp32,
-                                 int32_t *status, cudaStream_t st);
-/* T~|b~> written straight into rows g0 .. g0 + n of the positional layout
-   (the rest of those rows zeroed); a register marginal read straight from
-   those rows (probs zeroed by the caller, accumulated by atomics) */
-cudaError_t qw_launch_tinit_pos(const QwSimDev &d, void *pbuf, int64_t g0, int64_t n, const double *b_re,
-                                const double *b_im, const double *scale, int fp32, cudaStream_t st);
-cudaError_t qw_launch_measure_pos(const QwSimDev &d, const void *pbuf, int64_t g0, int64_t n, int fp32,
-                                  const double *scale, int reg, double *probs, int64_t len, cudaStream_t st);
+/* positional layout (qw_pos.cuh; 32: complex64, 64: complex128): the launch
+   shape, walk steps, T~|b~> written into rows g0 .. g0 + n, a register
+   marginal of those rows (probs zeroed by the caller; x0, nx: the rows'
+   extras), and the conversions
+   from and to the row buckets (pack: pbuf zeroed by the caller, a branch
+   without a place sets QW_ST_POS_UNREP; unpack: the buckets cleared by the
+   caller); full: plane B1 is in use */
+#define QW_POS_DECLARE(SUFFIX)                                                                                        \
+    QwPosPlan qw_pos_plan##SUFFIX(const QwSimDev &d);                                                                 \
+    cudaError_t qw_launch_walk_pos##SUFFIX(const QwSimDev &d, const QwPosPlan &pl, const QwPosArgs &p,                \
+                                           const QwStepArgs &a, int full, cudaStream_t st);                           \
+    cudaError_t qw_launch_tinit_pos##SUFFIX(const QwSimDev &d, void *pbuf, int64_t g0, int64_t n, int64_t x0,         \
+                                            int64_t nx, const double *b_re, const double *b_im, const double *scale,  \
+                                            cudaStream_t st);                                                         \
+    cudaError_t qw_launch_measure_pos##SUFFIX(const QwSimDev &d, const void *pbuf, int full, int64_t g0, int64_t n,   \
+                                              const double *scale, int reg, double *probs, int64_t len,               \
+                                              cudaStream_t st);                                                       \
+    cudaError_t qw_launch_pos_pack##SUFFIX(const QwSimDev &d, const QwBufDev &buf, void *pbuf, int32_t *status,       \
+                                           cudaStream_t st);                                                          \
+    cudaError_t qw_launch_pos_unpack##SUFFIX(const QwSimDev &d, const void *pbuf, int full, const QwBufDev &buf,      \
+                                             int32_t *status, cudaStream_t st);
+QW_POS_DECLARE(32)
+QW_POS_DECLARE(64)
+#undef QW_POS_DECLARE
+static inline QwPosPlan qw_pos_plan(const QwSimDev &d, int fp32) { return fp32 ? qw_pos_plan32(d) : qw_pos_plan64(d); }
+static inline cudaError_t qw_launch_walk_pos(const QwSimDev &d, const QwPosPlan &pl, const QwPosArgs &p,
+                                             const QwStepArgs &a, int fp32, int full, cudaStream_t st)
+{
+    return fp32 ? qw_launch_walk_pos32(d, pl, p, a, full, st) : qw_launch_walk_pos64(d, pl, p, a, full, st);
+}
+static inline cudaError_t qw_launch_tinit_pos(const QwSimDev &d, void *pbuf, int64_t g0, int64_t n, int64_t x0,
+                                              int64_t nx, const double *b_re, const double *b_im, const double *scale,
+                                              int fp32, cudaStream_t st)
+{
+    return fp32 ? qw_launch_tinit_pos32(d, pbuf, g0, n, x0, nx, b_re, b_im, scale, st)
+                : qw_launch_tinit_pos64(d, pbuf, g0, n, x0, nx, b_re, b_im, scale, st);
+}
+static inline cudaError_t qw_launch_measure_pos(const QwSimDev &d, const void *pbuf, int full, int64_t g0, int64_t n,
+                                                int fp32, const double *scale, int reg, double *probs, int64_t len,
+                                                cudaStream_t st)
+{
+    return fp32 ? qw_launch_measure_pos32(d, pbuf, full, g0, n, scale, reg, probs, len, st)
+                : qw_launch_measure_pos64(d, pbuf, full, g0, n, scale, reg, probs, len, st);
+}
+static inline cudaError_t qw_launch_pos_pack(const QwSimDev &d, const QwBufDev &buf, void *pbuf, int fp32,
+                                             int32_t *status, cudaStream_t st)
+{
+    return fp32 ? qw_launch_pos_pack32(d, buf, pbuf, status, st) : qw_launch_pos_pack64(d, buf, pbuf, status, st);
+}
+static inline cudaError_t qw_launch_pos_unpack(const QwSimDev &d, const void *pbuf, int full, const QwBufDev &buf,
+                                               int fp32, int32_t *status, cudaStream_t st)
+{
+    return fp32 ? qw_launch_pos_unpack32(d, pbuf, full, buf, status, st)
+                : qw_launch_pos_unpack64(d, pbuf, full, buf, status, st);
+}
 int qw_step_grid(const QwSimDev &d, int fp32, int mode);
 cudaError_t qw_launch_clear(const QwSimDev &d, const QwBufDev &buf, int64_t lo, int64_t hi,
                             int clear_spill, cudaStream_t st);
@@ -196,11 +255,12 @@ cudaError_t qw_launch_export(const QwSimDev &d, const QwBufDev &buf, int inst, i
 cudaError_t qw_launch_measure(const QwSimDev &d, const QwBufDev &buf, int inst, int fp32,
                               const double *scale, int reg, double *probs, int64_t len,
                               cudaStream_t st);
-/* pbuf (nullable): read rows g0 .. g0 + pn of the positional layout instead of buf */
+/* pbuf (nullable): read rows g0 .. g0 + pn of the positional layout (pfull:
+   plane B1 in use) instead of buf */
 cudaError_t qw_launch_measure_noalloc(const QwSimDev &d, const QwBufDev &buf, int inst, int fp32,
                                       const double *scale, int reg, double *host_probs,
                                       int64_t len, int device, cudaStream_t st, const void *pbuf = nullptr,
-                                      int64_t g0 = 0, int64_t pn = 0);
+                                      int pfull = 0, int64_t g0 = 0, int64_t pn = 0);
 cudaError_t qw_launch_count(const QwSimDev &d, const QwBufDev &buf, int inst,
                             unsigned long long *counter, cudaStream_t st);
 cudaError_t qw_launch_qls_norm(const double2 *y, int n, double *p, int64_t *jctr, cudaStream_t st);

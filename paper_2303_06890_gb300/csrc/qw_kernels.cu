@@ -925,7 +925,8 @@ __device__ void reflect_zero_list(const QwSimDev &d, const Row &r, WalkSink<AmpT
             p.lossy = z.lossy != 0;
             bool d0;
             key = x.key;
-            pair_reflect<AmpT>(d, sum, x.t, x.A, x.sneg, sink.zp[2 * u], sink.zp[2 * u + 1], x.u, z.m, p, r0, r1, d0);
+            pair_reflect<AmpT>(d, sum, x.t, x.A, x.sneg, sink.zp[2 * u], sink.zp[2 * u + 1],
+                               Amp<AmpT>::approx2(Amp<AmpT>::narrow(x.u)), z.m, p, r0, r1, d0);
             kept = (d0 ? 1u : 0u) + (p.c1 ? 1u : 0u);
             e0 = Amp<AmpT>::keep(d, r0);
             e1 = Amp<AmpT>::keep(d, r1);
@@ -1800,7 +1801,7 @@ __global__ void __launch_bounds__(WARPS * 32, 4) k_walk_slot(QwSimDev d, QwBufDe
             sum.scale_pow2(d.two_over_s);
             AmpT r0, r1;
             bool d0;
-            pair_reflect<AmpT>(d, sum, rv, val, sneg, p0, p1, u, m, ps, r0, r1, d0);
+            pair_reflect<AmpT>(d, sum, rv, val, sneg, p0, p1, Amp<AmpT>::approx2(Amp<AmpT>::narrow(u)), m, ps, r0, r1, d0);
             __syncwarp();
             st.hph += __popc(__ballot_sync(FULL, d0)) + __popc(__ballot_sync(FULL, ps.c1));
             const bool e0 = Amp<AmpT>::keep(d, r0), e1 = Amp<AmpT>::keep(d, r1);
@@ -1965,543 +1966,6 @@ __global__ void __launch_bounds__(WARPS * 32, 4) k_walk_slot(QwSimDev d, QwBufDe
         *a.deferred_ctr = 0u;
         *a.work_ctr = 0u;
         *a.done_ctr = 0u;
-    }
-}
-
-/* ==== positional walk step (walk_variant 7) ==================================== */
-/*
- * The state of a one-instance walk held by position instead of by key.  At a
- * step boundary every branch that the walk reaches from T~|b~> sits in a row
- * (jc = 0, j < N, b1) with kc = A = 0, and its k is either a column of row j
- * (W = S (2 T~ Pi T~^dag - 1): the branches of T~ Pi's range are those of
- * T~'s rows, the swapped ones have k = a row whose padded column list holds j)
- * -- position 2 l + b2 for the column in slot l -- or one of the E_j rows x
- * whose slot l_x holds column j while row j holds no column x (a padded, so
- * unpaired, entry) -- position 2 s + 2 e + b2.  Row (j, b1) is pos_R = 2 s +
- * 2 pos_E amplitudes at (2 j + b1) pos_R; an absent branch is 0, so the
- * position is the key.
- *
- * The lane of slot (j, l) runs the slot kernel's arithmetic on the pairs of
- * both rows of j at positions 2 l, 2 l + 1 (T~^dag's maps take them to (l, 0),
- * T~'s back to k = col): R^dag, H P H (the zero-type sum over the unit's
- * lanes for b1 = 0, -1 for b1 = 1), R; S sends its b2 = 0 / 1 outputs to rows
- * (col, 0) / (col, 1) at position tp(j, l) + b1, where tp is the position of
- * k = j in row col.  An extra (j, b1, e) is outside every zero-type group and
- * its maps leave A = 0 (kc = x ^ col(j, 0) != 0 after O_s'^dag, so O_A' does
- * not fire): R(0) (-1) R(0)^dag = -1 on its pair, sent to positions 2 l_x + b1
- * of rows (x, 0 / 1).  Every position of the output has exactly
- * one writer, and pruned outputs are written as 0: no counts, atomics,
- * searches or keys, and nothing to clear between steps.
- */
-/* launch shape of k_walk_pos per amplitude type (measured on GB300 at
-   N = 16384, s = 16): complex64 runs fastest with 16 warps per SM and up to
-   128 registers a thread (the next group's inputs held in registers while
-   the current one computes), complex128 -- bound by the FP64 pipe -- with
-   blocks of 4 warps, 5 per SM */
-template <typename AmpT> struct PosCfg;
-template <> struct PosCfg<float2> {
-    static constexpr int warps = 8, blocks = 2;
-    static constexpr bool even = true; /* grid: as many groups for every warp */
-};
-template <> struct PosCfg<double2> {
-    static constexpr int warps = 4, blocks = 4;
-    static constexpr bool even = false; /* grid: every resident block (FP64-pipe bound) */
-};
-
-template <typename AmpT> struct PosPair;
-template <> struct PosPair<float2> {
-    __device__ static void load(const float2 *p, float2 &a0, float2 &a1)
-    {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
-        a0 = make_float2(v.x, v.y);
-        a1 = make_float2(v.z, v.w);
-    }
-    __device__ static void store(float2 *p, float2 a0, float2 a1)
-    {
-        *reinterpret_cast<float4 *>(p) = make_float4(a0.x, a0.y, a1.x, a1.y);
-    }
-};
-template <> struct PosPair<double2> {
-    __device__ static void load(const double2 *p, double2 &a0, double2 &a1)
-    {
-        a0 = __ldg(p);
-        a1 = __ldg(p + 1);
-    }
-    __device__ static void store(double2 *p, double2 a0, double2 a1)
-    {
-        p[0] = a0;
-        p[1] = a1;
-    }
-};
-
-/* per-lane branch counters of the positional step, summed over the warp at
-   the end (the same quantities as WalkStats) */
-struct PosStats {
-    unsigned int rows = 0, in = 0, rdag = 0, hph = 0, out = 0;
-    __device__ void flush(const QwStepArgs &a)
-    {
-        unsigned int v[5] = {rows, in, rdag, hph, out};
-#pragma unroll
-        for (int i = 0; i < 5; ++i)
-            for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(FULL, v[i], o);
-        if (a.stats && lane_id() == 0 && v[1]) {
-            atomicAdd(a.stats + QW_STAT_ROWS, (unsigned long long)v[0]);
-            atomicAdd(a.stats + QW_STAT_IN, (unsigned long long)v[1]);
-            atomicAdd(a.stats + QW_STAT_RDAG, (unsigned long long)v[2]);
-            atomicAdd(a.stats + QW_STAT_HPH, (unsigned long long)v[3]);
-            atomicAdd(a.stats + QW_STAT_OUT, (unsigned long long)v[4]);
-        }
-    }
-};
-
-template <typename AmpT, int S, int PW>
-__global__ void __launch_bounds__(PW * 32, PosCfg<AmpT>::blocks / (S > 32 ? 2 : 1))
-    k_walk_pos(QwSimDev d, const AmpT *__restrict__ pin, AmpT *__restrict__ pout, QwStepArgs a)
-{
-    typedef typename Amp<AmpT>::RotVal RotVal;
-    /* a unit (one j) on SW lanes, each lane holding SPL of its slots (l = lb
-       + 32 k); RPP units per warp */
-    constexpr int SW = S > 32 ? 32 : S, SPL = S / SW, RPP = 32 / SW;
-    __shared__ double block_part[PW];
-    __shared__ double scale_sm;
-    __shared__ int is_last;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool skip = *(volatile int32_t *)a.status != 0;
-    const bool rescale = a.scale_in != nullptr;
-    const bool rot_in_place = Amp<AmpT>::kRotCode && d.rot_calc;
-    typename Amp<AmpT>::Norm nrm;
-    PosStats st;
-    const AmpT zero = Amp<AmpT>::zero();
-    /* 32-bit indices: the host keeps 2 N pos_R below 2^31 */
-    const uint32_t R = (uint32_t)d.pos_R;
-    const int E = d.pos_E;
-    const uint32_t n = (uint32_t)d.pos_rows; /* rows of all instances */
-    const uint32_t nall = (n + RPP - 1) / RPP, ngroups = skip ? 0u : nall;
-    const uint32_t nwarps = gridDim.x * PW;
-    const int ul = lane / SW, lb = lane % SW;
-    const int nx = RPP * 2 * E; /* extra items of a group: (unit, b1, e) */
-    /* the lane's first extra item is the same in every group */
-    int x_u = 0, x_b1 = 0, x_e = 0;
-    if (lane < nx) {
-        x_u = lane / (2 * E);
-        const int rem = lane - x_u * 2 * E;
-        x_b1 = rem / E;
-        x_e = rem - x_b1 * E;
-    }
-    /* a group's inputs, loaded one group ahead: the next group's loads are in
-       flight while the current one computes */
-    struct In {
-        uint32_t rb;       /* first row of the row's instance */
-        uint32_t w[SPL];   /* QRAM words */
-        RotVal t[SPL];
-        int tp[SPL];
-        AmpT a0[SPL], a1[SPL], q0[SPL], q1[SPL];
-        uint32_t xe; /* the lane's first extra item: x << 8 | l_x, 0xffffffff if none */
-        AmpT x0, x1;
-    };
-    /* extra item (u, b1, e) of group gg: its entry and pair (none past the
-       row's extras count) */
-    auto fetch_extra = [&](uint32_t gg, int u, int b1, int e, uint32_t &xe, AmpT &x0, AmpT &x1) {
-        const uint32_t jx = gg * RPP + u;
-        xe = 0xffffffffu;
-        x0 = x1 = zero;
-        if (gg < nall && jx < n && e < (int)__ldg(d.pos_xcnt + jx)) {
-            xe = __ldg(d.pos_xin + jx * (uint32_t)E + e);
-            PosPair<AmpT>::load(pin + (2 * jx + b1) * R + 2 * S + 2 * e, x0, x1);
-        }
-    };
-    auto fetch = [&](uint32_t gg, In &x) {
-        const uint32_t jj = gg * RPP + ul;
-        const bool have = gg < nall && jj < n;
-        x.rb = 0;
-        if (have && d.pos_rowbase) x.rb = __ldg(d.pos_rowbase + jj);
-#pragma unroll
-        for (int k = 0; k < SPL; ++k) {
-            const uint32_t l = lb + 32 * k;
-            x.w[k] = 0;
-            x.t[k] = Amp<AmpT>::rot_zero();
-            x.tp[k] = 0;
-            x.a0[k] = x.a1[k] = x.q0[k] = x.q1[k] = zero;
-            if (have) {
-                const uint32_t at = jj * S + l;
-                x.w[k] = __ldg(d.img + at);
-                if (!rot_in_place) x.t[k] = __ldg(static_cast<const RotVal *>(d.slot_rot) + at);
-                x.tp[k] = __ldg(d.pos_tp + at);
-                PosPair<AmpT>::load(pin + 2 * jj * R + 2 * l, x.a0[k], x.a1[k]);
-                PosPair<AmpT>::load(pin + (2 * jj + 1) * R + 2 * l, x.q0[k], x.q1[k]);
-            }
-        }
-        x.xe = 0xffffffffu;
-        x.x0 = x.x1 = zero;
-        if (lane < nx) fetch_extra(gg, x_u, x_b1, x_e, x.xe, x.x0, x.x1);
-    };
-    In nxt;
-    fetch(blockIdx.x * PW + warp, nxt);
-    /* the renormalisation factor, staged once per block while the first
-       group's loads are in flight */
-    if (threadIdx.x == 0) Amp<AmpT>::Scale::to_shared(rescale ? *a.scale_in : 1.0, &scale_sm);
-    __syncthreads();
-    const typename Amp<AmpT>::Scale scale = Amp<AmpT>::Scale::from_shared(&scale_sm);
-    for (uint32_t g = blockIdx.x * PW + warp; g < ngroups; g += nwarps) {
-        const In cur = nxt;
-        fetch(g + nwarps, nxt);
-        const uint32_t j = g * RPP + ul;
-        const bool valid = j < n;
-        RotVal rv[SPL];
-        uint32_t val[SPL], gc[SPL];
-        bool sneg[SPL];
-        AmpT a0[SPL], a1[SPL], q0[SPL], q1[SPL];
-        unsigned int nin = 0;
-#pragma unroll
-        for (int k = 0; k < SPL; ++k) {
-            const uint32_t w = cur.w[k];
-            val[k] = w & 0xffffu;
-            /* a 0 element rotates by R(0); complex64 derives the float pairs
-               from the value word (4 MB less read per step than the per-slot
-               table at N = 16384, s = 16) */
-            rv[k] = val[k] == 0 ? Amp<AmpT>::rot_zero() : (rot_in_place ? Amp<AmpT>::rot_code(val[k]) : cur.t[k]);
-            gc[k] = cur.rb + (w >> 16); /* the column's row among all instances' rows */
-            sneg[k] = j > gc[k];        /* j > col within the instance */
-            a0[k] = cur.a0[k];
-            a1[k] = cur.a1[k];
-            q0[k] = cur.q0[k];
-            q1[k] = cur.q1[k];
-            if (valid && rescale) {
-                a0[k] = scale.apply(a0[k]);
-                a1[k] = scale.apply(a1[k]);
-                q0[k] = scale.apply(q0[k]);
-                q1[k] = scale.apply(q1[k]);
-            }
-            nin += nz(a0[k]) + nz(a1[k]) + nz(q0[k]) + nz(q1[k]);
-        }
-        st.in += nin;
-        {
-            const unsigned m = __ballot_sync(FULL, nin != 0);
-            const unsigned um = SW == 32 ? m : (m >> (ul * SW)) & ((1u << (SW & 31)) - 1u);
-            if (lb == 0 && um != 0) st.rows += 1; /* units holding branches */
-        }
-
-        /* b1 = 0: R^dag, H P H on the zero-type group (the unit's slots), R */
-        AmpT rA0[SPL], rA1[SPL];
-        bool eA0[SPL], eA1[SPL];
-        {
-            typename Amp<AmpT>::Wide u[SPL];
-            PairState<AmpT> ps[SPL];
-            float m[SPL];
-#pragma unroll
-            for (int k = 0; k < SPL; ++k) {
-                ps[k] = pair_tdag<AmpT>(d, rv[k], val[k], sneg[k], a0[k], a1[k], u[k], m[k]);
-                st.rdag += (ps[k].c0 ? 1u : 0u) + (ps[k].c1 ? 1u : 0u);
-            }
-            __syncwarp();
-            typename Amp<AmpT>::Sum sum;
-            sum.set(u[0]);
-#pragma unroll
-            for (int k = 1; k < SPL; ++k) sum.add(u[k]);
-            sum.reduce(SW, SW);
-            if (a.qls_readout && valid && lb == 0) {
-                const double2 sv = sum.value();
-                const double coef = a.qls_coefs[*a.qls_j];
-                double2 acc = a.qls_y[j];
-                acc.x += coef * (d.inv_sqrt_s * sv.x);
-                acc.y += coef * (d.inv_sqrt_s * sv.y);
-                a.qls_y[j] = acc;
-            }
-            sum.scale_pow2(d.two_over_s);
-#pragma unroll
-            for (int k = 0; k < SPL; ++k) {
-                bool d0;
-                pair_reflect<AmpT>(d, sum, rv[k], val[k], sneg[k], a0[k], a1[k], u[k], m[k], ps[k], rA0[k], rA1[k], d0);
-                st.hph += (d0 ? 1u : 0u) + (ps[k].c1 ? 1u : 0u);
-                eA0[k] = Amp<AmpT>::keep(d, rA0[k]);
-                eA1[k] = Amp<AmpT>::keep(d, rA1[k]);
-            }
-        }
-        /* b1 = 1: R^dag, -1, R, then S: rows (col, 0) and (col, 1), positions
-           tp (from b1 = 0) and tp + 1 (from b1 = 1) */
-#pragma unroll
-        for (int k = 0; k < SPL; ++k) {
-            AmpT rB0, rB1;
-            const unsigned int kept = pair_negate<AmpT>(d, rv[k], val[k], sneg[k], q0[k], q1[k], rB0, rB1);
-            st.rdag += kept;
-            st.hph += kept;
-            const bool eB0 = Amp<AmpT>::keep(d, rB0), eB1 = Amp<AmpT>::keep(d, rB1);
-            if (valid) {
-                const AmpT s0 = eA0[k] ? rA0[k] : zero, s1 = eB0 ? rB0 : zero;
-                const AmpT s2 = eA1[k] ? rA1[k] : zero, s3 = eB1 ? rB1 : zero;
-                if (eA0[k]) nrm.add(rA0[k]);
-                if (eB0) nrm.add(rB0);
-                if (eA1[k]) nrm.add(rA1[k]);
-                if (eB1) nrm.add(rB1);
-                st.out += (eA0[k] ? 1u : 0u) + (eB0 ? 1u : 0u) + (eA1[k] ? 1u : 0u) + (eB1 ? 1u : 0u);
-                const uint32_t tp = (uint32_t)cur.tp[k];
-                PosPair<AmpT>::store(pout + 2 * gc[k] * R + tp, s0, s1);
-                PosPair<AmpT>::store(pout + (2 * gc[k] + 1) * R + tp, s2, s3);
-            }
-        }
-
-        /* the extras of the group's rows: the lane's first item prefetched, any
-           further ones (more than 32 per group) loaded here */
-        for (int it = lane; it < nx; it += 32) {
-            int xb1 = x_b1;
-            uint32_t xe = cur.xe;
-            AmpT x0 = cur.x0, x1 = cur.x1;
-            if (it != lane) {
-                const int uu = it / (2 * E), rem = it - uu * 2 * E;
-                xb1 = rem / E;
-                fetch_extra(g, uu, xb1, rem - xb1 * E, xe, x0, x1);
-            }
-            if (xe == 0xffffffffu) continue;
-            if (rescale) {
-                x0 = scale.apply(x0);
-                x1 = scale.apply(x1);
-            }
-            st.in += nz(x0) + nz(x1);
-            /* R(0) (-1) R(0)^dag with R(0) = [[0, -1], [1, 0]]: R(0)^dag gives
-               (x1, -x0), -1 and R(0) give (-x0, -x1) -- each output the
-               negated input, kept where the input is (every product is by
-               0 or 1, so this is the general rotation's result exactly) */
-            const bool k0 = Amp<AmpT>::keep(d, x0), k1 = Amp<AmpT>::keep(d, x1);
-            const unsigned int kept = (k0 ? 1u : 0u) + (k1 ? 1u : 0u);
-            st.rdag += kept;
-            st.hph += kept;
-            st.out += kept;
-            const AmpT r0 = Amp<AmpT>::neg(x0), r1 = Amp<AmpT>::neg(x1);
-            if (k0) nrm.add(r0);
-            if (k1) nrm.add(r1);
-            const uint32_t x = xe >> 8, px = 2 * (xe & 0xffu) + (uint32_t)xb1;
-            pout[2 * x * R + px] = k0 ? r0 : zero;
-            pout[(2 * x + 1) * R + px] = k1 ? r1 : zero;
-        }
-    }
-    st.flush(a);
-
-    /* end of the step: block partial of the norm, the last block reduces */
-    const double nv = nrm.warp_total();
-    if (lane == 0) block_part[warp] = nv;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double sum = 0.0;
-        for (int w = 0; w < PW; ++w) sum += block_part[w];
-        a.partials[blockIdx.x] = sum;
-        __threadfence();
-        const unsigned prev = atomicAdd(a.done_ctr, 1u);
-        is_last = (prev == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    double v = 0.0;
-    for (unsigned bb = threadIdx.x; bb < gridDim.x; bb += blockDim.x) v += __ldcg(a.partials + bb);
-    v = warp_sum(v);
-    if (lane == 0) block_part[warp] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int w = 0; w < PW; ++w) tot += block_part[w];
-        const bool clean = *(volatile int32_t *)a.status == 0;
-        if (clean) {
-            *a.norm_out = tot;
-            if (a.scale_out) *a.scale_out = (a.renorm && tot > 0.0) ? sqrt(*a.renorm_target / tot) : 1.0;
-            if (a.steps_done) *a.steps_done += 1;
-            if (a.stats) a.stats[QW_STAT_STEPS] += 1;
-        }
-        *a.done_ctr = 0u;
-    }
-}
-
-/* T~|b~> written straight into the positional layout for rows g0 .. g0 + n
- * of pbuf (one instance): |b~> holds one branch per row, a = b_j (divided by
- * the pending renormalisation factor when other instances share the state);
- * T~'s Hadamard gives (l, z = 0) with a / sqrt(s) for every slot l, its maps
- * take slot l to k = col(j, l), and R(A_jl) on (a / sqrt(s), 0) gives the
- * pair at positions 2 l, 2 l + 1 of row (j, b1 = 0) -- the arithmetic of
- * k_tinit.  Every other position of both rows is written 0.  One thread per
- * position. */
-template <typename AmpT>
-__global__ void k_tinit_pos(QwSimDev d, AmpT *pbuf, int64_t g0, int64_t n, const double *b_re, const double *b_im,
-                            const double *scale)
-{
-    typedef typename Amp<AmpT>::RotVal RotVal;
-    const int S = d.s;
-    const int64_t R = d.pos_R, total = 2 * n * R;
-    const AmpT zero = Amp<AmpT>::zero();
-    const bool rot_in_place = Amp<AmpT>::kRotCode && d.rot_calc;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = i / R, j = r >> 1;
-        const int q = (int)(i - r * R);
-        AmpT out = zero;
-        if ((r & 1) == 0 && q < 2 * S) {
-            double2 v = make_double2(b_re[j], b_im ? b_im[j] : 0.0);
-            if (scale) v = make_double2(v.x / *scale, v.y / *scale);
-            const double2 a = Amp<AmpT>::to_d(Amp<AmpT>::from_d(v)); /* as stored by |b~> */
-            const AmpT h = Amp<AmpT>::from_d(make_double2(d.inv_sqrt_s * a.x, d.inv_sqrt_s * a.y));
-            if ((v.x != 0.0 || v.y != 0.0) && Amp<AmpT>::keep(d, h)) {
-                const int64_t at = (g0 + j) * S + (q >> 1);
-                const uint32_t w = __ldg(d.img + at), val = w & 0xffffu;
-                const RotVal rv = val == 0 ? Amp<AmpT>::rot_zero()
-                                           : (rot_in_place ? Amp<AmpT>::rot_code(val)
-                                                           : __ldg(static_cast<const RotVal *>(d.slot_rot) + at));
-                AmpT o0, o1;
-                Amp<AmpT>::rot(rv, val, false, (uint32_t)j > (w >> 16), h, zero, o0, o1); /* R */
-                const AmpT o = (q & 1) ? o1 : o0;
-                if (Amp<AmpT>::keep(d, o)) out = o;
-            }
-        }
-        pbuf[2 * g0 * R + i] = out;
-    }
-}
-
-/* Marginal of one register over instance rows g0 .. g0 + n of the
- * positional layout (the key of a position: jc = kc = 0, j = its row, b1, k
- * = the slot's column or the extra's row, b2 = position & 1).  A warp per j
- * reads both rows whole (positions past a row's extras are 0), all loads in
- * flight together; the row registers (jc, j, b1) add their sums once. */
-template <typename AmpT>
-__global__ void k_measure_pos(QwSimDev d, const AmpT *pbuf, int64_t g0, int64_t n, const double *scale, int reg,
-                              double *probs, int64_t len)
-{
-    const int S = d.s, E = d.pos_E;
-    const int R = d.pos_R;
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const double sc = scale ? *scale : 1.0;
-    for (int64_t j = warp; j < n; j += nw) {
-        const int64_t g = g0 + j;
-        const AmpT *rows = pbuf + 2 * g * R; /* rows (j, 0) and (j, 1) */
-        double acc[2] = {0.0, 0.0};
-        for (int q2 = lane; q2 < 2 * R; q2 += 32) {
-            double2 a = Amp<AmpT>::to_d(rows[q2]);
-            if (a.x == 0.0 && a.y == 0.0) continue;
-            if (scale) a = make_double2(sc * a.x, sc * a.y);
-            const double p = a.x * a.x + a.y * a.y;
-            const int b1 = q2 >= R ? 1 : 0, q = q2 - b1 * R;
-            if (reg <= 2) {
-                acc[reg == 2 ? b1 : 0] += p;
-                continue;
-            }
-            uint64_t v = 0; /* kc = 0 */
-            if (reg == 4) v = q < 2 * S ? (d.img[g * S + (q >> 1)] >> 16)
-                                        : (uint64_t)((d.pos_xin[g * E + ((q - 2 * S) >> 1)] >> 8) - (uint32_t)g0);
-            else if (reg == 5) v = (uint64_t)(q & 1);
-            if ((int64_t)v < len) atomicAdd(probs + v, p);
-        }
-        if (reg <= 2) {
-            for (int t = 0; t < 2; ++t)
-                for (int o = 16; o > 0; o >>= 1) acc[t] += __shfl_xor_sync(FULL, acc[t], o);
-            if (lane == 0) {
-                if (reg == 1) {
-                    if (j < len && acc[0] != 0.0) atomicAdd(probs + j, acc[0]);
-                } else {
-                    for (int t = 0; t < 2; ++t) {
-                        const int64_t v = reg == 2 ? t : 0;
-                        if (v < len && acc[t] != 0.0) atomicAdd(probs + v, acc[t]);
-                    }
-                }
-            }
-        }
-    }
-}
-
-/* the row buckets into the positional layout (pbuf zeroed by the caller):
-   one thread per bucket slot */
-template <typename AmpT>
-__global__ void k_pos_pack(QwSimDev d, QwBufDev buf, AmpT *pbuf, int32_t *status)
-{
-    const int S = d.s, E = d.pos_E;
-    const int64_t total = d.total_buckets * (int64_t)d.cap_row;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = i / d.cap_row;
-        const int p = (int)(i - b * d.cap_row);
-        if (p >= buf.count[b]) continue;
-        if (b >= d.dense_buckets) { /* a row with jc != 0 */
-            atomicOr(status, QW_ST_POS_UNREP);
-            continue;
-        }
-        int64_t j = b >> 1, n = d.n_single, g0 = 0;
-        if (d.ninst > 1) {
-            const int inst = d.unit_inst[b >> 1];
-            j = (b - d.inst_bkt[inst]) >> 1;
-            n = d.inst_n[inst];
-            g0 = d.inst_img[inst] / S;
-        }
-        if (j >= n) { /* a row j >= N */
-            atomicOr(status, QW_ST_POS_UNREP);
-            continue;
-        }
-        const int64_t gr = g0 + j; /* the row among all instances' rows */
-        const Regs x = decode_r(buf.key[i], d.nb);
-        int pos = -1;
-        if (x.kc == 0 && x.A == 0) {
-            const uint32_t *row = d.img + gr * S;
-            int lo = 0, hi = S; /* lower bound of k among the row's sorted columns */
-            while (lo < hi) {
-                const int m = (lo + hi) >> 1;
-                if ((row[m] >> 16) < x.k) lo = m + 1;
-                else hi = m;
-            }
-            if (lo < S && (row[lo] >> 16) == x.k) {
-                pos = 2 * lo + (int)x.b2;
-            } else {
-                const int ne = d.pos_xcnt[gr];
-                for (int e = 0; e < ne; ++e)
-                    if ((d.pos_xin[gr * E + e] >> 8) - g0 == x.k) {
-                        pos = 2 * S + 2 * e + (int)x.b2;
-                        break;
-                    }
-            }
-        }
-        if (pos < 0) {
-            atomicOr(status, QW_ST_POS_UNREP);
-            continue;
-        }
-        pbuf[(2 * gr + (b & 1)) * d.pos_R + pos] = static_cast<const AmpT *>(buf.amp)[i];
-    }
-}
-
-/* the positional layout into the row buckets (cleared by the caller): one
-   thread per position, non-zero amplitudes appended to their row */
-template <typename AmpT>
-__global__ void k_pos_unpack(QwSimDev d, const AmpT *pbuf, QwBufDev buf, int32_t *status)
-{
-    const int S = d.s, E = d.pos_E;
-    const int64_t R = d.pos_R, total = 2 * d.pos_rows * R;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const AmpT v = pbuf[i];
-        if (v.x == 0 && v.y == 0) continue;
-        const int64_t r = i / R;
-        const int q = (int)(i - r * R);
-        const int64_t gr = r >> 1; /* the row among all instances' rows */
-        int64_t g0 = 0, bk = r;    /* the instance's first row; the bucket */
-        if (d.ninst > 1) {
-            const int inst = d.pos_rowinst[gr];
-            g0 = d.inst_img[inst] / S;
-            bk = d.inst_bkt[inst] + 2 * (gr - g0) + (r & 1);
-        }
-        Regs x;
-        x.kc = 0;
-        x.A = 0;
-        x.b2 = (uint32_t)(q & 1);
-        if (q < 2 * S) {
-            x.k = d.img[gr * S + (q >> 1)] >> 16;
-        } else {
-            const int e = (q - 2 * S) >> 1;
-            if (e >= (int)d.pos_xcnt[gr]) { /* never written: not a branch */
-                atomicOr(status, QW_ST_POS_UNREP);
-                continue;
-            }
-            x.k = (d.pos_xin[gr * E + e] >> 8) - (uint32_t)g0;
-        }
-        const int64_t r_b = bk;
-        const int p = atomicAdd(buf.count + r_b, 1);
-        if (p >= d.cap_row) {
-            atomicOr(status, QW_ST_ROW_OVERFLOW);
-            continue;
-        }
-        const int64_t sl = r_b * d.cap_row + p;
-        buf.key[sl] = encode_r(x, d.nb);
-        static_cast<AmpT *>(buf.amp)[sl] = v;
     }
 }
 
@@ -2932,54 +2396,6 @@ size_t slot_smem_bytes(const QwSimDev &d)
     return (size_t)WARPS * (key32_fits(d) ? slot_per_warp<AmpT, uint32_t>(d) : slot_per_warp<AmpT, uint64_t>(d));
 }
 
-template <typename AmpT, int S>
-int pos_grid_s(const QwSimDev &d)
-{
-    constexpr int PW = PosCfg<AmpT>::warps;
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_walk_pos<AmpT, S, PW>, PW * 32, 0);
-    if (per_sm < 1) per_sm = 1;
-    /* complex64: as many groups for every warp -- with k = ceil(groups /
-       resident warps) groups a warp, the fewest blocks that cover them (a warp
-       with fewer groups than the others would wait for them at the end of the
-       step); complex128, bound by each SM's FP64 pipe: every resident block,
-       so that every SM holds the same share (measured at N = 16384: 24.0 vs
-       25.4 us per flushed complex64 step, 57.0 vs 51.2 us complex128) */
-    constexpr int RPP = 32 / (S > 32 ? 32 : S);
-    const int64_t groups = (d.pos_rows + RPP - 1) / RPP;
-    const int64_t cap = (int64_t)per_sm * qw_sm_count();
-    const int64_t want = (groups + PW - 1) / PW;
-    int64_t g = want < cap ? want : cap;
-    if (PosCfg<AmpT>::even) {
-        const int64_t k = (groups + cap * PW - 1) / (cap * PW);
-        g = (groups + k * PW - 1) / (k * PW);
-    }
-    return (int)(g < 1 ? 1 : g);
-}
-
-template <typename AmpT>
-int pos_grid_t(const QwSimDev &d)
-{
-    if (d.s == 8) return pos_grid_s<AmpT, 8>(d);
-    if (d.s == 16) return pos_grid_s<AmpT, 16>(d);
-    if (d.s == 32) return pos_grid_s<AmpT, 32>(d);
-    return pos_grid_s<AmpT, 64>(d);
-}
-
-template <typename AmpT>
-cudaError_t launch_pos_t(const QwSimDev &d, const void *pin, void *pout, const QwStepArgs &a, int grid,
-                         cudaStream_t st)
-{
-    const AmpT *i = static_cast<const AmpT *>(pin);
-    AmpT *o = static_cast<AmpT *>(pout);
-    constexpr int PW = PosCfg<AmpT>::warps;
-    if (d.s == 8) k_walk_pos<AmpT, 8, PW><<<grid, PW * 32, 0, st>>>(d, i, o, a);
-    else if (d.s == 16) k_walk_pos<AmpT, 16, PW><<<grid, PW * 32, 0, st>>>(d, i, o, a);
-    else if (d.s == 32) k_walk_pos<AmpT, 32, PW><<<grid, PW * 32, 0, st>>>(d, i, o, a);
-    else k_walk_pos<AmpT, 64, PW><<<grid, PW * 32, 0, st>>>(d, i, o, a);
-    return cudaGetLastError();
-}
-
 } // namespace
 
 /* SM count of the current device, cached per device (launch shapes follow
@@ -3073,60 +2489,6 @@ cudaError_t qw_launch_clear(const QwSimDev &d, const QwBufDev &buf, int64_t lo, 
     if (grid < 1) grid = 1;
     if (grid > 4 * qw_sm_count()) grid = 4 * qw_sm_count();
     k_clear<<<grid, 256, 0, st>>>(buf, lo, hi, d.spill_slots, clear_spill);
-    return cudaGetLastError();
-}
-
-int qw_pos_grid(const QwSimDev &d, int fp32)
-{
-    return fp32 ? pos_grid_t<float2>(d) : pos_grid_t<double2>(d);
-}
-
-cudaError_t qw_launch_walk_pos(const QwSimDev &d, const void *pin, void *pout, const QwStepArgs &a, int fp32,
-                               int grid, cudaStream_t st)
-{
-    if (!qw_pos_supported(d)) return cudaErrorInvalidValue;
-    return fp32 ? launch_pos_t<float2>(d, pin, pout, a, grid, st) : launch_pos_t<double2>(d, pin, pout, a, grid, st);
-}
-
-cudaError_t qw_launch_tinit_pos(const QwSimDev &d, void *pbuf, int64_t g0, int64_t n, const double *b_re,
-                                const double *b_im, const double *scale, int fp32, cudaStream_t st)
-{
-    const int grid = 4 * qw_sm_count();
-    if (fp32) k_tinit_pos<float2><<<grid, 256, 0, st>>>(d, static_cast<float2 *>(pbuf), g0, n, b_re, b_im, scale);
-    else k_tinit_pos<double2><<<grid, 256, 0, st>>>(d, static_cast<double2 *>(pbuf), g0, n, b_re, b_im, scale);
-    return cudaGetLastError();
-}
-
-cudaError_t qw_launch_measure_pos(const QwSimDev &d, const void *pbuf, int64_t g0, int64_t n, int fp32,
-                                  const double *scale, int reg, double *probs, int64_t len, cudaStream_t st)
-{
-    /* a warp per j: enough blocks that every j's loads are in flight at once */
-    int64_t want = (n + 7) / 8;
-    const int64_t cap = 32 * (int64_t)qw_sm_count();
-    const int grid = (int)(want < 1 ? 1 : (want < cap ? want : cap));
-    if (fp32)
-        k_measure_pos<float2><<<grid, 256, 0, st>>>(d, static_cast<const float2 *>(pbuf), g0, n, scale, reg, probs, len);
-    else
-        k_measure_pos<double2><<<grid, 256, 0, st>>>(d, static_cast<const double2 *>(pbuf), g0, n, scale, reg, probs,
-                                                     len);
-    return cudaGetLastError();
-}
-
-cudaError_t qw_launch_pos_pack(const QwSimDev &d, const QwBufDev &buf, void *pbuf, int fp32, int32_t *status,
-                               cudaStream_t st)
-{
-    const int grid = 4 * qw_sm_count();
-    if (fp32) k_pos_pack<float2><<<grid, 256, 0, st>>>(d, buf, static_cast<float2 *>(pbuf), status);
-    else k_pos_pack<double2><<<grid, 256, 0, st>>>(d, buf, static_cast<double2 *>(pbuf), status);
-    return cudaGetLastError();
-}
-
-cudaError_t qw_launch_pos_unpack(const QwSimDev &d, const void *pbuf, const QwBufDev &buf, int fp32,
-                                 int32_t *status, cudaStream_t st)
-{
-    const int grid = 4 * qw_sm_count();
-    if (fp32) k_pos_unpack<float2><<<grid, 256, 0, st>>>(d, static_cast<const float2 *>(pbuf), buf, status);
-    else k_pos_unpack<double2><<<grid, 256, 0, st>>>(d, static_cast<const double2 *>(pbuf), buf, status);
     return cudaGetLastError();
 }
 
@@ -3238,8 +2600,8 @@ double *g_scratch_addr[kMaxDevices] = {nullptr};
 
 cudaError_t qw_launch_measure_noalloc(const QwSimDev &d, const QwBufDev &buf, int inst, int fp32,
                                       const double *scale, int reg, double *host_probs,
-                                      int64_t len, int device, cudaStream_t st, const void *pbuf, int64_t g0,
-                                      int64_t pn)
+                                      int64_t len, int device, cudaStream_t st, const void *pbuf, int pfull,
+                                      int64_t g0, int64_t pn)
 {
     if (device < 0 || device >= kMaxDevices || len < 1 || len > QW_MEASURE_NOALLOC_MAX_LEN)
         return cudaErrorInvalidValue;
@@ -3262,7 +2624,7 @@ cudaError_t qw_launch_measure_noalloc(const QwSimDev &d, const QwBufDev &buf, in
     cudaError_t e = cudaMemsetAsync(scratch, 0, (size_t)len * sizeof(double), st);
     if (e != cudaSuccess) return e;
     const int grid = 4 * qw_sm_count();
-    if (pbuf) e = qw_launch_measure_pos(d, pbuf, g0, pn, fp32, scale, reg, scratch, len, st);
+    if (pbuf) e = qw_launch_measure_pos(d, pbuf, pfull, g0, pn, fp32, scale, reg, scratch, len, st);
     else if (fp32) k_measure<float2><<<grid, 256, 0, st>>>(d, buf, inst, scale, reg, scratch, len);
     else k_measure<double2><<<grid, 256, 0, st>>>(d, buf, inst, scale, reg, scratch, len);
     if (!pbuf) e = cudaGetLastError();

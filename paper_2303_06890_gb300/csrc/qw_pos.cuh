@@ -1,0 +1,969 @@
+/*
+ * qw_pos.cuh -- the positional layout (walk_variant 7): kernels and launchers,
+ * instantiated for complex128 (qw_pos64.cu) and complex64 (qw_pos32.cu).
+ */
+#ifndef QW_POS_CUH
+#define QW_POS_CUH
+
+#include "qw_amp.cuh"
+#include "qw_device.cuh"
+#include "qw_internal.h"
+
+namespace {
+
+/* ==== positional walk steps ==================================================== */
+/*
+ * The state of the walk held by position instead of by key.  At a step
+ * boundary every branch that the walk reaches from T~|b~> sits in a row
+ * (jc = 0, j < N, b1) with kc = A = 0, and its k is either a column of row j
+ * (W = S (2 T~ Pi T~^dag - 1): the branches of T~ Pi's range are those of
+ * T~'s rows, the swapped ones have k = a row whose padded column list holds j)
+ * -- entry g s + l for the column in slot l of row g -- or one of the rows x
+ * whose slot l_x holds column j while row j holds no column x (a padded, so
+ * unpaired, entry): an extra, entry N s + e in a list of all rows' extras in
+ * row order.  Over these T entries three planes hold the amplitudes:
+ * A[2 i + b2] of row (j, b1 = 0), its b2 pair side by side, and B0[i], B1[i] of
+ * row (j, b1 = 1), b2 = 0 and 1.  An absent branch is 0, so the place is the
+ * key.
+ *
+ * B1 stays empty: S gives a b1 = b2 = 1 branch only from one of the same kind,
+ * and T~|b~> has none.  It is neither read nor written (3/4 of the state's
+ * bytes) unless an imported state put something there (FULL).
+ *
+ * The lane of slot (j, l) runs the walk operator on the slot's two pairs
+ * (T~^dag's maps take them to (l, 0), T~'s back to k = col): b1 = 0 reflected
+ * in the zero-type group (the unit's lanes), b1 = 1 negated; S sends the
+ * outputs to entry dst(j, l) -- that of k = j in row col(j, l) -- A from the two
+ * b2 = 0 outputs, B0 and B1 from the b2 = 1 ones.  An extra is outside every
+ * zero-type group and its maps leave A = 0 (kc = x ^ col(j, 0) != 0 after
+ * O_s'^dag, so O_A' does not fire): R(0) (-1) R(0)^dag = -1 on its pair
+ * (each output the negated input, kept where the input is), sent to slot
+ * (x, l_x); extras run 32 to a warp on their own.  Every entry of the output has
+ * exactly one writer and pruned outputs are written as 0: no counts, atomics,
+ * searches or keys, and nothing to clear between steps.
+ *
+ * Several steps run in one launch: a grid of at most one block per SM,
+ * launched cooperatively, with a barrier over the grid between steps that
+ * also carries the norm.  What a step needs of the matrix --
+ * each slot's rotation, destination and flags -- is laid out once per launch
+ * in shared memory (TAB) in the order the block's lanes use it, so that a
+ * step reads the state and nothing else.
+ *
+ * Bounds: a step at small N is a chain of latencies -- state load, rotation,
+ * group sum, store, barrier -- and one launch per step added the launch and
+ * the last block's reduction to it.  At large N the state's 24 (48) bytes per
+ * slot in and out come from L2.
+ */
+constexpr int kPosMaxWarps = 16; /* 512 threads: up to 128 registers a thread */
+
+/* state accesses go to L2 (another SM wrote what this one reads) */
+__device__ __forceinline__ void pos_load2(const float2 *p, float2 &a0, float2 &a1)
+{
+    const float4 v = __ldcg(reinterpret_cast<const float4 *>(p));
+    a0 = make_float2(v.x, v.y);
+    a1 = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void pos_load2(const double2 *p, double2 &a0, double2 &a1)
+{
+    a0 = __ldcg(p);
+    a1 = __ldcg(p + 1);
+}
+__device__ __forceinline__ void pos_store2(float2 *p, float2 a0, float2 a1)
+{
+    __stcg(reinterpret_cast<float4 *>(p), make_float4(a0.x, a0.y, a1.x, a1.y));
+}
+__device__ __forceinline__ void pos_store2(double2 *p, double2 a0, double2 a1)
+{
+    __stcg(p, a0);
+    __stcg(p + 1, a1);
+}
+
+/* ---- barrier over the grid, with the norm ---------------------------------- */
+/*
+ * One 64-bit word per step: every block adds 1 to its count (bits 56 up) and
+ * its share of the norm as a fixed-point number (bits 0 .. 55), so one atomic
+ * per block is both its arrival and its term of the sum, whose value does not
+ * depend on the order of arrival.  The unit is a power of two of which the
+ * renormalisation target holds 2^53 to 2^54: rounding a block's share to it
+ * costs 2^-55 of the target, below what the FP64 sum of the shares would.
+ * Four words take turns; passing step t, block 0 clears the word of step t + 2,
+ * which every block has left (it was step t - 2's).
+ */
+constexpr int kCountShift = 56;
+constexpr unsigned long long kShareMask = (1ull << kCountShift) - 1ull;
+
+struct PosNorm { /* per launch, in shared memory */
+    double unit_inv;                  /* 2^k: shares times this are in units */
+    unsigned long long target;        /* the renormalisation target in units */
+    float target_inv;                 /* 1 / target */
+};
+
+__device__ __forceinline__ void pos_norm_setup(const QwStepArgs &a, PosNorm &pn)
+{
+    const double t = *a.renorm_target;
+    int e = 0;
+    if (t > 0.0 && t < 1e300) frexp(t, &e);
+    e = max(e, -70); /* 2^(54 - e) is an FP32 number too */
+    pn.unit_inv = ldexp(1.0, 54 - e);
+    pn.target = (unsigned long long)__double2ll_rn(t > 0.0 && t < 1e300 ? t * pn.unit_inv : 0.0);
+    pn.target_inv = pn.target ? (float)(1.0 / (double)pn.target) : 0.0f;
+}
+
+/* a lane's norm share in units; poisoned (not finite, or beyond what the word
+   can sum) shares count as 0 and set the flag */
+__device__ __forceinline__ unsigned long long to_units(const Amp<double2>::Norm &n, double unit_inv, bool &bad)
+{
+    const double v = n.get() * unit_inv;
+    bad = !(v >= 0.0 && v < 0x1p54);
+    return bad ? 0ull : (unsigned long long)__double2ll_rn(v);
+}
+__device__ __forceinline__ unsigned long long to_units(const Amp<float2>::Norm &n, float unit_inv, bool &bad)
+{
+    /* the scaling by a power of two is exact; hi has 24 bits, lo is rounded
+       to a unit */
+    const float h = n.hi * unit_inv, l = n.lo * unit_inv;
+    bad = !(h >= 0.0f && h < 0x1p54f);
+    return bad ? 0ull : (unsigned long long)(__float2ll_rn(h) + __float2ll_rn(l));
+}
+/* the warp's sum of values below 2^57, exact: three limbs through the integer
+   reduction */
+__device__ __forceinline__ unsigned long long warp_sum_units(unsigned long long v)
+{
+    const unsigned a = __reduce_add_sync(FULL, (unsigned)(v & 0x3ffffffull));
+    const unsigned b = __reduce_add_sync(FULL, (unsigned)((v >> 26) & 0x3ffffffull));
+    const unsigned c = __reduce_add_sync(FULL, (unsigned)(v >> 52));
+    return (unsigned long long)a + ((unsigned long long)b << 26) + ((unsigned long long)c << 52);
+}
+
+__device__ __forceinline__ void word_add(unsigned long long *p, unsigned long long v)
+{
+    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ unsigned long long word_load(const unsigned long long *p)
+{
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+/* The renormalisation factor of a norm of `sum` units, as 1 + c in FP32 pair
+ * form (h, l) and in FP64.  sqrt(target / sum) = (1 - x)^(-1/2) with x = (target
+ * - sum) / target: within 2^-20 the series to second order is exact to 2^-60
+ * and needs no FP64 arithmetic (square root and division there take over a
+ * thousand cycles, between every two steps); otherwise FP64. */
+__device__ __noinline__ double pos_scale_exact(double target, double norm)
+{
+    return norm > 0.0 ? sqrt(target / norm) : 1.0;
+}
+__device__ __forceinline__ bool pos_scale(const PosNorm &pn, unsigned long long sum, float &c)
+{
+    const float x = (float)(long long)(pn.target - sum) * pn.target_inv;
+    c = fmaf(0.375f * x, x, 0.5f * x);
+    return fabsf(x) < 0x1p-20f;
+}
+
+/* FP64 work of the read-out and of a complex128 norm, out of line: a
+   predicated-off FP64 instruction takes its slot of the 1/64-rate pipe */
+__device__ __noinline__ double pos_readout(double2 *y, double unit, double sx, double sy)
+{
+    double2 acc = __ldcg(y);
+    acc.x += unit * sx;
+    acc.y += unit * sy;
+    __stcg(y, acc);
+    return fma(acc.x, acc.x, acc.y * acc.y);
+}
+__device__ __noinline__ double norm_c128(double v, double2 a) { return fma(a.x, a.x, fma(a.y, a.y, v)); }
+__device__ __forceinline__ void norm_add(Amp<double2>::Norm &n, double2 a) { n.v = norm_c128(n.v, a); }
+__device__ __forceinline__ void norm_add(Amp<float2>::Norm &n, float2 a) { n.add(a); }
+
+/* The pruning rule on a value of which m = inf_norm: above thr32 kept, the
+   rest exactly (0 is the common case there) */
+template <typename AmpT> __device__ __noinline__ bool keep_exact(const QwSimDev &d, AmpT a)
+{
+    return Amp<AmpT>::keep(d, a);
+}
+__device__ __forceinline__ bool pos_keep(const QwSimDev &d, double2 a)
+{
+    const float m = Amp<double2>::inf_norm(a);
+    bool k = m > d.thr32;
+    if (!k && m > 0.0f) k = keep_exact<double2>(d, a);
+    return k;
+}
+__device__ __forceinline__ bool pos_keep(const QwSimDev &d, float2 a) { return Amp<float2>::keep(d, a); }
+
+/* both rows of a slot where the FP32 bounds leave a decision open: the kept
+   flags by the exact values (bits 0, 1: u, v; bit 2: a non-zero one dropped) */
+template <typename AmpT>
+__device__ __noinline__ void negate_exact(const QwSimDev &d, typename Amp<AmpT>::RotVal t, uint32_t A, bool sneg,
+                                          AmpT q0, AmpT q1, AmpT &r0, AmpT &r1, unsigned &kept)
+{
+    const unsigned e = pair_exact<AmpT>(d, t, A, sneg, q0, q1);
+    kept = (e & 1u) + ((e >> 1) & 1u);
+    if (e & 4u) pair_literal<AmpT>(d, t, A, sneg, q0, q1, (e & 1u) != 0u, (e & 2u) != 0u, false, Amp<AmpT>::zero(), r0, r1);
+}
+
+/* branch counters of a lane, packed 8 bits each (in, rdag, hph, out) so that
+   one predicated addition counts a branch in several; unpacked before a field
+   can overflow */
+constexpr uint32_t kCntIn = 1u, kCntRdag = 1u << 8, kCntHph = 1u << 16, kCntOut = 1u << 24;
+struct PosStats {
+    unsigned int rows = 0, in = 0, rdag = 0, hph = 0, out = 0;
+    __device__ __forceinline__ void take(uint32_t &c)
+    {
+        in += c & 0xffu;
+        rdag += (c >> 8) & 0xffu;
+        hph += (c >> 16) & 0xffu;
+        out += c >> 24;
+        c = 0;
+    }
+    __device__ void flush(const QwStepArgs &a)
+    {
+        unsigned int v[5] = {rows, in, rdag, hph, out};
+#pragma unroll
+        for (int i = 0; i < 5; ++i) v[i] = __reduce_add_sync(FULL, v[i]);
+        if (a.stats && lane_id() == 0 && v[1]) {
+            atomicAdd(a.stats + QW_STAT_ROWS, (unsigned long long)v[0]);
+            atomicAdd(a.stats + QW_STAT_IN, (unsigned long long)v[1]);
+            atomicAdd(a.stats + QW_STAT_RDAG, (unsigned long long)v[2]);
+            atomicAdd(a.stats + QW_STAT_HPH, (unsigned long long)v[3]);
+            atomicAdd(a.stats + QW_STAT_OUT, (unsigned long long)v[4]);
+        }
+    }
+};
+
+template <typename AmpT, int S, bool FULLST, bool TAB>
+__global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, QwPosArgs p, QwStepArgs a)
+{
+    typedef typename Amp<AmpT>::RotVal RotVal;
+    /* a unit (one j) on SW lanes, each lane holding SPL of its slots (l = lb
+       + 32 k); RPP units per warp (a group) */
+    constexpr int SW = S > 32 ? 32 : S, SPL = S / SW, RPP = 32 / SW;
+    constexpr int LOG2S = S == 8 ? 3 : S == 16 ? 4 : S == 32 ? 5 : 6;
+    constexpr float kHalfS = 0.5f * S, kErr = Amp<AmpT>::kApproxErr;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ unsigned long long part_u[kPosMaxWarps];
+    __shared__ double part_d[kPosMaxWarps];
+    __shared__ double scale_sm;
+    __shared__ PosNorm pn;
+    __shared__ int flag_sm, bad_sm;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, PW = blockDim.x >> 5;
+    if (*(volatile int32_t *)a.status != 0) return; /* after a failed step: nothing (the whole grid alike) */
+    const bool rot_in_place = Amp<AmpT>::kRotCode && d.rot_calc;
+    const AmpT zero = Amp<AmpT>::zero();
+    const uint32_t n = (uint32_t)d.pos_rows, T = (uint32_t)d.pos_T; /* rows, entries; 4 T < 2^31 */
+    const uint32_t X = T - n * S;                                     /* extras */
+    const uint32_t ngroups = (n + RPP - 1) / RPP, xgroups = (X + 31) / 32, nwarps = gridDim.x * PW;
+    const uint32_t g0 = blockIdx.x * PW + warp, x0 = nwarps - 1 - g0; /* extras from the last warp down */
+    const int ul = lane / SW, lb = lane % SW;
+
+    /* per-launch tables of the block's groups, [turn][warp] */
+    const uint32_t turns = (ngroups + nwarps - 1) / nwarps, xturns = (xgroups + nwarps - 1) / nwarps;
+    RotVal *t_rot = reinterpret_cast<RotVal *>(smem);
+    uint32_t *t_dst = reinterpret_cast<uint32_t *>(t_rot + (size_t)turns * PW * 32 * SPL);
+    uint32_t *t_x = t_dst + (size_t)turns * PW * 32 * SPL;
+    /* a slot's rotation, its destination entry with flags: bit 31 sigma = -1,
+       bit 30 a negative element */
+    auto slot_table = [&](uint32_t at, RotVal &t, uint32_t &dst) {
+        const uint32_t w = __ldg(d.img + at), val = w & 0xffffu;
+        /* a 0 element rotates by R(0) */
+        t = val == 0 ? Amp<AmpT>::rot_zero()
+                     : (rot_in_place ? Amp<AmpT>::rot_code(val) : __ldg(static_cast<const RotVal *>(d.slot_rot) + at));
+        dst = __ldg(d.pos_dst + at) | ((val & 0x8000u) << 15);
+    };
+    if (TAB) {
+        for (uint32_t k = 0; k < turns; ++k) {
+            const uint32_t g = g0 + k * nwarps, jj = g * RPP + ul;
+#pragma unroll
+            for (int q = 0; q < SPL; ++q) {
+                RotVal t = Amp<AmpT>::rot_zero();
+                uint32_t dst = 0;
+                if (g < ngroups && jj < n) slot_table(jj * S + lb + 32 * q, t, dst);
+                const uint32_t at = ((k * PW + warp) * SPL + q) * 32 + lane;
+                t_rot[at] = t;
+                t_dst[at] = dst;
+            }
+        }
+        for (uint32_t k = 0; k < xturns; ++k) {
+            const uint32_t x = (x0 + k * nwarps) * 32 + lane;
+            t_x[(k * PW + warp) * 32 + lane] = x < X ? __ldg(d.pos_xdst + x) : 0u;
+        }
+        __syncwarp(); /* a warp reads only what it wrote */
+    }
+
+    /* a group's state, loaded one group ahead */
+    struct In {
+        AmpT a0[SPL], a1[SPL], q0[SPL], q1[FULLST ? SPL : 1];
+    };
+    auto fetch = [&](const AmpT *A, uint32_t gg, In &x) {
+        const uint32_t jj = gg * RPP + ul;
+        const bool have = gg < ngroups && jj < n;
+        const uint32_t i0 = jj * S + lb;
+#pragma unroll
+        for (int q = 0; q < SPL; ++q) {
+            x.a0[q] = x.a1[q] = x.q0[q] = zero;
+            if (FULLST) x.q1[q] = zero;
+            if (have) {
+                const uint32_t i = i0 + 32 * q;
+                pos_load2(A + 2 * i, x.a0[q], x.a1[q]);
+                x.q0[q] = __ldcg(A + 2 * T + i);
+                if (FULLST) x.q1[q] = __ldcg(A + 3 * T + i);
+            }
+        }
+    };
+
+    PosStats st;
+    uint32_t cnt = 0;
+    const AmpT *A = static_cast<const AmpT *>(p.in); /* planes A, B0 (at 2 T), B1 (at 3 T) */
+    bool rescale = a.scale_in != nullptr;
+    if (threadIdx.x == 0) {
+        Amp<AmpT>::Scale::to_shared(rescale ? *a.scale_in : 1.0, &scale_sm);
+        if (a.renorm) pos_norm_setup(a, pn);
+        bad_sm = 0;
+    }
+    __syncthreads();
+    for (int step = 0; step < p.nsteps; ++step) {
+        AmpT *O = static_cast<AmpT *>((step & 1) ? p.out1 : p.out0);
+        const bool readout = p.qls ? (step & 1) != 0 : a.qls_readout != 0;
+        double unit = 0.0, pshare = 0.0;
+        if (readout) /* u here is scaled by 2 / s */
+            unit = (p.qls ? a.qls_coefs[p.qls_term + (step >> 1)] : a.qls_coefs[*a.qls_j]) * (d.inv_sqrt_s * (0.5 * S));
+        const typename Amp<AmpT>::Scale scale = Amp<AmpT>::Scale::from_shared(&scale_sm);
+        typename Amp<AmpT>::Norm nrm;
+        In nxt;
+        fetch(A, g0, nxt);
+        for (uint32_t k = 0, g = g0; g < ngroups; ++k, g += nwarps) {
+            const In cur = nxt;
+            fetch(A, g + nwarps, nxt);
+            const uint32_t j = g * RPP + ul;
+            const bool valid = j < n;
+            RotVal rv[SPL];
+            uint32_t dst[SPL];
+#pragma unroll
+            for (int q = 0; q < SPL; ++q) {
+                if (TAB) {
+                    const uint32_t at = ((k * PW + warp) * SPL + q) * 32 + lane;
+                    rv[q] = t_rot[at];
+                    dst[q] = t_dst[at];
+                } else {
+                    rv[q] = Amp<AmpT>::rot_zero();
+                    dst[q] = 0;
+                    if (valid) slot_table(j * S + lb + 32 * q, rv[q], dst[q]);
+                }
+            }
+            AmpT a0[SPL], a1[SPL], q0[SPL], q1[SPL];
+            float A0[SPL], A1[SPL], Q0[SPL];
+            bool any = false;
+#pragma unroll
+            for (int q = 0; q < SPL; ++q) {
+                a0[q] = cur.a0[q];
+                a1[q] = cur.a1[q];
+                q0[q] = cur.q0[q];
+                q1[q] = FULLST ? cur.q1[q] : zero;
+                if (rescale) {
+                    a0[q] = scale.apply(a0[q]);
+                    a1[q] = scale.apply(a1[q]);
+                    q0[q] = scale.apply(q0[q]);
+                    if (FULLST) q1[q] = scale.apply(q1[q]);
+                }
+                A0[q] = Amp<AmpT>::inf_norm(a0[q]);
+                A1[q] = Amp<AmpT>::inf_norm(a1[q]);
+                Q0[q] = Amp<AmpT>::inf_norm(q0[q]);
+                const bool n0 = A0[q] != 0.0f, n1 = A1[q] != 0.0f, m0 = Q0[q] != 0.0f, m1 = FULLST && nz(q1[q]) != 0u;
+                if (n0) cnt += kCntIn;
+                if (n1) cnt += kCntIn;
+                if (m0) cnt += kCntIn;
+                if (m1) cnt += kCntIn;
+                any = any || n0 || n1 || m0 || m1;
+            }
+            {
+                const unsigned m = __ballot_sync(FULL, any);
+                const unsigned um = SW == 32 ? m : (m >> (ul * SW)) & ((1u << (SW & 31)) - 1u);
+                if (lb == 0 && um != 0) st.rows += 1; /* units holding branches */
+            }
+            /* b1 = 0: R^dag's b2 = 0 output u (its exact value, scaled by 2 / s),
+               and whether u and v are kept: |v| >= | f |a1| - g |a0| | in the
+               maximum norm, which the phases leave alone, so the norms decide
+               unless they nearly cancel */
+            typename Amp<AmpT>::Wide u[SPL];
+            PairState<AmpT> ps[SPL];
+            float f[SPL], g_[SPL], U[SPL];
+#pragma unroll
+            for (int q = 0; q < SPL; ++q) {
+                const uint32_t sgn = (dst[q] & 0x40000000u) >> 15; /* the value's sign bit (bit 15) */
+                const bool sneg = (dst[q] >> 31) != 0u;
+                f[q] = Amp<AmpT>::rot_f(rv[q]);
+                g_[q] = Amp<AmpT>::rot_g(rv[q]);
+                u[q] = Amp<AmpT>::rdag0(Amp<AmpT>::prescale(rv[q], LOG2S - 1), sgn, sneg, a0[q], a1[q]);
+                U[q] = kHalfS * Amp<AmpT>::inf_norm(Amp<AmpT>::narrow(u[q]));
+                const float fa = f[q] * A1[q], ga = g_[q] * A0[q];
+                ps[q].c0 = U[q] > d.thr32;
+                ps[q].c1 = fabsf(fa - ga) > fmaf(kErr, fa + ga, d.thr32);
+                ps[q].lossy = false;
+                if ((!ps[q].c0 && U[q] > 0.0f) || (!ps[q].c1 && fa + ga > 0.0f)) {
+                    const unsigned e = pair_exact<AmpT>(d, rv[q], sgn, sneg, a0[q], a1[q]);
+                    ps[q].c0 = (e & 1u) != 0u;
+                    ps[q].c1 = (e & 2u) != 0u;
+                    ps[q].lossy = (e & 4u) != 0u;
+                    if (!ps[q].c0) {
+                        u[q] = Amp<AmpT>::wide_zero();
+                        U[q] = 0.0f;
+                    }
+                }
+                if (ps[q].c0) cnt += kCntRdag;
+                if (ps[q].c1) cnt += kCntRdag + kCntHph;
+            }
+            __syncwarp();
+            typename Amp<AmpT>::Sum sum;
+            sum.set(u[0]);
+#pragma unroll
+            for (int q = 1; q < SPL; ++q) sum.add(u[q]);
+            sum.reduce(SW, SW);
+            if (readout && valid && lb == 0) { /* flag-0 amplitude (1/sqrt s) sum u: the QLS accumulator */
+                const double2 sv = sum.value();
+                pshare += pos_readout(a.qls_y + j, unit, sv.x, sv.y);
+            }
+            const float Rn = Amp<AmpT>::inf_norm(Amp<AmpT>::sum_amp(sum));
+#pragma unroll
+            for (int q = 0; q < SPL; ++q) {
+                const uint32_t sgn = (dst[q] & 0x40000000u) >> 15, to = dst[q] & 0x3fffffffu;
+                const bool sneg = (dst[q] >> 31) != 0u;
+                /* the reflected r - u, then R: (f r - a0, g r - a1) */
+                AmpT rA0, rA1;
+                bool d0 = fabsf(Rn - U[q]) > fmaf(kErr, Rn + U[q], d.thr32);
+                Amp<AmpT>::reflect(sum, rv[q], sgn, sneg, a0[q], a1[q], rA0, rA1);
+                if (ps[q].lossy || (!d0 && Rn + U[q] > 0.0f))
+                    d0 = pair_reflect_exact<AmpT>(d, sum, rv[q], sgn, sneg, a0[q], a1[q], ps[q], rA0, rA1);
+                if (d0) cnt += kCntHph;
+                /* b1 = 1: R^dag, -1, R */
+                AmpT rB0 = Amp<AmpT>::neg(q0[q]), rB1 = Amp<AmpT>::neg(q1[q]);
+                if (FULLST) {
+                    const unsigned kept = pair_negate<AmpT>(d, rv[q], sgn, sneg, q0[q], q1[q], rB0, rB1);
+                    cnt += kept * (kCntRdag + kCntHph);
+                } else { /* q1 = 0: |u| = f |q0|, |v| = g |q0| */
+                    const float fq = f[q] * Q0[q], gq = g_[q] * Q0[q], lim = fmaf(kErr, Q0[q], d.thr32);
+                    const bool c0 = fq > lim, c1 = gq > lim;
+                    unsigned kept = (c0 ? 1u : 0u) + (c1 ? 1u : 0u);
+                    if ((!c0 && fq > 0.0f) || (!c1 && gq > 0.0f))
+                        negate_exact<AmpT>(d, rv[q], sgn, sneg, q0[q], zero, rB0, rB1, kept);
+                    cnt += kept * (kCntRdag + kCntHph);
+                }
+                const bool eA0 = pos_keep(d, rA0), eA1 = pos_keep(d, rA1);
+                const bool eB0 = pos_keep(d, rB0), eB1 = FULLST && pos_keep(d, rB1);
+                if (valid) {
+                    if (a.renorm) {
+                        if (eA0) norm_add(nrm, rA0);
+                        if (eB0) norm_add(nrm, rB0);
+                        if (eA1) norm_add(nrm, rA1);
+                        if (FULLST && eB1) norm_add(nrm, rB1);
+                    }
+                    pos_store2(O + 2 * to, eA0 ? rA0 : zero, eB0 ? rB0 : zero);
+                    __stcg(O + 2 * T + to, eA1 ? rA1 : zero);
+                    if (FULLST) __stcg(O + 3 * T + to, eB1 ? rB1 : zero);
+                }
+                if (eA0) cnt += kCntOut;
+                if (eB0) cnt += kCntOut;
+                if (eA1) cnt += kCntOut;
+                if (eB1) cnt += kCntOut;
+            }
+            if ((k & 7u) == 7u) st.take(cnt);
+        }
+        st.take(cnt);
+        /* the extras, 32 at a time */
+        for (uint32_t k = 0, x = x0 * 32 + lane; k < xturns; ++k, x += nwarps * 32) {
+            if (x >= X) break;
+            const uint32_t i = n * S + x;
+            const uint32_t to = TAB ? t_x[(k * PW + warp) * 32 + lane] : __ldg(d.pos_xdst + x);
+            AmpT a0, a1, q0 = __ldcg(A + 2 * T + i), q1 = FULLST ? __ldcg(A + 3 * T + i) : zero;
+            pos_load2(A + 2 * i, a0, a1);
+            if (rescale) {
+                a0 = scale.apply(a0);
+                a1 = scale.apply(a1);
+                q0 = scale.apply(q0);
+                if (FULLST) q1 = scale.apply(q1);
+            }
+            const bool k0 = pos_keep(d, a0), k1 = pos_keep(d, a1), h0 = pos_keep(d, q0), h1 = FULLST && pos_keep(d, q1);
+            const uint32_t kept = (k0 ? 1u : 0u) + (k1 ? 1u : 0u) + (h0 ? 1u : 0u) + (h1 ? 1u : 0u);
+            cnt += (nz(a0) + nz(a1) + nz(q0) + (FULLST ? nz(q1) : 0u)) * kCntIn + kept * (kCntRdag + kCntHph + kCntOut);
+            if (a.renorm) {
+                if (k0) norm_add(nrm, a0);
+                if (k1) norm_add(nrm, a1);
+                if (h0) norm_add(nrm, q0);
+                if (FULLST && h1) norm_add(nrm, q1);
+            }
+            pos_store2(O + 2 * to, k0 ? Amp<AmpT>::neg(a0) : zero, h0 ? Amp<AmpT>::neg(q0) : zero);
+            __stcg(O + 2 * T + to, k1 ? Amp<AmpT>::neg(a1) : zero);
+            if (FULLST) __stcg(O + 3 * T + to, h1 ? Amp<AmpT>::neg(q1) : zero);
+            if ((k & 15u) == 15u) st.take(cnt);
+        }
+        st.take(cnt);
+        __syncwarp();
+        /* the warp's shares of the norm and of ||Y||^2 */
+        if (a.renorm) {
+            bool bad;
+            const unsigned long long v = warp_sum_units(to_units(nrm, pn.unit_inv, bad));
+            if (lane == 0) part_u[warp] = v;
+            if (bad) bad_sm = 1;
+        }
+        if (p.qls && readout) {
+            const double pv = warp_sum(pshare);
+            if (lane == 0) part_d[warp] = pv;
+        }
+        __syncthreads();
+        A = O;
+        const bool last = step == p.nsteps - 1;
+        if (p.words == nullptr) break; /* one step: finished below by the last block */
+        unsigned long long *word = p.words + ((p.epoch + (unsigned long long)step) & 3ull);
+        double *pshares = p.pshare + ((unsigned)(step >> 1) & 1u) * gridDim.x;
+        if (warp == 0) {
+            unsigned long long share = 0;
+            if (a.renorm) share = warp_sum_units(lane < PW ? part_u[lane] : 0ull);
+            if (p.qls && readout) {
+                const double ps = warp_sum(lane < PW ? part_d[lane] : 0.0);
+                if (lane == 0) __stcg(pshares + blockIdx.x, ps);
+            }
+            if (lane == 0) {
+                if (bad_sm || share >= 1ull << (kCountShift - 1)) { /* (the norm stays near the target) */
+                    atomicOr(p.poison, 1u);
+                    share = 0;
+                }
+                __threadfence();
+                word_add(word, (1ull << kCountShift) + share);
+                bool ok = true;
+                if (!last || blockIdx.x == 0) {
+                    unsigned long long w = 0;
+                    ok = false;
+                    for (int polls = 0; polls < (1 << 22) && !ok; ++polls) {
+                        w = word_load(word);
+                        ok = (w >> kCountShift) == (unsigned long long)gridDim.x;
+                    }
+                    if (!ok) atomicOr(a.status, QW_ST_GRID_WAIT);
+                    if (ok && blockIdx.x == 0) p.words[(p.epoch + (unsigned long long)step + 2ull) & 3ull] = 0ull;
+                    double fac = 1.0;
+                    if (a.renorm) {
+                        const unsigned long long sum = w & kShareMask;
+                        float c;
+                        if (pos_scale(pn, sum, c)) {
+                            Amp<AmpT>::scale_one_plus(c, &scale_sm);
+                            if (last) fac = 1.0 + (double)c;
+                        } else {
+                            const bool nan = *(volatile unsigned int *)p.poison != 0u;
+                            fac = nan ? 1.0 : pos_scale_exact(*a.renorm_target, (double)sum / pn.unit_inv);
+                            Amp<AmpT>::Scale::to_shared(fac, &scale_sm);
+                        }
+                    }
+                    if (last && ok) {
+                        *p.poison = 0u;
+                        *a.norm_out = a.renorm ? (double)(w & kShareMask) / pn.unit_inv : 0.0;
+                        if (a.scale_out) *a.scale_out = fac;
+                        if (a.steps_done) *a.steps_done += p.nsteps;
+                        if (a.stats) a.stats[QW_STAT_STEPS] += p.nsteps;
+                    }
+                }
+                flag_sm = ok ? 1 : 0;
+            }
+        }
+        __syncthreads();
+        if (flag_sm == 0) break;
+        rescale = a.renorm != 0;
+        /* p_j = ||Y||^2 of the term: the shares of all blocks, by one warp of a
+           block that changes from term to term, while the others go on */
+        if (p.qls && readout && warp == PW - 1) {
+            const unsigned who = last ? 0u : (unsigned)(step >> 1) % gridDim.x;
+            if (blockIdx.x == who) {
+                double v = 0.0;
+                for (unsigned b = lane; b < gridDim.x; b += 32) v += __ldcg(pshares + b);
+                v = warp_sum(v);
+                if (lane == 0) a.qls_p[p.qls_term + (step >> 1)] = v;
+            }
+        }
+    }
+    st.flush(a);
+    if (p.words != nullptr) return;
+
+    /* one step: the block's share of the norm, the last block reduces */
+    if (warp == 0) {
+        unsigned long long share = 0;
+        if (a.renorm) share = warp_sum_units(lane < PW ? part_u[lane] : 0ull);
+        if (lane == 0) {
+            a.partials[blockIdx.x] = bad_sm ? -1.0 : (double)share;
+            __threadfence();
+            const unsigned prev = atomicAdd(a.done_ctr, 1u);
+            flag_sm = prev == gridDim.x - 1;
+        }
+        __syncwarp();
+        if (!flag_sm) return;
+        __threadfence();
+        double v = 0.0;
+        bool bad = false;
+        if (a.renorm) {
+            for (unsigned bb = lane; bb < gridDim.x; bb += 32) {
+                const double w = __ldcg(a.partials + bb);
+                bad = bad || w < 0.0;
+                v += w;
+            }
+            v = warp_sum(v);
+            bad = __any_sync(FULL, bad);
+        }
+        if (lane == 0) {
+            if (*(volatile int32_t *)a.status == 0) {
+                const double norm = a.renorm ? v / pn.unit_inv : 0.0;
+                *a.norm_out = norm;
+                if (a.scale_out) *a.scale_out = a.renorm && !bad ? pos_scale_exact(*a.renorm_target, norm) : 1.0;
+                if (a.steps_done) *a.steps_done += 1;
+                if (a.stats) a.stats[QW_STAT_STEPS] += 1;
+            }
+            *a.done_ctr = 0u;
+        }
+    }
+}
+
+/* T~|b~> written straight into rows g0 .. g0 + n (one instance): |b~> holds one
+ * branch per row, a = b_j (divided by the pending renormalisation factor when
+ * other instances share the state); T~'s Hadamard gives (l, z = 0) with
+ * a / sqrt(s) for every slot l, its maps take slot l to k = col(j, l), and
+ * R(A_jl) on (a / sqrt(s), 0) gives the pair of the slot's entry in plane A --
+ * the arithmetic of k_tinit.  B0 of the slots and both planes of the rows'
+ * extras (x0 .. x0 + nx) are written 0.  One thread per entry: bound by the
+ * writes. */
+template <typename AmpT>
+__global__ void k_tinit_pos(QwSimDev d, AmpT *pbuf, uint32_t g0, uint32_t n, uint32_t x0, uint32_t nx,
+                            const double *b_re, const double *b_im, const double *scale)
+{
+    typedef typename Amp<AmpT>::RotVal RotVal;
+    const uint32_t S = (uint32_t)d.s, T = (uint32_t)d.pos_T, ns = n * S, total = ns + nx;
+    const AmpT zero = Amp<AmpT>::zero();
+    const bool rot_in_place = Amp<AmpT>::kRotCode && d.rot_calc;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        AmpT o0 = zero, o1 = zero;
+        uint32_t at = (uint32_t)d.pos_rows * S + x0 + (i - ns);
+        if (i < ns) {
+            const uint32_t j = i / S;
+            at = g0 * S + i;
+            double2 v = make_double2(b_re[j], b_im ? b_im[j] : 0.0);
+            if (scale) v = make_double2(v.x / *scale, v.y / *scale);
+            const double2 a = Amp<AmpT>::to_d(Amp<AmpT>::from_d(v)); /* as stored by |b~> */
+            const AmpT h = Amp<AmpT>::from_d(make_double2(d.inv_sqrt_s * a.x, d.inv_sqrt_s * a.y));
+            if ((v.x != 0.0 || v.y != 0.0) && Amp<AmpT>::keep(d, h)) {
+                const uint32_t w = __ldg(d.img + at), val = w & 0xffffu;
+                const RotVal rv = val == 0 ? Amp<AmpT>::rot_zero()
+                                           : (rot_in_place ? Amp<AmpT>::rot_code(val)
+                                                           : __ldg(static_cast<const RotVal *>(d.slot_rot) + at));
+                Amp<AmpT>::rot(rv, val, false, j > (w >> 16), h, zero, o0, o1); /* R */
+                if (!Amp<AmpT>::keep(d, o0)) o0 = zero;
+                if (!Amp<AmpT>::keep(d, o1)) o1 = zero;
+            }
+        }
+        pos_store2(pbuf + 2 * (size_t)at, o0, o1);
+        pbuf[2 * (size_t)T + at] = zero;
+    }
+}
+
+/* |a|^2 in FP64 */
+template <typename AmpT> __device__ __forceinline__ double amp_norm2(AmpT a)
+{
+    if (nz(a) == 0u) return 0.0;
+    const double2 v = Amp<AmpT>::to_d(a);
+    return fma(v.x, v.x, v.y * v.y);
+}
+
+/* Marginal of one register over rows g0 .. g0 + n (the key of an entry: jc =
+ * kc = 0, j = its row, b1 and b2 by plane, k = the slot's column or the
+ * extra's row), one warp per row.  j: the row's own entries.  k: a gather
+ * instead of an atomic per branch -- the branches with k = v sit at dst(v, l)
+ * for every slot l of row v (the entry of k = v in row col(v, l)) and at slot
+ * (x, l_x) for every extra x of row v.  The other registers: the sums by plane,
+ * one atomic per block. */
+template <typename AmpT>
+__global__ void __launch_bounds__(256) k_measure_pos(QwSimDev d, const AmpT *pbuf, int full, int64_t g0, int64_t n,
+                                                     const double *scale, int reg, double *probs, int64_t len)
+{
+    __shared__ double acc_sm[4][8];
+    const uint32_t S = (uint32_t)d.s, T = (uint32_t)d.pos_T, N = (uint32_t)d.pos_rows;
+    const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
+    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const double sc = scale ? *scale * *scale : 1.0;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0}; /* by (b1, b2) */
+    for (int64_t j = warp; j < n; j += nw) {
+        const uint32_t g = (uint32_t)(g0 + j), x0 = __ldg(d.pos_xptr + g), P = S + __ldg(d.pos_xptr + g + 1) - x0;
+        double row = 0.0;
+        for (uint32_t i = lane; i < P; i += 32) {
+            uint32_t at = i < S ? g * S + i : N * S + x0 + (i - S);
+            if (reg == 4) at = i < S ? (__ldg(d.pos_dst + at) & 0x3fffffffu) : __ldg(d.pos_xdst + x0 + (i - S));
+            AmpT a0, a1;
+            pos_load2(pbuf + 2 * (size_t)at, a0, a1);
+            const AmpT q0 = pbuf[2 * (size_t)T + at];
+            const double p[4] = {amp_norm2(a0), amp_norm2(a1), amp_norm2(q0),
+                                 full ? amp_norm2(pbuf[3 * (size_t)T + at]) : 0.0};
+            if (reg == 1 || reg == 4) {
+                row += (p[0] + p[1]) + (p[2] + p[3]);
+            } else {
+#pragma unroll
+                for (int t = 0; t < 4; ++t) acc[t] += p[t];
+            }
+        }
+        if (reg == 1 || reg == 4) {
+            row = warp_sum(row);
+            if (lane == 0 && j < len) probs[j] = sc * row;
+        }
+    }
+    if (reg == 1 || reg == 4) return;
+    for (int t = 0; t < 4; ++t) {
+        acc[t] = warp_sum(acc[t]);
+        if (lane == 0) acc_sm[t][wb] = acc[t];
+    }
+    __syncthreads();
+    if (threadIdx.x < 4) {
+        double v = 0.0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += acc_sm[threadIdx.x][w];
+        const int b1 = threadIdx.x >> 1, b2 = threadIdx.x & 1;
+        const int64_t bin = reg == 2 ? b1 : reg == 5 ? b2 : 0; /* jc = kc = 0 */
+        if (bin < len && v != 0.0) atomicAdd(probs + bin, sc * v);
+    }
+}
+
+/* the row buckets into the positional layout (pbuf zeroed by the caller):
+   one thread per bucket slot; a branch in B1 sets QW_ST_POS_FULL */
+template <typename AmpT>
+__global__ void k_pos_pack(QwSimDev d, QwBufDev buf, AmpT *pbuf, int32_t *status)
+{
+    const int S = d.s;
+    AmpT *B0 = pbuf + 2 * d.pos_T, *B1 = pbuf + 3 * d.pos_T;
+    const int64_t total = d.total_buckets * (int64_t)d.cap_row;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t b = i / d.cap_row;
+        const int p = (int)(i - b * d.cap_row);
+        if (p >= buf.count[b]) continue;
+        if (b >= d.dense_buckets) { /* a row with jc != 0 */
+            atomicOr(status, QW_ST_POS_UNREP);
+            continue;
+        }
+        int64_t j = b >> 1, n = d.n_single, g0 = 0;
+        if (d.ninst > 1) {
+            const int inst = d.unit_inst[b >> 1];
+            j = (b - d.inst_bkt[inst]) >> 1;
+            n = d.inst_n[inst];
+            g0 = d.inst_img[inst] / S;
+        }
+        if (j >= n) { /* a row j >= N */
+            atomicOr(status, QW_ST_POS_UNREP);
+            continue;
+        }
+        const int64_t gr = g0 + j; /* the row among all instances' rows */
+        const Regs x = decode_r(buf.key[i], d.nb);
+        int64_t at = -1;
+        if (x.kc == 0 && x.A == 0) {
+            const uint32_t *row = d.img + gr * S;
+            int lo = 0, hi = S; /* lower bound of k among the row's sorted columns */
+            while (lo < hi) {
+                const int m = (lo + hi) >> 1;
+                if ((row[m] >> 16) < x.k) lo = m + 1;
+                else hi = m;
+            }
+            if (lo < S && (row[lo] >> 16) == x.k) {
+                at = gr * S + lo;
+            } else {
+                for (uint32_t e = d.pos_xptr[gr]; e < d.pos_xptr[gr + 1]; ++e)
+                    if (d.pos_xdst[e] / (uint32_t)S - g0 == x.k) {
+                        at = d.pos_rows * S + e;
+                        break;
+                    }
+            }
+        }
+        if (at < 0) {
+            atomicOr(status, QW_ST_POS_UNREP);
+            continue;
+        }
+        const AmpT v = static_cast<const AmpT *>(buf.amp)[i];
+        if ((b & 1) == 0) {
+            pbuf[2 * at + x.b2] = v;
+        } else if (x.b2 == 0) {
+            B0[at] = v;
+        } else {
+            B1[at] = v;
+            if (nz(v)) atomicOr(status, QW_ST_POS_FULL);
+        }
+    }
+}
+
+/* the positional layout into the row buckets (cleared by the caller): one
+   thread per entry and plane, non-zero amplitudes appended to their row */
+template <typename AmpT>
+__global__ void k_pos_unpack(QwSimDev d, const AmpT *pbuf, int full, QwBufDev buf, int32_t *status)
+{
+    const int64_t S = d.s, T = d.pos_T, total = (full ? 4 : 3) * T;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const AmpT v = pbuf[i];
+        if (v.x == 0 && v.y == 0) continue;
+        const int b1 = i >= 2 * T ? 1 : 0;
+        const int64_t at = b1 ? (i >= 3 * T ? i - 3 * T : i - 2 * T) : i >> 1;
+        int64_t gr = at / S; /* the row among all instances' rows */
+        uint32_t k;          /* the branch's k, a row among all instances' for an extra */
+        if (gr < d.pos_rows) {
+            k = d.img[at] >> 16;
+        } else { /* the extra's row: the last one whose extras start at or before it */
+            const uint32_t e = (uint32_t)(at - d.pos_rows * S);
+            int64_t lo = 0, hi = d.pos_rows - 1;
+            while (lo < hi) {
+                const int64_t m = (lo + hi + 1) >> 1;
+                if (d.pos_xptr[m] <= e) lo = m;
+                else hi = m - 1;
+            }
+            gr = lo;
+            k = d.pos_xdst[e] / (uint32_t)S;
+        }
+        int64_t g0 = 0, b = 2 * gr + b1; /* the instance's first row; the bucket */
+        if (d.ninst > 1) {
+            const int inst = d.pos_rowinst[gr];
+            g0 = d.inst_img[inst] / S;
+            b = d.inst_bkt[inst] + 2 * (gr - g0) + b1;
+        }
+        Regs x;
+        x.kc = 0;
+        x.A = 0;
+        x.b2 = b1 ? (i >= 3 * T ? 1u : 0u) : (uint32_t)(i & 1);
+        x.k = at < d.pos_rows * S ? k : k - (uint32_t)g0;
+        const int p = atomicAdd(buf.count + b, 1);
+        if (p >= d.cap_row) {
+            atomicOr(status, QW_ST_ROW_OVERFLOW);
+            continue;
+        }
+        const int64_t sl = b * d.cap_row + p;
+        buf.key[sl] = encode_r(x, d.nb);
+        static_cast<AmpT *>(buf.amp)[sl] = v;
+    }
+}
+
+/* ---- launch shapes ------------------------------------------------------------- */
+
+template <typename AmpT, bool FULLST, bool TAB>
+void *pos_kernel(int s)
+{
+    if (s == 8) return (void *)k_walk_pos<AmpT, 8, FULLST, TAB>;
+    if (s == 16) return (void *)k_walk_pos<AmpT, 16, FULLST, TAB>;
+    if (s == 32) return (void *)k_walk_pos<AmpT, 32, FULLST, TAB>;
+    return (void *)k_walk_pos<AmpT, 64, FULLST, TAB>;
+}
+
+/* One block per SM: every group of rows has a warp within a few turns, with
+ * as many groups for each warp as for the others (54 groups an SM at N =
+ * 16384, s = 16: 4 turns of 14 warps instead of 16, 16, 16, 6); the tables
+ * fit shared memory up to about 300 groups a block (46 000 in all).  At least
+ * 4 warps a block, one per scheduler. */
+template <typename AmpT>
+QwPosPlan pos_plan(const QwSimDev &d)
+{
+    QwPosPlan pl{};
+    const int s = d.s, rpp = s >= 32 ? 1 : 32 / s, spl = s > 32 ? s / 32 : 1;
+    const int64_t xgroups = (d.pos_T - d.pos_rows * s + 31) / 32;
+    const int64_t groups = (d.pos_rows + rpp - 1) / rpp, sms = qw_sm_count();
+    const int64_t per_sm = (groups + sms - 1) / sms;
+    const int64_t turns = (per_sm + kPosMaxWarps - 1) / kPosMaxWarps;
+    int64_t pw = (per_sm + turns - 1) / turns;
+    if (pw < 4) pw = 4;
+    int64_t grid = (groups + pw * turns - 1) / (pw * turns);
+    if (grid > sms) grid = sms;
+    pl.warps = (int)pw;
+    pl.grid = (int)(grid < 1 ? 1 : grid);
+    const int64_t t = (groups + pl.grid * pw - 1) / (pl.grid * pw);
+    const int64_t xt = (xgroups + pl.grid * pw - 1) / (pl.grid * pw);
+    pl.smem = (size_t)(t * pw * 32) * (size_t)(spl * 20) + (size_t)(xt * pw * 32) * 4;
+    int dev = 0, optin = 0, coop = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    pl.tab = pl.smem + 1024 <= (size_t)optin; /* beside the kernel's static arrays */
+    if (!pl.tab) pl.smem = 0;
+    pl.coop = coop != 0 && pl.grid < 256; /* the barrier word's count has 8 bits */
+    if (pl.tab) cudaFuncSetAttribute(pos_kernel<AmpT, false, true>(s), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
+    return pl;
+}
+
+template <typename AmpT>
+cudaError_t launch_pos_t(const QwSimDev &d, const QwPosPlan &pl, const QwPosArgs &p, const QwStepArgs &a, int full,
+                         cudaStream_t st)
+{
+    /* one step reads each table entry once: straight from memory */
+    const bool tab = pl.tab && p.nsteps > 1 && !full;
+    void *k = full ? pos_kernel<AmpT, true, false>(d.s)
+                   : (tab ? pos_kernel<AmpT, false, true>(d.s) : pos_kernel<AmpT, false, false>(d.s));
+    QwSimDev dd = d;
+    QwPosArgs pp = p;
+    QwStepArgs aa = a;
+    void *args[] = {&dd, &pp, &aa};
+    const dim3 grid((unsigned)pl.grid), block((unsigned)pl.warps * 32);
+    if (p.words) return cudaLaunchCooperativeKernel(k, grid, block, args, tab ? pl.smem : 0, st);
+    return cudaLaunchKernel(k, grid, block, args, 0, st);
+}
+
+template <typename AmpT>
+cudaError_t launch_tinit_pos_t(const QwSimDev &d, void *pbuf, int64_t g0, int64_t n, int64_t x0, int64_t nx,
+                               const double *b_re, const double *b_im, const double *scale, cudaStream_t st)
+{
+    const int64_t want = (n * d.s + nx + 255) / 256, cap = 16 * (int64_t)qw_sm_count();
+    k_tinit_pos<AmpT><<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(
+        d, static_cast<AmpT *>(pbuf), (uint32_t)g0, (uint32_t)n, (uint32_t)x0, (uint32_t)nx, b_re, b_im, scale);
+    return cudaGetLastError();
+}
+
+template <typename AmpT>
+cudaError_t launch_measure_pos_t(const QwSimDev &d, const void *pbuf, int full, int64_t g0, int64_t n,
+                                 const double *scale, int reg, double *probs, int64_t len, cudaStream_t st)
+{
+    /* a warp per j: enough blocks that every j's loads are in flight at once;
+       the plane sums with one atomic per block: fewer blocks */
+    const int64_t want = (n + 7) / 8, cap = (reg == 1 || reg == 4 ? 32 : 4) * (int64_t)qw_sm_count();
+    k_measure_pos<AmpT><<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(
+        d, static_cast<const AmpT *>(pbuf), full, g0, n, scale, reg, probs, len);
+    return cudaGetLastError();
+}
+
+template <typename AmpT>
+cudaError_t launch_pos_pack_t(const QwSimDev &d, const QwBufDev &buf, void *pbuf, int32_t *status, cudaStream_t st)
+{
+    k_pos_pack<AmpT><<<4 * qw_sm_count(), 256, 0, st>>>(d, buf, static_cast<AmpT *>(pbuf), status);
+    return cudaGetLastError();
+}
+
+template <typename AmpT>
+cudaError_t launch_pos_unpack_t(const QwSimDev &d, const void *pbuf, int full, const QwBufDev &buf, int32_t *status,
+                                cudaStream_t st)
+{
+    k_pos_unpack<AmpT><<<4 * qw_sm_count(), 256, 0, st>>>(d, static_cast<const AmpT *>(pbuf), full, buf, status);
+    return cudaGetLastError();
+}
+
+} // namespace
+
+/* the launchers of one precision (declared in qw_internal.h) */
+#define QW_POS_INSTANTIATE(SUFFIX, AmpT)                                                                              \
+    QwPosPlan qw_pos_plan##SUFFIX(const QwSimDev &d) { return pos_plan<AmpT>(d); }                                    \
+    cudaError_t qw_launch_walk_pos##SUFFIX(const QwSimDev &d, const QwPosPlan &pl, const QwPosArgs &p,                \
+                                           const QwStepArgs &a, int full, cudaStream_t st)                            \
+    {                                                                                                                 \
+        return launch_pos_t<AmpT>(d, pl, p, a, full, st);                                                             \
+    }                                                                                                                 \
+    cudaError_t qw_launch_tinit_pos##SUFFIX(const QwSimDev &d, void *pbuf, int64_t g0, int64_t n, int64_t x0,         \
+                                            int64_t nx, const double *b_re, const double *b_im, const double *scale,  \
+                                            cudaStream_t st)                                                          \
+    {                                                                                                                 \
+        return launch_tinit_pos_t<AmpT>(d, pbuf, g0, n, x0, nx, b_re, b_im, scale, st);                               \
+    }                                                                                                                 \
+    cudaError_t qw_launch_measure_pos##SUFFIX(const QwSimDev &d, const void *pbuf, int full, int64_t g0, int64_t n,   \
+                                              const double *scale, int reg, double *probs, int64_t len,               \
+                                              cudaStream_t st)                                                        \
+    {                                                                                                                 \
+        return launch_measure_pos_t<AmpT>(d, pbuf, full, g0, n, scale, reg, probs, len, st);                          \
+    }                                                                                                                 \
+    cudaError_t qw_launch_pos_pack##SUFFIX(const QwSimDev &d, const QwBufDev &buf, void *pbuf, int32_t *status,       \
+                                           cudaStream_t st)                                                           \
+    {                                                                                                                 \
+        return launch_pos_pack_t<AmpT>(d, buf, pbuf, status, st);                                                     \
+    }                                                                                                                 \
+    cudaError_t qw_launch_pos_unpack##SUFFIX(const QwSimDev &d, const void *pbuf, int full, const QwBufDev &buf,      \
+                                             int32_t *status, cudaStream_t st)                                        \
+    {                                                                                                                 \
+        return launch_pos_unpack_t<AmpT>(d, pbuf, full, buf, status, st);                                             \
+    }
+
+#endif /* QW_POS_CUH */
