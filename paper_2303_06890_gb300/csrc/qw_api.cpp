@@ -1551,15 +1551,8 @@ extern "C" int qw_state_init(qw_sim *sim, int32_t inst, const double *b_re, cons
         int64_t g0 = 0;
         for (int i = 0; i < inst; ++i) g0 += sim->n_of[(size_t)i];
         const int64_t x0 = sim->pos_xrow[(size_t)inst], nx = sim->pos_xrow[(size_t)inst + 1] - x0;
-        if (all) {
-            sim->pos_full = false;
-        } else if (sim->pos_full) { /* the instance has no b1 = b2 = 1 branches now */
-            const size_t amp = sim->fp32 ? sizeof(float2) : sizeof(double2), s = (size_t)sim->d.s;
-            unsigned char *B1 = static_cast<unsigned char *>(sim->pbuf[sim->cur]) + 3 * (size_t)sim->d.pos_T * amp;
-            QW_CUDA(sim, cudaMemsetAsync(B1 + (size_t)g0 * s * amp, 0, (size_t)n * s * amp, sim->stream));
-            QW_CUDA(sim, cudaMemsetAsync(B1 + ((size_t)sim->d.pos_rows * s + x0) * amp, 0, (size_t)nx * amp, sim->stream));
-        }
-        QW_CUDA(sim, qw_launch_tinit_pos(sim->d, sim->pbuf[sim->cur], g0, n, x0, nx, dre, dim,
+        if (all) sim->pos_full = false;
+        QW_CUDA(sim, qw_launch_tinit_pos(sim->d, sim->pbuf[sim->cur], sim->pos_full, g0, n, x0, nx, dre, dim,
                                          all ? nullptr : pending_scale(sim), sim->fp32, sim->stream));
         sim->launches++;
         sim->pos_live = true;

@@ -190,14 +190,15 @@ size_t qw_step_smem_bytes(const QwSimDev &d, int fp32, int mode);
    extras), and the conversions
    from and to the row buckets (pack: pbuf zeroed by the caller, a branch
    without a place sets QW_ST_POS_UNREP; unpack: the buckets cleared by the
-   caller); full: plane B1 is in use */
+   caller); full: the state has b1 = b2 = 1
+   branches */
 #define QW_POS_DECLARE(SUFFIX)                                                                                        \
     QwPosPlan qw_pos_plan##SUFFIX(const QwSimDev &d);                                                                 \
     cudaError_t qw_launch_walk_pos##SUFFIX(const QwSimDev &d, const QwPosPlan &pl, const QwPosArgs &p,                \
                                            const QwStepArgs &a, int full, cudaStream_t st);                           \
-    cudaError_t qw_launch_tinit_pos##SUFFIX(const QwSimDev &d, void *pbuf, int64_t g0, int64_t n, int64_t x0,         \
-                                            int64_t nx, const double *b_re, const double *b_im, const double *scale,  \
-                                            cudaStream_t st);                                                         \
+    cudaError_t qw_launch_tinit_pos##SUFFIX(const QwSimDev &d, void *pbuf, int full, int64_t g0, int64_t n,           \
+                                            int64_t x0, int64_t nx, const double *b_re, const double *b_im,           \
+                                            const double *scale, cudaStream_t st);                                                         \
     cudaError_t qw_launch_measure_pos##SUFFIX(const QwSimDev &d, const void *pbuf, int full, int64_t g0, int64_t n,   \
                                               const double *scale, int reg, double *probs, int64_t len,               \
                                               cudaStream_t st);                                                       \
@@ -214,12 +215,12 @@ static inline cudaError_t qw_launch_walk_pos(const QwSimDev &d, const QwPosPlan 
 {
     return fp32 ? qw_launch_walk_pos32(d, pl, p, a, full, st) : qw_launch_walk_pos64(d, pl, p, a, full, st);
 }
-static inline cudaError_t qw_launch_tinit_pos(const QwSimDev &d, void *pbuf, int64_t g0, int64_t n, int64_t x0,
-                                              int64_t nx, const double *b_re, const double *b_im, const double *scale,
-                                              int fp32, cudaStream_t st)
+static inline cudaError_t qw_launch_tinit_pos(const QwSimDev &d, void *pbuf, int full, int64_t g0, int64_t n,
+                                              int64_t x0, int64_t nx, const double *b_re, const double *b_im,
+                                              const double *scale, int fp32, cudaStream_t st)
 {
-    return fp32 ? qw_launch_tinit_pos32(d, pbuf, g0, n, x0, nx, b_re, b_im, scale, st)
-                : qw_launch_tinit_pos64(d, pbuf, g0, n, x0, nx, b_re, b_im, scale, st);
+    return fp32 ? qw_launch_tinit_pos32(d, pbuf, full, g0, n, x0, nx, b_re, b_im, scale, st)
+                : qw_launch_tinit_pos64(d, pbuf, full, g0, n, x0, nx, b_re, b_im, scale, st);
 }
 static inline cudaError_t qw_launch_measure_pos(const QwSimDev &d, const void *pbuf, int full, int64_t g0, int64_t n,
                                                 int fp32, const double *scale, int reg, double *probs, int64_t len,
@@ -256,7 +257,7 @@ cudaError_t qw_launch_measure(const QwSimDev &d, const QwBufDev &buf, int inst, 
                               const double *scale, int reg, double *probs, int64_t len,
                               cudaStream_t st);
 /* pbuf (nullable): read rows g0 .. g0 + pn of the positional layout (pfull:
-   plane B1 in use) instead of buf */
+   b1 = b2 = 1 branches too) instead of buf */
 cudaError_t qw_launch_measure_noalloc(const QwSimDev &d, const QwBufDev &buf, int inst, int fp32,
                                       const double *scale, int reg, double *host_probs,
                                       int64_t len, int device, cudaStream_t st, const void *pbuf = nullptr,

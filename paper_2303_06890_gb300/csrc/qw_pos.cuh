@@ -21,14 +21,22 @@ namespace {
  * -- entry g s + l for the column in slot l of row g -- or one of the rows x
  * whose slot l_x holds column j while row j holds no column x (a padded, so
  * unpaired, entry): an extra, entry N s + e in a list of all rows' extras in
- * row order.  Over these T entries three planes hold the amplitudes:
- * A[2 i + b2] of row (j, b1 = 0), its b2 pair side by side, and B0[i], B1[i] of
- * row (j, b1 = 1), b2 = 0 and 1.  An absent branch is 0, so the place is the
- * key.
+ * row order.  An entry holds four amplitudes: A0, A1 of row (j, b1 = 0), b2 = 0
+ * and 1, and B0, B1 of row (j, b1 = 1).  An absent branch is 0, so the place is
+ * the key.
  *
  * B1 stays empty: S gives a b1 = b2 = 1 branch only from one of the same kind,
- * and T~|b~> has none.  It is neither read nor written (3/4 of the state's
- * bytes) unless an imported state put something there (FULL).
+ * and T~|b~> has none.  The arithmetic takes it as 0 unless an imported state
+ * put something there (FULLST).
+ *
+ * Layout (PosMem): S scatters a slot's outputs to one entry, and what a step
+ * costs at large N is the 32-byte sectors it writes (each counted twice in L2,
+ * which has a part on either die).  complex64: an entry is one sector {A0, A1,
+ * B0, B1}, read and written by one 32-byte access -- one full sector a slot
+ * instead of two partial ones with A and B apart.  complex128: A0, A1 are one
+ * sector, B0 and B1 planes of their own, B1 not touched (48 bytes a slot: with
+ * B0, B1 as a second sector the state of Table 1's E would be 134 MB a step in
+ * and out, more than L2 holds).
  *
  * The lane of slot (j, l) runs the walk operator on the slot's two pairs
  * (T~^dag's maps take them to (l, 0), T~'s back to k = col): b1 = 0 reflected
@@ -51,32 +59,52 @@ namespace {
  *
  * Bounds: a step at small N is a chain of latencies -- state load, rotation,
  * group sum, store, barrier -- and one launch per step added the launch and
- * the last block's reduction to it.  At large N the state's 24 (48) bytes per
- * slot in and out come from L2.
+ * the last block's reduction to it.  At large N: the sectors written, and the
+ * FP64 pipe for complex128 (12 FP64 instructions a slot, 16 cycles each on an
+ * SM).
  */
 constexpr int kPosMaxWarps = 16; /* 512 threads: up to 128 registers a thread */
 
-/* state accesses go to L2 (another SM wrote what this one reads) */
-__device__ __forceinline__ void pos_load2(const float2 *p, float2 &a0, float2 &a1)
-{
-    const float4 v = __ldcg(reinterpret_cast<const float4 *>(p));
-    a0 = make_float2(v.x, v.y);
-    a1 = make_float2(v.z, v.w);
-}
-__device__ __forceinline__ void pos_load2(const double2 *p, double2 &a0, double2 &a1)
-{
-    a0 = __ldcg(p);
-    a1 = __ldcg(p + 1);
-}
-__device__ __forceinline__ void pos_store2(float2 *p, float2 a0, float2 a1)
-{
-    __stcg(reinterpret_cast<float4 *>(p), make_float4(a0.x, a0.y, a1.x, a1.y));
-}
-__device__ __forceinline__ void pos_store2(double2 *p, double2 a0, double2 a1)
-{
-    __stcg(p, a0);
-    __stcg(p + 1, a1);
-}
+/* An entry's four amplitudes; state accesses go to L2 (another SM wrote what
+   this one reads). */
+template <typename AmpT> struct Entry {
+    AmpT a0, a1, b0, b1;
+};
+template <typename AmpT> struct PosMem;
+template <> struct PosMem<float2> {
+    /* index of one amplitude of entry i (T entries in all) */
+    __device__ static size_t at(size_t, size_t i, int b1, int b2) { return 4 * i + 2 * b1 + b2; }
+    template <bool FULLST> __device__ static void load(const float2 *p, uint32_t, uint32_t i, Entry<float2> &e)
+    {
+        asm volatile("ld.global.cg.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(e.a0.x), "=f"(e.a0.y), "=f"(e.a1.x), "=f"(e.a1.y), "=f"(e.b0.x), "=f"(e.b0.y),
+                       "=f"(e.b1.x), "=f"(e.b1.y)
+                     : "l"(p + 4 * (size_t)i));
+    }
+    template <bool FULLST> __device__ static void store(float2 *p, uint32_t, uint32_t i, const Entry<float2> &e)
+    {
+        asm volatile("st.global.cg.v8.f32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"f"(e.a0.x), "f"(e.a0.y),
+                     "f"(e.a1.x), "f"(e.a1.y), "f"(e.b0.x), "f"(e.b0.y), "f"(e.b1.x), "f"(e.b1.y), "l"(p + 4 * (size_t)i)
+                     : "memory");
+    }
+};
+template <> struct PosMem<double2> {
+    __device__ static size_t at(size_t T, size_t i, int b1, int b2) { return b1 ? (2 + b2) * T + i : 2 * i + b2; }
+    template <bool FULLST> __device__ static void load(const double2 *p, uint32_t T, uint32_t i, Entry<double2> &e)
+    {
+        asm volatile("ld.global.cg.v4.f64 {%0, %1, %2, %3}, [%4];"
+                     : "=d"(e.a0.x), "=d"(e.a0.y), "=d"(e.a1.x), "=d"(e.a1.y) : "l"(p + 2 * (size_t)i));
+        e.b0 = __ldcg(p + 2 * (size_t)T + i);
+        if (FULLST) e.b1 = __ldcg(p + 3 * (size_t)T + i);
+    }
+    template <bool FULLST> __device__ static void store(double2 *p, uint32_t T, uint32_t i, const Entry<double2> &e)
+    {
+        asm volatile("st.global.cg.v4.f64 [%4], {%0, %1, %2, %3};" ::"d"(e.a0.x), "d"(e.a0.y), "d"(e.a1.x), "d"(e.a1.y),
+                     "l"(p + 2 * (size_t)i) : "memory");
+        __stcg(p + 2 * (size_t)T + i, e.b0);
+        if (FULLST) __stcg(p + 3 * (size_t)T + i, e.b1);
+    }
+};
 
 /* ---- barrier over the grid, with the norm ---------------------------------- */
 /*
@@ -292,7 +320,7 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
 
     /* a group's state, loaded one group ahead */
     struct In {
-        AmpT a0[SPL], a1[SPL], q0[SPL], q1[FULLST ? SPL : 1];
+        Entry<AmpT> e[SPL];
     };
     auto fetch = [&](const AmpT *A, uint32_t gg, In &x) {
         const uint32_t jj = gg * RPP + ul;
@@ -300,20 +328,14 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
         const uint32_t i0 = jj * S + lb;
 #pragma unroll
         for (int q = 0; q < SPL; ++q) {
-            x.a0[q] = x.a1[q] = x.q0[q] = zero;
-            if (FULLST) x.q1[q] = zero;
-            if (have) {
-                const uint32_t i = i0 + 32 * q;
-                pos_load2(A + 2 * i, x.a0[q], x.a1[q]);
-                x.q0[q] = __ldcg(A + 2 * T + i);
-                if (FULLST) x.q1[q] = __ldcg(A + 3 * T + i);
-            }
+            x.e[q].a0 = x.e[q].a1 = x.e[q].b0 = x.e[q].b1 = zero;
+            if (have) PosMem<AmpT>::template load<FULLST>(A, T, i0 + 32 * q, x.e[q]);
         }
     };
 
     PosStats st;
     uint32_t cnt = 0;
-    const AmpT *A = static_cast<const AmpT *>(p.in); /* planes A, B0 (at 2 T), B1 (at 3 T) */
+    const AmpT *A = static_cast<const AmpT *>(p.in);
     bool rescale = a.scale_in != nullptr;
     if (threadIdx.x == 0) {
         Amp<AmpT>::Scale::to_shared(rescale ? *a.scale_in : 1.0, &scale_sm);
@@ -355,10 +377,10 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
             bool any = false;
 #pragma unroll
             for (int q = 0; q < SPL; ++q) {
-                a0[q] = cur.a0[q];
-                a1[q] = cur.a1[q];
-                q0[q] = cur.q0[q];
-                q1[q] = FULLST ? cur.q1[q] : zero;
+                a0[q] = cur.e[q].a0;
+                a1[q] = cur.e[q].a1;
+                q0[q] = cur.e[q].b0;
+                q1[q] = FULLST ? cur.e[q].b1 : zero;
                 if (rescale) {
                     a0[q] = scale.apply(a0[q]);
                     a1[q] = scale.apply(a1[q]);
@@ -456,9 +478,9 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
                         if (eA1) norm_add(nrm, rA1);
                         if (FULLST && eB1) norm_add(nrm, rB1);
                     }
-                    pos_store2(O + 2 * to, eA0 ? rA0 : zero, eB0 ? rB0 : zero);
-                    __stcg(O + 2 * T + to, eA1 ? rA1 : zero);
-                    if (FULLST) __stcg(O + 3 * T + to, eB1 ? rB1 : zero);
+                    /* S: (k, b2) <-> (j, b1) */
+                    const Entry<AmpT> o = {eA0 ? rA0 : zero, eB0 ? rB0 : zero, eA1 ? rA1 : zero, eB1 ? rB1 : zero};
+                    PosMem<AmpT>::template store<FULLST>(O, T, to, o);
                 }
                 if (eA0) cnt += kCntOut;
                 if (eB0) cnt += kCntOut;
@@ -473,8 +495,9 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
             if (x >= X) break;
             const uint32_t i = n * S + x;
             const uint32_t to = TAB ? t_x[(k * PW + warp) * 32 + lane] : __ldg(d.pos_xdst + x);
-            AmpT a0, a1, q0 = __ldcg(A + 2 * T + i), q1 = FULLST ? __ldcg(A + 3 * T + i) : zero;
-            pos_load2(A + 2 * i, a0, a1);
+            Entry<AmpT> e;
+            PosMem<AmpT>::template load<FULLST>(A, T, i, e);
+            AmpT a0 = e.a0, a1 = e.a1, q0 = e.b0, q1 = FULLST ? e.b1 : zero;
             if (rescale) {
                 a0 = scale.apply(a0);
                 a1 = scale.apply(a1);
@@ -490,9 +513,9 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
                 if (h0) norm_add(nrm, q0);
                 if (FULLST && h1) norm_add(nrm, q1);
             }
-            pos_store2(O + 2 * to, k0 ? Amp<AmpT>::neg(a0) : zero, h0 ? Amp<AmpT>::neg(q0) : zero);
-            __stcg(O + 2 * T + to, k1 ? Amp<AmpT>::neg(a1) : zero);
-            if (FULLST) __stcg(O + 3 * T + to, h1 ? Amp<AmpT>::neg(q1) : zero);
+            const Entry<AmpT> o = {k0 ? Amp<AmpT>::neg(a0) : zero, h0 ? Amp<AmpT>::neg(q0) : zero,
+                                   k1 ? Amp<AmpT>::neg(a1) : zero, h1 ? Amp<AmpT>::neg(q1) : zero};
+            PosMem<AmpT>::template store<FULLST>(O, T, to, o);
             if ((k & 15u) == 15u) st.take(cnt);
         }
         st.take(cnt);
@@ -526,7 +549,6 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
                     atomicOr(p.poison, 1u);
                     share = 0;
                 }
-                __threadfence();
                 word_add(word, (1ull << kCountShift) + share);
                 bool ok = true;
                 if (!last || blockIdx.x == 0) {
@@ -621,12 +643,11 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
  * branch per row, a = b_j (divided by the pending renormalisation factor when
  * other instances share the state); T~'s Hadamard gives (l, z = 0) with
  * a / sqrt(s) for every slot l, its maps take slot l to k = col(j, l), and
- * R(A_jl) on (a / sqrt(s), 0) gives the pair of the slot's entry in plane A --
- * the arithmetic of k_tinit.  B0 of the slots and both planes of the rows'
- * extras (x0 .. x0 + nx) are written 0.  One thread per entry: bound by the
- * writes. */
+ * R(A_jl) on (a / sqrt(s), 0) gives A0, A1 of the slot's entry -- the
+ * arithmetic of k_tinit.  The rest, the rows' extras (x0 .. x0 + nx) included,
+ * is written 0.  One thread per entry: bound by the writes. */
 template <typename AmpT>
-__global__ void k_tinit_pos(QwSimDev d, AmpT *pbuf, uint32_t g0, uint32_t n, uint32_t x0, uint32_t nx,
+__global__ void k_tinit_pos(QwSimDev d, AmpT *pbuf, int full, uint32_t g0, uint32_t n, uint32_t x0, uint32_t nx,
                             const double *b_re, const double *b_im, const double *scale)
 {
     typedef typename Amp<AmpT>::RotVal RotVal;
@@ -653,8 +674,9 @@ __global__ void k_tinit_pos(QwSimDev d, AmpT *pbuf, uint32_t g0, uint32_t n, uin
                 if (!Amp<AmpT>::keep(d, o1)) o1 = zero;
             }
         }
-        pos_store2(pbuf + 2 * (size_t)at, o0, o1);
-        pbuf[2 * (size_t)T + at] = zero;
+        const Entry<AmpT> e = {o0, o1, zero, zero};
+        if (full) PosMem<AmpT>::template store<true>(pbuf, T, at, e);
+        else PosMem<AmpT>::template store<false>(pbuf, T, at, e);
     }
 }
 
@@ -690,11 +712,10 @@ __global__ void __launch_bounds__(256) k_measure_pos(QwSimDev d, const AmpT *pbu
         for (uint32_t i = lane; i < P; i += 32) {
             uint32_t at = i < S ? g * S + i : N * S + x0 + (i - S);
             if (reg == 4) at = i < S ? (__ldg(d.pos_dst + at) & 0x3fffffffu) : __ldg(d.pos_xdst + x0 + (i - S));
-            AmpT a0, a1;
-            pos_load2(pbuf + 2 * (size_t)at, a0, a1);
-            const AmpT q0 = pbuf[2 * (size_t)T + at];
-            const double p[4] = {amp_norm2(a0), amp_norm2(a1), amp_norm2(q0),
-                                 full ? amp_norm2(pbuf[3 * (size_t)T + at]) : 0.0};
+            Entry<AmpT> e;
+            if (full) PosMem<AmpT>::template load<true>(pbuf, T, at, e);
+            else PosMem<AmpT>::template load<false>(pbuf, T, at, e);
+            const double p[4] = {amp_norm2(e.a0), amp_norm2(e.a1), amp_norm2(e.b0), full ? amp_norm2(e.b1) : 0.0};
             if (reg == 1 || reg == 4) {
                 row += (p[0] + p[1]) + (p[2] + p[3]);
             } else {
@@ -723,12 +744,11 @@ __global__ void __launch_bounds__(256) k_measure_pos(QwSimDev d, const AmpT *pbu
 }
 
 /* the row buckets into the positional layout (pbuf zeroed by the caller):
-   one thread per bucket slot; a branch in B1 sets QW_ST_POS_FULL */
+   one thread per bucket slot; a branch with b1 = b2 = 1 sets QW_ST_POS_FULL */
 template <typename AmpT>
 __global__ void k_pos_pack(QwSimDev d, QwBufDev buf, AmpT *pbuf, int32_t *status)
 {
     const int S = d.s;
-    AmpT *B0 = pbuf + 2 * d.pos_T, *B1 = pbuf + 3 * d.pos_T;
     const int64_t total = d.total_buckets * (int64_t)d.cap_row;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = i / d.cap_row;
@@ -775,28 +795,23 @@ __global__ void k_pos_pack(QwSimDev d, QwBufDev buf, AmpT *pbuf, int32_t *status
             continue;
         }
         const AmpT v = static_cast<const AmpT *>(buf.amp)[i];
-        if ((b & 1) == 0) {
-            pbuf[2 * at + x.b2] = v;
-        } else if (x.b2 == 0) {
-            B0[at] = v;
-        } else {
-            B1[at] = v;
-            if (nz(v)) atomicOr(status, QW_ST_POS_FULL);
-        }
+        pbuf[PosMem<AmpT>::at((size_t)d.pos_T, (size_t)at, (int)(b & 1), (int)x.b2)] = v;
+        if ((b & 1) != 0 && x.b2 != 0 && nz(v)) atomicOr(status, QW_ST_POS_FULL);
     }
 }
 
 /* the positional layout into the row buckets (cleared by the caller): one
-   thread per entry and plane, non-zero amplitudes appended to their row */
+   thread per amplitude, non-zero ones appended to their row */
 template <typename AmpT>
 __global__ void k_pos_unpack(QwSimDev d, const AmpT *pbuf, int full, QwBufDev buf, int32_t *status)
 {
-    const int64_t S = d.s, T = d.pos_T, total = (full ? 4 : 3) * T;
+    const int64_t S = d.s, T = d.pos_T, total = 4 * T;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const AmpT v = pbuf[i];
+        const int64_t at = i >> 2;
+        const int b1 = (int)(i >> 1) & 1, b2 = (int)i & 1;
+        if (b1 && b2 && !full) continue;
+        const AmpT v = pbuf[PosMem<AmpT>::at((size_t)T, (size_t)at, b1, b2)];
         if (v.x == 0 && v.y == 0) continue;
-        const int b1 = i >= 2 * T ? 1 : 0;
-        const int64_t at = b1 ? (i >= 3 * T ? i - 3 * T : i - 2 * T) : i >> 1;
         int64_t gr = at / S; /* the row among all instances' rows */
         uint32_t k;          /* the branch's k, a row among all instances' for an extra */
         if (gr < d.pos_rows) {
@@ -821,7 +836,7 @@ __global__ void k_pos_unpack(QwSimDev d, const AmpT *pbuf, int full, QwBufDev bu
         Regs x;
         x.kc = 0;
         x.A = 0;
-        x.b2 = b1 ? (i >= 3 * T ? 1u : 0u) : (uint32_t)(i & 1);
+        x.b2 = (uint32_t)b2;
         x.k = at < d.pos_rows * S ? k : k - (uint32_t)g0;
         const int p = atomicAdd(buf.count + b, 1);
         if (p >= d.cap_row) {
@@ -897,12 +912,12 @@ cudaError_t launch_pos_t(const QwSimDev &d, const QwPosPlan &pl, const QwPosArgs
 }
 
 template <typename AmpT>
-cudaError_t launch_tinit_pos_t(const QwSimDev &d, void *pbuf, int64_t g0, int64_t n, int64_t x0, int64_t nx,
+cudaError_t launch_tinit_pos_t(const QwSimDev &d, void *pbuf, int full, int64_t g0, int64_t n, int64_t x0, int64_t nx,
                                const double *b_re, const double *b_im, const double *scale, cudaStream_t st)
 {
     const int64_t want = (n * d.s + nx + 255) / 256, cap = 16 * (int64_t)qw_sm_count();
     k_tinit_pos<AmpT><<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(
-        d, static_cast<AmpT *>(pbuf), (uint32_t)g0, (uint32_t)n, (uint32_t)x0, (uint32_t)nx, b_re, b_im, scale);
+        d, static_cast<AmpT *>(pbuf), full, (uint32_t)g0, (uint32_t)n, (uint32_t)x0, (uint32_t)nx, b_re, b_im, scale);
     return cudaGetLastError();
 }
 
@@ -943,11 +958,12 @@ cudaError_t launch_pos_unpack_t(const QwSimDev &d, const void *pbuf, int full, c
     {                                                                                                                 \
         return launch_pos_t<AmpT>(d, pl, p, a, full, st);                                                             \
     }                                                                                                                 \
-    cudaError_t qw_launch_tinit_pos##SUFFIX(const QwSimDev &d, void *pbuf, int64_t g0, int64_t n, int64_t x0,         \
-                                            int64_t nx, const double *b_re, const double *b_im, const double *scale,  \
+    cudaError_t qw_launch_tinit_pos##SUFFIX(const QwSimDev &d, void *pbuf, int full, int64_t g0, int64_t n,           \
+                                            int64_t x0, int64_t nx, const double *b_re, const double *b_im,           \
+                                            const double *scale,                                                      \
                                             cudaStream_t st)                                                          \
     {                                                                                                                 \
-        return launch_tinit_pos_t<AmpT>(d, pbuf, g0, n, x0, nx, b_re, b_im, scale, st);                               \
+        return launch_tinit_pos_t<AmpT>(d, pbuf, full, g0, n, x0, nx, b_re, b_im, scale, st);                               \
     }                                                                                                                 \
     cudaError_t qw_launch_measure_pos##SUFFIX(const QwSimDev &d, const void *pbuf, int full, int64_t g0, int64_t n,   \
                                               const double *scale, int reg, double *probs, int64_t len,               \
