@@ -180,10 +180,11 @@ int qw_sim_create(const qw_csc *mats, int32_t num_instances, const qw_sim_opts *
  * Set instance inst to |b~> = sum_j b_j |jc=0, j, b1=0, kc=0, k=0, b2=0>
  * (Sec. IV, |j~>), b = b_re + i b_im (b_im may be NULL), n = that instance's N;
  * exact zeros are not stored.  With apply_T != 0 the state becomes T~|b~>
- * (Alg. T~).  Other instances are not touched.  b_re and b_im are copied to
- * the device directly (an asynchronous copy when they are pinned); the call
- * synchronises the simulator's stream before it returns, so they may be
- * reused afterwards.
+ * (Alg. T~).  Other instances are not touched.  b_re and b_im may be reused
+ * when the call returns: it copies them to the device (asynchronously when they
+ * are pinned) and synchronises the simulator's stream, or, for T~|b~> written
+ * straight into the positional layout (walk_variant 7 below), copies them to
+ * pinned memory of its own that the device reads, without synchronising.
  * Errors: QW_ERR_ARG, QW_ERR_CAPACITY, QW_ERR_CUDA, QW_ERR_DEVICE_STATUS (T~
  * met a row of the instance that was not |b~>).
  */

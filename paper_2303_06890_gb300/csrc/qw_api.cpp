@@ -44,6 +44,8 @@ struct StatusView {
     int64_t done;
 };
 static_assert(offsetof(Scalars, steps_done) == offsetof(StatusView, done), "Scalars head layout");
+static_assert(sizeof(Scalars) % 8 == 0 && sizeof(Scalars) / 8 <= 20, "Scalars as words (QwScalarWords)");
+static_assert(sizeof(StatusView) == 16, "the status head is two words");
 
 thread_local std::string g_create_error;
 
@@ -123,6 +125,13 @@ struct qw_sim {
     int64_t qls_p_cap = 0;
     double *b_dev = nullptr;     /* |b> staging: re then im, b_stride doubles each */
     int64_t b_stride = 0;
+    /* pinned host memory of the positional layout's own transfers, which its
+       kernels read and write directly: each instance's |b> (re, im), whether
+       the device may still be reading it, and a register marginal */
+    double *h_b = nullptr;
+    std::vector<char> h_b_busy;
+    double *h_probs = nullptr;
+    int64_t h_probs_cap = 0;
     double *meas_dev = nullptr;  /* register marginal scratch */
     int64_t meas_cap = 0;
     Scalars *h_sc = nullptr;     /* pinned host copies: Scalars reset, status read */
@@ -654,6 +663,8 @@ extern "C" int qw_sim_destroy(qw_sim *sim)
     cudaFree(sim->qls_c);
     cudaFree(sim->b_dev);
     cudaFree(sim->meas_dev);
+    cudaFreeHost(sim->h_b);
+    cudaFreeHost(sim->h_probs);
     cudaFreeHost(sim->h_sc);
     cudaFreeHost(sim->h_st);
     delete sim;
@@ -688,12 +699,22 @@ static const double *pending_scale(qw_sim *sim)
  * an error, steps issued after the failing one did nothing on the device, so
  * the state is the output of the last clean step: move the host view there.
  * Then clear the status and map it to an error code. */
+static int status_read(qw_sim *sim, const char *where);
+
 static int check_status(qw_sim *sim, const char *where)
 {
-    cudaError_t e = cudaMemcpyAsync(sim->h_st, &sim->sc->status, sizeof(StatusView), cudaMemcpyDeviceToHost,
-                                    sim->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(sim->stream);
+    const cudaError_t e = cudaMemcpyAsync(sim->h_st, &sim->sc->status, sizeof(StatusView), cudaMemcpyDeviceToHost,
+                                          sim->stream);
     if (e != cudaSuccess) return cuda_fail(sim, e, where);
+    return status_read(sim, where);
+}
+
+/* check_status with the status head already on its way to h_st */
+static int status_read(qw_sim *sim, const char *where)
+{
+    const cudaError_t e = cudaStreamSynchronize(sim->stream);
+    if (e != cudaSuccess) return cuda_fail(sim, e, where);
+    std::fill(sim->h_b_busy.begin(), sim->h_b_busy.end(), 0);
     const StatusView h = *sim->h_st;
     const int64_t good = h.done - sim->sync_done;
     sim->last_good = good;
@@ -1228,6 +1249,8 @@ static int pos_build(qw_sim *sim)
     d.pos_xptr = sim->pos_xptr;
     d.pos_xdst = sim->pos_xdst;
     d.pos_rowinst = sim->pos_rowinst;
+    sim->h_b_busy.assign((size_t)ninst, 0);
+    if (!sim->h_b) QW_CUDA(sim, cudaMallocHost((void **)&sim->h_b, 2 * (size_t)nrows * sizeof(double)));
     sim->pos_plan = qw_pos_plan(d, sim->fp32);
     const size_t words = 5 + 2 * (size_t)sim->pos_plan.grid;
     QW_CUDA(sim, dalloc(sim, &sim->pos_words, words));
@@ -1489,6 +1512,71 @@ extern "C" int qw_faithful_end(qw_sim *sim, int32_t keep)
     return rc;
 }
 
+/* T~|b~> of one instance straight into the positional layout: |b> is copied to
+ * pinned memory, which the kernel reads (one launch, no transfer of its own
+ * and no synchronisation -- the kernel has no error to report). */
+static int pos_state_init(qw_sim *sim, int32_t inst, const double *b_re, const double *b_im, int32_t n)
+{
+    const bool all = sim->d.ninst == 1;
+    const int64_t g0 = pos_row0(sim, inst);
+    if (sim->h_b_busy[(size_t)inst]) { /* set again before anything synchronised */
+        QW_CUDA(sim, cudaStreamSynchronize(sim->stream));
+        std::fill(sim->h_b_busy.begin(), sim->h_b_busy.end(), 0);
+    }
+    double *dre = sim->h_b + 2 * g0, *dim = b_im ? dre + n : nullptr;
+    double part[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    auto take = [&](const double *src, double *dst) {
+        int32_t j = 0;
+        for (; j + 8 <= n; j += 8)
+            for (int t = 0; t < 8; ++t) {
+                const double v = src[j + t];
+                dst[j + t] = v;
+                part[t] += v * v;
+            }
+        for (; j < n; ++j) {
+            dst[j] = src[j];
+            part[j & 7] += src[j] * src[j];
+        }
+    };
+    take(b_re, dre);
+    if (b_im) take(b_im, dim);
+    const double nb2 = ((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]));
+    sim->init_norm2[(size_t)inst] = nb2;
+    QwScalarWords words{};
+    if (all) {
+        Scalars z{};
+        z.scale[0] = z.scale[1] = 1.0;
+        z.renorm_target = nb2;
+        words.dst = reinterpret_cast<unsigned long long *>(sim->sc);
+        words.n = (int)(sizeof(Scalars) / 8);
+        std::memcpy(words.w, &z, sizeof(Scalars));
+        sim->scale_slot = sim->sync_slot = 0;
+        sim->cur = sim->sync_cur = 0;
+        sim->sync_done = 0;
+        sim->issued = 0;
+        sim->pos_issued = false;
+        sim->pos_full = false;
+    } else {
+        double target = 0.0;
+        for (double v : sim->init_norm2) target += v;
+        words.dst = reinterpret_cast<unsigned long long *>(&sim->sc->renorm_target);
+        words.n = 1;
+        std::memcpy(words.w, &target, 8);
+    }
+    const int64_t x0 = sim->pos_xrow[(size_t)inst], nx = sim->pos_xrow[(size_t)inst + 1] - x0;
+    QW_CUDA(sim, qw_launch_tinit_pos(sim->d, sim->pbuf[sim->cur], sim->pos_full, g0, n, x0, nx, dre, dim,
+                                     all ? nullptr : pending_scale(sim), words, sim->fp32, sim->stream));
+    sim->launches++;
+    sim->h_b_busy[(size_t)inst] = 1;
+    sim->pos_live = true;
+    sim->has_state = true;
+    sim->fresh_T = true;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(sim->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
+        return check_status(sim, "qw_state_init"); /* refused, as everywhere (it cannot synchronise) */
+    return QW_OK;
+}
+
 extern "C" int qw_state_init(qw_sim *sim, int32_t inst, const double *b_re, const double *b_im,
                              int32_t n, int32_t apply_T)
 {
@@ -1500,7 +1588,9 @@ extern "C" int qw_state_init(qw_sim *sim, int32_t inst, const double *b_re, cons
        instance, or several already there); otherwise into the row buckets */
     const bool pos_init = apply_T && sim->mode == QW_MODE_WALK_POS && sim->pos_built &&
                           (sim->d.ninst == 1 || sim->pos_live);
-    if (!pos_init) {
+    if (pos_init) {
+        sim->pos_try = true;
+    } else {
         if (sim->d.ninst > 1) { /* the other instances keep their state: back into the buckets */
             const int prc = pos_unpack(sim);
             if (prc != QW_OK) return prc;
@@ -1508,6 +1598,7 @@ extern "C" int qw_state_init(qw_sim *sim, int32_t inst, const double *b_re, cons
         sim->pos_live = false; /* the state is replaced in the row buckets */
     }
     sim->pos_try = true;
+    if (pos_init) return pos_state_init(sim, inst, b_re, b_im, n);
     /* |b> goes straight from the caller's arrays to the device (asynchronous
        when they are pinned); the previous call's copies ended at its sync */
     double *dre = sim->b_dev, *dim = b_im ? sim->b_dev + sim->b_stride : nullptr;
@@ -1518,12 +1609,12 @@ extern "C" int qw_state_init(qw_sim *sim, int32_t inst, const double *b_re, cons
     const bool all = sim->d.ninst == 1;
     /* clear the instance's rows in every buffer (the whole state for a single
        instance, garbage-row table included) */
-    for (int bi = 0; bi < 3 && !pos_init; ++bi) {
+    for (int bi = 0; bi < 3; ++bi) {
         QW_CUDA(sim, qw_launch_clear(sim->d, sim->buf[bi], all ? 0 : lo,
                                      all ? sim->d.total_buckets : hi, all ? 1 : 0, sim->stream));
         sim->launches++;
     }
-    if (apply_T && !pos_init && sim->opts.overflow_fallback && sim->d.cap_row < 2 * sim->d.s) {
+    if (apply_T && sim->opts.overflow_fallback && sim->d.cap_row < 2 * sim->d.s) {
         /* T~ gives a row of |b~> up to 2 s branches */
         int rc = grow_rows(sim, 2 * (int64_t)sim->d.s);
         if (rc != QW_OK) return rc;
@@ -1547,21 +1638,10 @@ extern "C" int qw_state_init(qw_sim *sim, int32_t inst, const double *b_re, cons
         QW_CUDA(sim, cudaMemcpyAsync(&sim->sc->renorm_target, &sim->host_target, 8,
                                      cudaMemcpyHostToDevice, sim->stream));
     }
-    if (pos_init) {
-        int64_t g0 = 0;
-        for (int i = 0; i < inst; ++i) g0 += sim->n_of[(size_t)i];
-        const int64_t x0 = sim->pos_xrow[(size_t)inst], nx = sim->pos_xrow[(size_t)inst + 1] - x0;
-        if (all) sim->pos_full = false;
-        QW_CUDA(sim, qw_launch_tinit_pos(sim->d, sim->pbuf[sim->cur], sim->pos_full, g0, n, x0, nx, dre, dim,
-                                         all ? nullptr : pending_scale(sim), sim->fp32, sim->stream));
-        sim->launches++;
-        sim->pos_live = true;
-    } else {
-        QW_CUDA(sim, qw_launch_init_b(sim->d, sim->buf[sim->cur], inst, dre, dim, n, sim->fp32,
-                                      all ? nullptr : pending_scale(sim), sim->stream));
-        sim->launches++;
-    }
-    if (apply_T && !pos_init) {
+    QW_CUDA(sim, qw_launch_init_b(sim->d, sim->buf[sim->cur], inst, dre, dim, n, sim->fp32,
+                                  all ? nullptr : pending_scale(sim), sim->stream));
+    sim->launches++;
+    if (apply_T) {
         /* T~ on |b~>: the one-branch-per-row kernel (a row that is not |b~>
            sets a status bit), or the literal sort-based schedule when that
            was asked for */
@@ -1917,11 +1997,31 @@ extern "C" int qw_measure_register(qw_sim *sim, int32_t inst, int32_t reg, doubl
         QW_CUDA(sim, cudaMalloc((void **)&sim->meas_dev, (size_t)len * sizeof(double)));
         sim->meas_cap = len;
     }
+    if (sim->pos_live && (reg == QW_REG_J || reg == QW_REG_K)) {
+        /* every bin written by one launch, into pinned memory, with the status
+           head beside it */
+        if (sim->h_probs_cap < len) {
+            QW_CUDA(sim, cudaStreamSynchronize(sim->stream));
+            cudaFreeHost(sim->h_probs);
+            sim->h_probs = nullptr;
+            sim->h_probs_cap = 0;
+            QW_CUDA(sim, cudaMallocHost((void **)&sim->h_probs, (size_t)len * sizeof(double)));
+            sim->h_probs_cap = len;
+        }
+        QW_CUDA(sim, qw_launch_measure_pos(sim->d, sim->pbuf[sim->cur], sim->pos_full, pos_row0(sim, inst),
+                                           sim->n_of[(size_t)inst], sim->fp32, pending_scale(sim), reg, sim->h_probs, len,
+                                           reinterpret_cast<const unsigned long long *>(&sim->sc->status),
+                                           reinterpret_cast<unsigned long long *>(sim->h_st), sim->stream));
+        sim->launches++;
+        const int rc = status_read(sim, "qw_measure_register");
+        std::memcpy(probs, sim->h_probs, (size_t)len * sizeof(double));
+        return rc;
+    }
     double *dp = sim->meas_dev;
     QW_CUDA(sim, cudaMemsetAsync(dp, 0, (size_t)len * sizeof(double), sim->stream));
     if (sim->pos_live) /* read the positional layout in place */
         QW_CUDA(sim, qw_launch_measure_pos(sim->d, sim->pbuf[sim->cur], sim->pos_full, pos_row0(sim, inst), sim->n_of[(size_t)inst],
-                                           sim->fp32, pending_scale(sim), reg, dp, len, sim->stream));
+                                           sim->fp32, pending_scale(sim), reg, dp, len, nullptr, nullptr, sim->stream));
     else
         QW_CUDA(sim, qw_launch_measure(sim->d, sim->buf[sim->cur], inst, sim->fp32, pending_scale(sim), reg,
                                        dp, len, sim->stream));

@@ -166,6 +166,11 @@ struct QwPosArgs {
     unsigned int *poison;     /* set when a block's norm share is not finite */
     double *pshare;           /* [2][grid]: the blocks' shares of p_j */
 };
+struct QwScalarWords { /* 8-byte words of the simulator's scalars a kernel sets */
+    unsigned long long *dst;
+    int n;
+    unsigned long long w[20];
+};
 struct QwPosPlan {
     int grid, warps; /* blocks, warps a block */
     int tab;         /* the matrix's tables fit shared memory */
@@ -185,9 +190,10 @@ int qw_pos_supported(const QwSimDev &d);
 /* dynamic shared memory per block of the step kernel of `mode` */
 size_t qw_step_smem_bytes(const QwSimDev &d, int fp32, int mode);
 /* positional layout (qw_pos.cuh; 32: complex64, 64: complex128): the launch
-   shape, walk steps, T~|b~> written into rows g0 .. g0 + n, a register
-   marginal of those rows (probs zeroed by the caller; x0, nx: the rows'
-   extras), and the conversions
+   shape, walk steps, T~|b~> written into rows g0 .. g0 + n (x0, nx: their
+   extras), a register marginal of those rows (j and k write every bin, the
+   others add to zeroed ones; probs and stat_dst may be pinned host memory),
+   and the conversions
    from and to the row buckets (pack: pbuf zeroed by the caller, a branch
    without a place sets QW_ST_POS_UNREP; unpack: the buckets cleared by the
    caller); full: the state has b1 = b2 = 1
@@ -198,9 +204,10 @@ size_t qw_step_smem_bytes(const QwSimDev &d, int fp32, int mode);
                                            const QwStepArgs &a, int full, cudaStream_t st);                           \
     cudaError_t qw_launch_tinit_pos##SUFFIX(const QwSimDev &d, void *pbuf, int full, int64_t g0, int64_t n,           \
                                             int64_t x0, int64_t nx, const double *b_re, const double *b_im,           \
-                                            const double *scale, cudaStream_t st);                                                         \
+                                            const double *scale, const QwScalarWords &words, cudaStream_t st);        \
     cudaError_t qw_launch_measure_pos##SUFFIX(const QwSimDev &d, const void *pbuf, int full, int64_t g0, int64_t n,   \
                                               const double *scale, int reg, double *probs, int64_t len,               \
+                                              const unsigned long long *stat_src, unsigned long long *stat_dst,       \
                                               cudaStream_t st);                                                       \
     cudaError_t qw_launch_pos_pack##SUFFIX(const QwSimDev &d, const QwBufDev &buf, void *pbuf, int32_t *status,       \
                                            cudaStream_t st);                                                          \
@@ -217,17 +224,19 @@ static inline cudaError_t qw_launch_walk_pos(const QwSimDev &d, const QwPosPlan 
 }
 static inline cudaError_t qw_launch_tinit_pos(const QwSimDev &d, void *pbuf, int full, int64_t g0, int64_t n,
                                               int64_t x0, int64_t nx, const double *b_re, const double *b_im,
-                                              const double *scale, int fp32, cudaStream_t st)
+                                              const double *scale, const QwScalarWords &words, int fp32,
+                                              cudaStream_t st)
 {
-    return fp32 ? qw_launch_tinit_pos32(d, pbuf, full, g0, n, x0, nx, b_re, b_im, scale, st)
-                : qw_launch_tinit_pos64(d, pbuf, full, g0, n, x0, nx, b_re, b_im, scale, st);
+    return fp32 ? qw_launch_tinit_pos32(d, pbuf, full, g0, n, x0, nx, b_re, b_im, scale, words, st)
+                : qw_launch_tinit_pos64(d, pbuf, full, g0, n, x0, nx, b_re, b_im, scale, words, st);
 }
 static inline cudaError_t qw_launch_measure_pos(const QwSimDev &d, const void *pbuf, int full, int64_t g0, int64_t n,
                                                 int fp32, const double *scale, int reg, double *probs, int64_t len,
+                                                const unsigned long long *stat_src, unsigned long long *stat_dst,
                                                 cudaStream_t st)
 {
-    return fp32 ? qw_launch_measure_pos32(d, pbuf, full, g0, n, scale, reg, probs, len, st)
-                : qw_launch_measure_pos64(d, pbuf, full, g0, n, scale, reg, probs, len, st);
+    return fp32 ? qw_launch_measure_pos32(d, pbuf, full, g0, n, scale, reg, probs, len, stat_src, stat_dst, st)
+                : qw_launch_measure_pos64(d, pbuf, full, g0, n, scale, reg, probs, len, stat_src, stat_dst, st);
 }
 static inline cudaError_t qw_launch_pos_pack(const QwSimDev &d, const QwBufDev &buf, void *pbuf, int fp32,
                                              int32_t *status, cudaStream_t st)

@@ -2624,7 +2624,7 @@ cudaError_t qw_launch_measure_noalloc(const QwSimDev &d, const QwBufDev &buf, in
     cudaError_t e = cudaMemsetAsync(scratch, 0, (size_t)len * sizeof(double), st);
     if (e != cudaSuccess) return e;
     const int grid = 4 * qw_sm_count();
-    if (pbuf) e = qw_launch_measure_pos(d, pbuf, pfull, g0, pn, fp32, scale, reg, scratch, len, st);
+    if (pbuf) e = qw_launch_measure_pos(d, pbuf, pfull, g0, pn, fp32, scale, reg, scratch, len, nullptr, nullptr, st);
     else if (fp32) k_measure<float2><<<grid, 256, 0, st>>>(d, buf, inst, scale, reg, scratch, len);
     else k_measure<double2><<<grid, 256, 0, st>>>(d, buf, inst, scale, reg, scratch, len);
     if (!pbuf) e = cudaGetLastError();

@@ -645,12 +645,17 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
  * a / sqrt(s) for every slot l, its maps take slot l to k = col(j, l), and
  * R(A_jl) on (a / sqrt(s), 0) gives A0, A1 of the slot's entry -- the
  * arithmetic of k_tinit.  The rest, the rows' extras (x0 .. x0 + nx) included,
- * is written 0.  One thread per entry: bound by the writes. */
+ * is written 0.  b lies in the simulator's pinned host memory and is read from
+ * there: S lanes share a value, so its bytes cross the link once, without a
+ * copy before the launch.  words: 8-byte words of the simulator's scalars to
+ * set (all of them for a single instance), so that no copy is needed for those
+ * either.  One thread per entry: bound by the writes. */
 template <typename AmpT>
 __global__ void k_tinit_pos(QwSimDev d, AmpT *pbuf, int full, uint32_t g0, uint32_t n, uint32_t x0, uint32_t nx,
-                            const double *b_re, const double *b_im, const double *scale)
+                            const double *b_re, const double *b_im, const double *scale, QwScalarWords words)
 {
     typedef typename Amp<AmpT>::RotVal RotVal;
+    if (blockIdx.x == 0 && (int)threadIdx.x < words.n) words.dst[threadIdx.x] = words.w[threadIdx.x];
     const uint32_t S = (uint32_t)d.s, T = (uint32_t)d.pos_T, ns = n * S, total = ns + nx;
     const AmpT zero = Amp<AmpT>::zero();
     const bool rot_in_place = Amp<AmpT>::kRotCode && d.rot_calc;
@@ -689,43 +694,56 @@ template <typename AmpT> __device__ __forceinline__ double amp_norm2(AmpT a)
 }
 
 /* Marginal of one register over rows g0 .. g0 + n (the key of an entry: jc =
- * kc = 0, j = its row, b1 and b2 by plane, k = the slot's column or the
- * extra's row), one warp per row.  j: the row's own entries.  k: a gather
+ * kc = 0, j = its row, b1 and b2 by member, k = the slot's column or the
+ * extra's row), LPR lanes a row.  j: the row's own entries.  k: a gather
  * instead of an atomic per branch -- the branches with k = v sit at dst(v, l)
  * for every slot l of row v (the entry of k = v in row col(v, l)) and at slot
- * (x, l_x) for every extra x of row v.  The other registers: the sums by plane,
- * one atomic per block. */
+ * (x, l_x) for every extra x of row v.  Both write every bin of probs (which may
+ * be host memory: a block's rows as one run of 8-byte words).  The other
+ * registers: sums by (b1, b2), one atomic per block into zeroed bins.
+ * stat_dst (host memory, nullable): the two words of the status head. */
 template <typename AmpT>
 __global__ void __launch_bounds__(256) k_measure_pos(QwSimDev d, const AmpT *pbuf, int full, int64_t g0, int64_t n,
-                                                     const double *scale, int reg, double *probs, int64_t len)
+                                                     const double *scale, int reg, double *probs, int64_t len,
+                                                     const unsigned long long *stat_src, unsigned long long *stat_dst)
 {
     __shared__ double acc_sm[4][8];
+    __shared__ double row_sm[256];
     const uint32_t S = (uint32_t)d.s, T = (uint32_t)d.pos_T, N = (uint32_t)d.pos_rows;
-    const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int lpr = S >= 32 ? 32 : (int)S, rpb = 256 / lpr; /* lanes a row, rows a block */
+    const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5, rl = threadIdx.x / lpr, lr = threadIdx.x % lpr;
     const double sc = scale ? *scale * *scale : 1.0;
+    const bool rows = reg == 1 || reg == 4;
+    if (stat_dst && blockIdx.x == 0 && threadIdx.x < 2) stat_dst[threadIdx.x] = __ldcg(stat_src + threadIdx.x);
     double acc[4] = {0.0, 0.0, 0.0, 0.0}; /* by (b1, b2) */
-    for (int64_t j = warp; j < n; j += nw) {
-        const uint32_t g = (uint32_t)(g0 + j), x0 = __ldg(d.pos_xptr + g), P = S + __ldg(d.pos_xptr + g + 1) - x0;
+    const int64_t end = rows && len > n ? len : n;
+    for (int64_t j0 = (int64_t)blockIdx.x * rpb; j0 < end; j0 += (int64_t)gridDim.x * rpb) {
+        const int64_t j = j0 + rl;
         double row = 0.0;
-        for (uint32_t i = lane; i < P; i += 32) {
-            uint32_t at = i < S ? g * S + i : N * S + x0 + (i - S);
-            if (reg == 4) at = i < S ? (__ldg(d.pos_dst + at) & 0x3fffffffu) : __ldg(d.pos_xdst + x0 + (i - S));
-            Entry<AmpT> e;
-            if (full) PosMem<AmpT>::template load<true>(pbuf, T, at, e);
-            else PosMem<AmpT>::template load<false>(pbuf, T, at, e);
-            const double p[4] = {amp_norm2(e.a0), amp_norm2(e.a1), amp_norm2(e.b0), full ? amp_norm2(e.b1) : 0.0};
-            if (reg == 1 || reg == 4) {
-                row += (p[0] + p[1]) + (p[2] + p[3]);
-            } else {
+        if (j < n) {
+            const uint32_t g = (uint32_t)(g0 + j), x0 = __ldg(d.pos_xptr + g), P = S + __ldg(d.pos_xptr + g + 1) - x0;
+            for (uint32_t i = lr; i < P; i += lpr) {
+                uint32_t at = i < S ? g * S + i : N * S + x0 + (i - S);
+                if (reg == 4) at = i < S ? (__ldg(d.pos_dst + at) & 0x3fffffffu) : __ldg(d.pos_xdst + x0 + (i - S));
+                Entry<AmpT> e;
+                if (full) PosMem<AmpT>::template load<true>(pbuf, T, at, e);
+                else PosMem<AmpT>::template load<false>(pbuf, T, at, e);
+                const double p[4] = {amp_norm2(e.a0), amp_norm2(e.a1), amp_norm2(e.b0), full ? amp_norm2(e.b1) : 0.0};
+                if (rows) {
+                    row += (p[0] + p[1]) + (p[2] + p[3]);
+                } else {
 #pragma unroll
-                for (int t = 0; t < 4; ++t) acc[t] += p[t];
+                    for (int t = 0; t < 4; ++t) acc[t] += p[t];
+                }
             }
         }
-        if (reg == 1 || reg == 4) {
-            row = warp_sum(row);
-            if (lane == 0 && j < len) probs[j] = sc * row;
+        if (rows) {
+            for (int o = lpr >> 1; o > 0; o >>= 1) row += __shfl_xor_sync(FULL, row, o);
+            if (lr == 0) row_sm[rl] = sc * row;
+            __syncthreads();
+            const int64_t v = j0 + threadIdx.x;
+            if ((int)threadIdx.x < rpb && v < len) probs[v] = row_sm[threadIdx.x];
+            __syncthreads();
         }
     }
     if (reg == 1 || reg == 4) return;
@@ -913,23 +931,27 @@ cudaError_t launch_pos_t(const QwSimDev &d, const QwPosPlan &pl, const QwPosArgs
 
 template <typename AmpT>
 cudaError_t launch_tinit_pos_t(const QwSimDev &d, void *pbuf, int full, int64_t g0, int64_t n, int64_t x0, int64_t nx,
-                               const double *b_re, const double *b_im, const double *scale, cudaStream_t st)
+                               const double *b_re, const double *b_im, const double *scale, const QwScalarWords &words,
+                               cudaStream_t st)
 {
     const int64_t want = (n * d.s + nx + 255) / 256, cap = 16 * (int64_t)qw_sm_count();
     k_tinit_pos<AmpT><<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(
-        d, static_cast<AmpT *>(pbuf), full, (uint32_t)g0, (uint32_t)n, (uint32_t)x0, (uint32_t)nx, b_re, b_im, scale);
+        d, static_cast<AmpT *>(pbuf), full, (uint32_t)g0, (uint32_t)n, (uint32_t)x0, (uint32_t)nx, b_re, b_im, scale, words);
     return cudaGetLastError();
 }
 
 template <typename AmpT>
 cudaError_t launch_measure_pos_t(const QwSimDev &d, const void *pbuf, int full, int64_t g0, int64_t n,
-                                 const double *scale, int reg, double *probs, int64_t len, cudaStream_t st)
+                                 const double *scale, int reg, double *probs, int64_t len,
+                                 const unsigned long long *stat_src, unsigned long long *stat_dst, cudaStream_t st)
 {
-    /* a warp per j: enough blocks that every j's loads are in flight at once;
-       the plane sums with one atomic per block: fewer blocks */
-    const int64_t want = (n + 7) / 8, cap = (reg == 1 || reg == 4 ? 32 : 4) * (int64_t)qw_sm_count();
+    /* j, k: enough blocks that every row's loads are in flight at once; the
+       other registers, with one atomic per block: fewer */
+    const bool rows = reg == 1 || reg == 4;
+    const int64_t rpb = 256 / (d.s >= 32 ? 32 : d.s), end = rows && len > n ? len : n;
+    const int64_t want = (end + rpb - 1) / rpb, cap = (rows ? 64 : 4) * (int64_t)qw_sm_count();
     k_measure_pos<AmpT><<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(
-        d, static_cast<const AmpT *>(pbuf), full, g0, n, scale, reg, probs, len);
+        d, static_cast<const AmpT *>(pbuf), full, g0, n, scale, reg, probs, len, stat_src, stat_dst);
     return cudaGetLastError();
 }
 
@@ -960,16 +982,16 @@ cudaError_t launch_pos_unpack_t(const QwSimDev &d, const void *pbuf, int full, c
     }                                                                                                                 \
     cudaError_t qw_launch_tinit_pos##SUFFIX(const QwSimDev &d, void *pbuf, int full, int64_t g0, int64_t n,           \
                                             int64_t x0, int64_t nx, const double *b_re, const double *b_im,           \
-                                            const double *scale,                                                      \
-                                            cudaStream_t st)                                                          \
+                                            const double *scale, const QwScalarWords &words, cudaStream_t st)         \
     {                                                                                                                 \
-        return launch_tinit_pos_t<AmpT>(d, pbuf, full, g0, n, x0, nx, b_re, b_im, scale, st);                               \
+        return launch_tinit_pos_t<AmpT>(d, pbuf, full, g0, n, x0, nx, b_re, b_im, scale, words, st);                  \
     }                                                                                                                 \
     cudaError_t qw_launch_measure_pos##SUFFIX(const QwSimDev &d, const void *pbuf, int full, int64_t g0, int64_t n,   \
                                               const double *scale, int reg, double *probs, int64_t len,               \
+                                              const unsigned long long *stat_src, unsigned long long *stat_dst,       \
                                               cudaStream_t st)                                                        \
     {                                                                                                                 \
-        return launch_measure_pos_t<AmpT>(d, pbuf, full, g0, n, scale, reg, probs, len, st);                          \
+        return launch_measure_pos_t<AmpT>(d, pbuf, full, g0, n, scale, reg, probs, len, stat_src, stat_dst, st);      \
     }                                                                                                                 \
     cudaError_t qw_launch_pos_pack##SUFFIX(const QwSimDev &d, const QwBufDev &buf, void *pbuf, int32_t *status,       \
                                            cudaStream_t st)                                                           \
