@@ -911,6 +911,25 @@ static cudaError_t flat_alloc(qw_sim *sim, size_t bytes, void **p)
     return cudaMallocFromPoolAsync(p, bytes < 16 ? 16 : bytes, sim->fpool, sim->stream);
 }
 
+/* Scratch of one call, given back to the pool on every way out. */
+struct FlatScratch {
+    qw_sim *sim;
+    std::vector<void *> all;
+    explicit FlatScratch(qw_sim *s) : sim(s) {}
+    FlatScratch(const FlatScratch &) = delete;
+    FlatScratch &operator=(const FlatScratch &) = delete;
+    ~FlatScratch()
+    {
+        for (void *p : all) cudaFreeAsync(p, sim->stream);
+    }
+    cudaError_t take(size_t bytes, void **p)
+    {
+        const cudaError_t e = flat_alloc(sim, bytes, p);
+        if (e == cudaSuccess) all.push_back(*p);
+        return e;
+    }
+};
+
 static void flat_release(qw_sim *sim, FlatList &L)
 {
     if (L.K) cudaFreeAsync(L.K, sim->stream);
@@ -936,8 +955,8 @@ static cudaError_t flat_gather(qw_sim *sim, FlatList &L, int kw)
     if ((e = flat_alloc(sim, (size_t)L.M * 8 * kw, &L.K)) != cudaSuccess) return e;
     if ((e = flat_alloc(sim, (size_t)L.M * 16, (void **)&L.A)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(&sim->sc->counter, 0, 8, st)) != cudaSuccess) return e;
-    return qw_flat_gather(sim->d, sim->buf[sim->cur], sim->fp32, pending_scale(sim), L.K, L.A, &sim->sc->counter, L.M,
-                          st, kw);
+    return qw_flat_gather(sim->d, sim->buf[sim->cur], -1, sim->fp32, pending_scale(sim), L.K, L.A, &sim->sc->counter,
+                          L.M, st, kw);
 }
 
 /* An interference op on the list (0 = R^dag, 1 = R, 2 = H): grouping by a
@@ -2082,12 +2101,6 @@ static uint64_t get_bits(const uint64_t *w, int pos, int width)
     return v;
 }
 
-static void put_bits(uint64_t *w, int pos, uint64_t v, int width)
-{
-    for (int b = 0; b < width; ++b)
-        if ((v >> b) & 1ull) w[(pos + b) >> 6] |= 1ull << ((pos + b) & 63);
-}
-
 extern "C" int qw_state_export(qw_sim *sim, int32_t inst, int32_t key_words, uint64_t *keys,
                                double *amps, int64_t cap, int64_t *count)
 {
@@ -2102,57 +2115,40 @@ extern "C" int qw_state_export(qw_sim *sim, int32_t inst, int32_t key_words, uin
     if (rc != QW_OK) return rc;
     *count = total;
     if (total == 0 || cap <= 0) return QW_OK;
-    uint64_t *drow = nullptr, *dloc = nullptr;
-    double2 *damp = nullptr;
-    QW_CUDA(sim, cudaMallocAsync((void **)&drow, (size_t)total * 8, sim->stream));
-    QW_CUDA(sim, cudaMallocAsync((void **)&dloc, (size_t)total * 8, sim->stream));
-    QW_CUDA(sim, cudaMallocAsync((void **)&damp, (size_t)total * 16, sim->stream));
-    QW_CUDA(sim, cudaMemsetAsync(&sim->sc->counter, 0, 8, sim->stream));
-    QW_CUDA(sim, qw_launch_export(sim->d, sim->buf[sim->cur], inst, sim->fp32, pending_scale(sim), drow,
-                                  dloc, damp, &sim->sc->counter, total, sim->stream));
+    /* gathered, sorted by key and laid out on the device; the caller's arrays
+       are written once the status is known to be clean */
+    cudaStream_t st = sim->stream;
+    FlatScratch scratch(sim);
+    const size_t M = (size_t)total, W = (size_t)key_words;
+    void *K = nullptr, *A = nullptr, *tk = nullptr, *ta = nullptr, *work = nullptr, *out = nullptr;
+    QW_CUDA(sim, scratch.take(M * 16, &K));
+    QW_CUDA(sim, scratch.take(M * 16, &A));
+    QW_CUDA(sim, scratch.take(M * 16, &tk));
+    QW_CUDA(sim, scratch.take(M * 16, &ta));
+    QW_CUDA(sim, scratch.take(qw_flat_sort_bytes(total), &work));
+    QW_CUDA(sim, cudaMemsetAsync(&sim->sc->counter, 0, 8, st));
+    QW_CUDA(sim, qw_flat_gather(sim->d, sim->buf[sim->cur], inst, sim->fp32, pending_scale(sim), K,
+                                static_cast<double2 *>(A), &sim->sc->counter, total, st, 2));
     sim->launches++;
-    std::vector<uint64_t> hrow((size_t)total), hloc((size_t)total);
-    std::vector<double2> hamp((size_t)total);
-    QW_CUDA(sim, cudaMemcpyAsync(hrow.data(), drow, (size_t)total * 8, cudaMemcpyDeviceToHost, sim->stream));
-    QW_CUDA(sim, cudaMemcpyAsync(hloc.data(), dloc, (size_t)total * 8, cudaMemcpyDeviceToHost, sim->stream));
-    QW_CUDA(sim, cudaMemcpyAsync(hamp.data(), damp, (size_t)total * 16, cudaMemcpyDeviceToHost, sim->stream));
-    QW_CUDA(sim, cudaFreeAsync(drow, sim->stream));
-    QW_CUDA(sim, cudaFreeAsync(dloc, sim->stream));
-    QW_CUDA(sim, cudaFreeAsync(damp, sim->stream));
+    int in_tmp = 0;
+    QW_CUDA(sim, qw_flat_sort(sim->d, K, static_cast<double2 *>(A), tk, static_cast<double2 *>(ta), total, 0, work,
+                              &sim->sc->status, st, 2, &in_tmp));
+    if (in_tmp) {
+        std::swap(K, tk);
+        std::swap(A, ta);
+    }
+    const int64_t nout = std::min(total, cap);
+    out = K;
+    if (W != 2) {
+        QW_CUDA(sim, scratch.take((size_t)nout * W * 8, &out));
+        QW_CUDA(sim, qw_io_store(K, key_words, nout, static_cast<uint64_t *>(out), st));
+        sim->launches++;
+    }
     rc = check_status(sim, "qw_state_export");
     if (rc != QW_OK) return rc;
-    /* pack: b2 | k | kc | b1 | j | jc | A | inst */
-    const size_t W = (size_t)key_words;
-    std::vector<uint64_t> packed((size_t)total * W, 0ull);
-    const uint64_t m = (1ull << nb) - 1;
-    for (int64_t i = 0; i < total; ++i) {
-        const uint64_t rk = hrow[(size_t)i], lk = hloc[(size_t)i];
-        uint64_t *w = packed.data() + (size_t)i * W;
-        int p = 0;
-        put_bits(w, p, lk & 1ull, 1); p += 1;                      /* b2 */
-        put_bits(w, p, (lk >> 1) & m, nb); p += nb;                /* k */
-        put_bits(w, p, (lk >> (1 + nb)) & m, nb); p += nb;         /* kc */
-        put_bits(w, p, rk & 1ull, 1); p += 1;                      /* b1 */
-        put_bits(w, p, (rk >> 1) & 0x7ffffull, nb); p += nb;       /* j */
-        put_bits(w, p, (rk >> 20) & 0xfffffull, nb); p += nb;      /* jc */
-        put_bits(w, p, (lk >> (1 + 2 * nb)) & 0xffffull, 16); p += 16; /* A */
-        put_bits(w, p, rk >> 40, 16);                              /* inst */
-    }
-    std::vector<int64_t> order((size_t)total);
-    for (int64_t i = 0; i < total; ++i) order[(size_t)i] = i;
-    std::sort(order.begin(), order.end(), [&](int64_t x, int64_t y) {
-        const uint64_t *a = packed.data() + (size_t)x * W, *b = packed.data() + (size_t)y * W;
-        for (size_t t = W; t-- > 0;)
-            if (a[t] != b[t]) return a[t] < b[t];
-        return false;
-    });
-    const int64_t nout = std::min(total, cap);
-    for (int64_t i = 0; i < nout; ++i) {
-        const int64_t src = order[(size_t)i];
-        std::memcpy(keys + (size_t)i * W, packed.data() + (size_t)src * W, W * 8);
-        amps[2 * i] = hamp[(size_t)src].x;
-        amps[2 * i + 1] = hamp[(size_t)src].y;
-    }
+    QW_CUDA(sim, cudaMemcpyAsync(keys, out, (size_t)nout * W * 8, cudaMemcpyDeviceToHost, st));
+    QW_CUDA(sim, cudaMemcpyAsync(amps, A, (size_t)nout * 16, cudaMemcpyDeviceToHost, st));
+    QW_CUDA(sim, cudaStreamSynchronize(st));
     return QW_OK;
 }
 
@@ -2165,6 +2161,34 @@ extern "C" int qw_step_stats(qw_sim *sim, int64_t *out, int32_t len, int32_t res
     QW_CUDA(sim, cudaStreamSynchronize(sim->stream));
     for (int i = 0; i < len && i < QW_NSTAT; ++i) out[i] = (int64_t)h[i];
     return QW_OK;
+}
+
+/* Which rule an imported list breaks: equal keys first, then the first key
+ * that the layout does not hold. */
+static int import_refused(qw_sim *sim, int32_t key_words, const uint64_t *keys, int64_t count)
+{
+    const size_t W = (size_t)key_words;
+    const int nb = sim->d.nb, layout = 4 * nb + 34;
+    std::vector<int64_t> order((size_t)count);
+    for (int64_t i = 0; i < count; ++i) order[(size_t)i] = i;
+    std::sort(order.begin(), order.end(), [&](int64_t x, int64_t y) {
+        const uint64_t *a = keys + (size_t)x * W, *b = keys + (size_t)y * W;
+        for (size_t t = W; t-- > 0;)
+            if (a[t] != b[t]) return a[t] < b[t];
+        return false;
+    });
+    for (int64_t i = 1; i < count; ++i)
+        if (std::memcmp(keys + (size_t)order[(size_t)i] * W, keys + (size_t)order[(size_t)i - 1] * W, W * 8) == 0)
+            return fail(sim, QW_ERR_ARG, "qw_state_import: duplicate key");
+    for (int64_t i = 0; i < count; ++i) {
+        const uint64_t *w = keys + (size_t)i * W;
+        for (int t = layout; t < (int)W * 64; ++t)
+            if ((w[t >> 6] >> (t & 63)) & 1ull) return fail(sim, QW_ERR_ARG, "qw_state_import: bits above the layout");
+        if (get_bits(w, 2 + 4 * nb, 16) != 0) return fail(sim, QW_ERR_ARG, "qw_state_import: register A must be 0");
+        if ((int64_t)get_bits(w, 18 + 4 * nb, 16) >= sim->d.ninst)
+            return fail(sim, QW_ERR_ARG, "qw_state_import: instance out of range");
+    }
+    return fail(sim, QW_ERR_DEVICE_STATUS, "qw_state_import: the keys changed while they were read");
 }
 
 extern "C" int qw_state_import(qw_sim *sim, int32_t key_words, const uint64_t *keys, const double *amps,
@@ -2181,52 +2205,52 @@ extern "C" int qw_state_import(qw_sim *sim, int32_t key_words, const uint64_t *k
     if (key_words < 1 || key_words > 10 || key_words * 64 < 4 * nb + 34)
         return fail(sim, QW_ERR_ARG, "key_words too small for the packed register layout");
     if (count < 0 || (count > 0 && (!keys || !amps))) return fail(sim, QW_ERR_ARG, "bad arrays");
-    const size_t W = (size_t)key_words;
-    /* distinct keys */
-    std::vector<int64_t> order((size_t)count);
-    for (int64_t i = 0; i < count; ++i) order[(size_t)i] = i;
-    std::sort(order.begin(), order.end(), [&](int64_t x, int64_t y) {
-        const uint64_t *a = keys + (size_t)x * W, *b = keys + (size_t)y * W;
-        for (size_t t = W; t-- > 0;)
-            if (a[t] != b[t]) return a[t] < b[t];
-        return false;
-    });
-    for (int64_t i = 1; i < count; ++i)
-        if (std::memcmp(keys + (size_t)order[(size_t)i] * W, keys + (size_t)order[(size_t)i - 1] * W, W * 8) == 0)
-            return fail(sim, QW_ERR_ARG, "qw_state_import: duplicate key");
-    std::vector<uint64_t> hrow((size_t)count), hloc((size_t)count);
-    std::vector<double2> hamp((size_t)count);
+    cudaStream_t st = sim->stream;
+    FlatScratch scratch(sim);
+    void *K = nullptr, *A = nullptr;
+    QwIoFlags *flags = nullptr;
     double norm2 = 0.0;
-    for (int64_t i = 0; i < count; ++i) {
-        const uint64_t *w = keys + (size_t)i * W;
-        int p = 0;
-        const uint64_t b2 = get_bits(w, p, 1); p += 1;
-        const uint64_t k = get_bits(w, p, nb); p += nb;
-        const uint64_t kc = get_bits(w, p, nb); p += nb;
-        const uint64_t b1 = get_bits(w, p, 1); p += 1;
-        const uint64_t j = get_bits(w, p, nb); p += nb;
-        const uint64_t jc = get_bits(w, p, nb); p += nb;
-        const uint64_t A = get_bits(w, p, 16); p += 16;
-        const uint64_t inst = get_bits(w, p, 16); p += 16;
-        for (int t = p; t < (int)W * 64; ++t)
-            if ((w[t >> 6] >> (t & 63)) & 1ull) return fail(sim, QW_ERR_ARG, "qw_state_import: bits above the layout");
-        if (A != 0) return fail(sim, QW_ERR_ARG, "qw_state_import: register A must be 0");
-        if ((int64_t)inst >= sim->d.ninst) return fail(sim, QW_ERR_ARG, "qw_state_import: instance out of range");
-        hrow[(size_t)i] = qw_rowkey((uint32_t)inst, (uint32_t)jc, (uint32_t)j, (uint32_t)b1);
-        hloc[(size_t)i] = b2 | (k << 1) | (kc << (1 + nb));
-        hamp[(size_t)i] = make_double2(amps[2 * i], amps[2 * i + 1]);
-        norm2 += amps[2 * i] * amps[2 * i] + amps[2 * i + 1] * amps[2 * i + 1];
-    }
-    if (sim->opts.overflow_fallback && count > 0) { /* a row longer than row_capacity: grow the buckets */
-        std::vector<uint64_t> rows(hrow);
-        std::sort(rows.begin(), rows.end());
-        int64_t longest = 0;
-        for (size_t i = 0, j = 0; i < rows.size(); i = j) {
-            while (j < rows.size() && rows[j] == rows[i]) ++j;
-            longest = std::max<int64_t>(longest, (int64_t)(j - i));
+    if (count > 0) {
+        const size_t M = (size_t)count;
+        void *in = nullptr;
+        QW_CUDA(sim, scratch.take(M * (size_t)key_words * 8, &in));
+        QW_CUDA(sim, scratch.take(M * 16, &K));
+        QW_CUDA(sim, scratch.take(M * 16, &A));
+        QW_CUDA(sim, scratch.take(sizeof(QwIoFlags), (void **)&flags));
+        QW_CUDA(sim, cudaMemsetAsync(flags, 0, sizeof(QwIoFlags), st));
+        QW_CUDA(sim, cudaMemcpyAsync(in, keys, M * (size_t)key_words * 8, cudaMemcpyHostToDevice, st));
+        QW_CUDA(sim, qw_io_load(sim->d, static_cast<uint64_t *>(in), key_words, count, K, flags, st));
+        QW_CUDA(sim, qw_io_order(sim->d, K, count, flags, st));
+        sim->launches += 2;
+        QW_CUDA(sim, cudaMemcpyAsync(A, amps, M * 16, cudaMemcpyHostToDevice, st));
+        for (int64_t i = 0; i < count; ++i) norm2 += amps[2 * i] * amps[2 * i] + amps[2 * i + 1] * amps[2 * i + 1];
+        QwIoFlags h{};
+        QW_CUDA(sim, cudaMemcpyAsync(&h, flags, sizeof h, cudaMemcpyDeviceToHost, st));
+        QW_CUDA(sim, cudaStreamSynchronize(st));
+        if (h.unsorted && !h.bad) { /* an exported list is sorted; any other is sorted here */
+            void *tk = nullptr, *ta = nullptr, *work = nullptr;
+            QW_CUDA(sim, scratch.take(M * 16, &tk));
+            QW_CUDA(sim, scratch.take(M * 16, &ta));
+            QW_CUDA(sim, scratch.take(qw_flat_sort_bytes(count), &work));
+            QW_CUDA(sim, cudaMemsetAsync(flags, 0, sizeof(QwIoFlags), st));
+            int in_tmp = 0;
+            QW_CUDA(sim, qw_flat_sort(sim->d, K, static_cast<double2 *>(A), tk, static_cast<double2 *>(ta), count, 0,
+                                      work, &flags->status, st, 2, &in_tmp));
+            if (in_tmp) {
+                std::swap(K, tk);
+                std::swap(A, ta);
+            }
+            QW_CUDA(sim, qw_io_order(sim->d, K, count, flags, st));
+            sim->launches++;
+            QW_CUDA(sim, cudaMemcpyAsync(&h, flags, sizeof h, cudaMemcpyDeviceToHost, st));
+            QW_CUDA(sim, cudaStreamSynchronize(st));
+            if (h.status != 0 || h.unsorted)
+                return fail(sim, QW_ERR_DEVICE_STATUS, "qw_state_import: the sort of the keys gave up waiting for a tile's count");
         }
-        if (longest > sim->d.cap_row) {
-            int rc = grow_rows(sim, longest);
+        if (h.bad || h.dup) return import_refused(sim, key_words, keys, count);
+        /* a row longer than row_capacity: grow the buckets */
+        if (sim->opts.overflow_fallback && (int64_t)h.longest > sim->d.cap_row) {
+            const int rc = grow_rows(sim, (int64_t)h.longest);
             if (rc != QW_OK) return rc;
         }
     }
@@ -2243,20 +2267,9 @@ extern "C" int qw_state_import(qw_sim *sim, int32_t key_words, const uint64_t *k
     sim->sync_done = 0;
     drop_graphs(sim);
     if (count > 0) {
-        uint64_t *drow = nullptr, *dloc = nullptr;
-        double2 *damp = nullptr;
-        QW_CUDA(sim, cudaMallocAsync((void **)&drow, (size_t)count * 8, sim->stream));
-        QW_CUDA(sim, cudaMallocAsync((void **)&dloc, (size_t)count * 8, sim->stream));
-        QW_CUDA(sim, cudaMallocAsync((void **)&damp, (size_t)count * 16, sim->stream));
-        QW_CUDA(sim, cudaMemcpyAsync(drow, hrow.data(), (size_t)count * 8, cudaMemcpyHostToDevice, sim->stream));
-        QW_CUDA(sim, cudaMemcpyAsync(dloc, hloc.data(), (size_t)count * 8, cudaMemcpyHostToDevice, sim->stream));
-        QW_CUDA(sim, cudaMemcpyAsync(damp, hamp.data(), (size_t)count * 16, cudaMemcpyHostToDevice, sim->stream));
-        QW_CUDA(sim, qw_launch_import(sim->d, sim->buf[sim->cur], drow, dloc, damp, count, sim->fp32,
-                                      &sim->sc->status, sim->stream));
+        QW_CUDA(sim, qw_flat_scatter(sim->d, sim->buf[sim->cur], sim->fp32, K, static_cast<double2 *>(A), count,
+                                     &sim->sc->status, &flags->maxrow, &flags->norm, st, 2));
         sim->launches++;
-        QW_CUDA(sim, cudaFreeAsync(drow, sim->stream));
-        QW_CUDA(sim, cudaFreeAsync(dloc, sim->stream));
-        QW_CUDA(sim, cudaFreeAsync(damp, sim->stream));
     }
     int rc = check_status(sim, "qw_state_import");
     if (rc != QW_OK) return rc;

@@ -206,7 +206,7 @@ __device__ __forceinline__ bool same_group(const FKeyN<NW> &a, const FKeyN<NW> &
 /* ---- gather, maps, phase ------------------------------------------------------ */
 
 template <typename AmpT, int NW>
-__global__ void k_f_gather(QwSimDev d, QwBufDev buf, const double *scale, FKeyN<NW> *keys, double2 *amps,
+__global__ void k_f_gather(QwSimDev d, QwBufDev buf, int inst, const double *scale, FKeyN<NW> *keys, double2 *amps,
                            unsigned long long *counter, int64_t cap)
 {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -220,9 +220,13 @@ __global__ void k_f_gather(QwSimDev d, QwBufDev buf, const double *scale, FKeyN<
         if (n > d.cap_row) n = d.cap_row;
         Row r;
         if (!row_of(d, buf, b, r)) continue;
+        if (inst >= 0 && r.inst != (uint32_t)inst) continue;
+        unsigned long long p0 = 0; /* a row's branches take adjacent places: one atomic a row */
+        if (lane == 0) p0 = atomicAdd(counter, (unsigned long long)n);
+        p0 = __shfl_sync(FULL, p0, 0);
         for (int i = lane; i < n; i += 32) {
             const int64_t slot = b * (int64_t)d.cap_row + i;
-            const unsigned long long p = atomicAdd(counter, 1ull);
+            const unsigned long long p = p0 + (unsigned long long)i;
             if ((int64_t)p >= cap) continue;
             FRegs f;
             f.inst = r.inst;
@@ -1103,6 +1107,7 @@ __global__ void k_f_scatter(QwSimDev d, QwBufDev out, const FKeyN<NW> *keys, con
     __shared__ double ws[8];
     const FLayout L = flayout(d.nb);
     double acc = 0.0;
+    unsigned int longest = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += (int64_t)gridDim.x * blockDim.x) {
         const FRegs f = fdecode(fbase_load(keys + i), L);
         if (f.x.A != 0) {
@@ -1112,7 +1117,7 @@ __global__ void k_f_scatter(QwSimDev d, QwBufDev out, const FKeyN<NW> *keys, con
         const int64_t b = bucket_of(d, out, f.inst, f.jc, f.j, f.b1, status);
         if (b < 0) continue;
         const int p = atomicAdd(out.count + b, 1);
-        atomicMax(maxrow, (unsigned int)(p + 1));
+        longest = max(longest, (unsigned int)(p + 1));
         if (p >= d.cap_row) {
             atomicOr(status, QW_ST_ROW_OVERFLOW);
             continue;
@@ -1122,7 +1127,11 @@ __global__ void k_f_scatter(QwSimDev d, QwBufDev out, const FKeyN<NW> *keys, con
         acc += store_amp<AmpT>(out.amp, slot, amps[i]);
     }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
+    longest = __reduce_max_sync(FULL, longest);
+    if ((threadIdx.x & 31) == 0) {
+        ws[threadIdx.x >> 5] = acc;
+        if (longest) atomicMax(maxrow, longest);
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
@@ -1151,6 +1160,76 @@ __global__ void k_f_finish(QwStepArgs a, const double *norm, unsigned long long 
     }
 }
 
+/* ---- state import and export ------------------------------------------------------ */
+/*
+ * A list of branches as the caller holds it: W 64-bit words a key, of which
+ * the layout takes the low 4 nb + 34 bits.  All passes are streams over 32 to
+ * 100 bytes a branch.  N = 2047, s = 8 (49 000 branches), an import, ten steps and
+ * an export: 12.30 ms with the keys packed bit by bit and sorted by comparison on
+ * the host, 0.74 ms so (what is left: launches, synchronisations and the copies
+ * from and to the caller's pageable arrays).
+ */
+
+/* keys of W words to the two-word layout, *bad set by one that the layout
+   does not hold: a bit above it, a non-zero A, an instance beyond the last */
+__global__ void k_io_load(const uint64_t *in, int W, int64_t M, FLayout L, uint32_t ninst, FKey *keys, QwIoFlags *f)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += (int64_t)gridDim.x * blockDim.x) {
+        FKey k;
+        k.w[0] = in[i * W];
+        k.w[1] = W > 1 ? in[i * W + 1] : 0ull;
+        uint64_t above = L.pinst + 16 < 64 ? k.w[1] | (k.w[0] >> (L.pinst + 16))
+                                           : (L.pinst + 16 == 64 ? k.w[1] : k.w[1] >> (L.pinst + 16 - 64));
+        for (int t = 2; t < W; ++t) above |= in[i * W + t];
+        if (above != 0ull || fget(k, L.pA, 16) != 0ull || fget(k, L.pinst, 16) >= ninst) f->bad = 1;
+        keys[i] = k;
+    }
+}
+
+/* the order of the list: *unsorted unless ascending, *dup if two neighbours
+   are equal, and the longest run of one row (inst, A, jc, j, b1: the bits from
+   b1 up), found from its first member by doubling and bisection -- a row's
+   length where the list is sorted */
+__global__ void k_io_order(const FKey *keys, int64_t M, FLayout L, QwIoFlags *f)
+{
+    unsigned int longest = 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += (int64_t)gridDim.x * blockDim.x) {
+        const FKey k = keys[i];
+        auto same_row = [&](const FKey &o) { return o.w[1] == k.w[1] && (o.w[0] >> L.pb1) == (k.w[0] >> L.pb1); };
+        if (i > 0) {
+            const FKey q = keys[i - 1];
+            if (q.w[1] == k.w[1] && q.w[0] == k.w[0]) f->dup = 1;
+            if (q.w[1] > k.w[1] || (q.w[1] == k.w[1] && q.w[0] > k.w[0])) f->unsorted = 1;
+            if (same_row(q)) continue;
+        }
+        int64_t in = i, step = 1; /* in: in the run */
+        while (in + step < M && same_row(keys[in + step])) {
+            in += step;
+            step <<= 1;
+        }
+        int64_t out = in + step < M ? in + step : M; /* beyond it */
+        while (out - in > 1) {
+            const int64_t m = (in + out) >> 1;
+            if (same_row(keys[m])) in = m;
+            else out = m;
+        }
+        const int64_t len = out - i;
+        longest = max(longest, (unsigned int)(len < 0x7fffffff ? len : 0x7fffffff));
+    }
+    longest = __reduce_max_sync(FULL, longest);
+    if ((threadIdx.x & 31) == 0 && longest) atomicMax(&f->longest, longest);
+}
+
+/* two-word keys to W words */
+__global__ void k_io_store(const FKey *keys, int W, int64_t M, uint64_t *out)
+{
+    const int64_t n = M * W;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t t = i % W;
+        out[i] = t < 2 ? keys[i / W].w[t] : 0ull;
+    }
+}
+
 int grid_for(int64_t n, int threads)
 {
     int64_t g = (n + threads - 1) / threads;
@@ -1168,21 +1247,21 @@ cudaError_t flat_sort_t(const QwSimDev &d, void *keys, double2 *amps, void *tmpk
 /* ---- launchers ------------------------------------------------------------------------ */
 /* kw: the key words (2, the export layout; 10, the register-faithful layout) */
 
-cudaError_t qw_flat_gather(const QwSimDev &d, const QwBufDev &buf, int fp32, const double *scale, void *keys,
-                           double2 *amps, unsigned long long *counter, int64_t cap, cudaStream_t st, int kw)
+cudaError_t qw_flat_gather(const QwSimDev &d, const QwBufDev &buf, int inst, int fp32, const double *scale,
+                           void *keys, double2 *amps, unsigned long long *counter, int64_t cap, cudaStream_t st, int kw)
 {
     const int grid = 4 * qw_sm_count();
     if (kw == NW_FAITH) {
         if (fp32)
-            k_f_gather<float2, NW_FAITH><<<grid, 256, 0, st>>>(d, buf, scale, static_cast<FKeyW *>(keys), amps,
+            k_f_gather<float2, NW_FAITH><<<grid, 256, 0, st>>>(d, buf, inst, scale, static_cast<FKeyW *>(keys), amps,
                                                                counter, cap);
         else
-            k_f_gather<double2, NW_FAITH><<<grid, 256, 0, st>>>(d, buf, scale, static_cast<FKeyW *>(keys), amps,
+            k_f_gather<double2, NW_FAITH><<<grid, 256, 0, st>>>(d, buf, inst, scale, static_cast<FKeyW *>(keys), amps,
                                                                 counter, cap);
     } else if (fp32) {
-        k_f_gather<float2, 2><<<grid, 256, 0, st>>>(d, buf, scale, static_cast<FKey *>(keys), amps, counter, cap);
+        k_f_gather<float2, 2><<<grid, 256, 0, st>>>(d, buf, inst, scale, static_cast<FKey *>(keys), amps, counter, cap);
     } else {
-        k_f_gather<double2, 2><<<grid, 256, 0, st>>>(d, buf, scale, static_cast<FKey *>(keys), amps, counter, cap);
+        k_f_gather<double2, 2><<<grid, 256, 0, st>>>(d, buf, inst, scale, static_cast<FKey *>(keys), amps, counter, cap);
     }
     return cudaGetLastError();
 }
@@ -1472,6 +1551,28 @@ cudaError_t qw_flat_finish(const QwStepArgs &a, const double *norm, const int64_
     k_f_finish<<<1, 1, 0, st>>>(a, norm, (unsigned long long)counts[0], (unsigned long long)counts[1],
                                 (unsigned long long)counts[2], (unsigned long long)counts[3],
                                 (unsigned long long)counts[4]);
+    return cudaGetLastError();
+}
+
+cudaError_t qw_io_load(const QwSimDev &d, const uint64_t *in, int words, int64_t M, void *keys, QwIoFlags *f,
+                       cudaStream_t st)
+{
+    if (M <= 0) return cudaSuccess;
+    k_io_load<<<grid_for(M, 256), 256, 0, st>>>(in, words, M, flayout(d.nb), (uint32_t)d.ninst, static_cast<FKey *>(keys), f);
+    return cudaGetLastError();
+}
+
+cudaError_t qw_io_order(const QwSimDev &d, const void *keys, int64_t M, QwIoFlags *f, cudaStream_t st)
+{
+    if (M <= 0) return cudaSuccess;
+    k_io_order<<<grid_for(M, 256), 256, 0, st>>>(static_cast<const FKey *>(keys), M, flayout(d.nb), f);
+    return cudaGetLastError();
+}
+
+cudaError_t qw_io_store(const void *keys, int words, int64_t M, uint64_t *out, cudaStream_t st)
+{
+    if (M <= 0) return cudaSuccess;
+    k_io_store<<<grid_for(M * words, 256), 256, 0, st>>>(static_cast<const FKey *>(keys), words, M, out);
     return cudaGetLastError();
 }
 

@@ -256,12 +256,6 @@ cudaError_t qw_launch_init_b(const QwSimDev &d, const QwBufDev &buf, int inst, c
                              const double *b_im, int n, int fp32, const double *scale, cudaStream_t st);
 cudaError_t qw_launch_tinit(const QwSimDev &d, const QwBufDev &buf, int64_t lo, int64_t hi, int fp32,
                             int32_t *status, cudaStream_t st);
-cudaError_t qw_launch_import(const QwSimDev &d, const QwBufDev &buf, const uint64_t *rowkey,
-                             const uint64_t *local, const double2 *amp, int64_t count, int fp32,
-                             int32_t *status, cudaStream_t st);
-cudaError_t qw_launch_export(const QwSimDev &d, const QwBufDev &buf, int inst, int fp32,
-                             const double *scale, uint64_t *rowkey, uint64_t *local, double2 *amp,
-                             unsigned long long *counter, int64_t cap, cudaStream_t st);
 cudaError_t qw_launch_measure(const QwSimDev &d, const QwBufDev &buf, int inst, int fp32,
                               const double *scale, int reg, double *probs, int64_t len,
                               cudaStream_t st);
@@ -289,8 +283,9 @@ cudaError_t qw_launch_regrow(const QwSimDev &d, const QwBufDev &from, int cap_ol
 #define QW_FLAT_S 4u
 #define QW_FLAT_A0 5u /* check A = 0 */
 #define QW_FAITH_WORDS 10
-cudaError_t qw_flat_gather(const QwSimDev &d, const QwBufDev &buf, int fp32, const double *scale, void *keys,
-                           double2 *amps, unsigned long long *counter, int64_t cap, cudaStream_t st, int kw);
+/* inst >= 0: that instance's branches only */
+cudaError_t qw_flat_gather(const QwSimDev &d, const QwBufDev &buf, int inst, int fp32, const double *scale,
+                           void *keys, double2 *amps, unsigned long long *counter, int64_t cap, cudaStream_t st, int kw);
 cudaError_t qw_flat_map(const QwSimDev &d, void *keys, int64_t M, uint32_t ops, int32_t *status, cudaStream_t st,
                         int kw);
 cudaError_t qw_flat_phase(const QwSimDev &d, const void *keys, double2 *amps, int64_t M, cudaStream_t st, int kw);
@@ -319,6 +314,18 @@ cudaError_t qw_flat_readout(const QwSimDev &d, const void *keys, const double2 *
                             cudaStream_t st, int kw);
 cudaError_t qw_flat_scatter(const QwSimDev &d, const QwBufDev &out, int fp32, const void *keys, const double2 *amps,
                             int64_t M, int32_t *status, unsigned int *maxrow, double *norm, cudaStream_t st, int kw);
+/* state import and export: the caller's keys of `words` 64-bit words to the
+   two-word layout and back, and what an import has to know of its list */
+struct QwIoFlags {
+    double norm;                  /* (the scatter's, unused) */
+    unsigned int maxrow, longest; /* longest: branches of the longest row (sorted list) */
+    int32_t status;               /* the sort's */
+    int32_t bad, unsorted, dup;
+};
+cudaError_t qw_io_load(const QwSimDev &d, const uint64_t *in, int words, int64_t M, void *keys, QwIoFlags *f,
+                       cudaStream_t st);
+cudaError_t qw_io_order(const QwSimDev &d, const void *keys, int64_t M, QwIoFlags *f, cudaStream_t st);
+cudaError_t qw_io_store(const void *keys, int words, int64_t M, uint64_t *out, cudaStream_t st);
 cudaError_t qw_flat_finish(const QwStepArgs &a, const double *norm, const int64_t *counts, cudaStream_t st);
 /* register-faithful sub-operations on 10-word keys (op codes QW_FQ_* of qwalk.h) */
 int qw_faithful_layout(const QwSimDev &d, int *addr_bits, int *layout_bits);

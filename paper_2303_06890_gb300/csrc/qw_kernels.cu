@@ -2082,28 +2082,6 @@ __global__ void k_init_b(QwSimDev d, QwBufDev buf, int inst, const double *b_re,
     buf.count[b] = 1;
 }
 
-/* Append imported branches (row key, local key, amplitude) to their rows. */
-template <typename AmpT>
-__global__ void k_import(QwSimDev d, QwBufDev buf, const uint64_t *rowkey, const uint64_t *local,
-                         const double2 *amp, int64_t count, int32_t *status)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count) return;
-    const uint64_t rk = rowkey[i];
-    const uint32_t inst = (uint32_t)(rk >> 40), jc = (uint32_t)((rk >> 20) & 0xfffffu);
-    const uint32_t j = (uint32_t)((rk >> 1) & 0x7ffffu), b1 = (uint32_t)(rk & 1);
-    const int64_t b = bucket_of(d, buf, inst, jc, j, b1, status);
-    if (b < 0) return;
-    const int pos = atomicAdd(buf.count + b, 1);
-    if (pos >= d.cap_row) {
-        atomicOr(status, QW_ST_ROW_OVERFLOW);
-        return;
-    }
-    const int64_t slot = b * (int64_t)d.cap_row + pos;
-    buf.key[slot] = local[i];
-    store_amp<AmpT>(buf.amp, slot, amp[i]);
-}
-
 /* Branches received from other partitions (their S outputs for rows this
  * partition owns) appended to the buckets of their rows. */
 /* one received entry appended to its row */
@@ -2154,36 +2132,6 @@ __global__ void k_part_scale(QwPartNorms nm, const double *target, double *scale
     double sum = 0.0;
     for (int p = 0; p < nm.n; ++p) sum += *nm.norm[p];
     *scale_out = (renorm && sum > 0.0) ? sqrt(*target / sum) : 1.0;
-}
-
-/* Every branch of instance inst (-1: all) to flat (row key, local key, amp). */
-template <typename AmpT>
-__global__ void k_export(QwSimDev d, QwBufDev buf, int inst, const double *scale, uint64_t *rowkey,
-                         uint64_t *local, double2 *amp, unsigned long long *counter, int64_t cap)
-{
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    const double sc = scale ? *scale : 1.0;
-    for (int64_t b = warp; b < d.total_buckets; b += nw) {
-        int n = buf.count[b];
-        if (n <= 0) continue;
-        if (n > d.cap_row) n = d.cap_row;
-        Row r;
-        if (!row_of(d, buf, b, r)) continue;
-        if (inst >= 0 && r.inst != (uint32_t)inst) continue;
-        const uint64_t rk = qw_rowkey(r.inst, r.jc, r.j, r.b1);
-        for (int i = lane; i < n; i += 32) {
-            const int64_t slot = b * (int64_t)d.cap_row + i;
-            const unsigned long long p = atomicAdd(counter, 1ull);
-            if ((int64_t)p >= cap) continue;
-            rowkey[p] = rk;
-            local[p] = buf.key[slot];
-            double2 v = load_amp<AmpT>(buf.amp, slot);
-            if (scale) v = cscale(sc, v);
-            amp[p] = v;
-        }
-    }
 }
 
 template <typename AmpT>
@@ -2501,18 +2449,6 @@ cudaError_t qw_launch_init_b(const QwSimDev &d, const QwBufDev &buf, int inst, c
     return cudaGetLastError();
 }
 
-cudaError_t qw_launch_export(const QwSimDev &d, const QwBufDev &buf, int inst, int fp32,
-                             const double *scale, uint64_t *rowkey, uint64_t *local, double2 *amp,
-                             unsigned long long *counter, int64_t cap, cudaStream_t st)
-{
-    const int grid = 4 * qw_sm_count();
-    if (fp32)
-        k_export<float2><<<grid, 256, 0, st>>>(d, buf, inst, scale, rowkey, local, amp, counter, cap);
-    else
-        k_export<double2><<<grid, 256, 0, st>>>(d, buf, inst, scale, rowkey, local, amp, counter, cap);
-    return cudaGetLastError();
-}
-
 cudaError_t qw_launch_measure(const QwSimDev &d, const QwBufDev &buf, int inst, int fp32,
                               const double *scale, int reg, double *probs, int64_t len,
                               cudaStream_t st)
@@ -2647,16 +2583,5 @@ cudaError_t qw_launch_tinit(const QwSimDev &d, const QwBufDev &buf, int64_t lo, 
         if (k32) launch_tinit_k<double2, uint32_t>(d, buf, lo, hi, grid, status, st);
         else launch_tinit_k<double2, uint64_t>(d, buf, lo, hi, grid, status, st);
     }
-    return cudaGetLastError();
-}
-
-cudaError_t qw_launch_import(const QwSimDev &d, const QwBufDev &buf, const uint64_t *rowkey,
-                             const uint64_t *local, const double2 *amp, int64_t count, int fp32,
-                             int32_t *status, cudaStream_t st)
-{
-    const int64_t grid = (count + 255) / 256;
-    if (grid < 1) return cudaSuccess;
-    if (fp32) k_import<float2><<<(unsigned)grid, 256, 0, st>>>(d, buf, rowkey, local, amp, count, status);
-    else k_import<double2><<<(unsigned)grid, 256, 0, st>>>(d, buf, rowkey, local, amp, count, status);
     return cudaGetLastError();
 }
