@@ -1345,17 +1345,14 @@ static int pos_prepare(qw_sim *sim)
 
 /* ---- register-faithful sub-operations (qw_flat.cu, 10-word keys) ---------- */
 
-/* One sub-operation (QW_FQ_*) on L.  The operators on the base registers are
- * preceded by the check that every working register is 0. */
-static cudaError_t faithful_op(qw_sim *sim, FlatList &L, int op, FaithCounts &fc)
+/* One operator on the base registers (QW_FQ_R .. QW_FQ_FREE_A) on L, whose
+ * working registers have been found 0. */
+static cudaError_t faithful_base_op(qw_sim *sim, FlatList &L, int op, FaithCounts &fc)
 {
     const QwSimDev &d = sim->d;
     cudaStream_t st = sim->stream;
     int32_t *status = &sim->sc->status;
-    if (op >= QW_FQ_ADDR_COL && op <= QW_FQ_QRAM_VAL) return qw_faithful_op(d, L.K, L.M, op, status, st);
-    if (op < QW_FQ_R || op > QW_FQ_FREE_A) return cudaErrorInvalidValue;
-    cudaError_t e = qw_faithful_check_idle(d, L.K, L.M, status, st);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     switch (op) {
     case QW_FQ_R:
         e = flat_stage(sim, L, 1);
@@ -1375,6 +1372,38 @@ static cudaError_t faithful_op(qw_sim *sim, FlatList &L, int op, FaithCounts &fc
     case QW_FQ_FREE_A: return qw_flat_map(d, L.K, L.M, QW_FLAT_A0, status, st, L.kw);
     default: return cudaSuccess; /* QW_FQ_ALLOC_A: A is 0 wherever it is free */
     }
+}
+
+/* A sequence of sub-operations (QW_FQ_*) on L.  Those on the working
+ * registers run up to QW_FQ_RUN to a launch; the operators on the base
+ * registers are preceded by the check that every working register is 0, which
+ * the run before makes (idle: already known of L -- the base operators leave the
+ * working registers alone).  readout (nullable): the QLS read-out after the first H. */
+static cudaError_t faithful_ops(qw_sim *sim, FlatList &L, const int32_t *ops, int n, FaithCounts &fc, bool idle,
+                                const QwStepArgs *readout)
+{
+    auto working = [](int op) { return op >= QW_FQ_ADDR_COL && op <= QW_FQ_QRAM_VAL; };
+    int32_t *status = &sim->sc->status;
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < n && e == cudaSuccess;) {
+        if (working(ops[i])) {
+            int j = i + 1;
+            while (j < n && j - i < QW_FQ_RUN && working(ops[j])) ++j;
+            idle = j < n && !working(ops[j]);
+            e = qw_faithful_run(sim->d, L.K, L.M, ops + i, j - i, idle, status, sim->stream);
+            i = j;
+        } else {
+            if (ops[i] < QW_FQ_R || ops[i] > QW_FQ_FREE_A) return cudaErrorInvalidValue;
+            if (!idle) e = qw_faithful_check_idle(sim->d, L.K, L.M, status, sim->stream);
+            idle = true;
+            if (e == cudaSuccess) e = faithful_base_op(sim, L, ops[i], fc);
+            if (e == cudaSuccess && readout && ops[i] == QW_FQ_H && fc.nh == 1)
+                e = qw_flat_readout(sim->d, L.K, L.A, L.M, *readout, sim->stream, L.kw);
+            ++i;
+        }
+        sim->launches++;
+    }
+    return e;
 }
 
 static bool faithful_fits(const qw_sim *sim)
@@ -1398,11 +1427,8 @@ static int faithful_walk_step(qw_sim *sim, int readout)
     a.qls_readout = readout;
     cudaError_t e = flat_gather(sim, L, QW_FQ_KEY_WORDS);
     fc.c[0] = L.M;
-    for (int i = 0; i < QW_FQ_STEP_LEN && e == cudaSuccess; ++i) {
-        e = faithful_op(sim, L, kStep[i], fc);
-        if (e == cudaSuccess && readout && kStep[i] == QW_FQ_H && fc.nh == 1)
-            e = qw_flat_readout(sim->d, L.K, L.A, L.M, a, sim->stream, L.kw);
-    }
+    /* a gathered list's working registers are 0 */
+    if (e == cudaSuccess) e = faithful_ops(sim, L, kStep, QW_FQ_STEP_LEN, fc, true, readout ? &a : nullptr);
     if (e != cudaSuccess) {
         flat_release(sim, L);
         return cuda_fail(sim, e, "register-faithful walk step");
@@ -1465,11 +1491,8 @@ extern "C" int qw_faithful_apply(qw_sim *sim, const int32_t *ops, int32_t nops)
     for (int32_t i = 0; i < nops; ++i)
         if (ops[i] < QW_FQ_ADDR_COL || ops[i] > QW_FQ_FREE_A)
             return fail(sim, QW_ERR_ARG, "unknown sub-operation code " + std::to_string(ops[i]));
-    for (int32_t i = 0; i < nops; ++i) {
-        cudaError_t e = faithful_op(sim, sim->fq, ops[i], sim->fq_counts);
-        if (e != cudaSuccess) return cuda_fail(sim, e, "qw_faithful_apply");
-        sim->launches++;
-    }
+    const cudaError_t e = faithful_ops(sim, sim->fq, ops, nops, sim->fq_counts, false, nullptr);
+    if (e != cudaSuccess) return cuda_fail(sim, e, "qw_faithful_apply");
     return check_status(sim, "qw_faithful_apply");
 }
 

@@ -313,13 +313,14 @@ struct FaithLayout {
     int p_addr, p_left, p_right, p_mid, p_midval, p_flag, p_cl, p_ce, p_stk, frame;
 };
 
-/* field access on a key held in shared memory (k_fq: one key per thread,
-   indexed by the field's word) */
+/* field access on a key held in shared memory (k_fq: word i of the thread's
+   key at w[256 i], so that a warp's accesses to one word are conflict-free) */
+constexpr int FQ_THREADS = 256;
 __device__ __forceinline__ uint64_t sget(const uint64_t *w, int pos, int n)
 {
     const int i = pos >> 6, o = pos & 63;
-    uint64_t v = w[i] >> o;
-    if (o + n > 64 && i + 1 < NW_FAITH) v |= w[i + 1] << (64 - o);
+    uint64_t v = w[i * FQ_THREADS] >> o;
+    if (o + n > 64 && i + 1 < NW_FAITH) v |= w[(i + 1) * FQ_THREADS] << (64 - o);
     return v & (n >= 64 ? ~0ull : ((1ull << n) - 1ull));
 }
 
@@ -327,16 +328,16 @@ __device__ __forceinline__ void sput(uint64_t *w, int pos, int n, uint64_t v)
 {
     v &= (n >= 64 ? ~0ull : ((1ull << n) - 1ull));
     const int i = pos >> 6, o = pos & 63;
-    w[i] |= v << o;
-    if (o + n > 64 && i + 1 < NW_FAITH) w[i + 1] |= v >> (64 - o);
+    w[i * FQ_THREADS] |= v << o;
+    if (o + n > 64 && i + 1 < NW_FAITH) w[(i + 1) * FQ_THREADS] |= v >> (64 - o);
 }
 
 __device__ __forceinline__ void sclear(uint64_t *w, int pos, int n)
 {
     const uint64_t m = (n >= 64 ? ~0ull : ((1ull << n) - 1ull));
     const int i = pos >> 6, o = pos & 63;
-    w[i] &= ~(m << o);
-    if (o + n > 64 && i + 1 < NW_FAITH) w[i + 1] &= ~(m >> (64 - o));
+    w[i * FQ_THREADS] &= ~(m << o);
+    if (o + n > 64 && i + 1 < NW_FAITH) w[(i + 1) * FQ_THREADS] &= ~(m >> (64 - o));
 }
 
 /* sub-operation codes (the same numbering as the oracle's) */
@@ -354,166 +355,186 @@ __device__ __forceinline__ uint64_t fq_qram(const QwSimDev &d, uint64_t addr, bo
     return (uint64_t)(__ldg(d.img + addr) & 0xffffu);
 }
 
-__global__ void __launch_bounds__(256) k_fq(QwSimDev d, FKeyW *keys, int64_t M, int op, FaithLayout F, int32_t *status)
+/* A run of sub-operations (their codes in `ops`, 4 bits each, from the lowest
+ * up) on every branch, its working registers held on chip from one to the
+ * next: the key is read once and written once a run instead of once per
+ * sub-operation.  QBS: the run holds Alg. 1 (or its uncomputation), whose
+ * frames live in the key's upper words -- the whole key goes to shared memory
+ * -- otherwise the address register (bits 128 .. 128 + aw - 1, in word 2) is
+ * the only working register touched and words 0..2 are read.  idle: the
+ * working registers must be 0 after the run (an interference op, P or S
+ * follows); words 2..9 are then written only where they changed from or to
+ * something else than 0.
+ * Bound: one launch per sub-operation moved 6 x 80 to 15 x 112 bytes a branch
+ * between two interference ops; now 80 to 96, and the time is the QRAM
+ * reads of Alg. 1's probes, L + 1 dependent ones each way.  A step at N = 8192, s = 32
+ * (with T~ and two marginals): 2097 -> 1458 us. */
+template <bool QBS>
+__global__ void __launch_bounds__(FQ_THREADS) k_fq(QwSimDev d, FKeyW *keys, int64_t M, uint64_t ops, FaithLayout F,
+                                                   int idle, int32_t *status)
 {
     const FLayout L = flayout(d.nb);
     const int aw = F.aw;
-    const uint64_t ns = (uint64_t)d.n_single * (uint64_t)d.s;
-    __shared__ FKeyW sk[256];
-    uint64_t *kw = sk[threadIdx.x].w;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += (int64_t)gridDim.x * blockDim.x) {
-        sk[threadIdx.x] = keys[i];
-        FKey b = fbase(sk[threadIdx.x]);
-        FRegs f = fdecode(b, L);
-        uint64_t addr = sget(kw, F.p_addr, aw);
-        const uint64_t offset = ns + (uint64_t)f.j * (uint64_t)d.s;
-        if (op == FQ_ADDR_COL) {
-            addr ^= offset + f.x.k;
-        } else if (op == FQ_QRAM_COL) {
-            f.x.kc ^= (uint32_t)fq_qram(d, addr, true);
-        } else if (op == FQ_ADDR_VAL) {
-            if (f.jc == 0 && f.x.kc == 0) addr ^= (uint64_t)f.j * (uint64_t)d.s + f.x.k;
-        } else if (op == FQ_QRAM_VAL) {
-            if (f.jc == 0 && f.x.kc == 0) f.x.A ^= (uint32_t)fq_qram(d, addr, false);
-        } else if (op == FQ_SWAP) {
-            const uint32_t t = f.x.k;
-            f.x.k = f.x.kc;
-            f.x.kc = t;
-        } else if (op == FQ_QBS_FWD || op == FQ_QBS_BWD) {
-            uint64_t left = sget(kw, F.p_left, aw), right = sget(kw, F.p_right, aw);
-            uint64_t mid = sget(kw, F.p_mid, aw), midval = sget(kw, F.p_midval, 16);
-            uint32_t flag = (uint32_t)sget(kw, F.p_flag, 1), cl = (uint32_t)sget(kw, F.p_cl, 1);
-            uint32_t ce = (uint32_t)sget(kw, F.p_ce, 1);
-            const uint64_t target = f.x.kc;
-            if (op == FQ_QBS_FWD) { /* Alg. 1's loop, every probe's registers pushed */
-                left ^= offset;
-                right ^= left + (uint64_t)d.s;
-                flag ^= 1u;
-                for (int it = 0; it <= d.L; ++it) {
-                    if (flag) mid ^= (left + right) / 2;
-                    if (flag) midval ^= fq_qram(d, mid, true);
-                    if (flag) {
-                        cl ^= (midval < target) ? 1u : 0u;
-                        ce ^= (midval == target) ? 1u : 0u;
-                    }
-                    if (ce) f.x.k ^= (uint32_t)(mid - offset);
-                    if (ce) flag ^= 1u;
-                    if (flag && cl) {
-                        const uint64_t t = mid;
-                        mid = left;
-                        left = t;
-                    }
-                    if (flag) cl ^= 1u;
-                    if (flag && cl) {
-                        const uint64_t t = mid;
-                        mid = right;
-                        right = t;
-                    }
-                    const int pf = F.p_stk + it * F.frame; /* push: the frame takes them, zeros stay */
-                    sput(kw, pf, aw, mid);
-                    sput(kw, pf + aw, 16, midval);
-                    sput(kw, pf + aw + 16, 1, cl);
-                    sput(kw, pf + aw + 17, 1, ce);
-                    mid = midval = 0;
-                    cl = ce = 0u;
-                }
-            } else { /* the loop undone in reverse: pop, then every step inverted */
-                for (int it = d.L; it >= 0; --it) {
-                    const int pf = F.p_stk + it * F.frame;
-                    mid = sget(kw, pf, aw);
-                    midval = sget(kw, pf + aw, 16);
-                    cl = (uint32_t)sget(kw, pf + aw + 16, 1);
-                    ce = (uint32_t)sget(kw, pf + aw + 17, 1);
-                    sclear(kw, pf, F.frame);
-                    if (flag && cl) {
-                        const uint64_t t = mid;
-                        mid = right;
-                        right = t;
-                    }
-                    if (flag) cl ^= 1u;
-                    if (flag && cl) {
-                        const uint64_t t = mid;
-                        mid = left;
-                        left = t;
-                    }
-                    if (ce) flag ^= 1u;
-                    if (flag) {
-                        cl ^= (midval < target) ? 1u : 0u;
-                        ce ^= (midval == target) ? 1u : 0u;
-                    }
-                    if (flag) midval ^= fq_qram(d, mid, true);
-                    if (flag) mid ^= (left + right) / 2;
-                    if (mid != 0 || midval != 0 || cl != 0 || ce != 0) atomicOr(status, QW_ST_ANCILLA);
-                    mid = midval = 0;
-                    cl = ce = 0u;
-                }
-                flag ^= 1u;
-                right ^= left + (uint64_t)d.s;
-                left ^= offset;
-                if (left != 0 || right != 0 || flag != 0) atomicOr(status, QW_ST_ANCILLA);
-                left = right = 0;
-                flag = 0u;
-            }
-            sclear(kw, F.p_left, aw);
-            sclear(kw, F.p_right, aw);
-            sclear(kw, F.p_mid, aw);
-            sclear(kw, F.p_midval, 16);
-            sclear(kw, F.p_flag, 3);
-            sput(kw, F.p_left, aw, left);
-            sput(kw, F.p_right, aw, right);
-            sput(kw, F.p_mid, aw, mid);
-            sput(kw, F.p_midval, 16, midval);
-            sput(kw, F.p_flag, 1, flag);
-            sput(kw, F.p_cl, 1, cl);
-            sput(kw, F.p_ce, 1, ce);
-        }
-        sclear(kw, F.p_addr, aw);
-        sput(kw, F.p_addr, aw, addr);
-        frewrite(b, f, L);
-        kw[0] = b.w[0];
-        kw[1] = b.w[1];
-        keys[i] = sk[threadIdx.x];
-    }
-}
-
-/* The sub-operations that touch only the base registers and the address
- * register (ADDR_COL, QRAM_COL, SWAP, ADDR_VAL, QRAM_VAL), as k_fq runs them,
- * reading words 0..2 of the 80-byte key (the address lies at bits 128 ..
- * 128 + aw - 1, in word 2 for aw <= 64) and writing back only the words the
- * operation changes: the address word, or the base registers' two. */
-__global__ void k_fq_light(QwSimDev d, FKeyW *keys, int64_t M, int op, int aw)
-{
-    const FLayout L = flayout(d.nb);
-    const uint64_t ns = (uint64_t)d.n_single * (uint64_t)d.s;
     const uint64_t am = aw >= 64 ? ~0ull : (1ull << aw) - 1ull;
-    const bool addr_op = op == FQ_ADDR_COL || op == FQ_ADDR_VAL;
+    const uint64_t ns = (uint64_t)d.n_single * (uint64_t)d.s;
+    __shared__ uint64_t sk[QBS ? NW_FAITH * FQ_THREADS : 1];
+    uint64_t *kw = sk + (QBS ? threadIdx.x : 0);
+    const bool whole = QBS || idle;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += (int64_t)gridDim.x * blockDim.x) {
-        ulonglong2 *base = reinterpret_cast<ulonglong2 *>(keys + i);
-        uint64_t *w2p = keys[i].w + 2;
-        const ulonglong2 b01 = *base;
+        ulonglong2 *g = reinterpret_cast<ulonglong2 *>(keys + i);
+        const ulonglong2 b01 = g[0];
         FKey b;
         b.w[0] = b01.x;
         b.w[1] = b01.y;
-        FRegs f = fdecode(b, L);
-        const uint64_t w2 = op == FQ_SWAP ? 0ull : *w2p;
-        uint64_t addr = w2 & am;
-        if (addr_op) {
-            if (op == FQ_ADDR_COL) addr ^= ns + (uint64_t)f.j * (uint64_t)d.s + f.x.k;
-            else if (f.jc == 0 && f.x.kc == 0) addr ^= (uint64_t)f.j * (uint64_t)d.s + f.x.k;
-            *w2p = (w2 & ~am) | (addr & am);
-            continue;
-        }
-        if (op == FQ_QRAM_COL) {
-            f.x.kc ^= (uint32_t)fq_qram(d, addr, true);
-        } else if (op == FQ_QRAM_VAL) {
-            if (f.jc == 0 && f.x.kc == 0) f.x.A ^= (uint32_t)fq_qram(d, addr, false);
+        uint64_t w2, upper = 0ull; /* upper: words 3..9 */
+        if (whole) {
+            ulonglong2 v = g[1];
+            w2 = v.x;
+            upper = v.y;
+            if (QBS) kw[3 * FQ_THREADS] = v.y;
+#pragma unroll
+            for (int t = 2; t < NW_FAITH / 2; ++t) {
+                v = g[t];
+                upper |= v.x | v.y;
+                if (QBS) {
+                    kw[2 * t * FQ_THREADS] = v.x;
+                    kw[(2 * t + 1) * FQ_THREADS] = v.y;
+                }
+            }
+            if (QBS) kw[2 * FQ_THREADS] = w2;
         } else {
-            const uint32_t t = f.x.k;
-            f.x.k = f.x.kc;
-            f.x.kc = t;
+            w2 = keys[i].w[2];
+        }
+        const uint64_t w2_in = w2;
+        FRegs f = fdecode(b, L);
+        uint64_t addr = w2 & am;
+        const uint64_t offset = ns + (uint64_t)f.j * (uint64_t)d.s;
+        for (uint64_t o = ops; o != 0; o >>= 4) {
+            const int op = (int)(o & 15u);
+            if (op == FQ_ADDR_COL) {
+                addr ^= offset + f.x.k;
+            } else if (op == FQ_QRAM_COL) {
+                f.x.kc ^= (uint32_t)fq_qram(d, addr, true);
+            } else if (op == FQ_ADDR_VAL) {
+                if (f.jc == 0 && f.x.kc == 0) addr ^= (uint64_t)f.j * (uint64_t)d.s + f.x.k;
+            } else if (op == FQ_QRAM_VAL) {
+                if (f.jc == 0 && f.x.kc == 0) f.x.A ^= (uint32_t)fq_qram(d, addr, false);
+            } else if (op == FQ_SWAP) {
+                const uint32_t t = f.x.k;
+                f.x.k = f.x.kc;
+                f.x.kc = t;
+            } else if (QBS) { /* FQ_QBS_FWD, FQ_QBS_BWD */
+                uint64_t left = sget(kw, F.p_left, aw), right = sget(kw, F.p_right, aw);
+                uint64_t mid = sget(kw, F.p_mid, aw), midval = sget(kw, F.p_midval, 16);
+                uint32_t flag = (uint32_t)sget(kw, F.p_flag, 1), cl = (uint32_t)sget(kw, F.p_cl, 1);
+                uint32_t ce = (uint32_t)sget(kw, F.p_ce, 1);
+                const uint64_t target = f.x.kc;
+                if (op == FQ_QBS_FWD) { /* Alg. 1's loop, every probe's registers pushed */
+                    left ^= offset;
+                    right ^= left + (uint64_t)d.s;
+                    flag ^= 1u;
+                    for (int it = 0; it <= d.L; ++it) {
+                        if (flag) mid ^= (left + right) / 2;
+                        if (flag) midval ^= fq_qram(d, mid, true);
+                        if (flag) {
+                            cl ^= (midval < target) ? 1u : 0u;
+                            ce ^= (midval == target) ? 1u : 0u;
+                        }
+                        if (ce) f.x.k ^= (uint32_t)(mid - offset);
+                        if (ce) flag ^= 1u;
+                        if (flag && cl) {
+                            const uint64_t t = mid;
+                            mid = left;
+                            left = t;
+                        }
+                        if (flag) cl ^= 1u;
+                        if (flag && cl) {
+                            const uint64_t t = mid;
+                            mid = right;
+                            right = t;
+                        }
+                        const int pf = F.p_stk + it * F.frame; /* push: the frame takes them, zeros stay */
+                        sput(kw, pf, aw, mid);
+                        sput(kw, pf + aw, 16, midval);
+                        sput(kw, pf + aw + 16, 1, cl);
+                        sput(kw, pf + aw + 17, 1, ce);
+                        mid = midval = 0;
+                        cl = ce = 0u;
+                    }
+                } else { /* the loop undone in reverse: pop, then every step inverted */
+                    for (int it = d.L; it >= 0; --it) {
+                        const int pf = F.p_stk + it * F.frame;
+                        mid = sget(kw, pf, aw);
+                        midval = sget(kw, pf + aw, 16);
+                        cl = (uint32_t)sget(kw, pf + aw + 16, 1);
+                        ce = (uint32_t)sget(kw, pf + aw + 17, 1);
+                        sclear(kw, pf, F.frame);
+                        if (flag && cl) {
+                            const uint64_t t = mid;
+                            mid = right;
+                            right = t;
+                        }
+                        if (flag) cl ^= 1u;
+                        if (flag && cl) {
+                            const uint64_t t = mid;
+                            mid = left;
+                            left = t;
+                        }
+                        if (ce) flag ^= 1u;
+                        if (flag) {
+                            cl ^= (midval < target) ? 1u : 0u;
+                            ce ^= (midval == target) ? 1u : 0u;
+                        }
+                        if (flag) midval ^= fq_qram(d, mid, true);
+                        if (flag) mid ^= (left + right) / 2;
+                        if (mid != 0 || midval != 0 || cl != 0 || ce != 0) atomicOr(status, QW_ST_ANCILLA);
+                        mid = midval = 0;
+                        cl = ce = 0u;
+                    }
+                    flag ^= 1u;
+                    right ^= left + (uint64_t)d.s;
+                    left ^= offset;
+                    if (left != 0 || right != 0 || flag != 0) atomicOr(status, QW_ST_ANCILLA);
+                    left = right = 0;
+                    flag = 0u;
+                }
+                sclear(kw, F.p_left, aw);
+                sclear(kw, F.p_right, aw);
+                sclear(kw, F.p_mid, aw);
+                sclear(kw, F.p_midval, 16);
+                sclear(kw, F.p_flag, 3);
+                sput(kw, F.p_left, aw, left);
+                sput(kw, F.p_right, aw, right);
+                sput(kw, F.p_mid, aw, mid);
+                sput(kw, F.p_midval, 16, midval);
+                sput(kw, F.p_flag, 1, flag);
+                sput(kw, F.p_cl, 1, cl);
+                sput(kw, F.p_ce, 1, ce);
+            }
+            /* a register holds what its field has room for */
+            addr &= am;
+            f.x.k &= (1u << L.nb) - 1u;
+            f.x.kc &= (1u << L.nb) - 1u;
+        }
+        uint64_t upper_out = upper;
+        if (QBS) {
+            w2 = kw[2 * FQ_THREADS];
+            upper_out = 0ull;
+#pragma unroll
+            for (int t = 3; t < NW_FAITH; ++t) upper_out |= kw[t * FQ_THREADS];
+        }
+        w2 = (w2 & ~am) | addr;
+        if (idle && (w2 | upper_out) != 0ull) atomicOr(status, QW_ST_ANCILLA);
+        if (QBS && (upper | upper_out) != 0ull) {
+            g[1] = make_ulonglong2(w2, kw[3 * FQ_THREADS]);
+#pragma unroll
+            for (int t = 2; t < NW_FAITH / 2; ++t)
+                g[t] = make_ulonglong2(kw[2 * t * FQ_THREADS], kw[(2 * t + 1) * FQ_THREADS]);
+        } else if (w2 != w2_in) {
+            keys[i].w[2] = w2;
         }
         frewrite(b, f, L);
-        *base = make_ulonglong2(b.w[0], b.w[1]);
+        if (b.w[0] != b01.x || b.w[1] != b01.y) g[0] = make_ulonglong2(b.w[0], b.w[1]);
     }
 }
 
@@ -1607,15 +1628,21 @@ int qw_faithful_layout(const QwSimDev &d, int *addr_bits, int *layout_bits)
     return bits <= 64 * NW_FAITH && d.L + 1 <= QW_FQ_FRAMES;
 }
 
-cudaError_t qw_faithful_op(const QwSimDev &d, void *keys, int64_t M, int op, int32_t *status, cudaStream_t st)
+cudaError_t qw_faithful_run(const QwSimDev &d, void *keys, int64_t M, const int32_t *ops, int n, int idle,
+                            int32_t *status, cudaStream_t st)
 {
-    if (M <= 0) return cudaSuccess;
-    const FaithLayout F = faith_layout(d);
-    const bool light = op == FQ_ADDR_COL || op == FQ_QRAM_COL || op == FQ_SWAP || op == FQ_ADDR_VAL ||
-                       op == FQ_QRAM_VAL;
-    if (light && F.p_addr == 128 && F.aw <= 64)
-        k_fq_light<<<grid_for(M, 256), 256, 0, st>>>(d, static_cast<FKeyW *>(keys), M, op, F.aw);
-    else k_fq<<<grid_for(M, 256), 256, 0, st>>>(d, static_cast<FKeyW *>(keys), M, op, F, status);
+    if (M <= 0 || n <= 0) return cudaSuccess;
+    if (n > QW_FQ_RUN) return cudaErrorInvalidValue;
+    uint64_t packed = 0;
+    bool qbs = false;
+    for (int i = 0; i < n; ++i) {
+        packed |= (uint64_t)ops[i] << (4 * i);
+        qbs = qbs || ops[i] == FQ_QBS_FWD || ops[i] == FQ_QBS_BWD;
+    }
+    FKeyW *k = static_cast<FKeyW *>(keys);
+    const int grid = grid_for(M, FQ_THREADS);
+    if (qbs) k_fq<true><<<grid, FQ_THREADS, 0, st>>>(d, k, M, packed, faith_layout(d), idle, status);
+    else k_fq<false><<<grid, FQ_THREADS, 0, st>>>(d, k, M, packed, faith_layout(d), idle, status);
     return cudaGetLastError();
 }
 

@@ -329,7 +329,9 @@ cudaError_t qw_io_store(const void *keys, int words, int64_t M, uint64_t *out, c
 cudaError_t qw_flat_finish(const QwStepArgs &a, const double *norm, const int64_t *counts, cudaStream_t st);
 /* register-faithful sub-operations on 10-word keys (op codes QW_FQ_* of qwalk.h) */
 int qw_faithful_layout(const QwSimDev &d, int *addr_bits, int *layout_bits);
-cudaError_t qw_faithful_op(const QwSimDev &d, void *keys, int64_t M, int op, int32_t *status, cudaStream_t st);
+#define QW_FQ_RUN 16 /* sub-operations of one launch */
+cudaError_t qw_faithful_run(const QwSimDev &d, void *keys, int64_t M, const int32_t *ops, int n, int idle,
+                            int32_t *status, cudaStream_t st);
 cudaError_t qw_faithful_check_idle(const QwSimDev &d, const void *keys, int64_t M, int32_t *status, cudaStream_t st);
 cudaError_t qw_faithful_export(const QwSimDev &d, const void *keys, int64_t M, uint64_t *table, cudaStream_t st);
 /* the other partitions' outbox segments toward this one (entries and device

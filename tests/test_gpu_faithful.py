@@ -171,3 +171,43 @@ def test_session_rules():
     o.apply("W")
     compare(gpu_state(sim), oracle_state(o), TOL64)
     sim.close()
+
+
+RUNS = {
+    "whole maps, then R^dag": qwalk.FQ_OSDAG + qwalk.FQ_OA + qwalk.FQ_OS + ("RDAG",),
+    "over a launch's 16": qwalk.FQ_OSDAG + qwalk.FQ_OA + qwalk.FQ_OS + qwalk.FQ_OSDAG + qwalk.FQ_OS,
+    "no search": qwalk.FQ_OA + ("SWAP",) + qwalk.FQ_OA + ("SWAP",),
+    "left inside Alg. 1": qwalk.FQ_OSDAG[:2],
+    "left with an address": qwalk.FQ_OSDAG[:4],
+    "a base operator between": ("SWAP", "P", "H") + qwalk.FQ_OSDAG + ("S",),
+}
+
+
+@pytest.mark.parametrize("name", RUNS)
+def test_a_run_of_sub_operations_equals_one_call_each(name):
+    """Sub-operations applied in one call leave every register as the same
+    ones applied by a call each, and the amplitudes within rounding of sums in
+    another order."""
+    w = wl.small_random(130, 16, 5)
+    lists = []
+    for calls in ((RUNS[name],), tuple((o,) for o in RUNS[name])):
+        sim = _sim(w)
+        sim.state_init(w.b)
+        sim.faithful_begin()
+        for ops in calls:
+            sim.faithful_apply(*ops)
+        lists.append(gpu_faithful(sim))
+    assert lists[0].keys() == lists[1].keys()
+    assert all(abs(lists[0][k] - lists[1][k]) <= 1e-15 for k in lists[0])
+
+
+def test_a_run_that_leaves_a_working_register_is_found():
+    """The check of a base operator after a run: the address register (no
+    search in the run) or Alg. 1's registers still hold something."""
+    w = wl.small_random(48, 8, 2)
+    for left in (("ADDR_COL",), qwalk.FQ_OSDAG[:2]):
+        sim = _sim(w)
+        sim.state_init(w.b)
+        sim.faithful_begin()
+        with pytest.raises(qwalk.QwError, match="register A not returned"):
+            sim.faithful_apply(*left, "P")
