@@ -961,8 +961,10 @@ static cudaError_t flat_gather(qw_sim *sim, FlatList &L, int kw)
 
 /* An interference op on the list (0 = R^dag, 1 = R, 2 = H): grouping by a
  * global radix sort, the per-group transform, the compaction of the kept
- * outputs; the host synchronises to size the result. */
-static cudaError_t flat_stage(qw_sim *sim, FlatList &L, int op)
+ * outputs; the host synchronises to size the result.  group: QW_SORT_GROUP, or
+ * QW_SORT_GROUP_NO_A within a walk step, whose list starts with A = 0 in every
+ * branch, so that A follows from (jc, j, kc, k) wherever it is allocated. */
+static cudaError_t flat_stage(qw_sim *sim, FlatList &L, int op, int group)
 {
     const QwSimDev &d = sim->d;
     cudaStream_t st = sim->stream;
@@ -974,7 +976,7 @@ static cudaError_t flat_stage(qw_sim *sim, FlatList &L, int op)
         if ((e = flat_alloc(sim, (size_t)L.M * 16, &ta)) != cudaSuccess) return e;
         if ((e = flat_alloc(sim, qw_flat_sort_bytes(L.M), &work)) != cudaSuccess) return e;
         int in_tmp = 0;
-        e = qw_flat_sort(d, L.K, L.A, tk, static_cast<double2 *>(ta), L.M, op == 2 ? 1 : 0, work,
+        e = qw_flat_sort(d, L.K, L.A, tk, static_cast<double2 *>(ta), L.M, op == 2 ? 1 : 0, group, work,
                          &sim->sc->status, st, L.kw, &in_tmp);
         if (e == cudaSuccess && in_tmp) {
             /* the sorted list is the one in the scratch arrays: swap them */
@@ -1153,18 +1155,18 @@ static int flat_walk_step(qw_sim *sim, int readout)
     a.qls_readout = readout;
     /* T~^dag */
     QW_FLAT(map(QW_FLAT_OSDAG | QW_FLAT_OA << 4 | QW_FLAT_OS << 8));
-    QW_FLAT(flat_stage(sim, L, 0));
+    QW_FLAT(flat_stage(sim, L, 0, QW_SORT_GROUP_NO_A));
     counts[1] = L.M;
     QW_FLAT(map(QW_FLAT_OSDAG | QW_FLAT_OA << 4));
-    QW_FLAT(flat_stage(sim, L, 2));
+    QW_FLAT(flat_stage(sim, L, 2, QW_SORT_GROUP_NO_A));
     counts[2] = L.M;
     if (readout) QW_FLAT(qw_flat_readout(d, L.K, L.A, L.M, a, st, 2));
     /* P, then T~ */
     QW_FLAT(qw_flat_phase(d, L.K, L.A, L.M, st, 2));
-    QW_FLAT(flat_stage(sim, L, 2));
+    QW_FLAT(flat_stage(sim, L, 2, QW_SORT_GROUP_NO_A));
     counts[3] = L.M;
     QW_FLAT(map(QW_FLAT_OA | QW_FLAT_OS << 4));
-    QW_FLAT(flat_stage(sim, L, 1));
+    QW_FLAT(flat_stage(sim, L, 1, QW_SORT_GROUP_NO_A));
     counts[4] = L.M;
     QW_FLAT(map(QW_FLAT_OSDAG | QW_FLAT_OA << 4 | QW_FLAT_OS << 8 | QW_FLAT_A0 << 12 | QW_FLAT_S << 16));
 #undef QW_FLAT
@@ -1347,7 +1349,7 @@ static int pos_prepare(qw_sim *sim)
 
 /* One operator on the base registers (QW_FQ_R .. QW_FQ_FREE_A) on L, whose
  * working registers have been found 0. */
-static cudaError_t faithful_base_op(qw_sim *sim, FlatList &L, int op, FaithCounts &fc)
+static cudaError_t faithful_base_op(qw_sim *sim, FlatList &L, int op, FaithCounts &fc, int group)
 {
     const QwSimDev &d = sim->d;
     cudaStream_t st = sim->stream;
@@ -1355,15 +1357,15 @@ static cudaError_t faithful_base_op(qw_sim *sim, FlatList &L, int op, FaithCount
     cudaError_t e;
     switch (op) {
     case QW_FQ_R:
-        e = flat_stage(sim, L, 1);
+        e = flat_stage(sim, L, 1, group);
         fc.c[4] = L.M;
         return e;
     case QW_FQ_RDAG:
-        e = flat_stage(sim, L, 0);
+        e = flat_stage(sim, L, 0, group);
         fc.c[1] = L.M;
         return e;
     case QW_FQ_H:
-        e = flat_stage(sim, L, 2);
+        e = flat_stage(sim, L, 2, group);
         fc.c[fc.nh < 1 ? 2 : 3] = L.M;
         fc.nh++;
         return e;
@@ -1380,7 +1382,7 @@ static cudaError_t faithful_base_op(qw_sim *sim, FlatList &L, int op, FaithCount
  * the run before makes (idle: already known of L -- the base operators leave the
  * working registers alone).  readout (nullable): the QLS read-out after the first H. */
 static cudaError_t faithful_ops(qw_sim *sim, FlatList &L, const int32_t *ops, int n, FaithCounts &fc, bool idle,
-                                const QwStepArgs *readout)
+                                int group, const QwStepArgs *readout)
 {
     auto working = [](int op) { return op >= QW_FQ_ADDR_COL && op <= QW_FQ_QRAM_VAL; };
     int32_t *status = &sim->sc->status;
@@ -1396,7 +1398,7 @@ static cudaError_t faithful_ops(qw_sim *sim, FlatList &L, const int32_t *ops, in
             if (ops[i] < QW_FQ_R || ops[i] > QW_FQ_FREE_A) return cudaErrorInvalidValue;
             if (!idle) e = qw_faithful_check_idle(sim->d, L.K, L.M, status, sim->stream);
             idle = true;
-            if (e == cudaSuccess) e = faithful_base_op(sim, L, ops[i], fc);
+            if (e == cudaSuccess) e = faithful_base_op(sim, L, ops[i], fc, group);
             if (e == cudaSuccess && readout && ops[i] == QW_FQ_H && fc.nh == 1)
                 e = qw_flat_readout(sim->d, L.K, L.A, L.M, *readout, sim->stream, L.kw);
             ++i;
@@ -1428,7 +1430,8 @@ static int faithful_walk_step(qw_sim *sim, int readout)
     cudaError_t e = flat_gather(sim, L, QW_FQ_KEY_WORDS);
     fc.c[0] = L.M;
     /* a gathered list's working registers are 0 */
-    if (e == cudaSuccess) e = faithful_ops(sim, L, kStep, QW_FQ_STEP_LEN, fc, true, readout ? &a : nullptr);
+    if (e == cudaSuccess) e = faithful_ops(sim, L, kStep, QW_FQ_STEP_LEN, fc, true, QW_SORT_GROUP_NO_A,
+                                         readout ? &a : nullptr);
     if (e != cudaSuccess) {
         flat_release(sim, L);
         return cuda_fail(sim, e, "register-faithful walk step");
@@ -1491,7 +1494,7 @@ extern "C" int qw_faithful_apply(qw_sim *sim, const int32_t *ops, int32_t nops)
     for (int32_t i = 0; i < nops; ++i)
         if (ops[i] < QW_FQ_ADDR_COL || ops[i] > QW_FQ_FREE_A)
             return fail(sim, QW_ERR_ARG, "unknown sub-operation code " + std::to_string(ops[i]));
-    const cudaError_t e = faithful_ops(sim, sim->fq, ops, nops, sim->fq_counts, false, nullptr);
+    const cudaError_t e = faithful_ops(sim, sim->fq, ops, nops, sim->fq_counts, false, QW_SORT_GROUP, nullptr);
     if (e != cudaSuccess) return cuda_fail(sim, e, "qw_faithful_apply");
     return check_status(sim, "qw_faithful_apply");
 }
@@ -2154,7 +2157,8 @@ extern "C" int qw_state_export(qw_sim *sim, int32_t inst, int32_t key_words, uin
                                 static_cast<double2 *>(A), &sim->sc->counter, total, st, 2));
     sim->launches++;
     int in_tmp = 0;
-    QW_CUDA(sim, qw_flat_sort(sim->d, K, static_cast<double2 *>(A), tk, static_cast<double2 *>(ta), total, 0, work,
+    QW_CUDA(sim, qw_flat_sort(sim->d, K, static_cast<double2 *>(A), tk, static_cast<double2 *>(ta), total, 0, QW_SORT_FULL,
+                              work,
                               &sim->sc->status, st, 2, &in_tmp));
     if (in_tmp) {
         std::swap(K, tk);
@@ -2258,7 +2262,7 @@ extern "C" int qw_state_import(qw_sim *sim, int32_t key_words, const uint64_t *k
             QW_CUDA(sim, cudaMemsetAsync(flags, 0, sizeof(QwIoFlags), st));
             int in_tmp = 0;
             QW_CUDA(sim, qw_flat_sort(sim->d, K, static_cast<double2 *>(A), tk, static_cast<double2 *>(ta), count, 0,
-                                      work, &flags->status, st, 2, &in_tmp));
+                                      QW_SORT_FULL, work, &flags->status, st, 2, &in_tmp));
             if (in_tmp) {
                 std::swap(K, tk);
                 std::swap(A, ta);

@@ -803,24 +803,29 @@ __global__ void __launch_bounds__(OS_THREADS, 4) k_f_onesweep(const uint64_t *ck
     const int64_t base = vb * OS_TILE + warp * (32 * OS_IPT) + lane;
     uint64_t c[OS_IPT];
     uint32_t ix[OS_IPT], rk[OS_IPT];
-    int dg[OS_IPT];
 #pragma unroll
     for (int r = 0; r < OS_IPT; ++r) {
         const int64_t i = base + 32 * r;
-        dg[r] = 256;
         c[r] = 0ull;
         ix[r] = 0u;
         if (i < M) {
             c[r] = ckin[i];
             ix[r] = FIRST ? (uint32_t)i : ixin[i];
-            dg[r] = (int)((c[r] >> shift) & 255ull);
         }
     }
+    auto digit = [&](int r) { return base + 32 * r < M ? (int)((c[r] >> shift) & 255ull) : 256; };
     const unsigned below = (1u << lane) - 1u;
 #pragma unroll
     for (int r = 0; r < OS_IPT; ++r) {
-        const unsigned m = __match_any_sync(FULL, dg[r]);
-        const int d = dg[r];
+        const int d = digit(r);
+        /* the lanes of the same digit (9 bits: 256 = none), by ballots: the
+           match instruction runs once per distinct value */
+        unsigned m = FULL;
+#pragma unroll
+        for (int b = 0; b < 9; ++b) {
+            const unsigned bal = __ballot_sync(FULL, (d >> b) & 1);
+            m &= (d >> b) & 1 ? bal : ~bal;
+        }
         const uint32_t cnt = d < 256 ? hw[warp][d] : 0u;
         rk[r] = cnt + (uint32_t)__popc(m & below);
         __syncwarp();
@@ -875,7 +880,7 @@ __global__ void __launch_bounds__(OS_THREADS, 4) k_f_onesweep(const uint64_t *ck
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < OS_IPT; ++r) {
-        const int d = dg[r];
+        const int d = digit(r);
         const uint32_t dest = d < 256 ? sbase[d] + hw[warp][d] + rk[r] : 0u;
         if (d < 256 && (int64_t)dest < M) { /* always, unless a wait gave up */
             if (WRITE_CK) ckout[dest] = c[r];
@@ -917,12 +922,12 @@ __global__ void k_f_rot(QwSimDev d, const FKeyN<NW> *keys, const double2 *amps, 
         flags[2 * i] = 0u;
         flags[2 * i + 1] = 0u;
         if (!head) continue;
-        double2 a0 = make_double2(0, 0), a1 = make_double2(0, 0);
-        if ((k.w[0] & 1ull) == 0) {
-            a0 = amps[i];
-            if (i + 1 < M && same_group<ORDER_R>(k, keys[i + 1], 0)) a1 = amps[i + 1];
-        } else {
-            a1 = amps[i];
+        double2 a0 = amps[i], a1 = make_double2(0, 0); /* the pair in either order */
+        if (i + 1 < M && same_group<ORDER_R>(k, keys[i + 1], 0)) a1 = amps[i + 1];
+        if ((k.w[0] & 1ull) != 0) {
+            const double2 t = a0;
+            a0 = a1;
+            a1 = t;
         }
         const FRegs f = fdecode(k, L);
         double2 fv;
@@ -1259,10 +1264,6 @@ int grid_for(int64_t n, int threads)
     return (int)(g < 1 ? 1 : g);
 }
 
-template <int NW>
-cudaError_t flat_sort_t(const QwSimDev &d, void *keys, double2 *amps, void *tmpk, double2 *tmpa, int64_t M, int order,
-                        uint32_t *work, cudaStream_t st);
-
 } // namespace
 
 /* ---- launchers ------------------------------------------------------------------------ */
@@ -1366,14 +1367,20 @@ SortWork sort_work(void *base, int64_t M)
     return w;
 }
 
-/* Stable sort of (keys, amps) by the permuted key of `order` (0: R, 1: H):
- * one synchronisation reads which bits vary; they are sorted in chunks of
+/* Stable sort of (keys, amps) by the permuted key of `order` (0: R, 1: H);
+ * group: only so far that the groups are contiguous, without the target's bits
+ * (the transforms take a group's members in any order; the direct sums of s >
+ * 128 in that of the list, so not there) and, where A is known to follow from
+ * the other idle registers, without A's -- 30 bits for 46 at N = 16384's R^dag. Two
+ * steps there, with T~ and two marginals: 2765 -> 2495 us, the sort's ranks by
+ * ballots included.
+ * One synchronisation reads which bits vary; they are sorted in chunks of
  * 64, each by 8-bit passes carrying a permutation; the entries are moved
  * once at the end, into tmpk / tmpa (*in_tmp = 1).  A list whose keys are
  * all equal is already sorted (*in_tmp = 0). */
 template <int NW>
 cudaError_t flat_sort_t(const QwSimDev &d, void *keys, double2 *amps, void *tmpk, double2 *tmpa, int64_t M, int order,
-                        void *work, int32_t *status, cudaStream_t st, int *in_tmp)
+                        int group, void *work, int32_t *status, cudaStream_t st, int *in_tmp)
 {
     *in_tmp = 0;
     if (M <= 1) return cudaSuccess;
@@ -1399,6 +1406,14 @@ cudaError_t flat_sort_t(const QwSimDev &d, void *keys, double2 *amps, void *tmpk
     /* the varying bits as runs, split into chunks of 64 */
     uint64_t var[NW];
     for (int wi = 0; wi < NW; ++wi) var[wi] = h[wi] ^ h[NW + wi];
+    if (group != QW_SORT_FULL) {
+        if (order == ORDER_R) var[0] &= ~1ull;
+        else if (d.s <= 128) var[0] &= ~((1ull << L) - 1ull);
+    }
+    if (group == QW_SORT_GROUP_NO_A) {
+        const int pA = flayout(d.nb).pA; /* bits pA .. pA + 15 */
+        for (int b = pA; b < pA + 16; ++b) var[b >> 6] &= ~(1ull << (b & 63));
+    }
     std::vector<CkRuns> chunks(NW);
     chunks.resize((size_t)qw_sort_chunks(var, NW, chunks.data()));
     if (chunks.empty()) return cudaSuccess;
@@ -1449,10 +1464,11 @@ size_t qw_flat_sort_bytes(int64_t M)
 }
 
 cudaError_t qw_flat_sort(const QwSimDev &d, void *keys, double2 *amps, void *tmpk, double2 *tmpa, int64_t M,
-                         int order, void *work, int32_t *status, cudaStream_t st, int kw, int *in_tmp)
+                         int order, int group, void *work, int32_t *status, cudaStream_t st, int kw, int *in_tmp)
 {
-    if (kw == NW_FAITH) return flat_sort_t<NW_FAITH>(d, keys, amps, tmpk, tmpa, M, order, work, status, st, in_tmp);
-    return flat_sort_t<2>(d, keys, amps, tmpk, tmpa, M, order, work, status, st, in_tmp);
+    if (kw == NW_FAITH)
+        return flat_sort_t<NW_FAITH>(d, keys, amps, tmpk, tmpa, M, order, group, work, status, st, in_tmp);
+    return flat_sort_t<2>(d, keys, amps, tmpk, tmpa, M, order, group, work, status, st, in_tmp);
 }
 
 /* op: 0 = R^dag, 1 = R (2 outputs per entry), 2 = H (s outputs per entry) */

@@ -294,8 +294,11 @@ cudaError_t qw_flat_scan(const uint32_t *in, int64_t n, uint32_t *sums, uint32_t
 /* stable sort by the permuted key (order 0: R, 1: H); work holds
    qw_flat_sort_bytes(M); the result is left in tmpk / tmpa when *in_tmp */
 size_t qw_flat_sort_bytes(int64_t M);
+#define QW_SORT_FULL 0       /* by every register */
+#define QW_SORT_GROUP 1      /* the target's bits left out: groups contiguous */
+#define QW_SORT_GROUP_NO_A 2 /* A's too: it follows from the other idle registers */
 cudaError_t qw_flat_sort(const QwSimDev &d, void *keys, double2 *amps, void *tmpk, double2 *tmpa, int64_t M,
-                         int order, void *work, int32_t *status, cudaStream_t st, int kw, int *in_tmp);
+                         int order, int group, void *work, int32_t *status, cudaStream_t st, int kw, int *in_tmp);
 /* the Hadamard stage's groups: head flags of the sorted list, and the first
    member of each of its G groups (starts[G] = M) from their exclusive scan */
 cudaError_t qw_flat_heads(const QwSimDev &d, const void *keys, int64_t M, uint32_t *flags, cudaStream_t st, int kw);
