@@ -960,8 +960,8 @@ static cudaError_t flat_gather(qw_sim *sim, FlatList &L, int kw)
 }
 
 /* An interference op on the list (0 = R^dag, 1 = R, 2 = H): grouping by a
- * global radix sort, the per-group transform, the compaction of the kept
- * outputs; the host synchronises to size the result.  group: QW_SORT_GROUP, or
+ * global radix sort, then the per-group transform with the kept outputs written
+ * one after another; the host synchronises to size the result.  group: QW_SORT_GROUP, or
  * QW_SORT_GROUP_NO_A within a walk step, whose list starts with A = 0 in every
  * branch, so that A follows from (jc, j, kc, k) wherever it is allocated. */
 static cudaError_t flat_stage(qw_sim *sim, FlatList &L, int op, int group)
@@ -990,93 +990,43 @@ static cudaError_t flat_stage(qw_sim *sim, FlatList &L, int op, int group)
         cudaFreeAsync(work, st);
         if (e != cudaSuccess) return e;
     }
-    /* H: the groups of the sorted list counted first (head flags and their
-       scan; the host reads the count) */
-    int64_t G = 0;
-    int64_t *starts = nullptr;
-    if (op == 2 && L.M > 0) {
-        void *heads = nullptr, *gidx = nullptr, *hsums = nullptr;
-        uint32_t g32 = 0;
-        if ((e = flat_alloc(sim, (size_t)L.M * 4, &heads)) != cudaSuccess) return e;
-        if ((e = flat_alloc(sim, (size_t)L.M * 4, &gidx)) != cudaSuccess) return e;
-        if ((e = flat_alloc(sim, qw_flat_scan_words(L.M) * 4, &hsums)) != cudaSuccess) return e;
-        e = qw_flat_heads(d, L.K, L.M, static_cast<uint32_t *>(heads), st, L.kw);
-        if (e == cudaSuccess)
-            e = qw_flat_scan(static_cast<uint32_t *>(heads), L.M, static_cast<uint32_t *>(hsums),
-                             static_cast<uint32_t *>(gidx), st);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(&g32, static_cast<uint32_t *>(hsums) + (L.M + 1023) / 1024, 4, cudaMemcpyDeviceToHost,
-                                st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        G = (int64_t)g32;
-        if (e == cudaSuccess) e = flat_alloc(sim, (size_t)(G + 1) * 8, (void **)&starts);
-        if (e == cudaSuccess)
-            e = qw_flat_starts(static_cast<uint32_t *>(heads), static_cast<uint32_t *>(gidx), L.M, G, starts, st);
-        for (void *p : {heads, gidx, hsums})
-            if (p) cudaFreeAsync(p, st);
+    if (L.M <= 0) return cudaSuccess;
+    FlatScratch scratch(sim);
+    void *tiles = nullptr, *starts = nullptr;
+    if ((e = scratch.take(qw_flat_tiles_bytes(L.M), &tiles)) != cudaSuccess) return e;
+    unsigned long long total = 0;
+    auto read_total = [&]() {
+        const cudaError_t r = cudaMemcpyAsync(&total, qw_flat_tiles_total(tiles), 8, cudaMemcpyDeviceToHost, st);
+        return r != cudaSuccess ? r : cudaStreamSynchronize(st);
+    };
+    /* H: the groups of the sorted list, their number read by the host; up to s
+       outputs each.  R, R^dag: up to two an entry. */
+    int64_t cap = 2 * L.M, G = 0;
+    if (op == 2) {
+        if ((e = scratch.take((size_t)(L.M + 1) * 8, &starts)) != cudaSuccess) return e;
+        e = qw_flat_starts(d, L.K, L.M, static_cast<int64_t *>(starts), tiles, &sim->sc->status, st, L.kw);
+        if (e == cudaSuccess) e = read_total();
         if (e != cudaSuccess) return e;
+        G = std::min<int64_t>((int64_t)total, L.M); /* (more only after a wait gave up) */
+        cap = G * d.s;
     }
     FlatList R;
     R.kw = L.kw;
-    uint32_t total = 0;
-    if (op == 2) {
-        /* H: the kept outputs of each group counted, scanned, then written */
-        void *cnt = nullptr, *gpos = nullptr, *sums = nullptr;
-        if (G > 0) {
-            if (e == cudaSuccess) e = flat_alloc(sim, (size_t)G * 4, &cnt);
-            if (e == cudaSuccess) e = flat_alloc(sim, (size_t)G * 4, &gpos);
-            if (e == cudaSuccess) e = flat_alloc(sim, qw_flat_scan_words(G) * 4, &sums);
-            if (e == cudaSuccess)
-                e = qw_flat_hgroups(d, L.K, L.A, starts, G, static_cast<uint32_t *>(cnt), nullptr, nullptr, nullptr, st,
-                                    L.kw);
-            if (e == cudaSuccess)
-                e = qw_flat_scan(static_cast<uint32_t *>(cnt), G, static_cast<uint32_t *>(sums),
-                                 static_cast<uint32_t *>(gpos), st);
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(&total, static_cast<uint32_t *>(sums) + (G + 1023) / 1024, 4,
-                                    cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        }
-        R.M = (int64_t)total;
-        if (e == cudaSuccess) e = flat_alloc(sim, (size_t)R.M * kb, &R.K);
-        if (e == cudaSuccess) e = flat_alloc(sim, (size_t)R.M * 16, (void **)&R.A);
-        if (e == cudaSuccess && total > 0)
-            e = qw_flat_hgroups(d, L.K, L.A, starts, G, static_cast<uint32_t *>(cnt), static_cast<uint32_t *>(gpos),
-                                R.K, R.A, st, L.kw);
-        for (void *p : {cnt, gpos, sums, (void *)starts})
-            if (p) cudaFreeAsync(p, st);
-        flat_release(sim, L);
-        L = R;
+    e = flat_alloc(sim, (size_t)cap * kb, &R.K);
+    if (e == cudaSuccess) e = flat_alloc(sim, (size_t)cap * 16, (void **)&R.A);
+    if (e == cudaSuccess)
+        e = op == 2 ? qw_flat_hgroups(d, L.K, L.A, L.M, static_cast<int64_t *>(starts), G, R.K, R.A, cap, tiles,
+                                      &sim->sc->status, st, L.kw)
+                    : qw_flat_rot(d, op, L.K, L.A, L.M, R.K, R.A, cap, tiles, &sim->sc->status, st, L.kw);
+    if (e == cudaSuccess) e = read_total();
+    if (e != cudaSuccess) {
+        flat_release(sim, R);
         return e;
     }
-    const int64_t n = L.M * 2;
-    void *ok = nullptr, *oa = nullptr, *flags = nullptr, *pos = nullptr, *sums = nullptr;
-    if ((e = flat_alloc(sim, (size_t)n * kb, &ok)) != cudaSuccess) return e;
-    if ((e = flat_alloc(sim, (size_t)n * 16, &oa)) != cudaSuccess) return e;
-    if ((e = flat_alloc(sim, (size_t)n * 4, &flags)) != cudaSuccess) return e;
-    if ((e = flat_alloc(sim, (size_t)n * 4, &pos)) != cudaSuccess) return e;
-    if ((e = flat_alloc(sim, qw_flat_scan_words(n) * 4, &sums)) != cudaSuccess) return e;
-    e = qw_flat_group(d, op, L.K, L.A, L.M, ok, static_cast<double2 *>(oa), static_cast<uint32_t *>(flags), st,
-                      L.kw);
-    if (e == cudaSuccess && n > 0) {
-        e = qw_flat_scan(static_cast<uint32_t *>(flags), n, static_cast<uint32_t *>(sums), static_cast<uint32_t *>(pos),
-                         st);
-        const int64_t nb = (n + 1023) / 1024;
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(&total, static_cast<uint32_t *>(sums) + nb, 4, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    }
-    R.M = (int64_t)total;
-    if (e == cudaSuccess) e = flat_alloc(sim, (size_t)R.M * kb, &R.K);
-    if (e == cudaSuccess) e = flat_alloc(sim, (size_t)R.M * 16, (void **)&R.A);
-    if (e == cudaSuccess)
-        e = qw_flat_compact(ok, static_cast<double2 *>(oa), static_cast<uint32_t *>(flags),
-                            static_cast<uint32_t *>(pos), n, R.K, R.A, st, L.kw);
-    for (void *p : {ok, oa, flags, pos, sums})
-        if (p) cudaFreeAsync(p, st);
+    R.M = std::min<int64_t>((int64_t)total, cap);
     flat_release(sim, L);
     L = R;
-    return e;
+    return cudaSuccess;
 }
 
 /* Store the list as the output of a step: X_cur+1 (and X_cur+2 cleared, as a

@@ -595,89 +595,107 @@ __global__ void k_fq_export(QwSimDev d, const FKeyW *keys, int64_t M, FaithLayou
     }
 }
 
-/* ---- device-wide exclusive scan of 32-bit counts ------------------------------ */
+/* ---- single-pass compaction ------------------------------------------------------ */
+/*
+ * Kernels that write a varying number of outputs per input take tiles of their
+ * input in the order blocks start (a counter), hold a tile's outputs in
+ * registers, and learn where they go from the counts of the tiles before, summed
+ * by looking back 32 tiles at a time (the single-pass prefix sum of the sort,
+ * one count a tile): the outputs are formed once and written once.  With flags, a
+ * three-kernel scan and a copy (R, R^dag) or a counting pass before the
+ * writing one (H) they were formed or moved twice.  Two flat steps at N = 16384,
+ * s = 16: 2495 -> 2224 us; one faithful step at N = 8192, s = 32: 1365 -> 1284.
+ */
+struct TileSum {            /* zeroed before the launch */
+    unsigned int next, pad; /* the next tile */
+    unsigned long long total;
+    unsigned long long tile[1]; /* per tile: 1 << 62 its count, 2 << 62 with the tiles before */
+};
+constexpr unsigned long long TS_AGG = 1ull << 62, TS_INC = 2ull << 62, TS_CNT = TS_AGG - 1ull;
+constexpr int TS_SPIN_LIMIT = 1 << 22;
 
-constexpr int SCAN_TILE = 1024; /* elements per block: 256 threads x 4 */
-
-__global__ void k_scan_reduce(const uint32_t *in, int64_t n, uint32_t *sums)
+/* the counts of the tiles before vb (called by one warp); count: this tile's.  A
+   wait that outlasts the limit sets the status; the outputs' places are then
+   wrong (and checked against the array's end), and the host reports it. */
+__device__ unsigned long long tile_before(TileSum *ts, int64_t vb, unsigned int count, int32_t *status)
 {
-    __shared__ uint32_t ws[8];
-    const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
-    uint32_t v = 0;
-    for (int t = 0; t < 4; ++t) {
-        const int64_t i = base + threadIdx.x * 4 + t;
-        if (i < n) v += in[i];
+    const int lane = threadIdx.x & 31;
+    volatile unsigned long long *t = ts->tile;
+    if (vb == 0) {
+        if (lane == 0) t[0] = TS_INC | count;
+        return 0ull;
     }
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t t = 0;
-        for (int w = 0; w < 8; ++w) t += ws[w];
-        sums[blockIdx.x] = t;
-    }
-}
-
-/* one block: exclusive scan of the block sums in place, total at sums[nb] */
-__global__ void k_scan_blocks(uint32_t *sums, int64_t nb)
-{
-    __shared__ uint32_t ws[32];
-    __shared__ uint32_t carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t base = 0; base < nb; base += blockDim.x) {
-        const int64_t i = base + threadIdx.x;
-        const uint32_t v = i < nb ? sums[i] : 0u;
-        uint32_t x = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(FULL, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) ws[warp] = x;
-        __syncthreads();
-        if (warp == 0) {
-            uint32_t w = lane < (int)(blockDim.x >> 5) ? ws[lane] : 0u;
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(FULL, w, o);
-                if (lane >= o) w += y;
+    if (lane == 0) t[vb] = TS_AGG | count;
+    unsigned long long before = 0ull;
+    int64_t p = vb - 1;
+    for (int spins = 0;;) {
+        unsigned long long v = TS_INC; /* before tile 0: an end of count 0 */
+        if (p >= lane) v = t[p - lane];
+        const unsigned empty = __ballot_sync(FULL, (v >> 62) == 0ull), inc = __ballot_sync(FULL, (v >> 62) == 2ull);
+        /* the tiles up to the nearest one that includes those before it */
+        const int end = inc ? __ffs(inc) - 1 : 31;
+        const unsigned need = end == 31 ? FULL : (2u << end) - 1u;
+        if (empty & need) {
+            if (++spins > TS_SPIN_LIMIT) {
+                if (lane == 0) atomicOr(status, QW_ST_SORT_WAIT);
+                break;
             }
-            ws[lane] = w;
+            if (spins > 32) __nanosleep(64);
+            continue;
         }
-        __syncthreads();
-        const uint32_t before = carry + (warp > 0 ? ws[warp - 1] : 0u) + x - v;
-        if (i < nb) sums[i] = before;
-        __syncthreads();
-        if (threadIdx.x == 0) carry += ws[(blockDim.x >> 5) - 1];
-        __syncthreads();
+        unsigned long long c = lane <= end ? v & TS_CNT : 0ull;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(FULL, c, o);
+        before += c;
+        if (inc) break;
+        p -= 32;
     }
-    if (threadIdx.x == 0) sums[nb] = carry;
+    if (lane == 0) t[vb] = TS_INC | (before + count);
+    return before;
 }
 
-__global__ void k_scan_apply(const uint32_t *in, int64_t n, const uint32_t *sums, uint32_t *out)
+/* A block's share of it: n outputs of this thread, the number of those of the
+   threads before it in the block and all before the tile; the last tile writes the total. */
+template <int THREADS>
+__device__ __forceinline__ unsigned long long tile_place(TileSum *ts, int64_t vb, int64_t ntiles, unsigned int n,
+                                                         int32_t *status)
 {
-    __shared__ uint32_t ws[8];
+    constexpr int W = THREADS / 32;
+    __shared__ unsigned int ws[W];
+    __shared__ unsigned long long base;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + threadIdx.x * 4;
-    uint32_t v[4], t = 0;
-    for (int k = 0; k < 4; ++k) {
-        v[k] = base + k < n ? in[base + k] : 0u;
-        t += v[k];
-    }
-    uint32_t x = t;
+    unsigned int x = n;
+#pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(FULL, x, o);
+        const unsigned int y = __shfl_up_sync(FULL, x, o);
         if (lane >= o) x += y;
     }
     if (lane == 31) ws[warp] = x;
     __syncthreads();
-    uint32_t wpre = 0;
-    for (int w = 0; w < warp; ++w) wpre += ws[w];
-    uint32_t run = sums[blockIdx.x] + wpre + x - t;
-    for (int k = 0; k < 4; ++k) {
-        if (base + k < n) out[base + k] = run;
-        run += v[k];
+    unsigned int pre = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        if (w < warp) pre += ws[w];
+        all += ws[w];
     }
+    if (warp == 0) {
+        const unsigned long long b = tile_before(ts, vb, all, status);
+        if (lane == 0) {
+            base = b;
+            if (vb == ntiles - 1) ts->total = b + all;
+        }
+    }
+    __syncthreads();
+    return base + pre + x - n;
+}
+
+/* the block's tile */
+__device__ __forceinline__ int64_t tile_take(TileSum *ts)
+{
+    __shared__ unsigned int vb;
+    if (threadIdx.x == 0) vb = atomicAdd(&ts->next, 1u);
+    __syncthreads();
+    return vb;
 }
 
 /* ---- radix sort ------------------------------------------------------------------ */
@@ -908,76 +926,99 @@ __global__ void k_f_permute(const FKeyN<NW> *kin, const double2 *ain, const uint
 
 /* ---- per-group transforms (the "computing" step) -------------------------------- */
 
-/* R (DAG = false) or R^dag on b2-pairs (sorted in ORDER_R): the head of each
- * pair writes both outputs at 2 i (b2 = 0) and 2 i + 1 (b2 = 1) with their
- * keep flags; R = [[f, -g], [g, conj f]] (Alg. T~ and the footnote of Sec. IV). */
+/* R (DAG = false) or R^dag on b2-pairs (the list sorted in ORDER_R, a pair in
+ * either order): the first member of each pair forms both outputs, R = [[f, -g],
+ * [g, conj f]] (Alg. T~ and the footnote of Sec. IV); the kept ones are written in
+ * the order of the pairs, b2 = 0 first, at most cap.  Bound by the keys read and
+ * written (a thread per entry, the neighbours' keys from L1). */
+constexpr int RT_THREADS = 256;
 template <bool DAG, int NW>
-__global__ void k_f_rot(QwSimDev d, const FKeyN<NW> *keys, const double2 *amps, int64_t M, FKeyN<NW> *okeys,
-                        double2 *oamps, uint32_t *flags)
+__global__ void __launch_bounds__(RT_THREADS) k_f_rot(QwSimDev d, const FKeyN<NW> *keys, const double2 *amps, int64_t M,
+                                                      FKeyN<NW> *okeys, double2 *oamps, int64_t cap, TileSum *ts,
+                                                      int32_t *status)
 {
     const FLayout L = flayout(d.nb);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += (int64_t)gridDim.x * blockDim.x) {
-        const FKeyN<NW> k = keys[i];
+    const int64_t vb = tile_take(ts), i = vb * RT_THREADS + threadIdx.x;
+    FKeyN<NW> k;
+    double2 o0 = make_double2(0, 0), o1 = o0;
+    bool k0 = false, k1 = false;
+    if (i < M) {
+        k = keys[i];
         const bool head = i == 0 || !same_group<ORDER_R>(keys[i - 1], k, 0);
-        flags[2 * i] = 0u;
-        flags[2 * i + 1] = 0u;
-        if (!head) continue;
-        double2 a0 = amps[i], a1 = make_double2(0, 0); /* the pair in either order */
-        if (i + 1 < M && same_group<ORDER_R>(k, keys[i + 1], 0)) a1 = amps[i + 1];
-        if ((k.w[0] & 1ull) != 0) {
-            const double2 t = a0;
-            a0 = a1;
-            a1 = t;
+        if (head) {
+            double2 a0 = amps[i], a1 = make_double2(0, 0);
+            if (i + 1 < M && same_group<ORDER_R>(k, keys[i + 1], 0)) a1 = amps[i + 1];
+            if ((k.w[0] & 1ull) != 0) {
+                const double2 t = a0;
+                a0 = a1;
+                a1 = t;
+            }
+            const FRegs f = fdecode(k, L);
+            double2 fv;
+            double g;
+            rot_fg(d, f.x.A, f.j, f.x.k, fv, g);
+            if (!DAG) {
+                o0 = csub(cmul(fv, a0), cscale(g, a1));
+                o1 = cadd(cscale(g, a0), cmul(cconj(fv), a1));
+            } else {
+                o0 = cadd(cmul(cconj(fv), a0), cscale(g, a1));
+                o1 = csub(cmul(fv, a1), cscale(g, a0));
+            }
+            k0 = keep(o0, d.tau2);
+            k1 = keep(o1, d.tau2);
         }
-        const FRegs f = fdecode(k, L);
-        double2 fv;
-        double g;
-        rot_fg(d, f.x.A, f.j, f.x.k, fv, g);
-        double2 o0, o1;
-        if (!DAG) {
-            o0 = csub(cmul(fv, a0), cscale(g, a1));
-            o1 = cadd(cscale(g, a0), cmul(cconj(fv), a1));
-        } else {
-            o0 = cadd(cmul(cconj(fv), a0), cscale(g, a1));
-            o1 = csub(cmul(fv, a1), cscale(g, a0));
-        }
-        FKeyN<NW> k0 = k;
-        k0.w[0] &= ~1ull;
-        FKeyN<NW> k1 = k0;
-        k1.w[0] |= 1ull;
-        okeys[2 * i] = k0;
-        okeys[2 * i + 1] = k1;
-        oamps[2 * i] = o0;
-        oamps[2 * i + 1] = o1;
-        flags[2 * i] = keep(o0, d.tau2) ? 1u : 0u;
-        flags[2 * i + 1] = keep(o1, d.tau2) ? 1u : 0u;
+    }
+    int64_t at = (int64_t)tile_place<RT_THREADS>(ts, vb, gridDim.x, (k0 ? 1u : 0u) + (k1 ? 1u : 0u), status);
+    if (k0 && at < cap) {
+        k.w[0] &= ~1ull;
+        okeys[at] = k;
+        oamps[at] = o0;
+        ++at;
+    }
+    if (k1 && at < cap) {
+        k.w[0] |= 1ull;
+        okeys[at] = k;
+        oamps[at] = o1;
     }
 }
 
-/* H on the low L bits of k (sorted in ORDER_H): the head of each group
- * writes the s outputs (1/sqrt s) sum_v (-1)^(u.v) a_v at s i + u. */
+/* The groups of H on the low L bits of k (the list sorted in ORDER_H): starts[g]
+ * = the first member of group g, starts[G] = M.  8 entries a thread. */
+constexpr int ST_THREADS = 256, ST_IPT = 8;
 template <int NW>
-__global__ void k_f_heads(QwSimDev d, const FKeyN<NW> *keys, int64_t M, uint32_t *flags)
+__global__ void __launch_bounds__(ST_THREADS) k_f_starts(QwSimDev d, const FKeyN<NW> *keys, int64_t M, int64_t *starts,
+                                                         TileSum *ts, int32_t *status)
 {
-    const int L = d.L;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += (int64_t)gridDim.x * blockDim.x)
-        flags[i] = (i == 0 || !same_group<ORDER_H>(keys[i - 1], keys[i], L)) ? 1u : 0u;
-}
-
-/* starts[g] = the first member of group g (gidx: the exclusive scan of the
-   head flags), starts[G] = M */
-__global__ void k_f_starts(const uint32_t *heads, const uint32_t *gidx, int64_t M, int64_t G, int64_t *starts)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += (int64_t)gridDim.x * blockDim.x) {
-        if (heads[i]) starts[gidx[i]] = i;
-        if (i == 0) starts[G] = M;
+    const int64_t vb = tile_take(ts), i0 = vb * (ST_THREADS * ST_IPT) + (threadIdx.x >> 5) * (32 * ST_IPT);
+    const int lane = threadIdx.x & 31;
+    /* a warp takes 256 entries in a row, 32 at a time */
+    unsigned heads[ST_IPT];
+    unsigned n = 0;
+#pragma unroll
+    for (int r = 0; r < ST_IPT; ++r) {
+        const int64_t i = i0 + 32 * r + lane;
+        const bool head = i < M && (i == 0 || !same_group<ORDER_H>(keys[i - 1], keys[i], d.L));
+        heads[r] = __ballot_sync(FULL, head);
+        n += __popc(heads[r]);
+    }
+    /* the warp's count on its first lane: every lane's place is its warp's */
+    unsigned long long at = tile_place<ST_THREADS>(ts, vb, gridDim.x, lane == 0 ? n : 0u, status);
+    at = __shfl_sync(FULL, at, 0);
+#pragma unroll
+    for (int r = 0; r < ST_IPT; ++r) {
+        const unsigned long long g = at + __popc(heads[r] & ((1u << lane) - 1u));
+        if ((heads[r] >> lane) & 1u) {
+            if (g < (unsigned long long)M) starts[g] = i0 + 32 * r + lane;
+        }
+        at += __popc(heads[r]);
+    }
+    /* the end of the last group */
+    if (vb == gridDim.x - 1 && threadIdx.x == 0) {
+        const unsigned long long G = *(volatile unsigned long long *)&ts->total;
+        if (G <= (unsigned long long)M) starts[G] = M;
     }
 }
 
-/* The s outputs of every Hadamard group (members equal but for the low L
- * bits of k, contiguous after the sort): one thread per (group, u), the
- * group's members read in list order, so each output is the same sum as a
- * dense s x s product on the zero-filled vector. */
 /* H on each group's zero-filled vector of 2^L = s entries (the groups of
  * the list sorted in ORDER_H, starts[g] .. starts[g + 1]): output u of a group
  * is s^-1/2 sum_m (-1)^{|u & v_m|} a_m over its members m (v_m: their low L
@@ -990,79 +1031,120 @@ __global__ void k_f_starts(const uint32_t *heads, const uint32_t *gidx, int64_t 
  * limit.  Larger s: s / 32 rounds of 32 outputs, each the direct sum over
  * the members in list order (a lane loads one member per round and the
  * warp's shuffles hand them to every output).
- * COUNT: the kept outputs of each group into cnt[g]; otherwise the kept
- * outputs are written, in order of u, from gpos[g] (the exclusive scan of
- * cnt) -- the clearing step without a list of all G s outputs. */
-template <int NW, bool COUNT, int FWHT_ROUNDS>
-__global__ void __launch_bounds__(256) k_f_hgroups(QwSimDev d, const FKeyN<NW> *keys, const double2 *amps,
-                                                   const int64_t *starts, int64_t G, uint32_t *cnt,
-                                                   const uint32_t *gpos, FKeyN<NW> *okeys, double2 *oamps)
+ * The kept outputs are written in the order of the groups and of u, at most cap
+ * (the fast transform: tiles of HG_ITERS x 8 warps' groups, the outputs held in
+ * registers until the counts of the tiles before are known).  The direct sums
+ * go over the groups twice -- their outputs, s / 32 a lane, do not fit registers. */
+constexpr int HG_WARPS = 8;
+template <int R> struct HgIters { static constexpr int n = R == 1 ? 4 : (R == 2 ? 2 : 1); }; /* R x n outputs a lane */
+template <int NW, int FWHT_ROUNDS>
+__global__ void __launch_bounds__(32 * HG_WARPS) k_f_hgroups(QwSimDev d, const FKeyN<NW> *keys, const double2 *amps,
+                                                             int64_t M, const int64_t *starts, int64_t G,
+                                                             FKeyN<NW> *okeys, double2 *oamps, int64_t cap, TileSum *ts, int32_t *status)
 {
     const int s = d.s;
     const int sw = s < 32 ? s : 32, gpw = 32 / sw, rounds = s / sw;
     const int lane = threadIdx.x & 31, sub = lane / sw, ul = lane - sub * sw, first = sub * sw;
-    const unsigned seg = sw == 32 ? FULL : ((1u << sw) - 1u) << first;
     const unsigned below = (1u << lane) - 1u;
     const uint64_t lowm = ((uint64_t)s - 1ull) << 1;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     constexpr int ZR = FWHT_ROUNDS > 0 ? FWHT_ROUNDS : 1;
-    const bool fwht = FWHT_ROUNDS > 0;
-    __shared__ double2 zv[8][32 * ZR];
-    double2 *vec = zv[threadIdx.x >> 5];
-    for (int64_t wg = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; wg * gpw < G; wg += nwarps) {
-        const int64_t g = wg * gpw + sub;
-        const bool act = g < G;
-        const int64_t b = act ? starts[g] : 0, nm = act ? starts[g + 1] - b : 0;
-        /* fast transform: entry q sw + ul of the group's zero-filled vector
-           in x[q], the butterflies of index bits below sw over shuffles, the
-           ones above between the lane's registers; x[q] is then output
-           u = q sw + ul */
-        double2 x[ZR];
-        if (fwht) {
+    constexpr bool fwht = FWHT_ROUNDS > 0;
+    constexpr int ITERS = HgIters<FWHT_ROUNDS>::n;
+    const int64_t vb = tile_take(ts), wg0 = (vb * HG_WARPS + (threadIdx.x >> 5)) * ITERS; /* the warp's first set of groups */
+    const int ns = rounds;
+    /* group g's first member and their number (in bounds whatever starts holds) */
+    auto group_at = [&](bool act, int64_t g, int64_t &b, int64_t &nm) {
+        b = act ? starts[g] : 0;
+        if (b < 0 || b >= M) b = 0;
+        const int64_t e = act ? starts[g + 1] : 0;
+        nm = e > b ? (e < M ? e : M) - b : 0;
+    };
+    if (fwht) {
+        __shared__ double2 zv[HG_WARPS][32 * ZR];
+        double2 *vec = zv[threadIdx.x >> 5];
+        /* entry q sw + ul of the group's zero-filled vector in x[it][q], the
+           butterflies of index bits below sw over shuffles, the ones above between
+           the lane's registers; x[it][q] is then output u = q sw + ul */
+        double2 x[ITERS][ZR];
+        unsigned kept[ITERS][ZR]; /* the warp's lanes whose output is kept */
+        int64_t b[ITERS];
+        unsigned n = 0;
+#pragma unroll
+        for (int it = 0; it < ITERS; ++it) {
+            const int64_t g = (wg0 + it) * gpw + sub;
+            const bool act = g < G;
+            int64_t nm;
+            group_at(act, g, b[it], nm);
 #pragma unroll
             for (int q = 0; q < ZR; ++q)
-                if (q < rounds) vec[first + q * sw + ul] = make_double2(0, 0);
+                if (q < ns) vec[first + q * sw + ul] = make_double2(0, 0);
             __syncwarp();
 #pragma unroll
             for (int q = 0; q < ZR; ++q) {
                 const int64_t mi = (int64_t)q * sw + ul;
-                if (q < rounds && mi < nm)
-                    vec[first + (int)((keys[b + mi].w[0] >> 1) & (uint64_t)(s - 1))] = amps[b + mi];
+                if (q < ns && mi < nm)
+                    vec[first + (int)((keys[b[it] + mi].w[0] >> 1) & (uint64_t)(s - 1))] = amps[b[it] + mi];
             }
             __syncwarp();
 #pragma unroll
-            for (int q = 0; q < ZR; ++q) x[q] = q < rounds ? vec[first + q * sw + ul] : make_double2(0, 0);
+            for (int q = 0; q < ZR; ++q) x[it][q] = q < ns ? vec[first + q * sw + ul] : make_double2(0, 0);
             __syncwarp();
             for (int h = 1; h < sw; h <<= 1) {
 #pragma unroll
                 for (int q = 0; q < ZR; ++q) {
-                    if (q >= rounds) continue;
-                    const double yx = __shfl_xor_sync(FULL, x[q].x, h), yy = __shfl_xor_sync(FULL, x[q].y, h);
-                    x[q] = (ul & h) ? make_double2(yx - x[q].x, yy - x[q].y)
-                                    : make_double2(x[q].x + yx, x[q].y + yy);
+                    if (q >= ns) continue;
+                    const double yx = __shfl_xor_sync(FULL, x[it][q].x, h), yy = __shfl_xor_sync(FULL, x[it][q].y, h);
+                    x[it][q] = (ul & h) ? make_double2(yx - x[it][q].x, yy - x[it][q].y)
+                                        : make_double2(x[it][q].x + yx, x[it][q].y + yy);
                 }
             }
 #pragma unroll
             for (int hq = 1; hq < ZR; hq <<= 1) {
 #pragma unroll
                 for (int q = 0; q < ZR; ++q) {
-                    if ((q & hq) || (q | hq) >= rounds) continue;
-                    const double2 lo = x[q], hi = x[q | hq];
-                    x[q] = make_double2(lo.x + hi.x, lo.y + hi.y);
-                    x[q | hq] = make_double2(lo.x - hi.x, lo.y - hi.y);
+                    if ((q & hq) || (q | hq) >= ns) continue;
+                    const double2 lo = x[it][q], hi = x[it][q | hq];
+                    x[it][q] = make_double2(lo.x + hi.x, lo.y + hi.y);
+                    x[it][q | hq] = make_double2(lo.x - hi.x, lo.y - hi.y);
                 }
             }
+#pragma unroll
+            for (int q = 0; q < ZR; ++q) {
+                x[it][q] = cscale(d.inv_sqrt_s, x[it][q]);
+                kept[it][q] = __ballot_sync(FULL, act && q < ns && keep(x[it][q], d.tau2));
+                n += __popc(kept[it][q]);
+            }
         }
-        uint32_t run = 0u;
+        unsigned long long at = tile_place<32 * HG_WARPS>(ts, vb, gridDim.x, lane == 0 ? n : 0u, status);
+        at = __shfl_sync(FULL, at, 0);
+#pragma unroll
+        for (int it = 0; it < ITERS; ++it) {
+            /* s < 32: one round, the warp's groups one after another; s >= 32: one group */
+#pragma unroll
+            for (int q = 0; q < ZR; ++q) {
+                const int64_t dst = (int64_t)at + __popc(kept[it][q] & below);
+                if (((kept[it][q] >> lane) & 1u) && dst < cap) {
+                    FKeyN<NW> ko = keys[b[it]];
+                    ko.w[0] = (ko.w[0] & ~lowm) | ((uint64_t)(q * sw + ul) << 1);
+                    okeys[dst] = ko;
+                    oamps[dst] = x[it][q];
+                }
+                at += __popc(kept[it][q]);
+            }
+        }
+        return;
+    }
+    /* s > 128: one group a warp */
+    const bool act = wg0 < G;
+    int64_t b, nm;
+    group_at(act, wg0, b, nm);
+    unsigned long long at = 0;
+    for (int pass = 0; pass < 2; ++pass) { /* counted, then written */
+        unsigned run = 0;
         for (int q = 0; q < rounds; ++q) {
             const uint32_t u = (uint32_t)(q * sw + ul);
             double2 o = make_double2(0, 0);
-            if (fwht) {
-#pragma unroll
-                for (int t = 0; t < ZR; ++t)
-                    if (t == q) o = x[t];
-            }
-            for (int q2 = 0; q2 < rounds && !fwht; ++q2) {
+            for (int q2 = 0; q2 < rounds; ++q2) {
                 const int64_t mi = (int64_t)q2 * sw + ul;
                 uint32_t mv = 0u;
                 double2 ma = make_double2(0, 0);
@@ -1081,31 +1163,20 @@ __global__ void __launch_bounds__(256) k_f_hgroups(QwSimDev d, const FKeyN<NW> *
                 }
             }
             o = cscale(d.inv_sqrt_s, o);
-            const bool kept = act && keep(o, d.tau2);
-            const unsigned bal = __ballot_sync(FULL, kept) & seg;
-            const uint32_t rank = run + (uint32_t)__popc(bal & below);
-            if (!COUNT && kept && rank < cnt[g]) { /* the count pass made the same decisions */
-                const int64_t dst = (int64_t)gpos[g] + rank;
+            const unsigned bal = __ballot_sync(FULL, act && keep(o, d.tau2));
+            const int64_t dst = (int64_t)at + run + __popc(bal & below);
+            if (pass == 1 && ((bal >> lane) & 1u) && dst < cap) {
                 FKeyN<NW> ko = keys[b];
                 ko.w[0] = (ko.w[0] & ~lowm) | ((uint64_t)u << 1);
                 okeys[dst] = ko;
                 oamps[dst] = o;
             }
-            run += (uint32_t)__popc(bal);
+            run += (unsigned)__popc(bal);
         }
-        if (COUNT && act && ul == 0) cnt[g] = run;
-    }
-}
-
-/* the "clearing" step: kept entries to their scanned positions */
-template <int NW>
-__global__ void k_f_compact(const FKeyN<NW> *keys, const double2 *amps, const uint32_t *flags, const uint32_t *pos,
-                            int64_t n, FKeyN<NW> *okeys, double2 *oamps)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        if (!flags[i]) continue;
-        okeys[pos[i]] = keys[i];
-        oamps[pos[i]] = amps[i];
+        if (pass == 0) {
+            at = tile_place<32 * HG_WARPS>(ts, vb, gridDim.x, lane == 0 ? run : 0u, status);
+            at = __shfl_sync(FULL, at, 0);
+        }
     }
 }
 
@@ -1306,21 +1377,6 @@ cudaError_t qw_flat_phase(const QwSimDev &d, const void *keys, double2 *amps, in
     return cudaGetLastError();
 }
 
-size_t qw_flat_scan_words(int64_t n)
-{
-    return (size_t)((n + SCAN_TILE - 1) / SCAN_TILE) + 1;
-}
-
-cudaError_t qw_flat_scan(const uint32_t *in, int64_t n, uint32_t *sums, uint32_t *out, cudaStream_t st)
-{
-    if (n <= 0) return cudaSuccess;
-    const int64_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
-    k_scan_reduce<<<(unsigned)nb, 256, 0, st>>>(in, n, sums);
-    k_scan_blocks<<<1, 1024, 0, st>>>(sums, nb);
-    k_scan_apply<<<(unsigned)nb, 256, 0, st>>>(in, n, sums, out);
-    return cudaGetLastError();
-}
-
 namespace {
 /* work layout of qw_flat_sort, in bytes: the tiles' status words, the
    digit counts of every chunk, the block counters of every pass, two
@@ -1471,88 +1527,99 @@ cudaError_t qw_flat_sort(const QwSimDev &d, void *keys, double2 *amps, void *tmp
     return flat_sort_t<2>(d, keys, amps, tmpk, tmpa, M, order, group, work, status, st, in_tmp);
 }
 
-/* op: 0 = R^dag, 1 = R (2 outputs per entry), 2 = H (s outputs per entry) */
-cudaError_t qw_flat_heads(const QwSimDev &d, const void *keys, int64_t M, uint32_t *flags, cudaStream_t st, int kw)
+/* The single-pass kernels' tile sums, zeroed: tiles of `per` inputs */
+size_t qw_flat_tiles_bytes(int64_t n)
 {
-    if (M <= 0) return cudaSuccess;
-    if (kw == NW_FAITH)
-        k_f_heads<NW_FAITH><<<grid_for(M, 256), 256, 0, st>>>(d, static_cast<const FKeyW *>(keys), M, flags);
-    else k_f_heads<2><<<grid_for(M, 256), 256, 0, st>>>(d, static_cast<const FKey *>(keys), M, flags);
-    return cudaGetLastError();
+    /* one word per tile; the smallest tiles are the direct sums', 8 groups */
+    return sizeof(TileSum) + (size_t)((n + HG_WARPS - 1) / HG_WARPS) * 8;
 }
 
-cudaError_t qw_flat_starts(const uint32_t *heads, const uint32_t *gidx, int64_t M, int64_t G, int64_t *starts,
-                           cudaStream_t st)
+namespace {
+cudaError_t tiles_clear(void *ts, int64_t ntiles, cudaStream_t st)
 {
-    if (M <= 0) return cudaSuccess;
-    k_f_starts<<<grid_for(M, 256), 256, 0, st>>>(heads, gidx, M, G, starts);
-    return cudaGetLastError();
+    return cudaMemsetAsync(ts, 0, sizeof(TileSum) + (size_t)ntiles * 8, st);
+}
+} // namespace
+
+/* where the number of outputs is found */
+const unsigned long long *qw_flat_tiles_total(const void *ts)
+{
+    return &static_cast<const TileSum *>(ts)->total;
 }
 
-cudaError_t qw_flat_group(const QwSimDev &d, int op, const void *keys, const double2 *amps, int64_t M, void *okeys,
-                          double2 *oamps, uint32_t *flags, cudaStream_t st, int kw)
+cudaError_t qw_flat_rot(const QwSimDev &d, int op, const void *keys, const double2 *amps, int64_t M, void *okeys,
+                        double2 *oamps, int64_t cap, void *tiles, int32_t *status, cudaStream_t st, int kw)
 {
     if (M <= 0) return cudaSuccess;
+    const int64_t nt = (M + RT_THREADS - 1) / RT_THREADS;
+    const cudaError_t e = tiles_clear(tiles, nt, st);
+    if (e != cudaSuccess) return e;
+    TileSum *ts = static_cast<TileSum *>(tiles);
+    const unsigned grid = (unsigned)nt;
     if (kw == NW_FAITH) {
         const FKeyW *k = static_cast<const FKeyW *>(keys);
         FKeyW *ok = static_cast<FKeyW *>(okeys);
-        if (op == 0) k_f_rot<true, NW_FAITH><<<grid_for(M, 256), 256, 0, st>>>(d, k, amps, M, ok, oamps, flags);
-        else k_f_rot<false, NW_FAITH><<<grid_for(M, 256), 256, 0, st>>>(d, k, amps, M, ok, oamps, flags);
+        if (op == 0) k_f_rot<true, NW_FAITH><<<grid, RT_THREADS, 0, st>>>(d, k, amps, M, ok, oamps, cap, ts, status);
+        else k_f_rot<false, NW_FAITH><<<grid, RT_THREADS, 0, st>>>(d, k, amps, M, ok, oamps, cap, ts, status);
     } else {
         const FKey *k = static_cast<const FKey *>(keys);
         FKey *ok = static_cast<FKey *>(okeys);
-        if (op == 0) k_f_rot<true, 2><<<grid_for(M, 256), 256, 0, st>>>(d, k, amps, M, ok, oamps, flags);
-        else k_f_rot<false, 2><<<grid_for(M, 256), 256, 0, st>>>(d, k, amps, M, ok, oamps, flags);
+        if (op == 0) k_f_rot<true, 2><<<grid, RT_THREADS, 0, st>>>(d, k, amps, M, ok, oamps, cap, ts, status);
+        else k_f_rot<false, 2><<<grid, RT_THREADS, 0, st>>>(d, k, amps, M, ok, oamps, cap, ts, status);
     }
+    return cudaGetLastError();
+}
+
+cudaError_t qw_flat_starts(const QwSimDev &d, const void *keys, int64_t M, int64_t *starts, void *tiles,
+                           int32_t *status, cudaStream_t st, int kw)
+{
+    if (M <= 0) return cudaSuccess;
+    const int64_t nt = (M + ST_THREADS * ST_IPT - 1) / (ST_THREADS * ST_IPT);
+    const cudaError_t e = tiles_clear(tiles, nt, st);
+    if (e != cudaSuccess) return e;
+    TileSum *ts = static_cast<TileSum *>(tiles);
+    const unsigned grid = (unsigned)nt;
+    if (kw == NW_FAITH)
+        k_f_starts<NW_FAITH><<<grid, ST_THREADS, 0, st>>>(d, static_cast<const FKeyW *>(keys), M, starts, ts, status);
+    else k_f_starts<2><<<grid, ST_THREADS, 0, st>>>(d, static_cast<const FKey *>(keys), M, starts, ts, status);
     return cudaGetLastError();
 }
 
 namespace {
 template <int NW, int R>
-void launch_hgroups(const QwSimDev &d, const FKeyN<NW> *k, const double2 *amps, const int64_t *starts, int64_t G,
-                    uint32_t *cnt, const uint32_t *gpos, FKeyN<NW> *ok, double2 *oamps, int grid, cudaStream_t st)
+cudaError_t launch_hgroups(const QwSimDev &d, const void *keys, const double2 *amps, int64_t M, const int64_t *starts,
+                           int64_t G, void *okeys, double2 *oamps, int64_t cap, void *tiles, int32_t *status, cudaStream_t st)
 {
-    if (gpos == nullptr) k_f_hgroups<NW, true, R><<<grid, 256, 0, st>>>(d, k, amps, starts, G, cnt, nullptr, nullptr, nullptr);
-    else k_f_hgroups<NW, false, R><<<grid, 256, 0, st>>>(d, k, amps, starts, G, cnt, gpos, ok, oamps);
+    const int64_t per = (int64_t)HG_WARPS * HgIters<R>::n * (d.s < 32 ? 32 / d.s : 1), nt = (G + per - 1) / per;
+    const cudaError_t e = tiles_clear(tiles, nt, st);
+    if (e != cudaSuccess) return e;
+    k_f_hgroups<NW, R><<<(unsigned)nt, 32 * HG_WARPS, 0, st>>>(d, static_cast<const FKeyN<NW> *>(keys), amps, M, starts, G,
+                                                             static_cast<FKeyN<NW> *>(okeys), oamps, cap,
+                                                             static_cast<TileSum *>(tiles), status);
+    return cudaGetLastError();
 }
 
 /* the fast transform's vector entries a lane: 1 (s <= 32), 2 (64), 4 (128);
    0: the direct sums (s > 128) */
 template <int NW>
-void launch_hgroups_s(const QwSimDev &d, const void *keys, const double2 *amps, const int64_t *starts, int64_t G,
-                      uint32_t *cnt, const uint32_t *gpos, void *okeys, double2 *oamps, int grid, cudaStream_t st)
+cudaError_t launch_hgroups_s(const QwSimDev &d, const void *keys, const double2 *amps, int64_t M, const int64_t *starts, int64_t G,
+                             void *okeys, double2 *oamps, int64_t cap, void *tiles, int32_t *status, cudaStream_t st)
 {
-    const FKeyN<NW> *k = static_cast<const FKeyN<NW> *>(keys);
-    FKeyN<NW> *ok = static_cast<FKeyN<NW> *>(okeys);
-    if (d.s <= 32) launch_hgroups<NW, 1>(d, k, amps, starts, G, cnt, gpos, ok, oamps, grid, st);
-    else if (d.s == 64) launch_hgroups<NW, 2>(d, k, amps, starts, G, cnt, gpos, ok, oamps, grid, st);
-    else if (d.s == 128) launch_hgroups<NW, 4>(d, k, amps, starts, G, cnt, gpos, ok, oamps, grid, st);
-    else launch_hgroups<NW, 0>(d, k, amps, starts, G, cnt, gpos, ok, oamps, grid, st);
+    if (d.s <= 32) return launch_hgroups<NW, 1>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, status, st);
+    if (d.s == 64) return launch_hgroups<NW, 2>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, status, st);
+    if (d.s == 128) return launch_hgroups<NW, 4>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, status, st);
+    return launch_hgroups<NW, 0>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, status, st);
 }
 } // namespace
 
-cudaError_t qw_flat_hgroups(const QwSimDev &d, const void *keys, const double2 *amps, const int64_t *starts, int64_t G,
-                            uint32_t *cnt, const uint32_t *gpos, void *okeys, double2 *oamps, cudaStream_t st, int kw)
+cudaError_t qw_flat_hgroups(const QwSimDev &d, const void *keys, const double2 *amps, int64_t M, const int64_t *starts, int64_t G,
+                            void *okeys, double2 *oamps, int64_t cap, void *tiles, int32_t *status, cudaStream_t st,
+                            int kw)
 {
     if (G <= 0) return cudaSuccess;
-    const int gpw = d.s < 32 ? 32 / d.s : 1;
-    const int grid = grid_for((G + gpw - 1) / gpw * 32, 256);
-    if (kw == NW_FAITH) launch_hgroups_s<NW_FAITH>(d, keys, amps, starts, G, cnt, gpos, okeys, oamps, grid, st);
-    else launch_hgroups_s<2>(d, keys, amps, starts, G, cnt, gpos, okeys, oamps, grid, st);
-    return cudaGetLastError();
-}
-
-cudaError_t qw_flat_compact(const void *keys, const double2 *amps, const uint32_t *flags, const uint32_t *pos,
-                            int64_t n, void *okeys, double2 *oamps, cudaStream_t st, int kw)
-{
-    if (n <= 0) return cudaSuccess;
     if (kw == NW_FAITH)
-        k_f_compact<NW_FAITH><<<grid_for(n, 256), 256, 0, st>>>(static_cast<const FKeyW *>(keys), amps, flags, pos, n,
-                                                                  static_cast<FKeyW *>(okeys), oamps);
-    else
-        k_f_compact<2><<<grid_for(n, 256), 256, 0, st>>>(static_cast<const FKey *>(keys), amps, flags, pos, n,
-                                                           static_cast<FKey *>(okeys), oamps);
-    return cudaGetLastError();
+        return launch_hgroups_s<NW_FAITH>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, status, st);
+    return launch_hgroups_s<2>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, status, st);
 }
 
 cudaError_t qw_flat_readout(const QwSimDev &d, const void *keys, const double2 *amps, int64_t M, const QwStepArgs &a,

@@ -289,8 +289,6 @@ cudaError_t qw_flat_gather(const QwSimDev &d, const QwBufDev &buf, int inst, int
 cudaError_t qw_flat_map(const QwSimDev &d, void *keys, int64_t M, uint32_t ops, int32_t *status, cudaStream_t st,
                         int kw);
 cudaError_t qw_flat_phase(const QwSimDev &d, const void *keys, double2 *amps, int64_t M, cudaStream_t st, int kw);
-size_t qw_flat_scan_words(int64_t n);
-cudaError_t qw_flat_scan(const uint32_t *in, int64_t n, uint32_t *sums, uint32_t *out, cudaStream_t st);
 /* stable sort by the permuted key (order 0: R, 1: H); work holds
    qw_flat_sort_bytes(M); the result is left in tmpk / tmpa when *in_tmp */
 size_t qw_flat_sort_bytes(int64_t M);
@@ -299,20 +297,22 @@ size_t qw_flat_sort_bytes(int64_t M);
 #define QW_SORT_GROUP_NO_A 2 /* A's too: it follows from the other idle registers */
 cudaError_t qw_flat_sort(const QwSimDev &d, void *keys, double2 *amps, void *tmpk, double2 *tmpa, int64_t M,
                          int order, int group, void *work, int32_t *status, cudaStream_t st, int kw, int *in_tmp);
-/* the Hadamard stage's groups: head flags of the sorted list, and the first
-   member of each of its G groups (starts[G] = M) from their exclusive scan */
-cudaError_t qw_flat_heads(const QwSimDev &d, const void *keys, int64_t M, uint32_t *flags, cudaStream_t st, int kw);
-cudaError_t qw_flat_starts(const uint32_t *heads, const uint32_t *gidx, int64_t M, int64_t G, int64_t *starts,
-                           cudaStream_t st);
-/* op 0 (R^dag) and 1 (R): 2 M outputs with their keep flags */
-cudaError_t qw_flat_group(const QwSimDev &d, int op, const void *keys, const double2 *amps, int64_t M, void *okeys,
-                          double2 *oamps, uint32_t *flags, cudaStream_t st, int kw);
-/* H on the G groups (starts): gpos == nullptr -- the kept outputs of each
-   group into cnt; otherwise the kept outputs written from gpos[g] on */
-cudaError_t qw_flat_hgroups(const QwSimDev &d, const void *keys, const double2 *amps, const int64_t *starts, int64_t G,
-                            uint32_t *cnt, const uint32_t *gpos, void *okeys, double2 *oamps, cudaStream_t st, int kw);
-cudaError_t qw_flat_compact(const void *keys, const double2 *amps, const uint32_t *flags, const uint32_t *pos,
-                            int64_t n, void *okeys, double2 *oamps, cudaStream_t st, int kw);
+/* Scratch of a single-pass kernel over n entries or groups, and where it
+   leaves the number of its outputs. */
+size_t qw_flat_tiles_bytes(int64_t n);
+const unsigned long long *qw_flat_tiles_total(const void *tiles);
+/* op 0 (R^dag) and 1 (R) on the sorted list: the kept outputs (up to 2 M; cap
+   is the room in okeys / oamps) */
+cudaError_t qw_flat_rot(const QwSimDev &d, int op, const void *keys, const double2 *amps, int64_t M, void *okeys,
+                        double2 *oamps, int64_t cap, void *tiles, int32_t *status, cudaStream_t st, int kw);
+/* the Hadamard stage's groups: the first member of each (their number G is the
+   kernel's total), starts[G] = M; starts has room for M + 1 */
+cudaError_t qw_flat_starts(const QwSimDev &d, const void *keys, int64_t M, int64_t *starts, void *tiles,
+                           int32_t *status, cudaStream_t st, int kw);
+/* H on the G groups: the kept outputs (up to G s) */
+cudaError_t qw_flat_hgroups(const QwSimDev &d, const void *keys, const double2 *amps, int64_t M, const int64_t *starts, int64_t G,
+                            void *okeys, double2 *oamps, int64_t cap, void *tiles, int32_t *status, cudaStream_t st,
+                            int kw);
 cudaError_t qw_flat_readout(const QwSimDev &d, const void *keys, const double2 *amps, int64_t M, const QwStepArgs &a,
                             cudaStream_t st, int kw);
 cudaError_t qw_flat_scatter(const QwSimDev &d, const QwBufDev &out, int fp32, const void *keys, const double2 *amps,
