@@ -908,7 +908,8 @@ QwPosPlan pos_plan(const QwSimDev &d)
     pl.tab = pl.smem + 1024 <= (size_t)optin; /* beside the kernel's static arrays */
     if (!pl.tab) pl.smem = 0;
     pl.coop = coop != 0 && pl.grid < 256; /* the barrier word's count has 8 bits */
-    if (pl.tab) cudaFuncSetAttribute(pos_kernel<AmpT, false, true>(s), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
+    if (pl.tab) /* the limit belongs to the process, not to this simulator: always the largest */
+        cudaFuncSetAttribute(pos_kernel<AmpT, false, true>(s), cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 1024);
     return pl;
 }
 
