@@ -240,8 +240,8 @@ int qw_sync(qw_sim *sim);
  * them with CUDA events on the simulator's stream, and keeps the fastest for
  * all later steps.  Segments are tried only when warp_capacity >= 2
  * row_capacity (true by default), the slot kernel only then and for s = 8, 16
- * or 32, the positional layout (variant 7) for s = 8, 16, 32 or 64 without
- * partitions (its tables are built first, and the move of the state into it
+ * or 32, the positional layout (variant 7) for s = 4, 8, 16, 32 or 64 without
+ * partitions (s = 4: here only, a simulator is not created with it; its tables are built first, and the move of the state into it
  * is not timed); the flat path and the register-faithful
  * schedule (variants 5 and 6) are never chosen; variants not tried are
  * reported as 0 us.  The state advances by steps_per_candidate walk steps per

@@ -411,7 +411,8 @@ extern "C" int qw_sim_create(const qw_csc *mats, int32_t ninst, const qw_sim_opt
         qw_sim_destroy(sim);
         return QW_ERR_ARG;
     }
-    if (sim->mode == QW_MODE_WALK_POS && !qw_pos_supported(d)) {
+    /* (s = 4: chosen by qw_autotune only) */
+    if (sim->mode == QW_MODE_WALK_POS && (!qw_pos_supported(d) || d.s < 8)) {
         g_create_error = "qw_sim_create: walk_variant 7 (positional layout) needs s = 8, 16, 32 or 64";
         qw_sim_destroy(sim);
         return QW_ERR_ARG;
@@ -1137,7 +1138,7 @@ static int pos_build(qw_sim *sim)
     if (sim->pos_built) return QW_OK;
     QwSimDev &d = sim->d;
     if (d.nparts != 1 || !qw_pos_supported(d))
-        return fail(sim, QW_ERR_ARG, "walk_variant 7 (positional) needs s = 8, 16, 32 or 64 and no partitions");
+        return fail(sim, QW_ERR_ARG, "walk_variant 7 (positional) needs s = 4, 8, 16, 32 or 64 and no partitions");
     const int s = d.s;
     const int ninst = d.ninst;
     /* rows of all instances in order: instance i starts at row inst_img[i] / s */
@@ -1793,13 +1794,17 @@ extern "C" int qw_autotune(qw_sim *sim, int32_t steps, int32_t *choice, double *
     /* candidates: walk_variant -> mode.  A segment holds two rows on chip:
        tried only when the warp buffer fits them; the slot kernel (which falls
        back to segments) also needs s = 8, 16 or 32; the positional layout
-       s = 8 .. 64 and no partitions (its tables are built first: they may
-       grow row_capacity, which the other kernels' launch shapes follow) */
+       s = 4 .. 64 and no partitions (its tables are built first: they may
+       grow row_capacity, which the other kernels' launch shapes follow).  At s = 4
+       the bucket kernels' step is ~17 us whatever N is (a launch and the last
+       block's reduction), a positional one 2 to 4: ten at N = 16 242 -> 80 us a job,
+       60 at N = 6000 (complex128) 1890 -> 296 */
     const bool slot = qw_slot_supported(sim->d);
-    const bool pos = qw_pos_supported(sim->d) && sim->d.nparts == 1;
+    bool pos = qw_pos_supported(sim->d) && sim->d.nparts == 1;
     if (pos) {
         const int rc = pos_build(sim);
-        if (rc != QW_OK) return rc;
+        if (rc != QW_OK && sim->d.s >= 8) return rc;
+        pos = rc == QW_OK; /* s = 4: a matrix it cannot hold keeps the bucket kernels */
     }
     const bool seg = sim->d.warp_cap >= 2 * sim->d.cap_row;
     std::vector<std::pair<int, int>> cand = {{0, QW_MODE_WALK_FUSED}, {1, QW_MODE_WALK_FUSED_PF}};

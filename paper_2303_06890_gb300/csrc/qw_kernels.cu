@@ -2369,7 +2369,7 @@ int qw_slot_supported(const QwSimDev &d)
 
 int qw_pos_supported(const QwSimDev &d)
 {
-    return d.s == 8 || d.s == 16 || d.s == 32 || d.s == 64;
+    return d.s == 4 || d.s == 8 || d.s == 16 || d.s == 32 || d.s == 64;
 }
 
 size_t qw_step_smem_bytes(const QwSimDev &d, int fp32, int mode)

@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
     /* a unit (one j) on SW lanes, each lane holding SPL of its slots (l = lb
        + 32 k); RPP units per warp (a group) */
     constexpr int SW = S > 32 ? 32 : S, SPL = S / SW, RPP = 32 / SW;
-    constexpr int LOG2S = S == 8 ? 3 : S == 16 ? 4 : S == 32 ? 5 : 6;
+    constexpr int LOG2S = S == 4 ? 2 : S == 8 ? 3 : S == 16 ? 4 : S == 32 ? 5 : 6;
     constexpr float kHalfS = 0.5f * S, kErr = Amp<AmpT>::kApproxErr;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long part_u[kPosMaxWarps];
@@ -872,6 +872,7 @@ __global__ void k_pos_unpack(QwSimDev d, const AmpT *pbuf, int full, QwBufDev bu
 template <typename AmpT, bool FULLST, bool TAB>
 void *pos_kernel(int s)
 {
+    if (s == 4) return (void *)k_walk_pos<AmpT, 4, FULLST, TAB>;
     if (s == 8) return (void *)k_walk_pos<AmpT, 8, FULLST, TAB>;
     if (s == 16) return (void *)k_walk_pos<AmpT, 16, FULLST, TAB>;
     if (s == 32) return (void *)k_walk_pos<AmpT, 32, FULLST, TAB>;
