@@ -88,6 +88,7 @@ struct qw_sim {
     cudaStream_t stream = nullptr;
     int device = 0;                  /* CUDA device current at creation */
     cudaMemPool_t fpool = nullptr;   /* flat-path scratch (flat_alloc) */
+    unsigned long long *h_flat = nullptr; /* pinned, with it: what the host reads between stages (kFlat*) */
     int fp32 = 0;
     int renorm = 0;
     int mode = QW_MODE_WALK_FUSED;
@@ -180,6 +181,9 @@ static bool host_staged(const qw_sim *sim)
 
 static const int kGraphSteps = 6; /* a multiple of the 3-buffer and 2-slot periods */
 static const int kGraphTerms = 3;  /* QLS terms per graph: 2 walk steps each */
+/* words of h_flat: outputs of a stage, branches of the state, longest row, flags
+   of an import (6), the sort's varying bits (2 x 10) */
+static const int kFlatTotal = 0, kFlatCount = 1, kFlatRow = 2, kFlatIo = 4, kFlatSort = 16, kFlatWords = 40;
 static const int64_t kPosSteps = 1024; /* walk steps of one positional launch: a few milliseconds */
 
 static void drop_graphs(qw_sim *sim)
@@ -632,6 +636,7 @@ extern "C" int qw_sim_destroy(qw_sim *sim)
     if (sim->stream) cudaStreamSynchronize(sim->stream);
     else cudaDeviceSynchronize();
     if (sim->fpool) cudaMemPoolDestroy(sim->fpool);
+    if (sim->h_flat) cudaFreeHost(sim->h_flat);
     cudaFree(sim->pos_dst);
     cudaFree(sim->pos_xdst);
     cudaFree(sim->pos_rowinst);
@@ -907,6 +912,12 @@ static cudaError_t flat_alloc(qw_sim *sim, size_t bytes, void **p)
             sim->fpool = nullptr;
             return e;
         }
+        if ((e = cudaMallocHost((void **)&sim->h_flat, kFlatWords * 8)) != cudaSuccess) {
+            cudaMemPoolDestroy(sim->fpool);
+            sim->fpool = nullptr;
+            sim->h_flat = nullptr;
+            return e;
+        }
         uint64_t keep = UINT64_MAX;
         if ((e = cudaMemPoolSetAttribute(sim->fpool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) return e;
     }
@@ -946,15 +957,17 @@ static void flat_release(qw_sim *sim, FlatList &L)
 static cudaError_t flat_gather(qw_sim *sim, FlatList &L, int kw)
 {
     cudaStream_t st = sim->stream;
-    unsigned long long hc = 0;
     cudaError_t e;
+    void *first = nullptr; /* (the pool and h_flat are there) */
+    if (!sim->fpool && (e = flat_alloc(sim, 16, &first)) != cudaSuccess) return e;
+    if (first) cudaFreeAsync(first, st);
     if ((e = cudaMemsetAsync(&sim->sc->counter, 0, 8, st)) != cudaSuccess) return e;
     if ((e = qw_launch_count(sim->d, sim->buf[sim->cur], -1, &sim->sc->counter, st)) != cudaSuccess) return e;
-    if ((e = cudaMemcpyAsync(&hc, &sim->sc->counter, 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
+    if ((e = cudaMemcpyAsync(sim->h_flat + kFlatCount, &sim->sc->counter, 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
     flat_release(sim, L);
     L.kw = kw;
-    L.M = (int64_t)hc;
+    L.M = (int64_t)sim->h_flat[kFlatCount];
     if ((e = flat_alloc(sim, (size_t)L.M * 8 * kw, &L.K)) != cudaSuccess) return e;
     if ((e = flat_alloc(sim, (size_t)L.M * 16, (void **)&L.A)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(&sim->sc->counter, 0, 8, st)) != cudaSuccess) return e;
@@ -981,7 +994,7 @@ static cudaError_t flat_stage(qw_sim *sim, FlatList &L, int op, int group)
         if ((e = flat_alloc(sim, (size_t)L.M * 16, &ta)) != cudaSuccess) return e;
         if ((e = flat_alloc(sim, qw_flat_sort_bytes(L.M), &work)) != cudaSuccess) return e;
         int in_tmp = 0;
-        e = qw_flat_sort(d, L.K, L.A, tk, static_cast<double2 *>(ta), L.M, op == 2 ? 1 : 0, group, work,
+        e = qw_flat_sort(d, L.K, L.A, tk, static_cast<double2 *>(ta), L.M, op == 2 ? 1 : 0, group, work, sim->h_flat + kFlatSort,
                          &sim->sc->status, st, L.kw, &in_tmp);
         if (e == cudaSuccess && in_tmp) {
             /* the sorted list is the one in the scratch arrays: swap them */
@@ -999,20 +1012,17 @@ static cudaError_t flat_stage(qw_sim *sim, FlatList &L, int op, int group)
     FlatScratch scratch(sim);
     void *tiles = nullptr, *starts = nullptr;
     if ((e = scratch.take(qw_flat_tiles_bytes(L.M), &tiles)) != cudaSuccess) return e;
-    unsigned long long total = 0;
-    auto read_total = [&]() {
-        const cudaError_t r = cudaMemcpyAsync(&total, qw_flat_tiles_total(tiles), 8, cudaMemcpyDeviceToHost, st);
-        return r != cudaSuccess ? r : cudaStreamSynchronize(st);
-    };
+    unsigned long long *const total = sim->h_flat + kFlatTotal;
+    *total = 0;
     /* H: the groups of the sorted list, their number read by the host; up to s
        outputs each.  R, R^dag: up to two an entry. */
     int64_t cap = 2 * L.M, G = 0;
     if (op == 2) {
         if ((e = scratch.take((size_t)(L.M + 1) * 8, &starts)) != cudaSuccess) return e;
-        e = qw_flat_starts(d, L.K, L.M, static_cast<int64_t *>(starts), tiles, &sim->sc->status, st, L.kw);
-        if (e == cudaSuccess) e = read_total();
+        e = qw_flat_starts(d, L.K, L.M, static_cast<int64_t *>(starts), tiles, total, &sim->sc->status, st, L.kw);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return e;
-        G = std::min<int64_t>((int64_t)total, L.M); /* (more only after a wait gave up) */
+        G = std::min<int64_t>((int64_t)*total, L.M); /* (more only after a wait gave up) */
         cap = G * d.s;
     }
     FlatList R;
@@ -1020,15 +1030,15 @@ static cudaError_t flat_stage(qw_sim *sim, FlatList &L, int op, int group)
     e = flat_alloc(sim, (size_t)cap * kb, &R.K);
     if (e == cudaSuccess) e = flat_alloc(sim, (size_t)cap * 16, (void **)&R.A);
     if (e == cudaSuccess)
-        e = op == 2 ? qw_flat_hgroups(d, L.K, L.A, L.M, static_cast<int64_t *>(starts), G, R.K, R.A, cap, tiles,
+        e = op == 2 ? qw_flat_hgroups(d, L.K, L.A, L.M, static_cast<int64_t *>(starts), G, R.K, R.A, cap, tiles, total,
                                       &sim->sc->status, st, L.kw)
-                    : qw_flat_rot(d, op, L.K, L.A, L.M, R.K, R.A, cap, tiles, &sim->sc->status, st, L.kw);
-    if (e == cudaSuccess) e = read_total();
+                    : qw_flat_rot(d, op, L.K, L.A, L.M, R.K, R.A, cap, tiles, total, &sim->sc->status, st, L.kw);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         flat_release(sim, R);
         return e;
     }
-    R.M = std::min<int64_t>((int64_t)total, cap);
+    R.M = std::min<int64_t>((int64_t)*total, cap);
     R.by_h = op == 2;
     flat_release(sim, L);
     L = R;
@@ -1055,16 +1065,15 @@ static int flat_store(qw_sim *sim, FlatList &L, const QwStepArgs &a, const int64
         QW_CUDA(sim, cudaMemsetAsync(maxrow, 0, 4, st));
         QW_CUDA(sim, qw_flat_scatter(d, sim->buf[nxt], sim->fp32, L.K, L.A, L.M, status,
                                      static_cast<unsigned int *>(maxrow), static_cast<double *>(norm), st, L.kw));
-        unsigned int hmax = 0;
         QW_CUDA(sim, cudaMemcpyAsync(sim->h_st, status, sizeof(StatusView), cudaMemcpyDeviceToHost, st));
-        QW_CUDA(sim, cudaMemcpyAsync(&hmax, maxrow, 4, cudaMemcpyDeviceToHost, st));
+        QW_CUDA(sim, cudaMemcpyAsync(sim->h_flat + kFlatRow, maxrow, 4, cudaMemcpyDeviceToHost, st));
         QW_CUDA(sim, cudaStreamSynchronize(st));
         if (sim->h_st->status != QW_ST_ROW_OVERFLOW || attempt == 1 || !sim->opts.overflow_fallback) break;
         /* a row of the result is longer than row_capacity: grow the buckets
            and store again */
         const int32_t zero = 0;
         QW_CUDA(sim, cudaMemcpyAsync(status, &zero, 4, cudaMemcpyHostToDevice, st));
-        rc = grow_rows(sim, (int64_t)hmax);
+        rc = grow_rows(sim, (int64_t)(unsigned int)sim->h_flat[kFlatRow]);
     }
     if (rc == QW_OK) {
         QW_CUDA(sim, qw_flat_finish(a, static_cast<double *>(norm), counts, st));
@@ -2124,7 +2133,7 @@ extern "C" int qw_state_export(qw_sim *sim, int32_t inst, int32_t key_words, uin
     sim->launches++;
     int in_tmp = 0;
     QW_CUDA(sim, qw_flat_sort(sim->d, K, static_cast<double2 *>(A), tk, static_cast<double2 *>(ta), total, 0, QW_SORT_FULL,
-                              work,
+                              work, sim->h_flat + kFlatSort,
                               &sim->sc->status, st, 2, &in_tmp));
     if (in_tmp) {
         std::swap(K, tk);
@@ -2217,8 +2226,9 @@ extern "C" int qw_state_import(qw_sim *sim, int32_t key_words, const uint64_t *k
         sim->launches += 2;
         QW_CUDA(sim, cudaMemcpyAsync(A, amps, M * 16, cudaMemcpyHostToDevice, st));
         for (int64_t i = 0; i < count; ++i) norm2 += amps[2 * i] * amps[2 * i] + amps[2 * i + 1] * amps[2 * i + 1];
-        QwIoFlags h{};
-        QW_CUDA(sim, cudaMemcpyAsync(&h, flags, sizeof h, cudaMemcpyDeviceToHost, st));
+        static_assert(sizeof(QwIoFlags) <= 8 * (kFlatSort - kFlatIo), "flags of an import");
+        const QwIoFlags &h = *reinterpret_cast<const QwIoFlags *>(sim->h_flat + kFlatIo);
+        QW_CUDA(sim, cudaMemcpyAsync(sim->h_flat + kFlatIo, flags, sizeof h, cudaMemcpyDeviceToHost, st));
         QW_CUDA(sim, cudaStreamSynchronize(st));
         if (h.unsorted && !h.bad) { /* an exported list is sorted; any other is sorted here */
             void *tk = nullptr, *ta = nullptr, *work = nullptr;
@@ -2228,14 +2238,14 @@ extern "C" int qw_state_import(qw_sim *sim, int32_t key_words, const uint64_t *k
             QW_CUDA(sim, cudaMemsetAsync(flags, 0, sizeof(QwIoFlags), st));
             int in_tmp = 0;
             QW_CUDA(sim, qw_flat_sort(sim->d, K, static_cast<double2 *>(A), tk, static_cast<double2 *>(ta), count, 0,
-                                      QW_SORT_FULL, work, &flags->status, st, 2, &in_tmp));
+                                      QW_SORT_FULL, work, sim->h_flat + kFlatSort, &flags->status, st, 2, &in_tmp));
             if (in_tmp) {
                 std::swap(K, tk);
                 std::swap(A, ta);
             }
             QW_CUDA(sim, qw_io_order(sim->d, K, count, flags, st));
             sim->launches++;
-            QW_CUDA(sim, cudaMemcpyAsync(&h, flags, sizeof h, cudaMemcpyDeviceToHost, st));
+            QW_CUDA(sim, cudaMemcpyAsync(sim->h_flat + kFlatIo, flags, sizeof h, cudaMemcpyDeviceToHost, st));
             QW_CUDA(sim, cudaStreamSynchronize(st));
             if (h.status != 0 || h.unsorted)
                 return fail(sim, QW_ERR_DEVICE_STATUS, "qw_state_import: the sort of the keys gave up waiting for a tile's count");

@@ -655,10 +655,11 @@ __device__ unsigned long long tile_before(TileSum *ts, int64_t vb, unsigned int 
 }
 
 /* A block's share of it: n outputs of this thread, the number of those of the
-   threads before it in the block and all before the tile; the last tile writes the total. */
+   threads before it in the block and all before the tile; the last tile writes the
+   total, to the host's pinned memory too. */
 template <int THREADS>
 __device__ __forceinline__ unsigned long long tile_place(TileSum *ts, int64_t vb, int64_t ntiles, unsigned int n,
-                                                         int32_t *status)
+                                                         int32_t *status, unsigned long long *host)
 {
     constexpr int W = THREADS / 32;
     __shared__ unsigned int ws[W];
@@ -682,7 +683,7 @@ __device__ __forceinline__ unsigned long long tile_place(TileSum *ts, int64_t vb
         const unsigned long long b = tile_before(ts, vb, all, status);
         if (lane == 0) {
             base = b;
-            if (vb == ntiles - 1) ts->total = b + all;
+            if (vb == ntiles - 1) ts->total = *host = b + all;
         }
     }
     __syncthreads();
@@ -700,36 +701,43 @@ __device__ __forceinline__ int64_t tile_take(TileSum *ts)
 
 /* ---- radix sort ------------------------------------------------------------------ */
 
-/* OR and AND of every permuted key, word by word: the bits that differ
-   between keys.  The key array is read as a flat array of 64-bit words; the
+/* OR of every permuted key and of its complement, word by word: a bit set in
+   both differs between keys.  acc and *done zeroed by the caller; the last block
+   writes the result to the host's pinned memory.  The key array is read as a flat array of 64-bit words; the
    grid's stride is a multiple of NW, so each thread always sees one word
    index. */
 template <int ORDER, int NW>
-__global__ void k_f_orand(const uint64_t *words, int64_t nwords, int L, unsigned long long *acc)
+__global__ void k_f_orand(const uint64_t *words, int64_t nwords, int L, unsigned long long *acc, unsigned int *done,
+                          unsigned long long *host)
 {
-    __shared__ unsigned long long s_or[NW], s_and[NW];
-    if (threadIdx.x < NW) {
-        s_or[threadIdx.x] = 0ull;
-        s_and[threadIdx.x] = ~0ull;
-    }
+    __shared__ unsigned long long s_or[NW], s_nor[NW];
+    __shared__ bool last;
+    if (threadIdx.x < NW) s_or[threadIdx.x] = s_nor[threadIdx.x] = 0ull;
     __syncthreads();
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int wi = (int)(g % NW);
-    uint64_t ov = 0ull, av = ~0ull;
+    uint64_t ov = 0ull, nv = 0ull;
     for (int64_t q = g; q < nwords; q += stride) {
         uint64_t v = words[q];
         if (wi == 0) v = permuted0<ORDER>(v, L);
         ov |= v;
-        av &= v;
+        nv |= ~v;
     }
     atomicOr(&s_or[wi], (unsigned long long)ov);
-    atomicAnd(&s_and[wi], (unsigned long long)av);
+    atomicOr(&s_nor[wi], (unsigned long long)nv);
     __syncthreads();
     if (threadIdx.x < NW) {
         atomicOr(acc + threadIdx.x, s_or[threadIdx.x]);
-        atomicAnd(acc + NW + threadIdx.x, s_and[threadIdx.x]);
+        atomicOr(acc + NW + threadIdx.x, s_nor[threadIdx.x]);
+        __threadfence();
     }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (threadIdx.x < 2 * NW) host[threadIdx.x] = __ldcg(acc + threadIdx.x);
 }
 
 /* The sort runs on a compacted key (the chunks of qw_sort_chunks.h).  LSD
@@ -935,7 +943,7 @@ constexpr int RT_THREADS = 256;
 template <bool DAG, int NW>
 __global__ void __launch_bounds__(RT_THREADS) k_f_rot(QwSimDev d, const FKeyN<NW> *keys, const double2 *amps, int64_t M,
                                                       FKeyN<NW> *okeys, double2 *oamps, int64_t cap, TileSum *ts,
-                                                      int32_t *status)
+                                                      int32_t *status, unsigned long long *host)
 {
     const FLayout L = flayout(d.nb);
     const int64_t vb = tile_take(ts), i = vb * RT_THREADS + threadIdx.x;
@@ -968,7 +976,7 @@ __global__ void __launch_bounds__(RT_THREADS) k_f_rot(QwSimDev d, const FKeyN<NW
             k1 = keep(o1, d.tau2);
         }
     }
-    int64_t at = (int64_t)tile_place<RT_THREADS>(ts, vb, gridDim.x, (k0 ? 1u : 0u) + (k1 ? 1u : 0u), status);
+    int64_t at = (int64_t)tile_place<RT_THREADS>(ts, vb, gridDim.x, (k0 ? 1u : 0u) + (k1 ? 1u : 0u), status, host);
     if (k0 && at < cap) {
         k.w[0] &= ~1ull;
         okeys[at] = k;
@@ -987,7 +995,7 @@ __global__ void __launch_bounds__(RT_THREADS) k_f_rot(QwSimDev d, const FKeyN<NW
 constexpr int ST_THREADS = 256, ST_IPT = 8;
 template <int NW>
 __global__ void __launch_bounds__(ST_THREADS) k_f_starts(QwSimDev d, const FKeyN<NW> *keys, int64_t M, int64_t *starts,
-                                                         TileSum *ts, int32_t *status)
+                                                         TileSum *ts, int32_t *status, unsigned long long *host)
 {
     const int64_t vb = tile_take(ts), i0 = vb * (ST_THREADS * ST_IPT) + (threadIdx.x >> 5) * (32 * ST_IPT);
     const int lane = threadIdx.x & 31;
@@ -1002,7 +1010,7 @@ __global__ void __launch_bounds__(ST_THREADS) k_f_starts(QwSimDev d, const FKeyN
         n += __popc(heads[r]);
     }
     /* the warp's count on its first lane: every lane's place is its warp's */
-    unsigned long long at = tile_place<ST_THREADS>(ts, vb, gridDim.x, lane == 0 ? n : 0u, status);
+    unsigned long long at = tile_place<ST_THREADS>(ts, vb, gridDim.x, lane == 0 ? n : 0u, status, host);
     at = __shfl_sync(FULL, at, 0);
 #pragma unroll
     for (int r = 0; r < ST_IPT; ++r) {
@@ -1040,7 +1048,8 @@ template <int R> struct HgIters { static constexpr int n = R == 1 ? 4 : (R == 2 
 template <int NW, int FWHT_ROUNDS>
 __global__ void __launch_bounds__(32 * HG_WARPS) k_f_hgroups(QwSimDev d, const FKeyN<NW> *keys, const double2 *amps,
                                                              int64_t M, const int64_t *starts, int64_t G,
-                                                             FKeyN<NW> *okeys, double2 *oamps, int64_t cap, TileSum *ts, int32_t *status)
+                                                             FKeyN<NW> *okeys, double2 *oamps, int64_t cap, TileSum *ts, int32_t *status,
+                                                             unsigned long long *host)
 {
     const int s = d.s;
     const int sw = s < 32 ? s : 32, gpw = 32 / sw, rounds = s / sw;
@@ -1115,7 +1124,7 @@ __global__ void __launch_bounds__(32 * HG_WARPS) k_f_hgroups(QwSimDev d, const F
                 n += __popc(kept[it][q]);
             }
         }
-        unsigned long long at = tile_place<32 * HG_WARPS>(ts, vb, gridDim.x, lane == 0 ? n : 0u, status);
+        unsigned long long at = tile_place<32 * HG_WARPS>(ts, vb, gridDim.x, lane == 0 ? n : 0u, status, host);
         at = __shfl_sync(FULL, at, 0);
 #pragma unroll
         for (int it = 0; it < ITERS; ++it) {
@@ -1174,7 +1183,7 @@ __global__ void __launch_bounds__(32 * HG_WARPS) k_f_hgroups(QwSimDev d, const F
             run += (unsigned)__popc(bal);
         }
         if (pass == 0) {
-            at = tile_place<32 * HG_WARPS>(ts, vb, gridDim.x, lane == 0 ? run : 0u, status);
+            at = tile_place<32 * HG_WARPS>(ts, vb, gridDim.x, lane == 0 ? run : 0u, status, host);
             at = __shfl_sync(FULL, at, 0);
         }
     }
@@ -1391,7 +1400,7 @@ struct SortWork {
     size_t zero_bytes, total;
 };
 
-constexpr int SORT_MAXPASSES = 64 * NW_FAITH / 8;
+constexpr int SORT_MAXPASSES = 64 * NW_FAITH / 8; /* counters: one a pass, the last for k_f_orand */
 
 size_t align256(size_t b)
 {
@@ -1412,9 +1421,9 @@ SortWork sort_work(void *base, int64_t M)
     };
     w.stat = reinterpret_cast<uint64_t *>(take((size_t)nblk * 256 * 8));
     w.ghist = reinterpret_cast<uint32_t *>(take((size_t)NW_FAITH * CK_MAXPASS * 256 * 4));
-    w.ctr = reinterpret_cast<unsigned int *>(take((size_t)SORT_MAXPASSES * 4));
-    w.zero_bytes = off;
+    w.ctr = reinterpret_cast<unsigned int *>(take((size_t)(SORT_MAXPASSES + 1) * 4));
     w.acc = reinterpret_cast<unsigned long long *>(take(2 * NW_FAITH * 8));
+    w.zero_bytes = off;
     w.ck[0] = reinterpret_cast<uint64_t *>(take((size_t)n * 8));
     w.ck[1] = reinterpret_cast<uint64_t *>(take((size_t)n * 8));
     w.ix[0] = reinterpret_cast<uint32_t *>(take((size_t)n * 4));
@@ -1436,32 +1445,26 @@ SortWork sort_work(void *base, int64_t M)
  * all equal is already sorted (*in_tmp = 0). */
 template <int NW>
 cudaError_t flat_sort_t(const QwSimDev &d, void *keys, double2 *amps, void *tmpk, double2 *tmpa, int64_t M, int order,
-                        int group, void *work, int32_t *status, cudaStream_t st, int *in_tmp)
+                        int group, void *work, unsigned long long *h, int32_t *status, cudaStream_t st, int *in_tmp)
 {
     *in_tmp = 0;
     if (M <= 1) return cudaSuccess;
     if (M > (int64_t)UINT32_MAX) return cudaErrorInvalidValue; /* 32-bit positions */
     const int L = d.L;
     const SortWork w = sort_work(work, M);
-    unsigned long long init[2 * NW];
-    for (int t = 0; t < NW; ++t) {
-        init[t] = 0ull;
-        init[NW + t] = ~0ull;
-    }
-    cudaError_t e = cudaMemcpyAsync(w.acc, init, sizeof init, cudaMemcpyHostToDevice, st);
+    cudaError_t e = cudaMemsetAsync(w.stat, 0, w.zero_bytes, st);
     if (e != cudaSuccess) return e;
     const int othreads = 32 * NW;
     const int ogrid = grid_for(M * NW, othreads);
     const uint64_t *kwords = static_cast<const uint64_t *>(keys);
-    if (order == ORDER_R) k_f_orand<ORDER_R, NW><<<ogrid, othreads, 0, st>>>(kwords, M * NW, L, w.acc);
-    else k_f_orand<ORDER_H, NW><<<ogrid, othreads, 0, st>>>(kwords, M * NW, L, w.acc);
-    if ((e = cudaMemsetAsync(w.stat, 0, w.zero_bytes, st)) != cudaSuccess) return e;
-    unsigned long long h[2 * NW];
-    if ((e = cudaMemcpyAsync(h, w.acc, sizeof h, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
+    unsigned int *done = w.ctr + SORT_MAXPASSES;
+    if (order == ORDER_R) k_f_orand<ORDER_R, NW><<<ogrid, othreads, 0, st>>>(kwords, M * NW, L, w.acc, done, h);
+    else k_f_orand<ORDER_H, NW><<<ogrid, othreads, 0, st>>>(kwords, M * NW, L, w.acc, done, h);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
     /* the varying bits as runs, split into chunks of 64 */
     uint64_t var[NW];
-    for (int wi = 0; wi < NW; ++wi) var[wi] = h[wi] ^ h[NW + wi];
+    for (int wi = 0; wi < NW; ++wi) var[wi] = h[wi] & h[NW + wi];
     if (group != QW_SORT_FULL) {
         if (order == ORDER_R) var[0] &= ~1ull;
         else if (d.s <= 128) var[0] &= ~((1ull << L) - 1ull);
@@ -1520,11 +1523,12 @@ size_t qw_flat_sort_bytes(int64_t M)
 }
 
 cudaError_t qw_flat_sort(const QwSimDev &d, void *keys, double2 *amps, void *tmpk, double2 *tmpa, int64_t M,
-                         int order, int group, void *work, int32_t *status, cudaStream_t st, int kw, int *in_tmp)
+                         int order, int group, void *work, unsigned long long *host, int32_t *status, cudaStream_t st,
+                         int kw, int *in_tmp)
 {
     if (kw == NW_FAITH)
-        return flat_sort_t<NW_FAITH>(d, keys, amps, tmpk, tmpa, M, order, group, work, status, st, in_tmp);
-    return flat_sort_t<2>(d, keys, amps, tmpk, tmpa, M, order, group, work, status, st, in_tmp);
+        return flat_sort_t<NW_FAITH>(d, keys, amps, tmpk, tmpa, M, order, group, work, host, status, st, in_tmp);
+    return flat_sort_t<2>(d, keys, amps, tmpk, tmpa, M, order, group, work, host, status, st, in_tmp);
 }
 
 /* The single-pass kernels' tile sums, zeroed: tiles of `per` inputs */
@@ -1541,14 +1545,9 @@ cudaError_t tiles_clear(void *ts, int64_t ntiles, cudaStream_t st)
 }
 } // namespace
 
-/* where the number of outputs is found */
-const unsigned long long *qw_flat_tiles_total(const void *ts)
-{
-    return &static_cast<const TileSum *>(ts)->total;
-}
-
 cudaError_t qw_flat_rot(const QwSimDev &d, int op, const void *keys, const double2 *amps, int64_t M, void *okeys,
-                        double2 *oamps, int64_t cap, void *tiles, int32_t *status, cudaStream_t st, int kw)
+                        double2 *oamps, int64_t cap, void *tiles, unsigned long long *host, int32_t *status,
+                        cudaStream_t st, int kw)
 {
     if (M <= 0) return cudaSuccess;
     const int64_t nt = (M + RT_THREADS - 1) / RT_THREADS;
@@ -1559,19 +1558,19 @@ cudaError_t qw_flat_rot(const QwSimDev &d, int op, const void *keys, const doubl
     if (kw == NW_FAITH) {
         const FKeyW *k = static_cast<const FKeyW *>(keys);
         FKeyW *ok = static_cast<FKeyW *>(okeys);
-        if (op == 0) k_f_rot<true, NW_FAITH><<<grid, RT_THREADS, 0, st>>>(d, k, amps, M, ok, oamps, cap, ts, status);
-        else k_f_rot<false, NW_FAITH><<<grid, RT_THREADS, 0, st>>>(d, k, amps, M, ok, oamps, cap, ts, status);
+        if (op == 0) k_f_rot<true, NW_FAITH><<<grid, RT_THREADS, 0, st>>>(d, k, amps, M, ok, oamps, cap, ts, status, host);
+        else k_f_rot<false, NW_FAITH><<<grid, RT_THREADS, 0, st>>>(d, k, amps, M, ok, oamps, cap, ts, status, host);
     } else {
         const FKey *k = static_cast<const FKey *>(keys);
         FKey *ok = static_cast<FKey *>(okeys);
-        if (op == 0) k_f_rot<true, 2><<<grid, RT_THREADS, 0, st>>>(d, k, amps, M, ok, oamps, cap, ts, status);
-        else k_f_rot<false, 2><<<grid, RT_THREADS, 0, st>>>(d, k, amps, M, ok, oamps, cap, ts, status);
+        if (op == 0) k_f_rot<true, 2><<<grid, RT_THREADS, 0, st>>>(d, k, amps, M, ok, oamps, cap, ts, status, host);
+        else k_f_rot<false, 2><<<grid, RT_THREADS, 0, st>>>(d, k, amps, M, ok, oamps, cap, ts, status, host);
     }
     return cudaGetLastError();
 }
 
 cudaError_t qw_flat_starts(const QwSimDev &d, const void *keys, int64_t M, int64_t *starts, void *tiles,
-                           int32_t *status, cudaStream_t st, int kw)
+                           unsigned long long *host, int32_t *status, cudaStream_t st, int kw)
 {
     if (M <= 0) return cudaSuccess;
     const int64_t nt = (M + ST_THREADS * ST_IPT - 1) / (ST_THREADS * ST_IPT);
@@ -1580,22 +1579,22 @@ cudaError_t qw_flat_starts(const QwSimDev &d, const void *keys, int64_t M, int64
     TileSum *ts = static_cast<TileSum *>(tiles);
     const unsigned grid = (unsigned)nt;
     if (kw == NW_FAITH)
-        k_f_starts<NW_FAITH><<<grid, ST_THREADS, 0, st>>>(d, static_cast<const FKeyW *>(keys), M, starts, ts, status);
-    else k_f_starts<2><<<grid, ST_THREADS, 0, st>>>(d, static_cast<const FKey *>(keys), M, starts, ts, status);
+        k_f_starts<NW_FAITH><<<grid, ST_THREADS, 0, st>>>(d, static_cast<const FKeyW *>(keys), M, starts, ts, status, host);
+    else k_f_starts<2><<<grid, ST_THREADS, 0, st>>>(d, static_cast<const FKey *>(keys), M, starts, ts, status, host);
     return cudaGetLastError();
 }
 
 namespace {
 template <int NW, int R>
 cudaError_t launch_hgroups(const QwSimDev &d, const void *keys, const double2 *amps, int64_t M, const int64_t *starts,
-                           int64_t G, void *okeys, double2 *oamps, int64_t cap, void *tiles, int32_t *status, cudaStream_t st)
+                           int64_t G, void *okeys, double2 *oamps, int64_t cap, void *tiles, unsigned long long *host, int32_t *status, cudaStream_t st)
 {
     const int64_t per = (int64_t)HG_WARPS * HgIters<R>::n * (d.s < 32 ? 32 / d.s : 1), nt = (G + per - 1) / per;
     const cudaError_t e = tiles_clear(tiles, nt, st);
     if (e != cudaSuccess) return e;
     k_f_hgroups<NW, R><<<(unsigned)nt, 32 * HG_WARPS, 0, st>>>(d, static_cast<const FKeyN<NW> *>(keys), amps, M, starts, G,
                                                              static_cast<FKeyN<NW> *>(okeys), oamps, cap,
-                                                             static_cast<TileSum *>(tiles), status);
+                                                             static_cast<TileSum *>(tiles), status, host);
     return cudaGetLastError();
 }
 
@@ -1603,23 +1602,23 @@ cudaError_t launch_hgroups(const QwSimDev &d, const void *keys, const double2 *a
    0: the direct sums (s > 128) */
 template <int NW>
 cudaError_t launch_hgroups_s(const QwSimDev &d, const void *keys, const double2 *amps, int64_t M, const int64_t *starts, int64_t G,
-                             void *okeys, double2 *oamps, int64_t cap, void *tiles, int32_t *status, cudaStream_t st)
+                             void *okeys, double2 *oamps, int64_t cap, void *tiles, unsigned long long *host, int32_t *status, cudaStream_t st)
 {
-    if (d.s <= 32) return launch_hgroups<NW, 1>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, status, st);
-    if (d.s == 64) return launch_hgroups<NW, 2>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, status, st);
-    if (d.s == 128) return launch_hgroups<NW, 4>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, status, st);
-    return launch_hgroups<NW, 0>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, status, st);
+    if (d.s <= 32) return launch_hgroups<NW, 1>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, host, status, st);
+    if (d.s == 64) return launch_hgroups<NW, 2>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, host, status, st);
+    if (d.s == 128) return launch_hgroups<NW, 4>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, host, status, st);
+    return launch_hgroups<NW, 0>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, host, status, st);
 }
 } // namespace
 
 cudaError_t qw_flat_hgroups(const QwSimDev &d, const void *keys, const double2 *amps, int64_t M, const int64_t *starts, int64_t G,
-                            void *okeys, double2 *oamps, int64_t cap, void *tiles, int32_t *status, cudaStream_t st,
-                            int kw)
+                            void *okeys, double2 *oamps, int64_t cap, void *tiles, unsigned long long *host,
+                            int32_t *status, cudaStream_t st, int kw)
 {
     if (G <= 0) return cudaSuccess;
     if (kw == NW_FAITH)
-        return launch_hgroups_s<NW_FAITH>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, status, st);
-    return launch_hgroups_s<2>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, status, st);
+        return launch_hgroups_s<NW_FAITH>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, host, status, st);
+    return launch_hgroups_s<2>(d, keys, amps, M, starts, G, okeys, oamps, cap, tiles, host, status, st);
 }
 
 cudaError_t qw_flat_readout(const QwSimDev &d, const void *keys, const double2 *amps, int64_t M, const QwStepArgs &a,

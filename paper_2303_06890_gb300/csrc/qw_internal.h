@@ -290,29 +290,31 @@ cudaError_t qw_flat_map(const QwSimDev &d, void *keys, int64_t M, uint32_t ops, 
                         int kw);
 cudaError_t qw_flat_phase(const QwSimDev &d, const void *keys, double2 *amps, int64_t M, cudaStream_t st, int kw);
 /* stable sort by the permuted key (order 0: R, 1: H); work holds
-   qw_flat_sort_bytes(M); the result is left in tmpk / tmpa when *in_tmp */
+   qw_flat_sort_bytes(M); host: 2 kw words of pinned memory for which bits vary
+   (synchronises to read them); the result is left in tmpk / tmpa when *in_tmp */
 size_t qw_flat_sort_bytes(int64_t M);
 #define QW_SORT_FULL 0       /* by every register */
 #define QW_SORT_GROUP 1      /* the target's bits left out: groups contiguous */
 #define QW_SORT_GROUP_NO_A 2 /* A's too: it follows from the other idle registers */
 cudaError_t qw_flat_sort(const QwSimDev &d, void *keys, double2 *amps, void *tmpk, double2 *tmpa, int64_t M,
-                         int order, int group, void *work, int32_t *status, cudaStream_t st, int kw, int *in_tmp);
-/* Scratch of a single-pass kernel over n entries or groups, and where it
-   leaves the number of its outputs. */
+                         int order, int group, void *work, unsigned long long *host, int32_t *status, cudaStream_t st,
+                         int kw, int *in_tmp);
+/* Scratch of a single-pass kernel over n entries or groups; it leaves the number
+   of its outputs in *host (pinned). */
 size_t qw_flat_tiles_bytes(int64_t n);
-const unsigned long long *qw_flat_tiles_total(const void *tiles);
 /* op 0 (R^dag) and 1 (R) on the sorted list: the kept outputs (up to 2 M; cap
    is the room in okeys / oamps) */
 cudaError_t qw_flat_rot(const QwSimDev &d, int op, const void *keys, const double2 *amps, int64_t M, void *okeys,
-                        double2 *oamps, int64_t cap, void *tiles, int32_t *status, cudaStream_t st, int kw);
+                        double2 *oamps, int64_t cap, void *tiles, unsigned long long *host, int32_t *status,
+                        cudaStream_t st, int kw);
 /* the Hadamard stage's groups: the first member of each (their number G is the
    kernel's total), starts[G] = M; starts has room for M + 1 */
 cudaError_t qw_flat_starts(const QwSimDev &d, const void *keys, int64_t M, int64_t *starts, void *tiles,
-                           int32_t *status, cudaStream_t st, int kw);
+                           unsigned long long *host, int32_t *status, cudaStream_t st, int kw);
 /* H on the G groups: the kept outputs (up to G s) */
 cudaError_t qw_flat_hgroups(const QwSimDev &d, const void *keys, const double2 *amps, int64_t M, const int64_t *starts, int64_t G,
-                            void *okeys, double2 *oamps, int64_t cap, void *tiles, int32_t *status, cudaStream_t st,
-                            int kw);
+                            void *okeys, double2 *oamps, int64_t cap, void *tiles, unsigned long long *host,
+                            int32_t *status, cudaStream_t st, int kw);
 cudaError_t qw_flat_readout(const QwSimDev &d, const void *keys, const double2 *amps, int64_t M, const QwStepArgs &a,
                             cudaStream_t st, int kw);
 cudaError_t qw_flat_scatter(const QwSimDev &d, const QwBufDev &out, int fp32, const void *keys, const double2 *amps,
