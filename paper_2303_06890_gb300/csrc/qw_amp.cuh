@@ -154,6 +154,7 @@ template <> struct Amp<double2> {
     __device__ static float rot_f(RotVal t) { return approx(t.x); }
     __device__ static float rot_g(RotVal t) { return approx(t.y); }
     __device__ static void scale_one_plus(float c, double *buf) { buf[0] = 1.0 + (double)c; }
+    __device__ static Scale scale_near_one(float c) { return Scale(1.0 + (double)c); }
     static constexpr float kApproxErr = 1.0f / 131072.0f; /* 2^-17 of the terms' magnitudes */
 };
 
@@ -405,6 +406,7 @@ template <> struct Amp<float2> {
         f[0] = 1.0f;
         f[1] = c;
     }
+    __device__ static Scale scale_near_one(float c) { return Scale(1.0f, c); }
     static constexpr float kApproxErr = 1.0f / 524288.0f; /* 2^-19 of the terms' magnitudes */
 };
 

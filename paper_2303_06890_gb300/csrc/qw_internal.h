@@ -176,6 +176,8 @@ struct QwPosPlan {
     int tab;         /* the matrix's tables fit shared memory */
     int coop;        /* the device takes cooperative launches */
     size_t smem;
+    int cl, cl_warps; /* runs go to one cluster of cl blocks (0: to the grid) */
+    size_t cl_smem;
 };
 
 /* launchers (qw_kernels.cu); all return cudaGetLastError() of the launch */

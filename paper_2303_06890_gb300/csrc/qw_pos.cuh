@@ -259,6 +259,136 @@ struct PosStats {
     }
 };
 
+/* The walk operator on a group's slots (both rows' pairs of each): the lane's
+ * SPL slots, rotations rv and flags dst (bit 31 sigma = -1, bit 30 a negative
+ * element) in, on_sum(the group sum, scaled by 2 / s) for the read-out, on_out(q,
+ * the entry that slot q sends to its destination). */
+template <typename AmpT, int S, bool FULLST, int SPL, typename OnSum, typename OnOut>
+__device__ __forceinline__ void pos_group(const QwSimDev &d, const typename Amp<AmpT>::RotVal (&rv)[SPL],
+                                          const uint32_t (&dst)[SPL], const Entry<AmpT> (&in)[SPL], bool rescale,
+                                          const typename Amp<AmpT>::Scale &scale, bool valid, bool renorm,
+                                          typename Amp<AmpT>::Norm &nrm, uint32_t &cnt, PosStats &st, OnSum on_sum,
+                                          OnOut on_out)
+{
+    constexpr int SW = S > 32 ? 32 : S;
+    constexpr int LOG2S = S == 4 ? 2 : S == 8 ? 3 : S == 16 ? 4 : S == 32 ? 5 : 6;
+    constexpr float kHalfS = 0.5f * S, kErr = Amp<AmpT>::kApproxErr;
+    const AmpT zero = Amp<AmpT>::zero();
+    const int lane = threadIdx.x & 31, ul = lane / SW, lb = lane % SW;
+                AmpT a0[SPL], a1[SPL], q0[SPL], q1[SPL];
+                float A0[SPL], A1[SPL], Q0[SPL];
+                bool any = false;
+    #pragma unroll
+                for (int q = 0; q < SPL; ++q) {
+                    a0[q] = in[q].a0;
+                    a1[q] = in[q].a1;
+                    q0[q] = in[q].b0;
+                    q1[q] = FULLST ? in[q].b1 : zero;
+                    if (rescale) {
+                        a0[q] = scale.apply(a0[q]);
+                        a1[q] = scale.apply(a1[q]);
+                        q0[q] = scale.apply(q0[q]);
+                        if (FULLST) q1[q] = scale.apply(q1[q]);
+                    }
+                    A0[q] = Amp<AmpT>::inf_norm(a0[q]);
+                    A1[q] = Amp<AmpT>::inf_norm(a1[q]);
+                    Q0[q] = Amp<AmpT>::inf_norm(q0[q]);
+                    const bool n0 = A0[q] != 0.0f, n1 = A1[q] != 0.0f, m0 = Q0[q] != 0.0f, m1 = FULLST && nz(q1[q]) != 0u;
+                    if (n0) cnt += kCntIn;
+                    if (n1) cnt += kCntIn;
+                    if (m0) cnt += kCntIn;
+                    if (m1) cnt += kCntIn;
+                    any = any || n0 || n1 || m0 || m1;
+                }
+                {
+                    const unsigned m = __ballot_sync(FULL, any);
+                    const unsigned um = SW == 32 ? m : (m >> (ul * SW)) & ((1u << (SW & 31)) - 1u);
+                    if (lb == 0 && um != 0) st.rows += 1; /* units holding branches */
+                }
+                /* b1 = 0: R^dag's b2 = 0 output u (its exact value, scaled by 2 / s),
+                   and whether u and v are kept: |v| >= | f |a1| - g |a0| | in the
+                   maximum norm, which the phases leave alone, so the norms decide
+                   unless they nearly cancel */
+                typename Amp<AmpT>::Wide u[SPL];
+                PairState<AmpT> ps[SPL];
+                float f[SPL], g_[SPL], U[SPL];
+    #pragma unroll
+                for (int q = 0; q < SPL; ++q) {
+                    const uint32_t sgn = (dst[q] & 0x40000000u) >> 15; /* the value's sign bit (bit 15) */
+                    const bool sneg = (dst[q] >> 31) != 0u;
+                    f[q] = Amp<AmpT>::rot_f(rv[q]);
+                    g_[q] = Amp<AmpT>::rot_g(rv[q]);
+                    u[q] = Amp<AmpT>::rdag0(Amp<AmpT>::prescale(rv[q], LOG2S - 1), sgn, sneg, a0[q], a1[q]);
+                    U[q] = kHalfS * Amp<AmpT>::inf_norm(Amp<AmpT>::narrow(u[q]));
+                    const float fa = f[q] * A1[q], ga = g_[q] * A0[q];
+                    ps[q].c0 = U[q] > d.thr32;
+                    ps[q].c1 = fabsf(fa - ga) > fmaf(kErr, fa + ga, d.thr32);
+                    ps[q].lossy = false;
+                    if ((!ps[q].c0 && U[q] > 0.0f) || (!ps[q].c1 && fa + ga > 0.0f)) {
+                        const unsigned e = pair_exact<AmpT>(d, rv[q], sgn, sneg, a0[q], a1[q]);
+                        ps[q].c0 = (e & 1u) != 0u;
+                        ps[q].c1 = (e & 2u) != 0u;
+                        ps[q].lossy = (e & 4u) != 0u;
+                        if (!ps[q].c0) {
+                            u[q] = Amp<AmpT>::wide_zero();
+                            U[q] = 0.0f;
+                        }
+                    }
+                    if (ps[q].c0) cnt += kCntRdag;
+                    if (ps[q].c1) cnt += kCntRdag + kCntHph;
+                }
+                __syncwarp();
+                typename Amp<AmpT>::Sum sum;
+                sum.set(u[0]);
+    #pragma unroll
+                for (int q = 1; q < SPL; ++q) sum.add(u[q]);
+                sum.reduce(SW, SW);
+                on_sum(sum);
+                const float Rn = Amp<AmpT>::inf_norm(Amp<AmpT>::sum_amp(sum));
+    #pragma unroll
+                for (int q = 0; q < SPL; ++q) {
+                    const uint32_t sgn = (dst[q] & 0x40000000u) >> 15;
+                    const bool sneg = (dst[q] >> 31) != 0u;
+                    /* the reflected r - u, then R: (f r - a0, g r - a1) */
+                    AmpT rA0, rA1;
+                    bool d0 = fabsf(Rn - U[q]) > fmaf(kErr, Rn + U[q], d.thr32);
+                    Amp<AmpT>::reflect(sum, rv[q], sgn, sneg, a0[q], a1[q], rA0, rA1);
+                    if (ps[q].lossy || (!d0 && Rn + U[q] > 0.0f))
+                        d0 = pair_reflect_exact<AmpT>(d, sum, rv[q], sgn, sneg, a0[q], a1[q], ps[q], rA0, rA1);
+                    if (d0) cnt += kCntHph;
+                    /* b1 = 1: R^dag, -1, R */
+                    AmpT rB0 = Amp<AmpT>::neg(q0[q]), rB1 = Amp<AmpT>::neg(q1[q]);
+                    if (FULLST) {
+                        const unsigned kept = pair_negate<AmpT>(d, rv[q], sgn, sneg, q0[q], q1[q], rB0, rB1);
+                        cnt += kept * (kCntRdag + kCntHph);
+                    } else { /* q1 = 0: |u| = f |q0|, |v| = g |q0| */
+                        const float fq = f[q] * Q0[q], gq = g_[q] * Q0[q], lim = fmaf(kErr, Q0[q], d.thr32);
+                        const bool c0 = fq > lim, c1 = gq > lim;
+                        unsigned kept = (c0 ? 1u : 0u) + (c1 ? 1u : 0u);
+                        if ((!c0 && fq > 0.0f) || (!c1 && gq > 0.0f))
+                            negate_exact<AmpT>(d, rv[q], sgn, sneg, q0[q], zero, rB0, rB1, kept);
+                        cnt += kept * (kCntRdag + kCntHph);
+                    }
+                    const bool eA0 = pos_keep(d, rA0), eA1 = pos_keep(d, rA1);
+                    const bool eB0 = pos_keep(d, rB0), eB1 = FULLST && pos_keep(d, rB1);
+                    if (valid) {
+                        if (renorm) {
+                            if (eA0) norm_add(nrm, rA0);
+                            if (eB0) norm_add(nrm, rB0);
+                            if (eA1) norm_add(nrm, rA1);
+                            if (FULLST && eB1) norm_add(nrm, rB1);
+                        }
+                        /* S: (k, b2) <-> (j, b1) */
+                        const Entry<AmpT> o = {eA0 ? rA0 : zero, eB0 ? rB0 : zero, eA1 ? rA1 : zero, eB1 ? rB1 : zero};
+                        on_out(q, o);
+                    }
+                    if (eA0) cnt += kCntOut;
+                    if (eB0) cnt += kCntOut;
+                    if (eA1) cnt += kCntOut;
+                    if (eB1) cnt += kCntOut;
+                }
+}
+
 template <typename AmpT, int S, bool FULLST, bool TAB>
 __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, QwPosArgs p, QwStepArgs a)
 {
@@ -266,8 +396,6 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
     /* a unit (one j) on SW lanes, each lane holding SPL of its slots (l = lb
        + 32 k); RPP units per warp (a group) */
     constexpr int SW = S > 32 ? 32 : S, SPL = S / SW, RPP = 32 / SW;
-    constexpr int LOG2S = S == 4 ? 2 : S == 8 ? 3 : S == 16 ? 4 : S == 32 ? 5 : 6;
-    constexpr float kHalfS = 0.5f * S, kErr = Amp<AmpT>::kApproxErr;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long part_u[kPosMaxWarps];
     __shared__ double part_d[kPosMaxWarps];
@@ -372,121 +500,15 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
                     if (valid) slot_table(j * S + lb + 32 * q, rv[q], dst[q]);
                 }
             }
-            AmpT a0[SPL], a1[SPL], q0[SPL], q1[SPL];
-            float A0[SPL], A1[SPL], Q0[SPL];
-            bool any = false;
-#pragma unroll
-            for (int q = 0; q < SPL; ++q) {
-                a0[q] = cur.e[q].a0;
-                a1[q] = cur.e[q].a1;
-                q0[q] = cur.e[q].b0;
-                q1[q] = FULLST ? cur.e[q].b1 : zero;
-                if (rescale) {
-                    a0[q] = scale.apply(a0[q]);
-                    a1[q] = scale.apply(a1[q]);
-                    q0[q] = scale.apply(q0[q]);
-                    if (FULLST) q1[q] = scale.apply(q1[q]);
-                }
-                A0[q] = Amp<AmpT>::inf_norm(a0[q]);
-                A1[q] = Amp<AmpT>::inf_norm(a1[q]);
-                Q0[q] = Amp<AmpT>::inf_norm(q0[q]);
-                const bool n0 = A0[q] != 0.0f, n1 = A1[q] != 0.0f, m0 = Q0[q] != 0.0f, m1 = FULLST && nz(q1[q]) != 0u;
-                if (n0) cnt += kCntIn;
-                if (n1) cnt += kCntIn;
-                if (m0) cnt += kCntIn;
-                if (m1) cnt += kCntIn;
-                any = any || n0 || n1 || m0 || m1;
-            }
-            {
-                const unsigned m = __ballot_sync(FULL, any);
-                const unsigned um = SW == 32 ? m : (m >> (ul * SW)) & ((1u << (SW & 31)) - 1u);
-                if (lb == 0 && um != 0) st.rows += 1; /* units holding branches */
-            }
-            /* b1 = 0: R^dag's b2 = 0 output u (its exact value, scaled by 2 / s),
-               and whether u and v are kept: |v| >= | f |a1| - g |a0| | in the
-               maximum norm, which the phases leave alone, so the norms decide
-               unless they nearly cancel */
-            typename Amp<AmpT>::Wide u[SPL];
-            PairState<AmpT> ps[SPL];
-            float f[SPL], g_[SPL], U[SPL];
-#pragma unroll
-            for (int q = 0; q < SPL; ++q) {
-                const uint32_t sgn = (dst[q] & 0x40000000u) >> 15; /* the value's sign bit (bit 15) */
-                const bool sneg = (dst[q] >> 31) != 0u;
-                f[q] = Amp<AmpT>::rot_f(rv[q]);
-                g_[q] = Amp<AmpT>::rot_g(rv[q]);
-                u[q] = Amp<AmpT>::rdag0(Amp<AmpT>::prescale(rv[q], LOG2S - 1), sgn, sneg, a0[q], a1[q]);
-                U[q] = kHalfS * Amp<AmpT>::inf_norm(Amp<AmpT>::narrow(u[q]));
-                const float fa = f[q] * A1[q], ga = g_[q] * A0[q];
-                ps[q].c0 = U[q] > d.thr32;
-                ps[q].c1 = fabsf(fa - ga) > fmaf(kErr, fa + ga, d.thr32);
-                ps[q].lossy = false;
-                if ((!ps[q].c0 && U[q] > 0.0f) || (!ps[q].c1 && fa + ga > 0.0f)) {
-                    const unsigned e = pair_exact<AmpT>(d, rv[q], sgn, sneg, a0[q], a1[q]);
-                    ps[q].c0 = (e & 1u) != 0u;
-                    ps[q].c1 = (e & 2u) != 0u;
-                    ps[q].lossy = (e & 4u) != 0u;
-                    if (!ps[q].c0) {
-                        u[q] = Amp<AmpT>::wide_zero();
-                        U[q] = 0.0f;
+            pos_group<AmpT, S, FULLST>(
+                d, rv, dst, cur.e, rescale, scale, valid, a.renorm != 0, nrm, cnt, st,
+                [&](const typename Amp<AmpT>::Sum &sum) {
+                    if (readout && valid && lb == 0) { /* flag-0 amplitude (1/sqrt s) sum u: the QLS accumulator */
+                        const double2 sv = sum.value();
+                        pshare += pos_readout(a.qls_y + j, unit, sv.x, sv.y);
                     }
-                }
-                if (ps[q].c0) cnt += kCntRdag;
-                if (ps[q].c1) cnt += kCntRdag + kCntHph;
-            }
-            __syncwarp();
-            typename Amp<AmpT>::Sum sum;
-            sum.set(u[0]);
-#pragma unroll
-            for (int q = 1; q < SPL; ++q) sum.add(u[q]);
-            sum.reduce(SW, SW);
-            if (readout && valid && lb == 0) { /* flag-0 amplitude (1/sqrt s) sum u: the QLS accumulator */
-                const double2 sv = sum.value();
-                pshare += pos_readout(a.qls_y + j, unit, sv.x, sv.y);
-            }
-            const float Rn = Amp<AmpT>::inf_norm(Amp<AmpT>::sum_amp(sum));
-#pragma unroll
-            for (int q = 0; q < SPL; ++q) {
-                const uint32_t sgn = (dst[q] & 0x40000000u) >> 15, to = dst[q] & 0x3fffffffu;
-                const bool sneg = (dst[q] >> 31) != 0u;
-                /* the reflected r - u, then R: (f r - a0, g r - a1) */
-                AmpT rA0, rA1;
-                bool d0 = fabsf(Rn - U[q]) > fmaf(kErr, Rn + U[q], d.thr32);
-                Amp<AmpT>::reflect(sum, rv[q], sgn, sneg, a0[q], a1[q], rA0, rA1);
-                if (ps[q].lossy || (!d0 && Rn + U[q] > 0.0f))
-                    d0 = pair_reflect_exact<AmpT>(d, sum, rv[q], sgn, sneg, a0[q], a1[q], ps[q], rA0, rA1);
-                if (d0) cnt += kCntHph;
-                /* b1 = 1: R^dag, -1, R */
-                AmpT rB0 = Amp<AmpT>::neg(q0[q]), rB1 = Amp<AmpT>::neg(q1[q]);
-                if (FULLST) {
-                    const unsigned kept = pair_negate<AmpT>(d, rv[q], sgn, sneg, q0[q], q1[q], rB0, rB1);
-                    cnt += kept * (kCntRdag + kCntHph);
-                } else { /* q1 = 0: |u| = f |q0|, |v| = g |q0| */
-                    const float fq = f[q] * Q0[q], gq = g_[q] * Q0[q], lim = fmaf(kErr, Q0[q], d.thr32);
-                    const bool c0 = fq > lim, c1 = gq > lim;
-                    unsigned kept = (c0 ? 1u : 0u) + (c1 ? 1u : 0u);
-                    if ((!c0 && fq > 0.0f) || (!c1 && gq > 0.0f))
-                        negate_exact<AmpT>(d, rv[q], sgn, sneg, q0[q], zero, rB0, rB1, kept);
-                    cnt += kept * (kCntRdag + kCntHph);
-                }
-                const bool eA0 = pos_keep(d, rA0), eA1 = pos_keep(d, rA1);
-                const bool eB0 = pos_keep(d, rB0), eB1 = FULLST && pos_keep(d, rB1);
-                if (valid) {
-                    if (a.renorm) {
-                        if (eA0) norm_add(nrm, rA0);
-                        if (eB0) norm_add(nrm, rB0);
-                        if (eA1) norm_add(nrm, rA1);
-                        if (FULLST && eB1) norm_add(nrm, rB1);
-                    }
-                    /* S: (k, b2) <-> (j, b1) */
-                    const Entry<AmpT> o = {eA0 ? rA0 : zero, eB0 ? rB0 : zero, eA1 ? rA1 : zero, eB1 ? rB1 : zero};
-                    PosMem<AmpT>::template store<FULLST>(O, T, to, o);
-                }
-                if (eA0) cnt += kCntOut;
-                if (eB0) cnt += kCntOut;
-                if (eA1) cnt += kCntOut;
-                if (eB1) cnt += kCntOut;
-            }
+                },
+                [&](int q, const Entry<AmpT> &o) { PosMem<AmpT>::template store<FULLST>(O, T, dst[q] & 0x3fffffffu, o); });
             if ((k & 7u) == 7u) st.take(cnt);
         }
         st.take(cnt);
@@ -636,6 +658,348 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
             }
             *a.done_ctr = 0u;
         }
+    }
+}
+
+/* ==== small states: several steps on one cluster, the state in shared memory ==== */
+/*
+ * A step of a small state is a chain of latencies, and over the grid most of it is
+ * L2: the state's load and store, the norm's atomic, the barrier word's polls --
+ * 3.5 us at N = 1000, whatever the arithmetic.  Up to a few hundred groups the
+ * blocks of one cluster hold the state instead, each its own warps' entries in
+ * shared memory (two buffers); S writes to the destination block's shared
+ * memory, each warp adds its share of the norm to all blocks' sums there, and the
+ * cluster's hardware barrier ends the step.  The QLS accumulator Y stays in
+ * shared memory too.  200 steps with T~ and two marginals, grid -> cluster: N = 256, s = 8
+ * complex128 776 -> 479 us, complex64 702 -> 492; N = 700 768 -> 634, 694 -> 539.  What
+ * is left is still latency: the arithmetic's chain and the barrier, 2.1 us a step at
+ * 64 groups, whatever the number of blocks they are on.
+ *
+ * Entry (k, warp, q, lane) of a block -- the order in which its lanes use them --
+ * is number ((k warps + warp) SPL + q) 32 + lane of its buffers, extras behind the
+ * slots; a destination is its block (bits 20 .. 23) and that
+ * index (bits 0 .. 19), with the flags of k_walk_pos above.  A buffer written in step
+ * t was last read in step t - 1, before the barrier that every block passed to
+ * start t; sums take turns three by three, cleared two steps ahead.
+ */
+constexpr int kPosCluster = 16; /* blocks of a cluster, at most (more than 8: opt-in) */
+
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t peer_addr(uint32_t a, uint32_t rank)
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void peer_store(uint32_t a, float2 v)
+{
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void peer_store(uint32_t a, double2 v)
+{
+    asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(v.x), "d"(v.y) : "memory");
+}
+__device__ __forceinline__ void peer_store_pair(uint32_t a, float2 u, float2 v)
+{
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(u.x), "f"(u.y), "f"(v.x), "f"(v.y)
+                 : "memory");
+}
+__device__ __forceinline__ void peer_store(uint32_t a, double v)
+{
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void peer_store(uint32_t a, uint32_t v)
+{
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void peer_add(uint32_t a, unsigned long long v)
+{
+    asm volatile("red.relaxed.cluster.shared::cluster.add.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+/* One buffer of E entries in shared memory.  complex64: (A0, A1) one 16-byte
+   access, B0 behind; complex128: three planes (16-byte accesses either way). */
+template <typename AmpT> struct ClusterBuf;
+template <> struct ClusterBuf<float2> {
+    static constexpr int kBytes = 24;
+    __device__ static void load(const unsigned char *b, uint32_t E, uint32_t at, Entry<float2> &e)
+    {
+        const float4 v = reinterpret_cast<const float4 *>(b)[at];
+        e.a0 = make_float2(v.x, v.y);
+        e.a1 = make_float2(v.z, v.w);
+        e.b0 = reinterpret_cast<const float2 *>(b + 16 * (size_t)E)[at];
+        e.b1 = make_float2(0.0f, 0.0f);
+    }
+    __device__ static void store(unsigned char *b, uint32_t E, uint32_t at, const Entry<float2> &e)
+    {
+        reinterpret_cast<float4 *>(b)[at] = make_float4(e.a0.x, e.a0.y, e.a1.x, e.a1.y);
+        reinterpret_cast<float2 *>(b + 16 * (size_t)E)[at] = e.b0;
+    }
+    __device__ static void send(uint32_t b, uint32_t E, uint32_t at, const Entry<float2> &e)
+    {
+        peer_store_pair(b + 16u * at, e.a0, e.a1);
+        peer_store(b + 16u * E + 8u * at, e.b0);
+    }
+};
+template <> struct ClusterBuf<double2> {
+    static constexpr int kBytes = 48;
+    __device__ static void load(const unsigned char *b, uint32_t E, uint32_t at, Entry<double2> &e)
+    {
+        const double2 *p = reinterpret_cast<const double2 *>(b);
+        e.a0 = p[at];
+        e.a1 = p[E + at];
+        e.b0 = p[2 * (size_t)E + at];
+        e.b1 = make_double2(0.0, 0.0);
+    }
+    __device__ static void store(unsigned char *b, uint32_t E, uint32_t at, const Entry<double2> &e)
+    {
+        double2 *p = reinterpret_cast<double2 *>(b);
+        p[at] = e.a0;
+        p[E + at] = e.a1;
+        p[2 * (size_t)E + at] = e.b0;
+    }
+    __device__ static void send(uint32_t b, uint32_t E, uint32_t at, const Entry<double2> &e)
+    {
+        peer_store(b + 16u * at, e.a0);
+        peer_store(b + 16u * (E + at), e.a1);
+        peer_store(b + 16u * (2u * E + at), e.b0);
+    }
+};
+/* FP64 out of line, as pos_readout; Y in shared memory */
+__device__ __noinline__ double pos_readout_sm(double2 *y, double unit, double sx, double sy)
+{
+    double2 acc = *y;
+    acc.x += unit * sx;
+    acc.y += unit * sy;
+    *y = acc;
+    return fma(acc.x, acc.x, acc.y * acc.y);
+}
+
+template <typename AmpT, int S>
+__global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_cluster(QwSimDev d, QwPosArgs p, QwStepArgs a)
+{
+    typedef typename Amp<AmpT>::RotVal RotVal;
+    constexpr int SW = S > 32 ? 32 : S, SPL = S / SW, RPP = 32 / SW;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ unsigned long long nsum[3];
+    __shared__ double pshares[2][kPosCluster * kPosMaxWarps];
+    __shared__ uint32_t poison;
+    __shared__ PosNorm pn;
+    if (*(volatile int32_t *)a.status != 0) return; /* after a failed step: nothing (every block alike) */
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, PW = blockDim.x >> 5;
+    const bool rot_in_place = Amp<AmpT>::kRotCode && d.rot_calc;
+    const AmpT zero = Amp<AmpT>::zero();
+    const uint32_t n = (uint32_t)d.pos_rows, T = (uint32_t)d.pos_T, X = T - n * S;
+    const uint32_t ngroups = (n + RPP - 1) / RPP, xgroups = (X + 31) / 32;
+    const uint32_t CL = gridDim.x, rank = blockIdx.x, nwarps = CL * PW; /* the grid is one cluster */
+    const uint32_t g0 = rank * PW + warp, x0 = nwarps - 1 - g0; /* extras from the last warp down */
+    const int ul = lane / SW, lb = lane % SW;
+    const uint32_t turns = (ngroups + nwarps - 1) / nwarps, xturns = (xgroups + nwarps - 1) / nwarps;
+    const uint32_t slots = turns * PW * 32 * SPL, E = slots + xturns * PW * 32;
+
+    typedef ClusterBuf<AmpT> Buf;
+    const uint32_t buf_bytes = E * (uint32_t)Buf::kBytes; /* (a multiple of 16: E is one of 32) */
+    RotVal *t_rot = reinterpret_cast<RotVal *>(smem + 2 * (size_t)buf_bytes);
+    double2 *y_sm = reinterpret_cast<double2 *>(t_rot + slots);
+    uint32_t *t_dst = reinterpret_cast<uint32_t *>(y_sm + (p.qls ? turns * PW * RPP : 0u));
+    uint32_t *t_x = t_dst + slots;
+    /* where entry e of the state lies */
+    auto place = [&](uint32_t e) {
+        uint32_t g, in;
+        if (e < n * S) {
+            const uint32_t j = e / S, l = e % S, gr = j / RPP, k = gr / nwarps;
+            g = gr % nwarps;
+            in = ((k * PW + g % PW) * SPL + l / SW) * 32 + (j % RPP) * SW + l % SW;
+        } else {
+            const uint32_t x = e - n * S, xg = x / 32, k = xg / nwarps;
+            g = nwarps - 1 - xg % nwarps;
+            in = slots + (k * PW + g % PW) * 32 + x % 32;
+        }
+        return (g / PW) << 20 | in;
+    };
+    auto load = [&](uint32_t at, uint32_t e, bool have) {
+        Entry<AmpT> v = {zero, zero, zero, zero};
+        if (have) PosMem<AmpT>::template load<false>(static_cast<const AmpT *>(p.in), T, e, v);
+        Buf::store(smem, E, at, v);
+    };
+    for (uint32_t k = 0; k < turns; ++k) {
+        const uint32_t jj = (g0 + k * nwarps) * RPP + ul;
+        const bool have = jj < n;
+#pragma unroll
+        for (int q = 0; q < SPL; ++q) {
+            const uint32_t at = ((k * PW + warp) * SPL + q) * 32 + lane, e = jj * S + lb + 32 * q;
+            RotVal t = Amp<AmpT>::rot_zero();
+            uint32_t dst = 0;
+            if (have) {
+                const uint32_t val = __ldg(d.img + e) & 0xffffu, to = __ldg(d.pos_dst + e);
+                if (val != 0)
+                    t = rot_in_place ? Amp<AmpT>::rot_code(val) : __ldg(static_cast<const RotVal *>(d.slot_rot) + e);
+                dst = place(to & 0x3fffffffu) | (to & 0x80000000u) | ((val & 0x8000u) << 15);
+            }
+            t_rot[at] = t;
+            t_dst[at] = dst;
+            load(at, e, have);
+        }
+        if (p.qls && lb == 0) y_sm[(k * PW + warp) * RPP + ul] = have ? __ldcg(a.qls_y + jj) : make_double2(0.0, 0.0);
+    }
+    for (uint32_t k = 0; k < xturns; ++k) {
+        const uint32_t x = (x0 + k * nwarps) * 32 + lane, at = (k * PW + warp) * 32 + lane;
+        t_x[at] = x < X ? place(__ldg(d.pos_xdst + x)) : 0u;
+        load(slots + at, n * S + x, x < X);
+    }
+    if (threadIdx.x == 0) {
+        nsum[0] = nsum[1] = nsum[2] = 0ull;
+        poison = 0u;
+        if (a.renorm) pos_norm_setup(a, pn);
+    }
+    const uint32_t buf_addr = smem_addr(smem);
+    const uint32_t peer = lane < CL ? lane : 0u; /* the block this lane adds the warp's norm to */
+    const uint32_t sum_peer = peer_addr(smem_addr(nsum), peer), poison_peer = peer_addr(smem_addr(&poison), peer);
+    auto send = [&](uint32_t out, uint32_t to, const Entry<AmpT> &o) { /* out: the buffer's own address */
+        Buf::send(peer_addr(out, (to >> 20) & 15u), E, to & 0xfffffu, o);
+    };
+
+    PosStats st;
+    uint32_t cnt = 0;
+    bool rescale = a.scale_in != nullptr;
+    typename Amp<AmpT>::Scale scale(rescale ? *a.scale_in : 1.0);
+    double coef = p.qls ? __ldg(a.qls_coefs + p.qls_term) : 0.0, coef_next = 0.0;
+    const double unit_of = d.inv_sqrt_s * (0.5 * S); /* u is scaled by 2 / s */
+    double fac = 1.0;
+    unsigned long long sum_u = 0ull;
+    cluster_sync(); /* every block's state, tables and sums are there */
+    for (int step = 0; step < p.nsteps; ++step) {
+        const unsigned char *A = smem + (size_t)(step & 1) * buf_bytes;
+        const uint32_t out = buf_addr + ((step & 1) ^ 1) * buf_bytes;
+        const bool readout = p.qls && (step & 1) != 0, last = step == p.nsteps - 1;
+        const int64_t term = p.qls_term + (step >> 1);
+        double unit = 0.0, pshare = 0.0;
+        if (readout) {
+            unit = coef * unit_of;
+            if (!last) coef_next = __ldg(a.qls_coefs + term + 1);
+        }
+        typename Amp<AmpT>::Norm nrm;
+        for (uint32_t k = 0, g = g0; g < ngroups; ++k, g += nwarps) {
+            const bool valid = g * RPP + ul < n;
+            RotVal rv[SPL];
+            uint32_t dst[SPL];
+            Entry<AmpT> in[SPL];
+#pragma unroll
+            for (int q = 0; q < SPL; ++q) {
+                const uint32_t at = ((k * PW + warp) * SPL + q) * 32 + lane;
+                rv[q] = t_rot[at];
+                dst[q] = t_dst[at];
+                Buf::load(A, E, at, in[q]);
+            }
+            pos_group<AmpT, S, false>(
+                d, rv, dst, in, rescale, scale, valid, a.renorm != 0, nrm, cnt, st,
+                [&](const typename Amp<AmpT>::Sum &sum) {
+                    if (readout && valid && lb == 0) {
+                        const double2 sv = sum.value();
+                        pshare += pos_readout_sm(y_sm + (k * PW + warp) * RPP + ul, unit, sv.x, sv.y);
+                    }
+                },
+                [&](int q, const Entry<AmpT> &o) { send(out, dst[q], o); });
+            if ((k & 7u) == 7u) st.take(cnt);
+        }
+        st.take(cnt);
+        for (uint32_t k = 0, x = x0 * 32 + lane; k < xturns; ++k, x += nwarps * 32) {
+            if (x >= X) break;
+            const uint32_t at = (k * PW + warp) * 32 + lane;
+            Entry<AmpT> e;
+            Buf::load(A, E, slots + at, e);
+            AmpT a0 = e.a0, a1 = e.a1, q0 = e.b0;
+            if (rescale) {
+                a0 = scale.apply(a0);
+                a1 = scale.apply(a1);
+                q0 = scale.apply(q0);
+            }
+            const bool k0 = pos_keep(d, a0), k1 = pos_keep(d, a1), h0 = pos_keep(d, q0);
+            const uint32_t kept = (k0 ? 1u : 0u) + (k1 ? 1u : 0u) + (h0 ? 1u : 0u);
+            cnt += (nz(a0) + nz(a1) + nz(q0)) * kCntIn + kept * (kCntRdag + kCntHph + kCntOut);
+            if (a.renorm) {
+                if (k0) norm_add(nrm, a0);
+                if (k1) norm_add(nrm, a1);
+                if (h0) norm_add(nrm, q0);
+            }
+            const Entry<AmpT> o = {k0 ? Amp<AmpT>::neg(a0) : zero, h0 ? Amp<AmpT>::neg(q0) : zero,
+                                   k1 ? Amp<AmpT>::neg(a1) : zero, zero};
+            send(out, t_x[at], o);
+            if ((k & 15u) == 15u) st.take(cnt);
+        }
+        st.take(cnt);
+        __syncwarp();
+        /* the warp's shares of the norm, to every block, and of ||Y||^2, to the
+           term's */
+        const uint32_t turn = (uint32_t)step % 3u;
+        const uint32_t who = last ? 0u : (uint32_t)(step >> 1) % CL;
+        if (a.renorm) {
+            bool bad;
+            unsigned long long v = warp_sum_units(to_units(nrm, pn.unit_inv, bad));
+            bad = __any_sync(FULL, bad) || v >= 1ull << 55; /* (the norm stays near the target) */
+            if (lane < CL) {
+                peer_add(sum_peer + 8u * turn, bad ? 0ull : v);
+                if (bad) peer_store(poison_peer, 1u);
+            }
+        }
+        double *const ps = pshares[(step >> 1) & 1];
+        if (readout) {
+            const double pv = warp_sum(pshare);
+            if (lane == 0) peer_store(peer_addr(smem_addr(ps + rank * PW + warp), who), pv);
+        }
+        cluster_sync();
+        if (a.renorm) {
+            sum_u = nsum[turn];
+            if (threadIdx.x == 0) nsum[(turn + 2u) % 3u] = 0ull;
+            float c;
+            if (pos_scale(pn, sum_u, c)) {
+                scale = Amp<AmpT>::scale_near_one(c);
+                if (last) fac = 1.0 + (double)c;
+            } else {
+                fac = *(volatile uint32_t *)&poison ? 1.0 : pos_scale_exact(*a.renorm_target, (double)sum_u / pn.unit_inv);
+                scale = typename Amp<AmpT>::Scale(fac);
+            }
+        }
+        rescale = a.renorm != 0;
+        if (readout) coef = coef_next;
+        /* p_j = ||Y||^2 of the term, by one warp of a block that changes from term to
+           term, while the others go on */
+        if (readout && warp == PW - 1 && rank == who) {
+            double v = 0.0;
+            for (uint32_t b = lane; b < nwarps; b += 32) v += ps[b];
+            v = warp_sum(v);
+            if (lane == 0) a.qls_p[term] = v;
+        }
+    }
+    st.flush(a);
+
+    /* the last barrier is passed: the other blocks' shared memory is left alone */
+    AmpT *O = static_cast<AmpT *>((p.nsteps & 1) ? p.out0 : p.out1);
+    const unsigned char *A = smem + (size_t)(p.nsteps & 1) * buf_bytes;
+    auto store = [&](uint32_t at, uint32_t e) {
+        Entry<AmpT> v;
+        Buf::load(A, E, at, v);
+        PosMem<AmpT>::template store<false>(O, T, e, v);
+    };
+    for (uint32_t k = 0; k < turns; ++k) {
+        const uint32_t jj = (g0 + k * nwarps) * RPP + ul;
+        if (jj >= n) continue;
+#pragma unroll
+        for (int q = 0; q < SPL; ++q) store(((k * PW + warp) * SPL + q) * 32 + lane, jj * S + lb + 32 * q);
+        if (p.qls && lb == 0) __stcg(a.qls_y + jj, y_sm[(k * PW + warp) * RPP + ul]);
+    }
+    for (uint32_t k = 0; k < xturns; ++k) {
+        const uint32_t x = (x0 + k * nwarps) * 32 + lane;
+        if (x < X) store(slots + (k * PW + warp) * 32 + lane, n * S + x);
+    }
+    if (rank == 0 && threadIdx.x == 0) {
+        *a.norm_out = a.renorm ? (double)sum_u / pn.unit_inv : 0.0;
+        if (a.scale_out) *a.scale_out = fac;
+        if (a.steps_done) *a.steps_done += p.nsteps;
+        if (a.stats) a.stats[QW_STAT_STEPS] += p.nsteps;
     }
 }
 
@@ -879,6 +1243,78 @@ void *pos_kernel(int s)
     return (void *)k_walk_pos<AmpT, 64, FULLST, TAB>;
 }
 
+/* Slots up to which a run goes to one cluster, either precision: 16 SMs then issue the
+   arithmetic of more than 12 warps each, and the grid's 152 make up for its
+   barrier -- 200 steps of 175 groups of 32 slots (N = 700, s = 8) 694 us on the
+   grid, 539 on the cluster (complex64), 768 and 634 (complex128); 100 steps of 256
+   groups (N = 1024) 378 and 386, 250 (N = 1000) 430 and 437. */
+constexpr int64_t kClusterSlots = 6144;
+constexpr int kClusterStatic = 8192; /* more than the kernel's static shared memory and what the system takes */
+
+inline void cluster_config(const QwPosPlan &pl, cudaLaunchConfig_t &c, cudaLaunchAttribute &at, cudaStream_t st)
+{
+    c = cudaLaunchConfig_t{};
+    at = cudaLaunchAttribute{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)pl.cl;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    c.gridDim = dim3((unsigned)pl.cl);
+    c.blockDim = dim3((unsigned)pl.cl_warps * 32);
+    c.dynamicSmemBytes = pl.cl_smem;
+    c.stream = st;
+    c.attrs = &at;
+    c.numAttrs = 1;
+}
+
+template <typename AmpT>
+void *cluster_kernel(int s)
+{
+    if (s == 4) return (void *)k_walk_cluster<AmpT, 4>;
+    if (s == 8) return (void *)k_walk_cluster<AmpT, 8>;
+    if (s == 16) return (void *)k_walk_cluster<AmpT, 16>;
+    if (s == 32) return (void *)k_walk_cluster<AmpT, 32>;
+    return (void *)k_walk_cluster<AmpT, 64>;
+}
+
+/* The launch of a run on one cluster, or cl = 0 where the grid is faster or the
+ * state does not fit.  Without the opt-in size of 16 blocks: 8. */
+template <typename AmpT>
+void cluster_plan(const QwSimDev &d, int64_t groups, int64_t xgroups, int spl, int rpp, int optin, QwPosPlan &pl)
+{
+    constexpr bool c128 = sizeof(AmpT) == 16;
+    const int64_t few = c128 ? 4 : 8; /* groups a block: fewer blocks, not slower (measured) */
+    pl.cl = 0;
+    if (groups * 32 * spl > kClusterSlots) return;
+    int cl = 1;
+    while (cl < kPosCluster && groups * spl > cl * few) cl *= 2;
+    for (; cl >= 1; cl /= 2) {
+        const int64_t per = (groups + cl - 1) / cl, t0 = (per + kPosMaxWarps - 1) / kPosMaxWarps;
+        int64_t pw = (per + t0 - 1) / t0;
+        if (pw < 4) pw = 4;
+        const int64_t turns = (groups + cl * pw - 1) / (cl * pw), xturns = (xgroups + cl * pw - 1) / (cl * pw);
+        const int64_t slots = turns * pw * 32 * spl, E = slots + xturns * pw * 32;
+        const int64_t smem = 2 * E * (int64_t)ClusterBuf<AmpT>::kBytes + slots * (int64_t)(sizeof(typename Amp<AmpT>::RotVal) + 4) +
+                             turns * pw * rpp * 16 + xturns * pw * 32 * 4;
+        if (E >= 1 << 20 || smem + kClusterStatic > optin) return; /* (fewer blocks would need more) */
+        void *k = cluster_kernel<AmpT>(d.s);
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - kClusterStatic) != cudaSuccess ||
+            (cl > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+            cudaGetLastError();
+            continue;
+        }
+        pl.cl = cl;
+        pl.cl_warps = (int)pw;
+        pl.cl_smem = (size_t)smem;
+        cudaLaunchConfig_t c;
+        cudaLaunchAttribute at;
+        cluster_config(pl, c, at, nullptr);
+        int fit = 0;
+        if (cudaOccupancyMaxActiveClusters(&fit, k, &c) == cudaSuccess && fit >= 1) return;
+        cudaGetLastError();
+        pl.cl = 0;
+    }
+}
+
 /* One block per SM: every group of rows has a warp within a few turns, with
  * as many groups for each warp as for the others (54 groups an SM at N =
  * 16384, s = 16: 4 turns of 14 warps instead of 16, 16, 16, 6); the tables
@@ -909,6 +1345,7 @@ QwPosPlan pos_plan(const QwSimDev &d)
     pl.tab = pl.smem + 1024 <= (size_t)optin; /* beside the kernel's static arrays */
     if (!pl.tab) pl.smem = 0;
     pl.coop = coop != 0 && pl.grid < 256; /* the barrier word's count has 8 bits */
+    cluster_plan<AmpT>(d, groups, xgroups, spl, rpp, optin, pl);
     if (pl.tab) /* the limit belongs to the process, not to this simulator: always the largest */
         cudaFuncSetAttribute(pos_kernel<AmpT, false, true>(s), cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 1024);
     return pl;
@@ -918,6 +1355,16 @@ template <typename AmpT>
 cudaError_t launch_pos_t(const QwSimDev &d, const QwPosPlan &pl, const QwPosArgs &p, const QwStepArgs &a, int full,
                          cudaStream_t st)
 {
+    if (p.words && pl.cl && !full) {
+        QwSimDev dc = d;
+        QwPosArgs pc = p;
+        QwStepArgs ac = a;
+        void *cargs[] = {&dc, &pc, &ac};
+        cudaLaunchConfig_t c;
+        cudaLaunchAttribute at;
+        cluster_config(pl, c, at, st);
+        return cudaLaunchKernelExC(&c, cluster_kernel<AmpT>(d.s), cargs);
+    }
     /* one step reads each table entry once: straight from memory */
     const bool tab = pl.tab && p.nsteps > 1 && !full;
     void *k = full ? pos_kernel<AmpT, true, false>(d.s)

@@ -1,6 +1,6 @@
-"""The positional layout's runs: many steps (or QLS terms) in one cooperative
-launch equal the same ones by single launches, at the edges of its tables and
-turns; s = 4, which the autotuner alone chooses; marginals read in place."""
+"""The positional layout's runs: many steps (or QLS terms) in one launch, over the
+grid or (up to 6144 slots) on one cluster, equal the same ones by single
+launches, at the edges of their tables and turns; s = 4, which the autotuner alone chooses; marginals read in place."""
 import numpy as np
 import pytest
 
@@ -12,8 +12,9 @@ from parity import compare, gpu_state, oracle_state
 
 pytestmark = pytest.mark.gpu
 
-# rows a warp, a block of 4 warps and the card hold, and one more or less
-SHAPES = [(8, 8), (9, 8), (33, 8), (127, 8), (129, 16), (1217, 8), (70, 32), (130, 64), (20001, 8)]
+# rows a warp, a block of 4 warps, a cluster and the card hold, and one more or less
+SHAPES = [(8, 8), (9, 8), (33, 8), (127, 8), (129, 16), (70, 32), (768, 8), (95, 64), (96, 64), (97, 64), (769, 8),
+          (1217, 8), (130, 64), (20001, 8)]
 
 
 def _matrix(n, s):
@@ -50,18 +51,19 @@ def test_a_run_equals_single_steps(n, s):
         assert np.array_equal(ka, kb) and np.array_equal(va, vb)
 
 
+@pytest.mark.parametrize("n", [100, 900])
 @pytest.mark.parametrize("precision,tol", [(qwalk.QW_FP64, 1e-12), (qwalk.QW_FP32_AMP, 1e-4)])
-def test_a_run_over_a_launchs_length(precision, tol):
+def test_a_run_over_a_launchs_length(precision, tol, n):
     """1025 steps: two launches, and (complex64) a renormalisation between any two
     steps; against the single steps, whose factor is computed another way.
     complex64: an amplitude takes a rounding of 2^-24 of itself a step from
     the factor's last bit, 1025 steps of it in the worst case 6e-5."""
-    m, b = _matrix(100, 8), _b(100, 2)
+    m, b = _matrix(n, 8), _b(n, 2)
     out = []
     for graphs in (True, False):
         sim = _positional(m, 8, b, precision=precision, graphs=graphs)
         sim.enqueue_walk_steps(1025)
-        out.append([sim.measure_register(r, 100) for r in ("j", "k")])
+        out.append([sim.measure_register(r, n) for r in ("j", "k")])
     for x, y in zip(*out):
         assert abs(x.sum() - 1.0) < tol and np.abs(x - y).max() < tol
 
@@ -82,7 +84,8 @@ def test_s4_matches_oracle(n, s):
         compare(gpu_state(sim), oracle_state(o), 1e-12)
 
 
-@pytest.mark.parametrize("n,s,terms", [(60, 4, 5), (100, 8, 1), (100, 8, 513), (140, 16, 8)])
+@pytest.mark.parametrize("n,s,terms", [(60, 4, 5), (100, 8, 1), (100, 8, 513), (140, 16, 8), (100, 64, 3),
+                                       (900, 8, 3)])
 def test_qls_terms_in_one_launch(n, s, terms):
     """Y and every p_j against the Chebyshev sum in numpy (1e-9 relative, the
     bound of the other QLS tests)."""
