@@ -924,21 +924,30 @@ static cudaError_t flat_alloc(qw_sim *sim, size_t bytes, void **p)
     return cudaMallocFromPoolAsync(p, bytes < 16 ? 16 : bytes, sim->fpool, sim->stream);
 }
 
-/* Scratch of one call, given back to the pool on every way out. */
+/* Scratch of one call, given back to the pool on every way out -- and, when a call
+ * outside the flat path (import, export) took more than kIoKeep, by the pool to
+ * the device: a simulator that never runs the flat path holds on to no more. */
+static const size_t kIoKeep = (size_t)256 << 20;
 struct FlatScratch {
     qw_sim *sim;
+    bool io;
+    size_t bytes = 0;
     std::vector<void *> all;
-    explicit FlatScratch(qw_sim *s) : sim(s) {}
+    explicit FlatScratch(qw_sim *s, bool io_ = false) : sim(s), io(io_) {}
     FlatScratch(const FlatScratch &) = delete;
     FlatScratch &operator=(const FlatScratch &) = delete;
     ~FlatScratch()
     {
         for (void *p : all) cudaFreeAsync(p, sim->stream);
+        if (io && bytes > kIoKeep && !host_staged(sim) && !sim->fq_open) {
+            cudaStreamSynchronize(sim->stream);
+            cudaMemPoolTrimTo(sim->fpool, kIoKeep);
+        }
     }
-    cudaError_t take(size_t bytes, void **p)
+    cudaError_t take(size_t n, void **p)
     {
-        const cudaError_t e = flat_alloc(sim, bytes, p);
-        if (e == cudaSuccess) all.push_back(*p);
+        const cudaError_t e = flat_alloc(sim, n, p);
+        if (e == cudaSuccess) all.push_back(*p), bytes += n;
         return e;
     }
 };
@@ -2119,7 +2128,7 @@ extern "C" int qw_state_export(qw_sim *sim, int32_t inst, int32_t key_words, uin
     /* gathered, sorted by key and laid out on the device; the caller's arrays
        are written once the status is known to be clean */
     cudaStream_t st = sim->stream;
-    FlatScratch scratch(sim);
+    FlatScratch scratch(sim, true);
     const size_t M = (size_t)total, W = (size_t)key_words;
     void *K = nullptr, *A = nullptr, *tk = nullptr, *ta = nullptr, *work = nullptr, *out = nullptr;
     QW_CUDA(sim, scratch.take(M * 16, &K));
@@ -2208,7 +2217,7 @@ extern "C" int qw_state_import(qw_sim *sim, int32_t key_words, const uint64_t *k
         return fail(sim, QW_ERR_ARG, "key_words too small for the packed register layout");
     if (count < 0 || (count > 0 && (!keys || !amps))) return fail(sim, QW_ERR_ARG, "bad arrays");
     cudaStream_t st = sim->stream;
-    FlatScratch scratch(sim);
+    FlatScratch scratch(sim, true);
     void *K = nullptr, *A = nullptr;
     QwIoFlags *flags = nullptr;
     double norm2 = 0.0;
