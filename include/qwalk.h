@@ -212,7 +212,7 @@ int qw_apply_walk_step(qw_sim *sim, int64_t nsteps);
  * walk_variant 7, a call made while the stream is not being captured first
  * moves a state that is not yet in the positional layout into it, which
  * synchronises once; during a capture such a state runs on the bucket
- * kernel of variant 4 (2 for s = 64) instead.  The flat and register-faithful schedules (variants 5
+ * kernel of variant 4 (2 for s = 4 and 64) instead.  The flat and register-faithful schedules (variants 5
  * and 6) synchronise between their stages.
  * Errors: QW_ERR_ARG, QW_ERR_STATE, QW_ERR_CUDA (launch failure).
  */
@@ -241,10 +241,13 @@ int qw_sync(qw_sim *sim);
  * all later steps.  Segments are tried only when warp_capacity >= 2
  * row_capacity (true by default), the slot kernel only then and for s = 8, 16
  * or 32, the positional layout (variant 7) for s = 4, 8, 16, 32 or 64 without
- * partitions (s = 4: here only, a simulator is not created with it; its tables are built first, and the move of the state into it
- * is not timed); the flat path and the register-faithful
- * schedule (variants 5 and 6) are never chosen; variants not tried are
- * reported as 0 us.  The state advances by steps_per_candidate walk steps per
+ * partitions (its tables are built first, and the move of the state into it is
+ * not timed); the flat path and the register-faithful schedule (variants 5 and
+ * 6) are never chosen; variants not tried are reported as 0 us.  s = 4: a
+ * simulator is not created with variant 7, so *choice names the fastest of the
+ * others, which one can be created with, while this simulator keeps the
+ * positional layout if us_per_step[7] is the least.
+ * The state advances by steps_per_candidate walk steps per
  * variant tried (the variants give the same results).  *choice (nullable)
  * receives the variant, *us_per_step (nullable, QW_WALK_VARIANTS doubles) the
  * measured times.  Synchronises.  Has no effect with fuse_reflection = 0.

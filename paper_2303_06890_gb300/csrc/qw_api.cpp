@@ -1885,7 +1885,16 @@ extern "C" int qw_autotune(qw_sim *sim, int32_t steps, int32_t *choice, double *
     sim->mode = best_mode;
     sim->grid_walk = best_mode == QW_MODE_WALK_POS ? sim->grid_alt : qw_step_grid(sim->d, sim->fp32, best_mode);
     drop_graphs(sim);
-    if (choice) *choice = best;
+    if (choice) {
+        *choice = best;
+        if (best_mode == QW_MODE_WALK_POS && sim->d.s < 8) { /* one that qw_sim_create takes */
+            int other = cand[0].first;
+            for (const auto &cv : cand)
+                if (cv.second != QW_MODE_WALK_POS && us[cv.first] > 0.0 && (us[other] <= 0.0 || us[cv.first] < us[other]))
+                    other = cv.first;
+            *choice = other;
+        }
+    }
     if (us_per_step)
         for (int v = 0; v < QW_WALK_VARIANTS; ++v) us_per_step[v] = us[v];
     return rc;
