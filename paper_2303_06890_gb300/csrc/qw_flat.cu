@@ -2,15 +2,16 @@
  * qw_flat.cu -- the walk step as the paper's simulator runs it, on one flat
  * list of branches in global memory (Sec. V-A): every register map applied to
  * every branch, and every interference operation as
- *   (1) grouping: a stable LSD radix sort of the whole list by all
- *       registers, with the target's bits moved below the others, so that
- *       the branches equal on every idle register are contiguous (8-bit
- *       digits over the bits that vary between keys, one single-pass
- *       kernel per digit carrying a permutation, the entries moved once);
+ *   (1) grouping: a stable LSD radix sort of the whole list by the registers
+ *       that make the groups, so that the branches equal on every idle
+ *       register are contiguous (8-bit digits over the bits that vary between
+ *       keys, one single-pass kernel per digit carrying a permutation, the
+ *       entries moved once);
  *   (2) computing: the small dense operator on each group's zero-filled
- *       vector (a thread per output; for H the groups are counted first, so
- *       that s outputs are formed per group, not per list entry);
- *   (3) clearing: outputs with |a| <= tau dropped by a stream compaction.
+ *       vector (for H the groups are found first, so that s outputs are
+ *       formed per group, not per list entry);
+ *   (3) clearing: outputs with |a| <= tau dropped as they are written, at places
+ *       from a single-pass prefix sum over the tiles of (2).
  * T~^dag, H, P, H, T~ and S run in the order of Alg. "Quantum walk operator",
  * with the element register A allocated for the whole step.  Nothing here is
  * bounded by the row buckets or the on-chip buffers of the step kernels, only
