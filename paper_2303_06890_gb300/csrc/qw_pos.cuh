@@ -417,14 +417,22 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
     RotVal *t_rot = reinterpret_cast<RotVal *>(smem);
     uint32_t *t_dst = reinterpret_cast<uint32_t *>(t_rot + (size_t)turns * PW * 32 * SPL);
     uint32_t *t_x = t_dst + (size_t)turns * PW * 32 * SPL;
-    /* a slot's rotation, its destination entry with flags: bit 31 sigma = -1,
-       bit 30 a negative element */
-    auto slot_table = [&](uint32_t at, RotVal &t, uint32_t &dst) {
-        const uint32_t w = __ldg(d.img + at), val = w & 0xffffu;
+    /* what a slot needs of the matrix, as it lies in memory; its rotation, its
+       destination entry with flags: bit 31 sigma = -1, bit 30 a negative element */
+    struct Slot {
+        uint32_t w, dst;
+        RotVal rot;
+    };
+    auto slot_load = [&](uint32_t at, Slot &x) {
+        x.w = __ldg(d.img + at);
+        x.dst = __ldg(d.pos_dst + at);
+        if (!rot_in_place) x.rot = __ldg(static_cast<const RotVal *>(d.slot_rot) + at);
+    };
+    auto slot_use = [&](const Slot &x, RotVal &t, uint32_t &dst) {
+        const uint32_t val = x.w & 0xffffu;
         /* a 0 element rotates by R(0) */
-        t = val == 0 ? Amp<AmpT>::rot_zero()
-                     : (rot_in_place ? Amp<AmpT>::rot_code(val) : __ldg(static_cast<const RotVal *>(d.slot_rot) + at));
-        dst = __ldg(d.pos_dst + at) | ((val & 0x8000u) << 15);
+        t = val == 0 ? Amp<AmpT>::rot_zero() : (rot_in_place ? Amp<AmpT>::rot_code(val) : x.rot);
+        dst = x.dst | ((val & 0x8000u) << 15);
     };
     if (TAB) {
         for (uint32_t k = 0; k < turns; ++k) {
@@ -433,7 +441,11 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
             for (int q = 0; q < SPL; ++q) {
                 RotVal t = Amp<AmpT>::rot_zero();
                 uint32_t dst = 0;
-                if (g < ngroups && jj < n) slot_table(jj * S + lb + 32 * q, t, dst);
+                if (g < ngroups && jj < n) {
+                    Slot x;
+                    slot_load(jj * S + lb + 32 * q, x);
+                    slot_use(x, t, dst);
+                }
                 const uint32_t at = ((k * PW + warp) * SPL + q) * 32 + lane;
                 t_rot[at] = t;
                 t_dst[at] = dst;
@@ -446,9 +458,14 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
         __syncwarp(); /* a warp reads only what it wrote */
     }
 
-    /* a group's state, loaded one group ahead */
+    /* a group's state, loaded one group ahead, and without the tables the words of
+       the matrix too: a single step meets them in DRAM (29.0 -> 25.3 us a flushed step at N = 16384
+       complex64, 28.5 -> 24.6 complex128; not where they
+       would spill: two complex128 slots a lane) */
+    constexpr bool kSlotAhead = SPL == 1 || sizeof(AmpT) == 8;
     struct In {
         Entry<AmpT> e[SPL];
+        Slot x[TAB ? 1 : SPL];
     };
     auto fetch = [&](const AmpT *A, uint32_t gg, In &x) {
         const uint32_t jj = gg * RPP + ul;
@@ -458,6 +475,10 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
         for (int q = 0; q < SPL; ++q) {
             x.e[q].a0 = x.e[q].a1 = x.e[q].b0 = x.e[q].b1 = zero;
             if (have) PosMem<AmpT>::template load<FULLST>(A, T, i0 + 32 * q, x.e[q]);
+            if (!TAB && kSlotAhead) {
+                x.x[TAB ? 0 : q].w = x.x[TAB ? 0 : q].dst = 0;
+                if (have) slot_load(i0 + 32 * q, x.x[TAB ? 0 : q]);
+            }
         }
     };
 
@@ -481,6 +502,14 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
         typename Amp<AmpT>::Norm nrm;
         In nxt;
         fetch(A, g0, nxt);
+        /* so are a single step's first extras */
+        constexpr bool kXAhead = !TAB && sizeof(AmpT) == 8;
+        Entry<AmpT> xe = {zero, zero, zero, zero};
+        uint32_t xto = 0;
+        if (kXAhead && x0 * 32 + lane < X) {
+            PosMem<AmpT>::template load<FULLST>(A, T, n * S + x0 * 32 + lane, xe);
+            xto = __ldg(d.pos_xdst + x0 * 32 + lane);
+        }
         for (uint32_t k = 0, g = g0; g < ngroups; ++k, g += nwarps) {
             const In cur = nxt;
             fetch(A, g + nwarps, nxt);
@@ -495,9 +524,12 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
                     rv[q] = t_rot[at];
                     dst[q] = t_dst[at];
                 } else {
-                    rv[q] = Amp<AmpT>::rot_zero();
-                    dst[q] = 0;
-                    if (valid) slot_table(j * S + lb + 32 * q, rv[q], dst[q]);
+                    Slot x = cur.x[TAB ? 0 : q];
+                    if (!kSlotAhead) {
+                        x.w = x.dst = 0;
+                        if (valid) slot_load(j * S + lb + 32 * q, x);
+                    }
+                    slot_use(x, rv[q], dst[q]);
                 }
             }
             pos_group<AmpT, S, FULLST>(
@@ -516,9 +548,12 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
         for (uint32_t k = 0, x = x0 * 32 + lane; k < xturns; ++k, x += nwarps * 32) {
             if (x >= X) break;
             const uint32_t i = n * S + x;
-            const uint32_t to = TAB ? t_x[(k * PW + warp) * 32 + lane] : __ldg(d.pos_xdst + x);
-            Entry<AmpT> e;
-            PosMem<AmpT>::template load<FULLST>(A, T, i, e);
+            uint32_t to = xto;
+            Entry<AmpT> e = xe;
+            if (!kXAhead || k > 0) {
+                to = TAB ? t_x[(k * PW + warp) * 32 + lane] : __ldg(d.pos_xdst + x);
+                PosMem<AmpT>::template load<FULLST>(A, T, i, e);
+            }
             AmpT a0 = e.a0, a1 = e.a1, q0 = e.b0, q1 = FULLST ? e.b1 : zero;
             if (rescale) {
                 a0 = scale.apply(a0);
