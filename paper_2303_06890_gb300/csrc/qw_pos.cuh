@@ -126,7 +126,7 @@ struct PosNorm { /* per launch, in shared memory */
     float target_inv;                 /* 1 / target */
 };
 
-__device__ __forceinline__ void pos_norm_setup(const QwStepArgs &a, PosNorm &pn)
+__device__ __forceinline__ void pos_norm_setup(const QwStepArgs &a, PosNorm &pn, bool series = true)
 {
     const double t = *a.renorm_target;
     int e = 0;
@@ -134,7 +134,8 @@ __device__ __forceinline__ void pos_norm_setup(const QwStepArgs &a, PosNorm &pn)
     e = max(e, -70); /* 2^(54 - e) is an FP32 number too */
     pn.unit_inv = ldexp(1.0, 54 - e);
     pn.target = (unsigned long long)__double2ll_rn(t > 0.0 && t < 1e300 ? t * pn.unit_inv : 0.0);
-    pn.target_inv = pn.target ? (float)(1.0 / (double)pn.target) : 0.0f;
+    pn.target_inv = 0.0f;
+    if (series) pn.target_inv = pn.target ? (float)(1.0 / (double)pn.target) : 0.0f;
 }
 
 /* a lane's norm share in units; poisoned (not finite, or beyond what the word
@@ -403,7 +404,6 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
     __shared__ PosNorm pn;
     __shared__ int flag_sm, bad_sm;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, PW = blockDim.x >> 5;
-    if (*(volatile int32_t *)a.status != 0) return; /* after a failed step: nothing (the whole grid alike) */
     const bool rot_in_place = Amp<AmpT>::kRotCode && d.rot_calc;
     const AmpT zero = Amp<AmpT>::zero();
     const uint32_t n = (uint32_t)d.pos_rows, T = (uint32_t)d.pos_T; /* rows, entries; 4 T < 2^31 */
@@ -434,30 +434,6 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
         t = val == 0 ? Amp<AmpT>::rot_zero() : (rot_in_place ? Amp<AmpT>::rot_code(val) : x.rot);
         dst = x.dst | ((val & 0x8000u) << 15);
     };
-    if (TAB) {
-        for (uint32_t k = 0; k < turns; ++k) {
-            const uint32_t g = g0 + k * nwarps, jj = g * RPP + ul;
-#pragma unroll
-            for (int q = 0; q < SPL; ++q) {
-                RotVal t = Amp<AmpT>::rot_zero();
-                uint32_t dst = 0;
-                if (g < ngroups && jj < n) {
-                    Slot x;
-                    slot_load(jj * S + lb + 32 * q, x);
-                    slot_use(x, t, dst);
-                }
-                const uint32_t at = ((k * PW + warp) * SPL + q) * 32 + lane;
-                t_rot[at] = t;
-                t_dst[at] = dst;
-            }
-        }
-        for (uint32_t k = 0; k < xturns; ++k) {
-            const uint32_t x = (x0 + k * nwarps) * 32 + lane;
-            t_x[(k * PW + warp) * 32 + lane] = x < X ? __ldg(d.pos_xdst + x) : 0u;
-        }
-        __syncwarp(); /* a warp reads only what it wrote */
-    }
-
     /* a group's state, loaded one group ahead, and without the tables the words of
        the matrix too: a single step meets them in DRAM (29.0 -> 25.3 us a flushed step at N = 16384
        complex64, 28.5 -> 24.6 complex128; not where they
@@ -482,13 +458,50 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
         }
     };
 
+    /* a single step issues its first loads before anything that waits for one (the
+       status, the norm's target: DRAM latencies too when the L2 is cold; 25.3 -> 25.0 us a flushed
+       step complex64, 24.6 -> 23.7 complex128) */
+    const AmpT *A = static_cast<const AmpT *>(p.in);
+    constexpr bool kFirst = !TAB && SPL == 1, kXAhead = kFirst && sizeof(AmpT) == 8;
+    In first;
+    Entry<AmpT> xe = {zero, zero, zero, zero};
+    uint32_t xto = 0;
+    if (kFirst) fetch(A, g0, first);
+    if (kXAhead && x0 * 32 + lane < X) {
+        PosMem<AmpT>::template load<FULLST>(A, T, n * S + x0 * 32 + lane, xe);
+        xto = __ldg(d.pos_xdst + x0 * 32 + lane);
+    }
+    if (*(volatile int32_t *)a.status != 0) return; /* after a failed step: nothing (the whole grid alike) */
+    if (TAB) {
+        for (uint32_t k = 0; k < turns; ++k) {
+            const uint32_t g = g0 + k * nwarps, jj = g * RPP + ul;
+#pragma unroll
+            for (int q = 0; q < SPL; ++q) {
+                RotVal t = Amp<AmpT>::rot_zero();
+                uint32_t dst = 0;
+                if (g < ngroups && jj < n) {
+                    Slot x;
+                    slot_load(jj * S + lb + 32 * q, x);
+                    slot_use(x, t, dst);
+                }
+                const uint32_t at = ((k * PW + warp) * SPL + q) * 32 + lane;
+                t_rot[at] = t;
+                t_dst[at] = dst;
+            }
+        }
+        for (uint32_t k = 0; k < xturns; ++k) {
+            const uint32_t x = (x0 + k * nwarps) * 32 + lane;
+            t_x[(k * PW + warp) * 32 + lane] = x < X ? __ldg(d.pos_xdst + x) : 0u;
+        }
+        __syncwarp(); /* a warp reads only what it wrote */
+    }
+
     PosStats st;
     uint32_t cnt = 0;
-    const AmpT *A = static_cast<const AmpT *>(p.in);
     bool rescale = a.scale_in != nullptr;
     if (threadIdx.x == 0) {
         Amp<AmpT>::Scale::to_shared(rescale ? *a.scale_in : 1.0, &scale_sm);
-        if (a.renorm) pos_norm_setup(a, pn);
+        if (a.renorm) pos_norm_setup(a, pn, p.words != nullptr);
         bad_sm = 0;
     }
     __syncthreads();
@@ -501,15 +514,8 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
         const typename Amp<AmpT>::Scale scale = Amp<AmpT>::Scale::from_shared(&scale_sm);
         typename Amp<AmpT>::Norm nrm;
         In nxt;
-        fetch(A, g0, nxt);
-        /* so are a single step's first extras */
-        constexpr bool kXAhead = !TAB && sizeof(AmpT) == 8;
-        Entry<AmpT> xe = {zero, zero, zero, zero};
-        uint32_t xto = 0;
-        if (kXAhead && x0 * 32 + lane < X) {
-            PosMem<AmpT>::template load<FULLST>(A, T, n * S + x0 * 32 + lane, xe);
-            xto = __ldg(d.pos_xdst + x0 * 32 + lane);
-        }
+        if (!kFirst || step > 0) fetch(A, g0, nxt);
+        else nxt = first;
         for (uint32_t k = 0, g = g0; g < ngroups; ++k, g += nwarps) {
             const In cur = nxt;
             fetch(A, g + nwarps, nxt);
@@ -550,7 +556,7 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
             const uint32_t i = n * S + x;
             uint32_t to = xto;
             Entry<AmpT> e = xe;
-            if (!kXAhead || k > 0) {
+            if (!kXAhead || k > 0 || step > 0) {
                 to = TAB ? t_x[(k * PW + warp) * 32 + lane] : __ldg(d.pos_xdst + x);
                 PosMem<AmpT>::template load<FULLST>(A, T, i, e);
             }
