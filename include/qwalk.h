@@ -238,7 +238,9 @@ int qw_sync(qw_sim *sim);
  * each variant of walk_variant (rows or segments of two rows, plain or
  * software-pipelined, one lane per QRAM slot, the positional layout), times
  * them with CUDA events on the simulator's stream, and keeps the fastest for
- * all later steps.  Segments are tried only when warp_capacity >= 2
+ * all later steps.  A step whose result is dropped goes before the timed ones,
+ * and the positional layout is timed as it will run: with graphs, over launches
+ * of at least 32 steps, dropped too.  Segments are tried only when warp_capacity >= 2
  * row_capacity (true by default), the slot kernel only then and for s = 8, 16
  * or 32, the positional layout (variant 7) for s = 4, 8, 16, 32 or 64 without
  * partitions (its tables are built first, and the move of the state into it is

@@ -185,6 +185,7 @@ static const int kGraphTerms = 3;  /* QLS terms per graph: 2 walk steps each */
    of an import (6), the sort's varying bits (2 x 10) */
 static const int kFlatTotal = 0, kFlatCount = 1, kFlatRow = 2, kFlatIo = 4, kFlatSort = 16, kFlatWords = 40;
 static const int64_t kPosSteps = 1024; /* walk steps of one positional launch: a few milliseconds */
+static const int64_t kTuneSteps = 32;  /* at least, of one the autotuner times: the launch is a small part */
 
 static void drop_graphs(qw_sim *sim)
 {
@@ -1811,6 +1812,52 @@ extern "C" int qw_apply_walk_step(qw_sim *sim, int64_t nsteps)
     return sync_walk(sim, "qw_apply_walk_step");
 }
 
+/* The least time of a step of the kernel in use, in us; the state advances by
+ * `steps`.  What a first launch takes beside its steps (a kernel's load, the
+ * first cooperative launch: tens of us in all) must not be divided by the few steps asked
+ * for -- over two of them it made a run of 8.5 us a step look slower than a
+ * bucket kernel's 20 -- so a launch whose results are dropped goes first, and a
+ * positional run is timed twice over at least kTuneSteps steps, dropped too.
+ * Both kinds leave their input as it is; the scalars (but the status) are put
+ * back, the bucket step's output is cleared.  Nothing waits in between: what is
+ * timed is queued before the device gets there. */
+static int tune_time(qw_sim *sim, int32_t steps, cudaEvent_t *ev, double *us)
+{
+    cudaStream_t st = sim->stream;
+    const bool runs = pos_runs(sim, false), buckets = sim->mode != QW_MODE_WALK_POS || !sim->pos_live;
+    const int64_t m = runs ? std::min(kPosSteps, std::max<int64_t>(steps, kTuneSteps)) : 1;
+    const int cur = sim->cur, slot = sim->scale_slot;
+    const int64_t issued = sim->issued;
+    const size_t head = offsetof(Scalars, steps_done);
+    QW_CUDA(sim, cudaMemcpyAsync(sim->h_sc, sim->sc, sizeof(Scalars), cudaMemcpyDeviceToHost, st));
+    QW_CUDA(sim, cudaStreamSynchronize(st));
+    for (int r = 0; r < (runs ? 3 : 1); ++r) {
+        if (r > 0) QW_CUDA(sim, cudaEventRecord(ev[r - 1], st));
+        const int rc = runs ? launch_pos(sim, m, -1, 0) : launch_walk(sim, 0);
+        sim->cur = cur;
+        sim->scale_slot = slot;
+        sim->issued = issued;
+        if (rc != QW_OK) return rc;
+    }
+    if (runs) QW_CUDA(sim, cudaEventRecord(ev[2], st));
+    if (buckets) QW_CUDA(sim, qw_launch_clear(sim->d, sim->buf[(cur + 1) % 3], 0, sim->d.total_buckets, 1, st));
+    QW_CUDA(sim, cudaMemcpyAsync((char *)sim->sc + head, (const char *)sim->h_sc + head, sizeof(Scalars) - head,
+                                 cudaMemcpyHostToDevice, st));
+    if (!runs) QW_CUDA(sim, cudaEventRecord(ev[0], st));
+    int rc = qw_enqueue_walk_steps(sim, steps);
+    if (rc != QW_OK) return rc;
+    if (!runs) QW_CUDA(sim, cudaEventRecord(ev[1], st));
+    rc = check_status(sim, "qw_autotune");
+    if (rc != QW_OK) return rc;
+    for (int r = 0; r < (runs ? 2 : 1); ++r) {
+        float ms = 0.f;
+        QW_CUDA(sim, cudaEventElapsedTime(&ms, ev[r], ev[r + 1]));
+        const double t = 1000.0 * ms / (double)(runs ? m : steps);
+        if (r == 0 || t < *us) *us = t;
+    }
+    return QW_OK;
+}
+
 extern "C" int qw_autotune(qw_sim *sim, int32_t steps, int32_t *choice, double *us_per_step)
 {
     if (!sim || steps < 1) return QW_ERR_ARG;
@@ -1845,10 +1892,10 @@ extern "C" int qw_autotune(qw_sim *sim, int32_t steps, int32_t *choice, double *
     if (pos) cand.push_back({7, QW_MODE_WALK_POS});
     double us[QW_WALK_VARIANTS];
     for (double &u : us) u = 0.0;
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    QW_CUDA(sim, cudaEventCreate(&e0));
-    QW_CUDA(sim, cudaEventCreate(&e1));
+    cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
     int rc = QW_OK;
+    for (cudaEvent_t &e : ev)
+        if (rc == QW_OK && cudaEventCreate(&e) != cudaSuccess) rc = fail(sim, QW_ERR_CUDA, "qw_autotune: cudaEventCreate");
     const int graphs = sim->opts.graphs;
     /* time the kernels themselves; the positional layout as it will run */
     for (size_t c = 0; c < cand.size() && rc == QW_OK; ++c) {
@@ -1858,20 +1905,12 @@ extern "C" int qw_autotune(qw_sim *sim, int32_t steps, int32_t *choice, double *
         sim->mode = mode;
         sim->opts.graphs = mode == QW_MODE_WALK_POS ? graphs : 0;
         sim->grid_walk = mode == QW_MODE_WALK_POS ? sim->grid_alt : qw_step_grid(sim->d, sim->fp32, mode);
-        if (mode == QW_MODE_WALK_POS) { /* the move into the layout is not timed */
-            rc = pos_prepare(sim);
-            if (rc != QW_OK) break;
-        }
-        cudaEventRecord(e0, sim->stream);
-        rc = qw_enqueue_walk_steps(sim, steps);
-        cudaEventRecord(e1, sim->stream);
-        if (rc == QW_OK) rc = check_status(sim, "qw_autotune");
-        float ms = 0.f;
-        if (rc == QW_OK && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) us[v] = 1000.0 * ms / steps;
+        if (mode == QW_MODE_WALK_POS) rc = pos_prepare(sim); /* the move into the layout is not timed */
+        if (rc == QW_OK) rc = tune_time(sim, steps, ev, &us[v]);
     }
     sim->opts.graphs = graphs;
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
+    for (cudaEvent_t e : ev)
+        if (e) cudaEventDestroy(e);
     int best = cand[0].first, best_mode = cand[0].second;
     for (const auto &cv : cand)
         if (us[cv.first] > 0.0 && (us[best] <= 0.0 || us[cv.first] < us[best])) {

@@ -1,0 +1,76 @@
+"""Host side of the C ABI (`qw_api.cpp`) without a GPU: compiled here with the host
+C++ compiler against a CUDA runtime and kernel launchers that run on the host
+(`fake_cuda/fake_cuda.cpp`), for what a sound device does not show: the autotuner's
+choice under given kernel times, and the state of the simulator after a wait
+on the device that gave up, an allocation that failed, a refused call."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2303_06890_gb300 import build as native
+from paper_2303_06890_gb300 import qwalk
+from paper_2303_06890_gb300 import workloads as wl
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(HERE, "..", "paper_2303_06890_gb300", "csrc")
+MODE = {0: 0, 1: 3, 2: 4, 3: 5, 4: 6}  # walk_variant -> kernel mode (qw_internal.h)
+GRID_WAIT, ROW_OVERFLOW, POS_FULL = 512, 1, 256
+
+
+@pytest.fixture(scope="module")
+def fake_path(tmp_path_factory):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(native.nvcc())), "include")
+    if cxx is None:
+        pytest.skip("no host C++ compiler")
+    so = str(tmp_path_factory.mktemp("hostapi") / "libfake.so")
+    subprocess.run([cxx, "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", cuda, "-I", CSRC, "-o", so,
+                    os.path.join(HERE, "fake_cuda", "fake_cuda.cpp"), os.path.join(CSRC, "qw_api.cpp")], check=True)
+    return so
+
+
+@pytest.fixture
+def fake(fake_path, monkeypatch):
+    monkeypatch.setattr(native, "LIB", fake_path)
+    monkeypatch.setattr(qwalk, "_lib", None)
+    lib = qwalk.load(build_if_missing=False)
+    for name in ("fake_live", "fake_sync_copies", "fake_map_lists", "fake_map_entries", "fake_tinits"):
+        getattr(lib, name).restype = ctypes.c_int64
+    lib.fake_word.restype = ctypes.c_ulonglong
+    lib.fake_set_step.argtypes = [ctypes.c_int, ctypes.c_double]
+    lib.fake_set_times.argtypes = [ctypes.c_double] * 4
+    lib.fake_reset()
+    yield lib
+    lib.fake_reset()
+
+
+def _b(n):
+    b = np.random.default_rng(n).standard_normal(n)
+    return b / np.linalg.norm(b)
+
+
+def _sim(n=64, s=8, **kw):
+    return qwalk.Sim(wl.random_symmetric(n, s, 1, n, n), s_pad=s, **kw)
+
+
+@pytest.mark.parametrize("steps", [1, 2, 3, 8])
+@pytest.mark.parametrize("graphs", [True, False])
+@pytest.mark.parametrize("slot,run,choice", [(20.0, 8.5, 7), (10.0, 3.5, 7), (6.0, 8.5, 4)])
+def test_autotuner_times_steps_not_first_launches(fake, steps, graphs, slot, run, choice):
+    """The fastest kernel a step is chosen whatever number of steps is asked for,
+    though each kind's first launch takes 60 us more, and a run 15 us beside
+    its steps; the state advances by the steps asked for, no more."""
+    for v, us in ((0, 40.0), (1, 38.0), (2, 45.0), (3, 44.0), (4, slot)):
+        fake.fake_set_step(MODE[v], us)
+    fake.fake_set_times(run, run, 15.0 if graphs else 0.0, 60.0)
+    with _sim(graphs=graphs) as sim:
+        sim.state_init(_b(64))
+        v, us = sim.autotune(steps)
+        assert v == choice
+        assert sim.step_stats()["steps"] == steps  # (the fake counts them for the positional layout)
+        tried = sum(u > 0.0 for u in us)
+        assert tried == 6 and abs(us[7] - run) <= (15.0 / 32 if graphs else 1e-6) + 1e-6
