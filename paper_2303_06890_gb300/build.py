@@ -30,7 +30,7 @@ def _stale(out: str, deps: list[str]) -> bool:
 
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
-    headers = [os.path.join(CSRC, f) for f in ("qw_internal.h", "qw_device.cuh", "qw_amp.cuh", "qw_pos.cuh")]
+    headers = [os.path.join(CSRC, f) for f in ("qw_internal.h", "qw_device.cuh", "qw_amp.cuh", "qw_pos.cuh", "qw_pos_norm.h")]
     headers.append(os.path.join(os.path.dirname(HERE), "include", "qwalk.h"))
     objs, procs = [], []
     for src in SOURCES:

@@ -161,7 +161,7 @@ struct qw_sim {
     void *pbuf[3] = {nullptr, nullptr, nullptr};
     size_t pbuf_bytes = 0;
     QwPosPlan pos_plan{};
-    unsigned long long *pos_words = nullptr; /* 4 barrier words, the poison flag, the p_j shares [2][grid] */
+    unsigned long long *pos_words = nullptr; /* barrier words (QW_POS_WORDS), the p_j shares [2][grid] */
     unsigned long long pos_epoch = 1; /* of the next step's barrier */
     bool pos_issued = false; /* positional steps issued since the last synchronising call */
     bool pos_built = false;
@@ -752,7 +752,7 @@ static int status_read(qw_sim *sim, const char *where)
     if (st & QW_ST_GRID_WAIT) m += " [a positional step gave up waiting for the other blocks]";
     if (pos_issued) { /* several steps share the arrays: no clean one to go back to */
         sim->has_state = sim->pos_live = false;
-        cudaMemsetAsync(sim->pos_words, 0, 5 * sizeof(unsigned long long), sim->stream);
+        cudaMemsetAsync(sim->pos_words, 0, QW_POS_WORDS * sizeof(unsigned long long), sim->stream);
         cudaStreamSynchronize(sim->stream);
         return fail(sim, QW_ERR_DEVICE_STATUS, m + "; the state is lost: initialise it again");
     }
@@ -809,8 +809,8 @@ static int launch_pos(qw_sim *sim, int64_t nsteps, int64_t qls_term, int readout
     if (nsteps > 1) {
         p.epoch = sim->pos_epoch;
         p.words = sim->pos_words;
-        p.poison = reinterpret_cast<unsigned int *>(sim->pos_words + 4);
-        p.pshare = reinterpret_cast<double *>(sim->pos_words + 5);
+        p.extra = reinterpret_cast<double *>(sim->pos_words + QW_POS_EXTRA);
+        p.pshare = reinterpret_cast<double *>(sim->pos_words + QW_POS_WORDS);
         sim->pos_epoch += (unsigned long long)nsteps;
     }
     const cudaError_t e = qw_launch_walk_pos(sim->d, sim->pos_plan, p, a, sim->fp32, sim->pos_full, sim->stream);
@@ -1251,7 +1251,7 @@ static int pos_build(qw_sim *sim)
     sim->h_b_busy.assign((size_t)ninst, 0);
     if (!sim->h_b) QW_CUDA(sim, cudaMallocHost((void **)&sim->h_b, 2 * (size_t)nrows * sizeof(double)));
     sim->pos_plan = qw_pos_plan(d, sim->fp32);
-    const size_t words = 5 + 2 * (size_t)sim->pos_plan.grid;
+    const size_t words = QW_POS_WORDS + 2 * (size_t)sim->pos_plan.grid;
     QW_CUDA(sim, dalloc(sim, &sim->pos_words, words));
     QW_CUDA(sim, cudaMemset(sim->pos_words, 0, words * sizeof(unsigned long long)));
     sim->mode_alt = d.warp_cap < 2 * d.cap_row ? QW_MODE_WALK_FUSED

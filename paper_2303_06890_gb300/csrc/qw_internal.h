@@ -161,11 +161,14 @@ struct QwPosArgs {
     int nsteps;
     int qls;                  /* QLS terms of two steps, read out on the second */
     int64_t qls_term;         /* index of the first */
-    unsigned long long epoch; /* of the first step: its barrier word is words[epoch & 3] */
-    unsigned long long *words; /* the barrier's 4 words, or null */
-    unsigned int *poison;     /* set when a block's norm share is not finite */
+    unsigned long long epoch; /* of the first step: its barrier's turn is epoch & 3 */
+    unsigned long long *words; /* [4][2]: the barrier's words; or null */
+    double *extra;            /* [4]: norm shares no word takes */
     double *pshare;           /* [2][grid]: the blocks' shares of p_j */
 };
+/* 8-byte words of the barrier's memory: words, extra (on a line of its own), then pshare */
+#define QW_POS_EXTRA 16
+#define QW_POS_WORDS 32
 struct QwScalarWords { /* 8-byte words of the simulator's scalars a kernel sets */
     unsigned long long *dst;
     int n;

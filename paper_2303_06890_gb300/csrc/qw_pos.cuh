@@ -8,6 +8,7 @@
 #include "qw_amp.cuh"
 #include "qw_device.cuh"
 #include "qw_internal.h"
+#include "qw_pos_norm.h"
 
 namespace {
 
@@ -108,65 +109,88 @@ template <> struct PosMem<double2> {
 
 /* ---- barrier over the grid, with the norm ---------------------------------- */
 /*
- * One 64-bit word per step: every block adds 1 to its count (bits 56 up) and
- * its share of the norm as a fixed-point number (bits 0 .. 55), so one atomic
- * per block is both its arrival and its term of the sum, whose value does not
- * depend on the order of arrival.  The unit is a power of two of which the
- * renormalisation target holds 2^53 to 2^54: rounding a block's share to it
- * costs 2^-55 of the target, below what the FP64 sum of the shares would.
- * Four words take turns; passing step t, block 0 clears the word of step t + 2,
- * which every block has left (it was step t - 2's).
+ * Two 64-bit words per step (qw_pos_norm.h): every block adds 1 to the count in
+ * their low 8 bits and its share of the norm above it, to one the share modulo
+ * 2^56 units, to the other its high part, so an atomic on each is both the
+ * block's arrival and its term of a sum that does not depend on the order of
+ * arrival, and that no norm carries into the count.  Without renormalisation
+ * only the first is used.  They lie side by side and are polled by one load; the
+ * second's add goes before the first's, which releases the block's stores.  A
+ * block that holds a share out of the units' range (or not finite) adds all of its
+ * own to the step's FP64 number and says so.  Four sets take turns; passing step t,
+ * block 0 clears that of step t + 2, which every block has left (it was step t - 2's).
+ * Beside one word with a lane's share rounded to 2^-54 of the target (QLS, N = 1024
+ * complex64: 4.44 us a step) the second word costs 0.1 us a step.
  */
-constexpr int kCountShift = 56;
-constexpr unsigned long long kShareMask = (1ull << kCountShift) - 1ull;
-
 struct PosNorm { /* per launch, in shared memory */
-    double unit_inv;                  /* 2^k: shares times this are in units */
-    unsigned long long target;        /* the renormalisation target in units */
-    float target_inv;                 /* 1 / target */
+    int k;                     /* units are 2^-k */
+    float s1, s2;              /* s1 s2 = 2^k */
+    unsigned long long target; /* the renormalisation target in units */
+    float target_inv;          /* 1 / target */
 };
 
-__device__ __forceinline__ void pos_norm_setup(const QwStepArgs &a, PosNorm &pn, bool series = true)
+__device__ __forceinline__ void pos_norm_setup(const QwStepArgs &a, PosNorm &pn)
 {
     const double t = *a.renorm_target;
-    int e = 0;
-    if (t > 0.0 && t < 1e300) frexp(t, &e);
-    e = max(e, -70); /* 2^(54 - e) is an FP32 number too */
-    pn.unit_inv = ldexp(1.0, 54 - e);
-    pn.target = (unsigned long long)__double2ll_rn(t > 0.0 && t < 1e300 ? t * pn.unit_inv : 0.0);
-    pn.target_inv = 0.0f;
-    if (series) pn.target_inv = pn.target ? (float)(1.0 / (double)pn.target) : 0.0f;
+    bool odd;
+    pn.k = pos_unit_exp(t);
+    pn.target = pos_units(t, pn.k, odd);
+    pn.target_inv = pn.target ? (float)(1.0 / (double)pn.target) : 0.0f;
+    /* (FP32 shares: 2^k in two factors; beyond 2^252 every non-zero share is odd) */
+    const int k = pn.k > 252 ? 252 : (pn.k < -252 ? -252 : pn.k), h = k >> 1;
+    pn.s1 = __int_as_float((127 + h) << 23);
+    pn.s2 = __int_as_float((127 + k - h) << 23);
 }
 
-/* a lane's norm share in units; poisoned (not finite, or beyond what the word
-   can sum) shares count as 0 and set the flag */
-__device__ __forceinline__ unsigned long long to_units(const Amp<double2>::Norm &n, double unit_inv, bool &bad)
+/* a lane's norm share in units */
+__device__ __forceinline__ unsigned long long to_units(const Amp<double2>::Norm &n, const PosNorm &pn, bool &odd)
 {
-    const double v = n.get() * unit_inv;
-    bad = !(v >= 0.0 && v < 0x1p54);
-    return bad ? 0ull : (unsigned long long)__double2ll_rn(v);
+    return pos_units(n.get(), pn.k, odd);
 }
-__device__ __forceinline__ unsigned long long to_units(const Amp<float2>::Norm &n, float unit_inv, bool &bad)
+__device__ __forceinline__ unsigned long long to_units(const Amp<float2>::Norm &n, const PosNorm &pn, bool &odd)
 {
-    /* the scaling by a power of two is exact; hi has 24 bits, lo is rounded
-       to a unit */
-    const float h = n.hi * unit_inv, l = n.lo * unit_inv;
-    bad = !(h >= 0.0f && h < 0x1p54f);
-    return bad ? 0ull : (unsigned long long)(__float2ll_rn(h) + __float2ll_rn(l));
+    /* the scaling by powers of two is exact; hi has 24 bits, lo is rounded to a unit */
+    const float h = n.hi * pn.s1 * pn.s2, l = n.lo * pn.s1 * pn.s2;
+    odd = !(h >= 0.0f && h < 0x1p63f);
+    return odd ? 0ull : (unsigned long long)(__float2ll_rn(h) + __float2ll_rn(l));
 }
-/* the warp's sum of values below 2^57, exact: three limbs through the integer
-   reduction */
-__device__ __forceinline__ unsigned long long warp_sum_units(unsigned long long v)
+/* Sums of shares below 2^63, exact through the integer reduction of three limbs,
+   of 22 bits and the rest: up to 512 lanes' fit 32 bits each */
+struct PosLimbs {
+    unsigned int a, b, c;
+    __device__ __forceinline__ void reduce()
+    {
+        a = __reduce_add_sync(FULL, a);
+        b = __reduce_add_sync(FULL, b);
+        c = __reduce_add_sync(FULL, c);
+    }
+    __device__ __forceinline__ unsigned long long low() const { return (unsigned long long)a + ((unsigned long long)b << 22); }
+    __device__ __forceinline__ unsigned long long fine() const { return low() + ((unsigned long long)c << 44); }
+    __device__ __forceinline__ unsigned long long coarse() const
+    {
+        return ((unsigned long long)c << (44 - kCoarseShift)) + (low() >> kCoarseShift);
+    }
+};
+__device__ __forceinline__ PosLimbs warp_sum_units(unsigned long long v)
 {
-    const unsigned a = __reduce_add_sync(FULL, (unsigned)(v & 0x3ffffffull));
-    const unsigned b = __reduce_add_sync(FULL, (unsigned)((v >> 26) & 0x3ffffffull));
-    const unsigned c = __reduce_add_sync(FULL, (unsigned)(v >> 52));
-    return (unsigned long long)a + ((unsigned long long)b << 26) + ((unsigned long long)c << 52);
+    PosLimbs l{(unsigned)(v & 0x3fffffull), (unsigned)((v >> 22) & 0x3fffffull), (unsigned)(v >> 44)};
+    l.reduce();
+    return l;
 }
 
 __device__ __forceinline__ void word_add(unsigned long long *p, unsigned long long v)
 {
     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ void word_add_relaxed(unsigned long long *p, unsigned long long v)
+{
+    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ ulonglong2 words_load(const unsigned long long *p) /* each word of its own moment */
+{
+    ulonglong2 v;
+    asm volatile("ld.acquire.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+    return v;
 }
 __device__ __forceinline__ unsigned long long word_load(const unsigned long long *p)
 {
@@ -175,20 +199,26 @@ __device__ __forceinline__ unsigned long long word_load(const unsigned long long
     return v;
 }
 
-/* The renormalisation factor of a norm of `sum` units, as 1 + c in FP32 pair
- * form (h, l) and in FP64.  sqrt(target / sum) = (1 - x)^(-1/2) with x = (target
- * - sum) / target: within 2^-20 the series to second order is exact to 2^-60
- * and needs no FP64 arithmetic (square root and division there take over a
- * thousand cycles, between every two steps); otherwise FP64. */
+/* The renormalisation factor sqrt(target / sum) of a sum of shares, as 1 + c: with x
+ * = (target - sum) / target it is (1 - x)^(-1/2), and within 2^-20 the series to
+ * second order is exact to 2^-60 and needs no FP64 arithmetic (square root and
+ * division there take over a thousand cycles, between every two steps); otherwise
+ * false, and FP64. */
 __device__ __noinline__ double pos_scale_exact(double target, double norm)
 {
     return norm > 0.0 ? sqrt(target / norm) : 1.0;
 }
-__device__ __forceinline__ bool pos_scale(const PosNorm &pn, unsigned long long sum, float &c)
+template <int FIELD>
+__device__ __forceinline__ bool pos_scale(const PosNorm &pn, unsigned long long fine, float &c) /* of a near sum */
 {
-    const float x = (float)(long long)(pn.target - sum) * pn.target_inv;
+    const float x = (float)pos_deviation<FIELD>(pn.target, fine) * pn.target_inv;
     c = fmaf(0.375f * x, x, 0.5f * x);
     return fabsf(x) < 0x1p-20f;
+}
+template <int FIELD>
+__device__ __noinline__ double pos_norm(const PosNorm &pn, unsigned long long fine, unsigned long long coarse, double extra)
+{
+    return pos_total<FIELD>(fine, coarse, extra, pn.k);
 }
 
 /* FP64 work of the read-out and of a complex128 norm, out of line: a
@@ -398,11 +428,12 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
        + 32 k); RPP units per warp (a group) */
     constexpr int SW = S > 32 ? 32 : S, SPL = S / SW, RPP = 32 / SW;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ unsigned long long part_u[kPosMaxWarps];
-    __shared__ double part_d[kPosMaxWarps];
+    __shared__ PosLimbs part_u[kPosMaxWarps]; /* the warps' shares of the norm */
+    __shared__ double part_n[kPosMaxWarps]; /* the same in FP64: of a single step, and with odd ones */
+    __shared__ double part_d[kPosMaxWarps]; /* ... of ||Y||^2 */
     __shared__ double scale_sm;
     __shared__ PosNorm pn;
-    __shared__ int flag_sm, bad_sm;
+    __shared__ int flag_sm, odd_sm;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, PW = blockDim.x >> 5;
     const bool rot_in_place = Amp<AmpT>::kRotCode && d.rot_calc;
     const AmpT zero = Amp<AmpT>::zero();
@@ -501,8 +532,8 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
     bool rescale = a.scale_in != nullptr;
     if (threadIdx.x == 0) {
         Amp<AmpT>::Scale::to_shared(rescale ? *a.scale_in : 1.0, &scale_sm);
-        if (a.renorm) pos_norm_setup(a, pn, p.words != nullptr);
-        bad_sm = 0;
+        if (a.renorm && p.words != nullptr) pos_norm_setup(a, pn);
+        odd_sm = 0;
     }
     __syncthreads();
     for (int step = 0; step < p.nsteps; ++step) {
@@ -584,11 +615,14 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
         st.take(cnt);
         __syncwarp();
         /* the warp's shares of the norm and of ||Y||^2 */
-        if (a.renorm) {
-            bool bad;
-            const unsigned long long v = warp_sum_units(to_units(nrm, pn.unit_inv, bad));
+        if (a.renorm && p.words == nullptr) {
+            const double v = nrm.warp_total();
+            if (lane == 0) part_n[warp] = v;
+        } else if (a.renorm) {
+            bool odd;
+            const PosLimbs v = warp_sum_units(to_units(nrm, pn, odd));
             if (lane == 0) part_u[warp] = v;
-            if (bad) bad_sm = 1;
+            if (odd) odd_sm = 1;
         }
         if (p.qls && readout) {
             const double pv = warp_sum(pshare);
@@ -598,47 +632,63 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
         A = O;
         const bool last = step == p.nsteps - 1;
         if (p.words == nullptr) break; /* one step: finished below by the last block */
-        unsigned long long *word = p.words + ((p.epoch + (unsigned long long)step) & 3ull);
+        const bool odd = a.renorm && odd_sm != 0;
+        if (odd) { /* (the whole block alike) */
+            const double v = nrm.warp_total();
+            if (lane == 0) part_n[warp] = v;
+            __syncthreads();
+            if (threadIdx.x == 0) odd_sm = 0;
+        }
+        const unsigned at = (unsigned)(p.epoch + (unsigned long long)step) & 3u, at2 = (at + 2u) & 3u;
         double *pshares = p.pshare + ((unsigned)(step >> 1) & 1u) * gridDim.x;
         if (warp == 0) {
-            unsigned long long share = 0;
-            if (a.renorm) share = warp_sum_units(lane < PW ? part_u[lane] : 0ull);
+            PosLimbs share{0u, 0u, 0u};
+            if (a.renorm) {
+                if (lane < PW) share = part_u[lane];
+                share.reduce();
+            }
+            double odd_share = 0.0;
+            if (odd) odd_share = warp_sum(lane < PW ? part_n[lane] : 0.0);
             if (p.qls && readout) {
                 const double ps = warp_sum(lane < PW ? part_d[lane] : 0.0);
                 if (lane == 0) __stcg(pshares + blockIdx.x, ps);
             }
             if (lane == 0) {
-                if (bad_sm || share >= 1ull << (kCountShift - 1)) { /* (the norm stays near the target) */
-                    atomicOr(p.poison, 1u);
-                    share = 0;
-                }
-                word_add(word, (1ull << kCountShift) + share);
+                unsigned long long *const word = p.words + 2 * at, *const clear = p.words + 2 * at2;
+                if (odd) atomicAdd(p.extra + at, odd_share);
+                if (a.renorm) word_add_relaxed(word + 1, ((odd ? kOddShare : share.coarse()) << kCountBits) + 1ull);
+                word_add(word, ((odd ? 0ull : share.fine()) << kCountBits) + 1ull);
                 bool ok = true;
                 if (!last || blockIdx.x == 0) {
-                    unsigned long long w = 0;
+                    ulonglong2 w = {0ull, 0ull};
                     ok = false;
                     for (int polls = 0; polls < (1 << 22) && !ok; ++polls) {
-                        w = word_load(word);
-                        ok = (w >> kCountShift) == (unsigned long long)gridDim.x;
+                        if (a.renorm) w = words_load(word);
+                        else w.x = w.y = word_load(word);
+                        ok = (w.x & kCountMask) == gridDim.x && (w.y & kCountMask) == gridDim.x;
                     }
                     if (!ok) atomicOr(a.status, QW_ST_GRID_WAIT);
-                    if (ok && blockIdx.x == 0) p.words[(p.epoch + (unsigned long long)step + 2ull) & 3ull] = 0ull;
-                    double fac = 1.0;
+                    if (ok && blockIdx.x == 0) {
+                        clear[0] = clear[1] = 0ull;
+                        if (a.renorm) p.extra[at2] = 0.0;
+                    }
+                    double fac = 1.0, norm = 0.0;
                     if (a.renorm) {
-                        const unsigned long long sum = w & kShareMask;
+                        const unsigned long long fine = w.x >> kCountBits, coarse = w.y >> kCountBits;
                         float c;
-                        if (pos_scale(pn, sum, c)) {
+                        const bool near = pos_near(pn.target, coarse) && pos_scale<kGridField>(pn, fine, c);
+                        if (!near || last)
+                            norm = pos_norm<kGridField>(pn, fine, coarse, coarse >= kOddShare ? __ldcg(p.extra + at) : 0.0);
+                        if (near) {
                             Amp<AmpT>::scale_one_plus(c, &scale_sm);
                             if (last) fac = 1.0 + (double)c;
                         } else {
-                            const bool nan = *(volatile unsigned int *)p.poison != 0u;
-                            fac = nan ? 1.0 : pos_scale_exact(*a.renorm_target, (double)sum / pn.unit_inv);
+                            fac = pos_scale_exact(*a.renorm_target, norm);
                             Amp<AmpT>::Scale::to_shared(fac, &scale_sm);
                         }
                     }
                     if (last && ok) {
-                        *p.poison = 0u;
-                        *a.norm_out = a.renorm ? (double)(w & kShareMask) / pn.unit_inv : 0.0;
+                        *a.norm_out = norm;
                         if (a.scale_out) *a.scale_out = fac;
                         if (a.steps_done) *a.steps_done += p.nsteps;
                         if (a.stats) a.stats[QW_STAT_STEPS] += p.nsteps;
@@ -665,12 +715,12 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
     st.flush(a);
     if (p.words != nullptr) return;
 
-    /* one step: the block's share of the norm, the last block reduces */
+    /* one step: the block's share of the norm, the last block reduces (FP64) */
     if (warp == 0) {
-        unsigned long long share = 0;
-        if (a.renorm) share = warp_sum_units(lane < PW ? part_u[lane] : 0ull);
+        double share = 0.0;
+        if (a.renorm) share = warp_sum(lane < PW ? part_n[lane] : 0.0);
         if (lane == 0) {
-            a.partials[blockIdx.x] = bad_sm ? -1.0 : (double)share;
+            a.partials[blockIdx.x] = share;
             __threadfence();
             const unsigned prev = atomicAdd(a.done_ctr, 1u);
             flag_sm = prev == gridDim.x - 1;
@@ -678,22 +728,15 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
         __syncwarp();
         if (!flag_sm) return;
         __threadfence();
-        double v = 0.0;
-        bool bad = false;
+        double norm = 0.0;
         if (a.renorm) {
-            for (unsigned bb = lane; bb < gridDim.x; bb += 32) {
-                const double w = __ldcg(a.partials + bb);
-                bad = bad || w < 0.0;
-                v += w;
-            }
-            v = warp_sum(v);
-            bad = __any_sync(FULL, bad);
+            for (unsigned bb = lane; bb < gridDim.x; bb += 32) norm += __ldcg(a.partials + bb);
+            norm = warp_sum(norm);
         }
         if (lane == 0) {
             if (*(volatile int32_t *)a.status == 0) {
-                const double norm = a.renorm ? v / pn.unit_inv : 0.0;
                 *a.norm_out = norm;
-                if (a.scale_out) *a.scale_out = a.renorm && !bad ? pos_scale_exact(*a.renorm_target, norm) : 1.0;
+                if (a.scale_out) *a.scale_out = a.renorm ? pos_scale_exact(*a.renorm_target, norm) : 1.0;
                 if (a.steps_done) *a.steps_done += 1;
                 if (a.stats) a.stats[QW_STAT_STEPS] += 1;
             }
@@ -721,7 +764,8 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
  * slots; a destination is its block (bits 20 .. 23) and that
  * index (bits 0 .. 19), with the flags of k_walk_pos above.  A buffer written in step
  * t was last read in step t - 1, before the barrier that every block passed to
- * start t; sums take turns three by three, cleared two steps ahead.
+ * start t; the norm's sums (qw_pos_norm.h, both words as wide as they are) take
+ * turns three by three, cleared two steps ahead.
  */
 constexpr int kPosCluster = 16; /* blocks of a cluster, at most (more than 8: opt-in) */
 
@@ -749,13 +793,13 @@ __device__ __forceinline__ void peer_store(uint32_t a, double v)
 {
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
 }
-__device__ __forceinline__ void peer_store(uint32_t a, uint32_t v)
-{
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
 __device__ __forceinline__ void peer_add(uint32_t a, unsigned long long v)
 {
     asm volatile("red.relaxed.cluster.shared::cluster.add.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
+}
+__device__ __forceinline__ void peer_add(uint32_t a, double v)
+{
+    asm volatile("red.relaxed.cluster.shared::cluster.add.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
 }
 __device__ __forceinline__ void cluster_sync()
 {
@@ -825,9 +869,9 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_cluster(QwSimDev 
     typedef typename Amp<AmpT>::RotVal RotVal;
     constexpr int SW = S > 32 ? 32 : S, SPL = S / SW, RPP = 32 / SW;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ unsigned long long nsum[3];
+    __shared__ unsigned long long nsum[2][3]; /* fine, coarse */
+    __shared__ double nodd[3];                /* the odd shares */
     __shared__ double pshares[2][kPosCluster * kPosMaxWarps];
-    __shared__ uint32_t poison;
     __shared__ PosNorm pn;
     if (*(volatile int32_t *)a.status != 0) return; /* after a failed step: nothing (every block alike) */
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, PW = blockDim.x >> 5;
@@ -892,13 +936,15 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_cluster(QwSimDev 
         load(slots + at, n * S + x, x < X);
     }
     if (threadIdx.x == 0) {
-        nsum[0] = nsum[1] = nsum[2] = 0ull;
-        poison = 0u;
+        for (int t = 0; t < 3; ++t) {
+            nsum[0][t] = nsum[1][t] = 0ull;
+            nodd[t] = 0.0;
+        }
         if (a.renorm) pos_norm_setup(a, pn);
     }
     const uint32_t buf_addr = smem_addr(smem);
     const uint32_t peer = lane < CL ? lane : 0u; /* the block this lane adds the warp's norm to */
-    const uint32_t sum_peer = peer_addr(smem_addr(nsum), peer), poison_peer = peer_addr(smem_addr(&poison), peer);
+    const uint32_t sum_peer = peer_addr(smem_addr(nsum), peer), odd_peer = peer_addr(smem_addr(nodd), peer);
     auto send = [&](uint32_t out, uint32_t to, const Entry<AmpT> &o) { /* out: the buffer's own address */
         Buf::send(peer_addr(out, (to >> 20) & 15u), E, to & 0xfffffu, o);
     };
@@ -909,8 +955,6 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_cluster(QwSimDev 
     typename Amp<AmpT>::Scale scale(rescale ? *a.scale_in : 1.0);
     double coef = p.qls ? __ldg(a.qls_coefs + p.qls_term) : 0.0, coef_next = 0.0;
     const double unit_of = d.inv_sqrt_s * (0.5 * S); /* u is scaled by 2 / s */
-    double fac = 1.0;
-    unsigned long long sum_u = 0ull;
     cluster_sync(); /* every block's state, tables and sums are there */
     for (int step = 0; step < p.nsteps; ++step) {
         const unsigned char *A = smem + (size_t)(step & 1) * buf_bytes;
@@ -978,12 +1022,15 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_cluster(QwSimDev 
         const uint32_t turn = (uint32_t)step % 3u;
         const uint32_t who = last ? 0u : (uint32_t)(step >> 1) % CL;
         if (a.renorm) {
-            bool bad;
-            unsigned long long v = warp_sum_units(to_units(nrm, pn.unit_inv, bad));
-            bad = __any_sync(FULL, bad) || v >= 1ull << 55; /* (the norm stays near the target) */
+            bool odd;
+            const PosLimbs v = warp_sum_units(to_units(nrm, pn, odd));
+            odd = __any_sync(FULL, odd);
+            double total = 0.0;
+            if (odd) total = __shfl_sync(FULL, nrm.warp_total(), 0);
             if (lane < CL) {
-                peer_add(sum_peer + 8u * turn, bad ? 0ull : v);
-                if (bad) peer_store(poison_peer, 1u);
+                peer_add(sum_peer + 8u * turn, odd ? 0ull : v.fine());
+                peer_add(sum_peer + 24u + 8u * turn, odd ? kOddShare : v.coarse());
+                if (odd) peer_add(odd_peer + 8u * turn, total);
             }
         }
         double *const ps = pshares[(step >> 1) & 1];
@@ -993,16 +1040,16 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_cluster(QwSimDev 
         }
         cluster_sync();
         if (a.renorm) {
-            sum_u = nsum[turn];
-            if (threadIdx.x == 0) nsum[(turn + 2u) % 3u] = 0ull;
-            float c;
-            if (pos_scale(pn, sum_u, c)) {
-                scale = Amp<AmpT>::scale_near_one(c);
-                if (last) fac = 1.0 + (double)c;
-            } else {
-                fac = *(volatile uint32_t *)&poison ? 1.0 : pos_scale_exact(*a.renorm_target, (double)sum_u / pn.unit_inv);
-                scale = typename Amp<AmpT>::Scale(fac);
+            if (threadIdx.x == 0) {
+                const uint32_t next = (turn + 2u) % 3u;
+                nsum[0][next] = nsum[1][next] = 0ull;
+                nodd[next] = 0.0;
             }
+            const unsigned long long fine = nsum[0][turn], coarse = nsum[1][turn];
+            float c;
+            if (pos_near(pn.target, coarse) && pos_scale<kClusterField>(pn, fine, c)) scale = Amp<AmpT>::scale_near_one(c);
+            else scale = typename Amp<AmpT>::Scale(
+                     pos_scale_exact(*a.renorm_target, pos_norm<kClusterField>(pn, fine, coarse, nodd[turn])));
         }
         rescale = a.renorm != 0;
         if (readout) coef = coef_next;
@@ -1037,7 +1084,15 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_cluster(QwSimDev 
         if (x < X) store(slots + (k * PW + warp) * 32 + lane, n * S + x);
     }
     if (rank == 0 && threadIdx.x == 0) {
-        *a.norm_out = a.renorm ? (double)sum_u / pn.unit_inv : 0.0;
+        double fac = 1.0, norm = 0.0;
+        if (a.renorm) {
+            const uint32_t turn = (uint32_t)(p.nsteps - 1) % 3u;
+            const unsigned long long fine = nsum[0][turn], coarse = nsum[1][turn];
+            float c;
+            norm = pos_norm<kClusterField>(pn, fine, coarse, nodd[turn]);
+            fac = pos_near(pn.target, coarse) && pos_scale<kClusterField>(pn, fine, c) ? 1.0 + (double)c : pos_scale_exact(*a.renorm_target, norm);
+        }
+        *a.norm_out = norm;
         if (a.scale_out) *a.scale_out = fac;
         if (a.steps_done) *a.steps_done += p.nsteps;
         if (a.stats) a.stats[QW_STAT_STEPS] += p.nsteps;

@@ -247,12 +247,12 @@ cudaError_t qw_launch_step(const QwSimDev &, const QwBufDev &, const QwBufDev &,
 
 static cudaError_t walk_pos(const QwPosArgs &p, const QwStepArgs &a)
 {
-    if (p.words) std::memcpy(F.words, p.words, 5 * sizeof(unsigned long long));
+    if (p.words) std::memcpy(F.words, p.words, 8 * sizeof(unsigned long long));
     if (!F.capturing && *a.status == 0) {
         if (F.give_up > 0) {
             --F.give_up;
             *a.status |= QW_ST_GRID_WAIT;
-            if (p.words) p.words[p.epoch & 3] = 7ull; /* some blocks had arrived */
+            if (p.words) p.words[2 * (p.epoch & 3)] = 7ull; /* some blocks had arrived */
         } else {
             *a.steps_done += p.nsteps;
             a.stats[QW_STAT_STEPS] += (unsigned long long)p.nsteps;
