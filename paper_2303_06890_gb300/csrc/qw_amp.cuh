@@ -109,6 +109,7 @@ template <> struct Amp<double2> {
         __device__ T apply(T a) const { return scale_c128(a, s); }
         /* staged once per block (the factor in 8 bytes of shared memory) */
         __device__ static void to_shared(double v, double *buf) { buf[0] = v; }
+        __device__ void store(double *buf) const { buf[0] = s; }
         __device__ static Scale from_shared(const double *buf) { return Scale(buf[0]); }
     };
     typedef double2 RotVal; /* (sqrt|a|, sqrt(1-|a|)) */
@@ -153,8 +154,6 @@ template <> struct Amp<double2> {
     }
     __device__ static float rot_f(RotVal t) { return approx(t.x); }
     __device__ static float rot_g(RotVal t) { return approx(t.y); }
-    __device__ static void scale_one_plus(float c, double *buf) { buf[0] = 1.0 + (double)c; }
-    __device__ static Scale scale_near_one(float c) { return Scale(1.0 + (double)c); }
     static constexpr float kApproxErr = 1.0f / 131072.0f; /* 2^-17 of the terms' magnitudes */
 };
 
@@ -323,6 +322,12 @@ template <> struct Amp<float2> {
             float *f = reinterpret_cast<float *>(buf);
             split(v, f[0], f[1]);
         }
+        __device__ void store(double *buf) const
+        {
+            float *f = reinterpret_cast<float *>(buf);
+            f[0] = sh;
+            f[1] = sl;
+        }
         __device__ static Scale from_shared(const double *buf)
         {
             const float *f = reinterpret_cast<const float *>(buf);
@@ -400,13 +405,6 @@ template <> struct Amp<float2> {
     __device__ static float inf_norm(T a) { return fmaxf(fabsf(a.x), fabsf(a.y)); }
     __device__ static float rot_f(RotVal t) { return t.x; }
     __device__ static float rot_g(RotVal t) { return t.z; }
-    __device__ static void scale_one_plus(float c, double *buf)
-    {
-        float *f = reinterpret_cast<float *>(buf);
-        f[0] = 1.0f;
-        f[1] = c;
-    }
-    __device__ static Scale scale_near_one(float c) { return Scale(1.0f, c); }
     static constexpr float kApproxErr = 1.0f / 524288.0f; /* 2^-19 of the terms' magnitudes */
 };
 

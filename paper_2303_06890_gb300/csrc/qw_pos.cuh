@@ -120,13 +120,13 @@ template <> struct PosMem<double2> {
  * own to the step's FP64 number and says so.  Four sets take turns; passing step t,
  * block 0 clears that of step t + 2, which every block has left (it was step t - 2's).
  * Beside one word with a lane's share rounded to 2^-54 of the target (QLS, N = 1024
- * complex64: 4.44 us a step) the second word costs 0.1 us a step.
+ * complex64: 4.44 us a step) the second word costs 0.05 us a step.
  */
 struct PosNorm { /* per launch, in shared memory */
     int k;                     /* units are 2^-k */
     float s1, s2;              /* s1 s2 = 2^k */
     unsigned long long target; /* the renormalisation target in units */
-    float target_inv;          /* 1 / target */
+    float inv_h, inv_l;        /* 2^24 / target */
 };
 
 __device__ __forceinline__ void pos_norm_setup(const QwStepArgs &a, PosNorm &pn)
@@ -135,7 +135,9 @@ __device__ __forceinline__ void pos_norm_setup(const QwStepArgs &a, PosNorm &pn)
     bool odd;
     pn.k = pos_unit_exp(t);
     pn.target = pos_units(t, pn.k, odd);
-    pn.target_inv = pn.target ? (float)(1.0 / (double)pn.target) : 0.0f;
+    const double inv = pn.target ? 16777216.0 / (double)pn.target : 0.0;
+    pn.inv_h = (float)inv;
+    pn.inv_l = (float)(inv - (double)pn.inv_h);
     /* (FP32 shares: 2^k in two factors; beyond 2^252 every non-zero share is odd) */
     const int k = pn.k > 252 ? 252 : (pn.k < -252 ? -252 : pn.k), h = k >> 1;
     pn.s1 = __int_as_float((127 + h) << 23);
@@ -199,21 +201,25 @@ __device__ __forceinline__ unsigned long long word_load(const unsigned long long
     return v;
 }
 
-/* The renormalisation factor sqrt(target / sum) of a sum of shares, as 1 + c: with x
- * = (target - sum) / target it is (1 - x)^(-1/2), and within 2^-20 the series to
- * second order is exact to 2^-60 and needs no FP64 arithmetic (square root and
- * division there take over a thousand cycles, between every two steps); otherwise
- * false, and FP64. */
+/* The renormalisation factor sqrt(target / sum) between two steps of a run, from a sum
+ * near the target, where FP32 arithmetic gives it as well as FP64's does: complex64,
+ * which applies it as a float pair, within 2^-14 (pos_factor_pair); complex128 where
+ * x = (target - sum) / target is below 2^-30 (what rounding alone leaves is 2^-50),
+ * as 1 + x / 2, off by 2^-54 at most before it is rounded to FP64.  Otherwise false,
+ * and pos_scale_exact; that too for the factor a launch leaves behind. */
 __device__ __noinline__ double pos_scale_exact(double target, double norm)
 {
     return norm > 0.0 ? sqrt(target / norm) : 1.0;
 }
-template <int FIELD>
-__device__ __forceinline__ bool pos_scale(const PosNorm &pn, unsigned long long fine, float &c) /* of a near sum */
+__device__ __forceinline__ bool pos_scale(const PosNorm &pn, int64_t dev, Amp<float2>::Scale &s)
 {
-    const float x = (float)pos_deviation<FIELD>(pn.target, fine) * pn.target_inv;
-    c = fmaf(0.375f * x, x, 0.5f * x);
-    return fabsf(x) < 0x1p-20f;
+    return pos_factor_pair(dev, pn.inv_h, pn.inv_l, s.sh, s.sl);
+}
+__device__ __forceinline__ bool pos_scale(const PosNorm &pn, int64_t dev, Amp<double2>::Scale &s)
+{
+    const float x = (float)dev * (pn.inv_h * 0x1p-24f);
+    s.s = 1.0 + (double)(0.5f * x);
+    return fabsf(x) < 0x1p-30f;
 }
 template <int FIELD>
 __device__ __noinline__ double pos_norm(const PosNorm &pn, unsigned long long fine, unsigned long long coarse, double extra)
@@ -675,14 +681,11 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_pos(QwSimDev d, Q
                     double fac = 1.0, norm = 0.0;
                     if (a.renorm) {
                         const unsigned long long fine = w.x >> kCountBits, coarse = w.y >> kCountBits;
-                        float c;
-                        const bool near = pos_near(pn.target, coarse) && pos_scale<kGridField>(pn, fine, c);
-                        if (!near || last)
-                            norm = pos_norm<kGridField>(pn, fine, coarse, coarse >= kOddShare ? __ldcg(p.extra + at) : 0.0);
-                        if (near) {
-                            Amp<AmpT>::scale_one_plus(c, &scale_sm);
-                            if (last) fac = 1.0 + (double)c;
+                        typename Amp<AmpT>::Scale f(1.0);
+                        if (!last && pos_near(pn.target, coarse) && pos_scale(pn, pos_deviation<kGridField>(pn.target, fine), f)) {
+                            f.store(&scale_sm);
                         } else {
+                            norm = pos_norm<kGridField>(pn, fine, coarse, coarse >= kOddShare ? __ldcg(p.extra + at) : 0.0);
                             fac = pos_scale_exact(*a.renorm_target, norm);
                             Amp<AmpT>::Scale::to_shared(fac, &scale_sm);
                         }
@@ -1046,10 +1049,9 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_cluster(QwSimDev 
                 nodd[next] = 0.0;
             }
             const unsigned long long fine = nsum[0][turn], coarse = nsum[1][turn];
-            float c;
-            if (pos_near(pn.target, coarse) && pos_scale<kClusterField>(pn, fine, c)) scale = Amp<AmpT>::scale_near_one(c);
-            else scale = typename Amp<AmpT>::Scale(
-                     pos_scale_exact(*a.renorm_target, pos_norm<kClusterField>(pn, fine, coarse, nodd[turn])));
+            if (!pos_near(pn.target, coarse) || !pos_scale(pn, pos_deviation<kClusterField>(pn.target, fine), scale))
+                scale = typename Amp<AmpT>::Scale(
+                    pos_scale_exact(*a.renorm_target, pos_norm<kClusterField>(pn, fine, coarse, nodd[turn])));
         }
         rescale = a.renorm != 0;
         if (readout) coef = coef_next;
@@ -1087,10 +1089,8 @@ __global__ void __launch_bounds__(kPosMaxWarps * 32, 1) k_walk_cluster(QwSimDev 
         double fac = 1.0, norm = 0.0;
         if (a.renorm) {
             const uint32_t turn = (uint32_t)(p.nsteps - 1) % 3u;
-            const unsigned long long fine = nsum[0][turn], coarse = nsum[1][turn];
-            float c;
-            norm = pos_norm<kClusterField>(pn, fine, coarse, nodd[turn]);
-            fac = pos_near(pn.target, coarse) && pos_scale<kClusterField>(pn, fine, c) ? 1.0 + (double)c : pos_scale_exact(*a.renorm_target, norm);
+            norm = pos_norm<kClusterField>(pn, nsum[0][turn], nsum[1][turn], nodd[turn]);
+            fac = pos_scale_exact(*a.renorm_target, norm);
         }
         *a.norm_out = norm;
         if (a.scale_out) *a.scale_out = fac;

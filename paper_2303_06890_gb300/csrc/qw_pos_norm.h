@@ -19,6 +19,7 @@
  * above them, so what they carry out of the word is lost, not counted.
  */
 #pragma once
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -87,6 +88,28 @@ QW_HD bool pos_near(uint64_t target, uint64_t coarse)
 template <int FIELD> QW_HD int64_t pos_deviation(uint64_t target, uint64_t fine) /* target - sum */
 {
     return (int64_t)((target - fine) << (64 - FIELD)) >> (64 - FIELD);
+}
+
+/* The factor sqrt(target / sum) = (1 - x)^(-1/2), x = dev / target, as a float pair h +
+ * l, in FP32 alone (square root and division in FP64 take over a thousand cycles on
+ * the device, between every two steps).  |x| < 2^-14 or false.  inv_h + inv_l:
+ * 2^24 / target.  x = p + e within 2^-46 of itself; the series' terms beyond the
+ * third are below 2^-57, its square and cube within 2^-50; h is 1 + p / 2 rounded,
+ * with what that leaves out and the rest in l: within 2^-48 in all, what the
+ * pair of a correctly rounded factor is. */
+QW_HD bool pos_factor_pair(int64_t dev, float inv_h, float inv_l, float &h, float &l)
+{
+    const int64_t top = dev >> 24;
+    if (top < -(1 << 23) || top >= 1 << 23) return false;
+    const float d = (float)(int)top, low = (float)(int)(dev & 0xffffff) * (1.0f / 16777216.0f);
+    const float p = d * inv_h;
+    float e = fmaf(d, inv_h, -p);
+    e = fmaf(d, inv_l, e);
+    e = fmaf(low, inv_h, e);
+    const float c = 0.5f * p;
+    h = 1.0f + c;
+    l = (c - (h - 1.0f)) + fmaf(p * p, fmaf(0.3125f, p, 0.375f), 0.5f * e);
+    return true;
 }
 
 /* v 2^e, e of any size, v a finite number */

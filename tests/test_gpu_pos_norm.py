@@ -1,6 +1,8 @@
 """The renormalisation of the positional layout's runs (over the grid, and on one
 cluster) against its single steps, whose norm is an FP64 sum: for a norm many
 times the target, and for targets far from 1."""
+import math
+
 import numpy as np
 import pytest
 
@@ -72,3 +74,21 @@ def test_complex64_renormalises_at_small_scale(n, s):
         out.append(sim.measure_register("j", n) / c**2)
         sim.close()
     assert np.abs(out[0] - out[1]).max() <= 1e-5 * out[0].max() and (np.abs(out[0] - out[1]) <= 1e-5 * out[0] + 1e-9).all()
+
+
+@pytest.mark.parametrize("n,s", [(100, 8), (900, 8)])
+@pytest.mark.parametrize("tau", [3e-5, 1e-4, 3e-4, 1e-3, 3e-3])
+def test_complex128_factor_is_fp64(n, s, tau):
+    """Steps whose pruning takes 1e-9 to 1e-3 of the norm: the state's norm is the
+    target's again to FP64.  A bin is a sum of at most 30 squares (5 roundings
+    deep), their sum 10 deep, the norm and the factor 4 roundings, squared: 2^-53 each,
+    30 in all at most."""
+    m = wl.random_symmetric(n, s, 1, (3 * n * s) // 8, n)
+    b = _b(n, 5)
+    for graphs in (True, False):
+        sim = qwalk.Sim(m, s_pad=s, walk_variant=7, renorm=1, prune_tau=tau, graphs=graphs)
+        sim.state_init(b)
+        for steps in (3, 4, 5):
+            sim.enqueue_walk_steps(steps)
+            assert abs(math.fsum(sim.measure_register("j", n)) / math.fsum(b * b) - 1.0) <= 30 * 2.0**-53
+        sim.close()

@@ -8,6 +8,7 @@ import math
 import os
 import shutil
 import subprocess
+from decimal import Decimal, getcontext
 from fractions import Fraction
 
 import numpy as np
@@ -22,6 +23,7 @@ int unit_exp(double t) { return pos_unit_exp(t); }
 uint64_t units(double v, int k, int *odd) { bool o; const uint64_t u = pos_units(v, k, o); *odd = o; return u; }
 int deviation56(uint64_t t, uint64_t f, uint64_t c, int64_t *d) { *d = pos_deviation<56>(t, f); return pos_near(t, c); }
 int deviation64(uint64_t t, uint64_t f, uint64_t c, int64_t *d) { *d = pos_deviation<64>(t, f); return pos_near(t, c); }
+int factor(int64_t dev, float ih, float il, float *h, float *l) { return pos_factor_pair(dev, ih, il, *h, *l); }
 double total56(uint64_t f, uint64_t c, double x, int k) { return pos_total<56>(f, c, x, k); }
 double total64(uint64_t f, uint64_t c, double x, int k) { return pos_total<64>(f, c, x, k); }
 }
@@ -41,6 +43,8 @@ def lib(tmp_path_factory):
     u64, i64, f64, i32 = ctypes.c_uint64, ctypes.c_int64, ctypes.c_double, ctypes.c_int
     lib.unit_exp.argtypes = [f64]
     lib.units.argtypes, lib.units.restype = [f64, i32, ctypes.POINTER(i32)], u64
+    f32 = ctypes.c_float
+    lib.factor.argtypes = [i64, f32, f32, ctypes.POINTER(f32), ctypes.POINTER(f32)]
     for n in (56, 64):
         getattr(lib, f"deviation{n}").argtypes = [u64, u64, u64, ctypes.POINTER(i64)]
         f = getattr(lib, f"total{n}")
@@ -144,3 +148,24 @@ def test_a_lane_beyond_the_integers_is_summed_in_fp64(lib):
     v[2, 1, 0] = math.nan
     fine, coarse, extra, _ = _sums(lib, v, k, 56)
     assert math.isnan(lib.total56(fine, coarse, extra, k))
+
+
+@pytest.mark.parametrize("target", [2**61, 2**61 + 12345678901, 3 * 2**60 + 7, 2**62 - 1])
+def test_factor_as_a_float_pair(lib, target):
+    """h + l is sqrt(target / sum) to 2^-48, h its rounding to FP32 or a neighbour, up to
+    2^-14 from the target (in 60-digit decimal arithmetic)."""
+    getcontext().prec = 60
+    rng = np.random.default_rng(target % 1000)
+    inv = 2.0**24 / target
+    ih = np.float32(inv)
+    il = np.float32(inv - float(ih))
+    devs = [0, 1, -1, 2**24, 2**24 - 1, -2**24, 2**47 - 1, -2**47]
+    devs += [int(s * 2.0**e) for e in rng.uniform(0, 47, 3000) for s in (1, -1)]
+    h, l = ctypes.c_float(), ctypes.c_float()
+    for dev in devs:
+        assert lib.factor(dev, ih, il, ctypes.byref(h), ctypes.byref(l))
+        want = (Decimal(target) / Decimal(target - dev)).sqrt()
+        assert abs(Decimal(h.value) + Decimal(l.value) - want) <= Decimal(2) ** -48
+        assert abs(l.value) <= 2.0**-23
+    for dev in (2**47, -2**47 - 1, 2**54):
+        assert not lib.factor(dev, ih, il, ctypes.byref(h), ctypes.byref(l))
