@@ -9,6 +9,7 @@
 #define QW_AMP_CUH
 
 #include "qw_device.cuh"
+#include "qw_pos_norm.h"
 
 namespace {
 
@@ -294,22 +295,10 @@ template <> struct Amp<float2> {
         return __fadd_rn(__fmul_rn(a.x, a.x), __fmul_rn(a.y, a.y)) > d.tau2f;
     }
     struct Scale { /* the FP64 factor as a float pair, applied with one rounding;
-                      within 2^-12 of 1 (always, but after an unusual pruning) as
-                      1 + sl, which takes one FMA */
+                      where its high part is 1 that takes one FMA */
         float sh, sl;
-        __device__ explicit Scale(double v) { split(v, sh, sl); }
+        __device__ explicit Scale(double v) { factor_split(v, sh, sl); }
         __device__ Scale(float h, float l) : sh(h), sl(l) {}
-        __device__ static void split(double v, float &h, float &l)
-        {
-            const double c = v - 1.0;
-            if (fabs(c) < 1.0 / 4096.0) {
-                h = 1.0f;
-                l = (float)c;
-            } else {
-                h = (float)v;
-                l = (float)(v - (double)h);
-            }
-        }
         __device__ T apply(T a) const
         {
             if (sh == 1.0f) return make_float2(__fmaf_rn(a.x, sl, a.x), __fmaf_rn(a.y, sl, a.y));
@@ -320,7 +309,7 @@ template <> struct Amp<float2> {
         __device__ static void to_shared(double v, double *buf)
         {
             float *f = reinterpret_cast<float *>(buf);
-            split(v, f[0], f[1]);
+            factor_split(v, f[0], f[1]);
         }
         __device__ void store(double *buf) const
         {

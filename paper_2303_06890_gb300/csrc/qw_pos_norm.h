@@ -6,8 +6,9 @@
  * A share is a number of units, of which the renormalisation target holds 2^61
  * to 2^62, whatever its exponent: a lane's rounding is 2^-62 of the target, so
  * that the sum over 78 000 lanes is off by 2^-54 of it in the mean (2^-46 at
- * most), as an FP64 sum of them is.  Sums of shares are exact, so they do not depend on the order of
- * arrival.  A sum travels as two words that are both added to:
+ * most), as an FP64 sum of them is.  Sums of shares are exact, so they do not
+ * depend on the order of arrival.  A sum travels as two words that are both added
+ * to:
  *   fine    the sum modulo 2^FIELD units,
  *   coarse  the sum of the shares' parts above 2^42 units (each cut down), and
  *           2^48 for every share that is kept out of the integer sums because it
@@ -88,6 +89,14 @@ QW_HD bool pos_near(uint64_t target, uint64_t coarse)
 template <int FIELD> QW_HD int64_t pos_deviation(uint64_t target, uint64_t fine) /* target - sum */
 {
     return (int64_t)((target - fine) << (64 - FIELD)) >> (64 - FIELD);
+}
+
+/* A factor as a float pair, 49 significant bits: h its rounding to FP32 (1 wherever it
+ * is within 2^-25 of that, as a step's renormalisation mostly is), l the rest. */
+QW_HD void factor_split(double v, float &h, float &l)
+{
+    h = (float)v;
+    l = (float)(v - (double)h);
 }
 
 /* The factor sqrt(target / sum) = (1 - x)^(-1/2), x = dev / target, as a float pair h +

@@ -24,6 +24,7 @@ uint64_t units(double v, int k, int *odd) { bool o; const uint64_t u = pos_units
 int deviation56(uint64_t t, uint64_t f, uint64_t c, int64_t *d) { *d = pos_deviation<56>(t, f); return pos_near(t, c); }
 int deviation64(uint64_t t, uint64_t f, uint64_t c, int64_t *d) { *d = pos_deviation<64>(t, f); return pos_near(t, c); }
 int factor(int64_t dev, float ih, float il, float *h, float *l) { return pos_factor_pair(dev, ih, il, *h, *l); }
+void split(double v, float *h, float *l) { factor_split(v, *h, *l); }
 double total56(uint64_t f, uint64_t c, double x, int k) { return pos_total<56>(f, c, x, k); }
 double total64(uint64_t f, uint64_t c, double x, int k) { return pos_total<64>(f, c, x, k); }
 }
@@ -44,6 +45,7 @@ def lib(tmp_path_factory):
     lib.unit_exp.argtypes = [f64]
     lib.units.argtypes, lib.units.restype = [f64, i32, ctypes.POINTER(i32)], u64
     f32 = ctypes.c_float
+    lib.split.argtypes = [f64, ctypes.POINTER(f32), ctypes.POINTER(f32)]
     lib.factor.argtypes = [i64, f32, f32, ctypes.POINTER(f32), ctypes.POINTER(f32)]
     for n in (56, 64):
         getattr(lib, f"deviation{n}").argtypes = [u64, u64, u64, ctypes.POINTER(i64)]
@@ -169,3 +171,13 @@ def test_factor_as_a_float_pair(lib, target):
         assert abs(l.value) <= 2.0**-23
     for dev in (2**47, -2**47 - 1, 2**54):
         assert not lib.factor(dev, ih, il, ctypes.byref(h), ctypes.byref(l))
+
+
+def test_a_factor_keeps_48_bits(lib):
+    """The float pair a factor is applied as: 2^-48 of it at any distance from 1."""
+    h, l = ctypes.c_float(), ctypes.c_float()
+    rng = np.random.default_rng(0)
+    for v in [1.0, 1.0 + 2.0**-30, *(1.0 + s * 2.0**-e for e in rng.uniform(1, 50, 2000) for s in (1, -1)), 1e-3, 700.3]:
+        lib.split(v, ctypes.byref(h), ctypes.byref(l))
+        assert abs(Fraction(h.value) + Fraction(l.value) - Fraction(v)) <= Fraction(v) / 2**48
+        assert h.value == np.float32(v)
