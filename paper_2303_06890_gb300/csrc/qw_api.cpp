@@ -2335,7 +2335,17 @@ extern "C" int qw_state_import(qw_sim *sim, int32_t key_words, const uint64_t *k
     if (rc != QW_OK) return rc;
     sim->has_state = true;
     sim->fresh_T = false;
+    /* each instance's share of the target, which setting one of them again replaces */
     for (auto &v : sim->init_norm2) v = 0.0;
+    if (sim->d.ninst == 1) sim->init_norm2[0] = norm2;
+    else {
+        const int at = (18 + 4 * nb) >> 6, off = (18 + 4 * nb) & 63; /* the instance's 16 bits */
+        for (int64_t i = 0; i < count; ++i) {
+            const uint64_t *w = keys + (size_t)i * (size_t)key_words + at;
+            const uint64_t inst = w[0] >> off | (off > 48 ? w[1] << (64 - off) : 0ull);
+            sim->init_norm2[(size_t)(inst & 0xffffull)] += amps[2 * i] * amps[2 * i] + amps[2 * i + 1] * amps[2 * i + 1];
+        }
+    }
     return QW_OK;
 }
 

@@ -35,6 +35,7 @@ struct Fake {
     int capturing = 0;
     unsigned long long words[8] = {0}; /* the barrier words a positional run started on */
     int64_t tinits = 0;
+    double target = 0.0; /* the renormalisation target of the last step */
 } F;
 
 template <typename T> T *handle() { return reinterpret_cast<T *>(std::malloc(16)); }
@@ -95,6 +96,7 @@ int64_t fake_sync_copies() { return F.sync_copies; }
 int64_t fake_map_lists() { return F.map_lists; }
 int64_t fake_map_entries() { return F.map_entries; }
 int64_t fake_tinits() { return F.tinits; }
+double fake_target() { return F.target; }
 int fake_launched(int kind) { return F.launched.count(kind) ? F.launched[kind] : 0; }
 unsigned long long fake_word(int i) { return F.words[i]; }
 int fake_last_error() { return (int)F.last; }
@@ -237,6 +239,7 @@ int qw_step_grid(const QwSimDev &, int, int) { return 152; }
 cudaError_t qw_launch_step(const QwSimDev &, const QwBufDev &, const QwBufDev &, const QwBufDev &, const QwStepArgs &a,
                            int, int, cudaStream_t)
 {
+    F.target = *a.renorm_target;
     if (!F.capturing && *a.status == 0) {
         *a.status |= F.status_bits;
         F.status_bits = 0;
@@ -247,6 +250,7 @@ cudaError_t qw_launch_step(const QwSimDev &, const QwBufDev &, const QwBufDev &,
 
 static cudaError_t walk_pos(const QwPosArgs &p, const QwStepArgs &a)
 {
+    F.target = *a.renorm_target;
     if (p.words) std::memcpy(F.words, p.words, 8 * sizeof(unsigned long long));
     if (!F.capturing && *a.status == 0) {
         if (F.give_up > 0) {

@@ -92,3 +92,24 @@ def test_complex128_factor_is_fp64(n, s, tau):
             sim.enqueue_walk_steps(steps)
             assert abs(math.fsum(sim.measure_register("j", n)) / math.fsum(b * b) - 1.0) <= 30 * 2.0**-53
         sim.close()
+
+
+@pytest.mark.parametrize("variant", [7, 4])
+def test_a_state_saved_and_resumed_takes_a_new_instance_as_before(variant):
+    """Setting one instance of a batch again after an import leaves the same state as
+    without the import in between (complex128, FP64 roundings)."""
+    mats = [_matrix(n, 8, n) for n in (40, 70, 100)]
+    out = []
+    for resume in (True, False):
+        sim = qwalk.Sim(mats, s_pad=8, walk_variant=variant, renorm=1)
+        for i, m in enumerate(mats):
+            sim.state_init(_b(m.n, i), inst=i)
+        sim.apply_walk_step(2)
+        if resume:
+            sim.state_import(*sim.state_export())
+        sim.state_init(3.0 * _b(70, 9), inst=1)
+        sim.apply_walk_step(3)
+        out.append([sim.measure_register("j", m.n, inst=i) for i, m in enumerate(mats)])
+        sim.close()
+    for x, y, norm in zip(*out, (1.0, 9.0, 1.0)):
+        assert abs(x.sum() - norm) < 1e-12 and np.abs(x - y).max() < 1e-13

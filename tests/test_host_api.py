@@ -41,6 +41,7 @@ def fake(fake_path, monkeypatch):
     for name in ("fake_live", "fake_sync_copies", "fake_map_lists", "fake_map_entries", "fake_tinits"):
         getattr(lib, name).restype = ctypes.c_int64
     lib.fake_word.restype = ctypes.c_ulonglong
+    lib.fake_target.restype = ctypes.c_double
     lib.fake_set_step.argtypes = [ctypes.c_int, ctypes.c_double]
     lib.fake_set_times.argtypes = [ctypes.c_double] * 4
     lib.fake_reset()
@@ -74,3 +75,20 @@ def test_autotuner_times_steps_not_first_launches(fake, steps, graphs, slot, run
         assert sim.step_stats()["steps"] == steps  # (the fake counts them for the positional layout)
         tried = sum(u > 0.0 for u in us)
         assert tried == 6 and abs(us[7] - run) <= (15.0 / 32 if graphs else 1e-6) + 1e-6
+
+
+def test_a_batch_imported_and_one_instance_set_again_keeps_the_target(fake):
+    """The renormalisation target is the sum of the instances' norms: of the imported
+    list's, and, where one instance is set again, of its new one and the
+    others' (which went out of it: the batch was then scaled to one instance's norm)."""
+    with qwalk.Sim([wl.random_symmetric(16, 8, 1, 16, i) for i in range(3)], s_pad=8, renorm=1) as sim:
+        regs = np.zeros((6, 8), dtype=np.uint64)
+        regs[:, 7] = [0, 0, 1, 2, 2, 2]  # inst
+        regs[:, 1] = [1, 2, 1, 1, 2, 3]  # j
+        amps = np.array([1.0, 2.0j, 3.0, 1.0, 1.0, 1.0 + 1.0j])
+        sim.state_import(sim.pack(regs), amps)
+        sim.enqueue_walk_steps(1)
+        assert fake.fake_target() == 5.0 + 9.0 + 4.0
+        sim.state_init(np.full(16, 0.5), inst=1)
+        sim.enqueue_walk_steps(1)
+        assert fake.fake_target() == 5.0 + 4.0 + 4.0
