@@ -1657,6 +1657,7 @@ extern "C" int qw_state_init(qw_sim *sim, int32_t inst, const double *b_re, cons
         sim->scale_slot = sim->sync_slot = 0;
         sim->cur = sim->sync_cur = 0;
         sim->sync_done = 0;
+        sim->pos_issued = false; /* what comes now is not their error */
     } else {
         double target = 0.0;
         for (double v : sim->init_norm2) target += v;
@@ -2325,6 +2326,7 @@ extern "C" int qw_state_import(qw_sim *sim, int32_t key_words, const uint64_t *k
     sim->scale_slot = sim->sync_slot = 0;
     sim->cur = sim->sync_cur = 0;
     sim->sync_done = 0;
+    sim->pos_issued = false; /* what comes now is not their error */
     drop_graphs(sim);
     if (count > 0) {
         QW_CUDA(sim, qw_flat_scatter(sim->d, sim->buf[sim->cur], sim->fp32, K, static_cast<double2 *>(A), count,

@@ -92,3 +92,16 @@ def test_a_batch_imported_and_one_instance_set_again_keeps_the_target(fake):
         sim.state_init(np.full(16, 0.5), inst=1)
         sim.enqueue_walk_steps(1)
         assert fake.fake_target() == 5.0 + 4.0 + 4.0
+
+
+def test_an_import_that_overflows_after_positional_steps_is_a_capacity_error(fake):
+    """The overflow is the import's, not that of the steps enqueued before it (whose
+    errors lose the state)."""
+    with _sim(walk_variant=7, overflow_fallback=False) as sim:
+        sim.state_init(_b(64))
+        sim.enqueue_walk_steps(2)
+        fake.fake_status(ROW_OVERFLOW)
+        regs = np.zeros((1, 8), dtype=np.uint64)
+        with pytest.raises(qwalk.QwError) as e:
+            sim.state_import(sim.pack(regs), np.ones(1))
+        assert e.value.code == qwalk.QW_ERR_CAPACITY
