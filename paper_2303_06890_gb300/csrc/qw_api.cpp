@@ -698,6 +698,17 @@ extern "C" int qw_sim_info(const qw_sim *sim, int32_t *nb, int32_t *s, int32_t *
 
 extern "C" int64_t qw_launch_count(const qw_sim *sim) { return sim ? sim->launches : 0; }
 
+/* Before the scalars, the device's status among them, are written anew while
+ * positional steps may still run: should one of those give up its wait, nobody
+ * reads that any more, and the next run must not start on the words it leaves
+ * behind (its count would be reached early, or never). */
+static cudaError_t pos_forget(qw_sim *sim)
+{
+    if (!sim->pos_issued) return cudaSuccess;
+    sim->pos_issued = false;
+    return cudaMemsetAsync(sim->pos_words, 0, QW_POS_WORDS * sizeof(unsigned long long), sim->stream);
+}
+
 static const double *pending_scale(qw_sim *sim)
 {
     return sim->renorm ? &sim->sc->scale[sim->scale_slot] : nullptr;
@@ -752,7 +763,8 @@ static int status_read(qw_sim *sim, const char *where)
     if (st & QW_ST_GRID_WAIT) m += " [a positional step gave up waiting for the other blocks]";
     if (pos_issued) { /* several steps share the arrays: no clean one to go back to */
         sim->has_state = sim->pos_live = false;
-        cudaMemsetAsync(sim->pos_words, 0, QW_POS_WORDS * sizeof(unsigned long long), sim->stream);
+        sim->pos_issued = true;
+        pos_forget(sim);
         cudaStreamSynchronize(sim->stream);
         return fail(sim, QW_ERR_DEVICE_STATUS, m + "; the state is lost: initialise it again");
     }
@@ -1580,7 +1592,7 @@ static int pos_state_init(qw_sim *sim, int32_t inst, const double *b_re, const d
         sim->cur = sim->sync_cur = 0;
         sim->sync_done = 0;
         sim->issued = 0;
-        sim->pos_issued = false;
+        QW_CUDA(sim, pos_forget(sim));
         sim->pos_full = false;
     } else {
         double target = 0.0;
@@ -1653,11 +1665,11 @@ extern "C" int qw_state_init(qw_sim *sim, int32_t inst, const double *b_re, cons
         z = Scalars{};
         z.scale[0] = z.scale[1] = 1.0;
         z.renorm_target = nb2;
+        QW_CUDA(sim, pos_forget(sim)); /* what comes now is not those steps' error */
         QW_CUDA(sim, cudaMemcpyAsync(sim->sc, sim->h_sc, sizeof(Scalars), cudaMemcpyHostToDevice, sim->stream));
         sim->scale_slot = sim->sync_slot = 0;
         sim->cur = sim->sync_cur = 0;
         sim->sync_done = 0;
-        sim->pos_issued = false; /* what comes now is not their error */
     } else {
         double target = 0.0;
         for (double v : sim->init_norm2) target += v;
@@ -2322,11 +2334,11 @@ extern "C" int qw_state_import(qw_sim *sim, int32_t key_words, const uint64_t *k
     Scalars z{};
     z.scale[0] = z.scale[1] = 1.0;
     z.renorm_target = norm2;
+    QW_CUDA(sim, pos_forget(sim)); /* what comes now is not those steps' error */
     QW_CUDA(sim, cudaMemcpyAsync(sim->sc, &z, sizeof z, cudaMemcpyHostToDevice, sim->stream));
     sim->scale_slot = sim->sync_slot = 0;
     sim->cur = sim->sync_cur = 0;
     sim->sync_done = 0;
-    sim->pos_issued = false; /* what comes now is not their error */
     drop_graphs(sim);
     if (count > 0) {
         QW_CUDA(sim, qw_flat_scatter(sim->d, sim->buf[sim->cur], sim->fp32, K, static_cast<double2 *>(A), count,

@@ -105,3 +105,24 @@ def test_an_import_that_overflows_after_positional_steps_is_a_capacity_error(fak
         with pytest.raises(qwalk.QwError) as e:
             sim.state_import(sim.pack(regs), np.ones(1))
         assert e.value.code == qwalk.QW_ERR_CAPACITY
+
+
+@pytest.mark.parametrize("how", ["init", "init without T", "import", "read", "sync"])
+def test_a_run_starts_on_clear_barrier_words_after_one_that_gave_up(fake, how):
+    """A launch that gives up its wait leaves words that some blocks arrived at.  They
+    are cleared with the status, whether somebody reads it or the state is replaced."""
+    with _sim(walk_variant=7) as sim:
+        sim.state_init(_b(64))
+        fake.fake_give_up(1)
+        sim.enqueue_walk_steps(2)
+        if how in ("read", "sync"):
+            with pytest.raises(qwalk.QwError, match="gave up waiting.*the state is lost") as e:
+                sim.measure_register("j", 64) if how == "read" else sim.sync()
+            assert e.value.code == qwalk.QW_ERR_DEVICE_STATUS
+        if how == "import":
+            sim.state_import(sim.pack(np.zeros((1, 8), dtype=np.uint64)), np.ones(1))
+        else:
+            sim.state_init(_b(64), apply_T=how != "init without T")
+        sim.enqueue_walk_steps(2)
+        assert [fake.fake_word(i) for i in range(8)] == [0] * 8
+        sim.sync()
