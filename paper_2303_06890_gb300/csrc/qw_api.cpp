@@ -823,13 +823,16 @@ static int launch_pos(qw_sim *sim, int64_t nsteps, int64_t qls_term, int readout
         p.words = sim->pos_words;
         p.extra = reinterpret_cast<double *>(sim->pos_words + QW_POS_EXTRA);
         p.pshare = reinterpret_cast<double *>(sim->pos_words + QW_POS_WORDS);
-        sim->pos_epoch += (unsigned long long)nsteps;
     }
     const cudaError_t e = qw_launch_walk_pos(sim->d, sim->pos_plan, p, a, sim->fp32, sim->pos_full, sim->stream);
+    if (e != cudaSuccess) {
+        cudaGetLastError(); /* not the next launch's error too */
+        return cuda_fail(sim, e, "walk step launch");
+    }
+    if (nsteps > 1) sim->pos_epoch += (unsigned long long)nsteps; /* (a refused launch leaves its words' turn) */
     sim->launches++;
     sim->issued += nsteps;
     sim->pos_issued = true;
-    if (e != cudaSuccess) return cuda_fail(sim, e, "walk step launch");
     sim->cur = (sim->cur + (nsteps & 1 ? 1 : 2)) % 3;
     sim->scale_slot ^= 1;
     return QW_OK;

@@ -35,6 +35,9 @@ struct Fake {
     int capturing = 0;
     unsigned long long words[8] = {0}; /* the barrier words a positional run started on */
     int64_t tinits = 0;
+    int refuse = 0;                 /* the next positional launch is refused */
+    unsigned long long epoch = 0;   /* of the last one that was not */
+    int64_t run_steps = 0;          /* steps of the runs since the last reset */
     double target = 0.0; /* the renormalisation target of the last step */
 } F;
 
@@ -96,6 +99,9 @@ int64_t fake_sync_copies() { return F.sync_copies; }
 int64_t fake_map_lists() { return F.map_lists; }
 int64_t fake_map_entries() { return F.map_entries; }
 int64_t fake_tinits() { return F.tinits; }
+void fake_refuse(int n) { F.refuse = n; }
+unsigned long long fake_epoch() { return F.epoch; }
+int64_t fake_run_steps() { return F.run_steps; }
 double fake_target() { return F.target; }
 int fake_launched(int kind) { return F.launched.count(kind) ? F.launched[kind] : 0; }
 unsigned long long fake_word(int i) { return F.words[i]; }
@@ -250,7 +256,15 @@ cudaError_t qw_launch_step(const QwSimDev &, const QwBufDev &, const QwBufDev &,
 
 static cudaError_t walk_pos(const QwPosArgs &p, const QwStepArgs &a)
 {
+    if (F.refuse > 0) {
+        --F.refuse;
+        return done(cudaErrorLaunchOutOfResources);
+    }
     F.target = *a.renorm_target;
+    if (p.words) {
+        F.epoch = p.epoch;
+        F.run_steps += p.nsteps;
+    }
     if (p.words) std::memcpy(F.words, p.words, 8 * sizeof(unsigned long long));
     if (!F.capturing && *a.status == 0) {
         if (F.give_up > 0) {

@@ -38,9 +38,9 @@ def fake(fake_path, monkeypatch):
     monkeypatch.setattr(native, "LIB", fake_path)
     monkeypatch.setattr(qwalk, "_lib", None)
     lib = qwalk.load(build_if_missing=False)
-    for name in ("fake_live", "fake_sync_copies", "fake_map_lists", "fake_map_entries", "fake_tinits"):
+    for name in ("fake_live", "fake_sync_copies", "fake_map_lists", "fake_map_entries", "fake_tinits", "fake_run_steps"):
         getattr(lib, name).restype = ctypes.c_int64
-    lib.fake_word.restype = ctypes.c_ulonglong
+    lib.fake_word.restype = lib.fake_epoch.restype = ctypes.c_ulonglong
     lib.fake_target.restype = ctypes.c_double
     lib.fake_set_step.argtypes = [ctypes.c_int, ctypes.c_double]
     lib.fake_set_times.argtypes = [ctypes.c_double] * 4
@@ -126,3 +126,20 @@ def test_a_run_starts_on_clear_barrier_words_after_one_that_gave_up(fake, how):
         sim.enqueue_walk_steps(2)
         assert [fake.fake_word(i) for i in range(8)] == [0] * 8
         sim.sync()
+
+
+def test_a_refused_launch_takes_no_turn_of_the_barrier(fake):
+    """The words of a run's turns are left clear for it by the runs before: a run that
+    was not launched has not passed its turns on."""
+    with _sim(walk_variant=7) as sim:
+        sim.state_init(_b(64))
+        sim.enqueue_walk_steps(3)
+        first = fake.fake_epoch()
+        fake.fake_refuse(1)
+        with pytest.raises(qwalk.QwError) as e:
+            sim.enqueue_walk_steps(2)
+        assert e.value.code == qwalk.QW_ERR_CUDA
+        sim.enqueue_walk_steps(2)
+        assert fake.fake_epoch() == first + 3
+        sim.sync()
+        assert sim.step_stats()["steps"] == 5
