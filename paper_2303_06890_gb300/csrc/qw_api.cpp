@@ -181,8 +181,9 @@ static bool host_staged(const qw_sim *sim)
 
 static const int kGraphSteps = 6; /* a multiple of the 3-buffer and 2-slot periods */
 static const int kGraphTerms = 3;  /* QLS terms per graph: 2 walk steps each */
-/* words of h_flat: outputs of a stage, branches of the state, longest row, flags
-   of an import (6), the sort's varying bits (2 x 10) */
+/* words of h_flat: outputs of a stage, branches of the state, longest row, whether
+   the stage gave up a wait (QW_TOTAL_WAIT), flags of an import (6), the sort's varying
+   bits (2 x 10) */
 static const int kFlatTotal = 0, kFlatCount = 1, kFlatRow = 2, kFlatIo = 4, kFlatSort = 16, kFlatWords = 40;
 static const int64_t kPosSteps = 1024; /* walk steps of one positional launch: a few milliseconds */
 static const int64_t kTuneSteps = 32;  /* at least, of one the autotuner times: the launch is a small part */
@@ -1002,7 +1003,8 @@ static cudaError_t flat_gather(qw_sim *sim, FlatList &L, int kw)
 
 /* An interference op on the list (0 = R^dag, 1 = R, 2 = H): grouping by a
  * global radix sort, then the per-group transform with the kept outputs written
- * one after another; the host synchronises to size the result.  group: QW_SORT_GROUP, or
+ * one after another; the host synchronises to size the result.  Where the device
+ * gave up a wait the list is left as before the op.  group: QW_SORT_GROUP, or
  * QW_SORT_GROUP_NO_A within a walk step, whose list starts with A = 0 in every
  * branch, so that A follows from (jc, j, kc, k) wherever it is allocated. */
 static cudaError_t flat_stage(qw_sim *sim, FlatList &L, int op, int group)
@@ -1038,7 +1040,7 @@ static cudaError_t flat_stage(qw_sim *sim, FlatList &L, int op, int group)
     void *tiles = nullptr, *starts = nullptr;
     if ((e = scratch.take(qw_flat_tiles_bytes(L.M), &tiles)) != cudaSuccess) return e;
     unsigned long long *const total = sim->h_flat + kFlatTotal;
-    *total = 0;
+    *total = total[QW_TOTAL_WAIT] = 0;
     /* H: the groups of the sorted list, their number read by the host; up to s
        outputs each.  R, R^dag: up to two an entry. */
     int64_t cap = 2 * L.M, G = 0;
@@ -1047,7 +1049,8 @@ static cudaError_t flat_stage(qw_sim *sim, FlatList &L, int op, int group)
         e = qw_flat_starts(d, L.K, L.M, static_cast<int64_t *>(starts), tiles, total, &sim->sc->status, st, L.kw);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return e;
-        G = std::min<int64_t>((int64_t)*total, L.M); /* (more only after a wait gave up) */
+        if (total[QW_TOTAL_WAIT]) return cudaSuccess; /* the list as it was; the status says so */
+        G = std::min<int64_t>((int64_t)*total, L.M);
         cap = G * d.s;
     }
     FlatList R;
@@ -1062,6 +1065,10 @@ static cudaError_t flat_stage(qw_sim *sim, FlatList &L, int op, int group)
     if (e != cudaSuccess) {
         flat_release(sim, R);
         return e;
+    }
+    if (total[QW_TOTAL_WAIT]) { /* the list as it was; the status says so */
+        flat_release(sim, R);
+        return cudaSuccess;
     }
     R.M = std::min<int64_t>((int64_t)*total, cap);
     R.by_h = op == 2;

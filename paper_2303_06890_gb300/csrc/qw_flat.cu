@@ -616,9 +616,11 @@ constexpr unsigned long long TS_AGG = 1ull << 62, TS_INC = 2ull << 62, TS_CNT = 
 constexpr int TS_SPIN_LIMIT = 1 << 22;
 
 /* the counts of the tiles before vb (called by one warp); count: this tile's.  A
-   wait that outlasts the limit sets the status; the outputs' places are then
-   wrong (and checked against the array's end), and the host reports it. */
-__device__ unsigned long long tile_before(TileSum *ts, int64_t vb, unsigned int count, int32_t *status)
+   wait that outlasts the limit sets the status and the host's word; the outputs'
+   places are then wrong (and checked against the array's end), and the host drops
+   them all: what it would find between them are not keys. */
+__device__ unsigned long long tile_before(TileSum *ts, int64_t vb, unsigned int count, int32_t *status,
+                                          unsigned long long *host)
 {
     const int lane = threadIdx.x & 31;
     volatile unsigned long long *t = ts->tile;
@@ -638,7 +640,10 @@ __device__ unsigned long long tile_before(TileSum *ts, int64_t vb, unsigned int 
         const unsigned need = end == 31 ? FULL : (2u << end) - 1u;
         if (empty & need) {
             if (++spins > TS_SPIN_LIMIT) {
-                if (lane == 0) atomicOr(status, QW_ST_SORT_WAIT);
+                if (lane == 0) {
+                    atomicOr(status, QW_ST_SORT_WAIT);
+                    *(volatile unsigned long long *)(host + QW_TOTAL_WAIT) = 1ull;
+                }
                 break;
             }
             if (spins > 32) __nanosleep(64);
@@ -681,7 +686,7 @@ __device__ __forceinline__ unsigned long long tile_place(TileSum *ts, int64_t vb
         all += ws[w];
     }
     if (warp == 0) {
-        const unsigned long long b = tile_before(ts, vb, all, status);
+        const unsigned long long b = tile_before(ts, vb, all, status, host);
         if (lane == 0) {
             base = b;
             if (vb == ntiles - 1) ts->total = *host = b + all;

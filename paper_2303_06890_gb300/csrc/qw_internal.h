@@ -305,7 +305,9 @@ cudaError_t qw_flat_sort(const QwSimDev &d, void *keys, double2 *amps, void *tmp
                          int order, int group, void *work, unsigned long long *host, int32_t *status, cudaStream_t st,
                          int kw, int *in_tmp);
 /* Scratch of a single-pass kernel over n entries or groups; it leaves the number
-   of its outputs in *host (pinned). */
+   of its outputs in *host (pinned), and a 1 in host[QW_TOTAL_WAIT] where one of its
+   waits gave up: its outputs then have holes, which hold no keys. */
+#define QW_TOTAL_WAIT 3
 size_t qw_flat_tiles_bytes(int64_t n);
 /* op 0 (R^dag) and 1 (R) on the sorted list: the kept outputs (up to 2 M; cap
    is the room in okeys / oamps) */

@@ -29,7 +29,7 @@ struct Fake {
     int give_up = 0;            /* the next positional launch gives up its wait */
     int status_bits = 0;        /* the next bucket step or scatter sets these */
     int flat_wait = 0;          /* the next single-pass launch of the flat path gives up */
-    int64_t map_lists = 0, map_entries = 0; /* non-empty lists given to qw_flat_map, their entries */
+    int64_t map_most = 0;       /* entries of the longest list given to qw_flat_map */
     int64_t live = 0;           /* device allocations not yet freed */
     int64_t sync_copies = 0;    /* cudaMemcpy: ordered on the default stream alone */
     int capturing = 0;
@@ -96,8 +96,7 @@ void fake_flat_wait(int n) { F.flat_wait = n; }
 void fake_capture(int on) { F.capturing = on; }
 int64_t fake_live() { return F.live; }
 int64_t fake_sync_copies() { return F.sync_copies; }
-int64_t fake_map_lists() { return F.map_lists; }
-int64_t fake_map_entries() { return F.map_entries; }
+int64_t fake_map_most() { return F.map_most; }
 int64_t fake_tinits() { return F.tinits; }
 void fake_refuse(int n) { F.refuse = n; }
 unsigned long long fake_epoch() { return F.epoch; }
@@ -368,8 +367,7 @@ cudaError_t qw_flat_gather(const QwSimDev &, const QwBufDev &, int, int, const d
 }
 cudaError_t qw_flat_map(const QwSimDev &, void *, int64_t M, uint32_t, int32_t *, cudaStream_t, int)
 {
-    F.map_lists += M > 0;
-    F.map_entries += M;
+    F.map_most = M > F.map_most ? M : F.map_most;
     return launch(114, 0.0);
 }
 cudaError_t qw_flat_phase(const QwSimDev &, const void *, double2 *, int64_t, cudaStream_t, int) { return launch(115, 0.0); }
@@ -383,15 +381,14 @@ cudaError_t qw_flat_sort(const QwSimDev &, void *, double2 *, void *, double2 *,
 size_t qw_flat_tiles_bytes(int64_t n) { return 64 + (size_t)n; }
 
 /* a single-pass kernel: as many outputs as inputs; one that gives up its wait
-   sets the status and says so beside the total */
+   sets the status, says so beside the total, and counts what it did not write */
 static cudaError_t single_pass(int64_t n, unsigned long long *host, int32_t *status)
 {
     host[0] = (unsigned long long)n;
     if (F.flat_wait > 0 && --F.flat_wait == 0) {
         *status |= QW_ST_SORT_WAIT;
-#ifdef QW_TOTAL_WAIT
+        host[0] = 2ull * (unsigned long long)n;
         host[QW_TOTAL_WAIT] = 1ull;
-#endif
     }
     return launch(117, 0.0);
 }

@@ -38,7 +38,7 @@ def fake(fake_path, monkeypatch):
     monkeypatch.setattr(native, "LIB", fake_path)
     monkeypatch.setattr(qwalk, "_lib", None)
     lib = qwalk.load(build_if_missing=False)
-    for name in ("fake_live", "fake_sync_copies", "fake_map_lists", "fake_map_entries", "fake_tinits", "fake_run_steps"):
+    for name in ("fake_live", "fake_sync_copies", "fake_map_most", "fake_tinits", "fake_run_steps"):
         getattr(lib, name).restype = ctypes.c_int64
     lib.fake_word.restype = lib.fake_epoch.restype = ctypes.c_ulonglong
     lib.fake_target.restype = ctypes.c_double
@@ -143,3 +143,19 @@ def test_a_refused_launch_takes_no_turn_of_the_barrier(fake):
         assert fake.fake_epoch() == first + 3
         sim.sync()
         assert sim.step_stats()["steps"] == 5
+
+
+@pytest.mark.parametrize("variant", [5, 6])
+@pytest.mark.parametrize("nth", range(1, 7))
+def test_a_flat_stage_that_gave_up_its_wait_leaves_its_list(fake, variant, nth):
+    """What such a stage has written has holes that hold no keys, whose instance and row
+    would be looked up: no later kernel is given them (the lists here have 1000
+    entries throughout).  The step is reported, the state kept."""
+    with _sim(walk_variant=variant) as sim:
+        sim.state_init(_b(64))
+        fake.fake_flat_wait(nth)
+        with pytest.raises(qwalk.QwError, match="gave up waiting.*state kept after 0 clean steps") as e:
+            sim.apply_walk_step(1)
+        assert e.value.code == qwalk.QW_ERR_DEVICE_STATUS
+        assert fake.fake_map_most() == 1000
+        sim.apply_walk_step(1)
