@@ -1182,9 +1182,8 @@ static int flat_walk_step(qw_sim *sim, int readout)
  * c, slot l' where row c holds column j there, else an extra of row c -- the
  * three state arrays and the barrier words.  The row buckets grow to hold a whole positional row (2 s +
  * 2 E branches). */
-static int pos_build(qw_sim *sim)
+static int pos_tables(qw_sim *sim)
 {
-    if (sim->pos_built) return QW_OK;
     QwSimDev &d = sim->d;
     if (d.nparts != 1 || !qw_pos_supported(d))
         return fail(sim, QW_ERR_ARG, "walk_variant 7 (positional) needs s = 4, 8, 16, 32 or 64 and no partitions");
@@ -1279,8 +1278,30 @@ static int pos_build(qw_sim *sim)
     sim->mode_alt = d.warp_cap < 2 * d.cap_row ? QW_MODE_WALK_FUSED
                     : (qw_slot_supported(d) ? QW_MODE_WALK_SLOT : QW_MODE_WALK_SEG);
     sim->grid_alt = qw_step_grid(d, sim->fp32, sim->mode_alt);
-    sim->pos_built = true;
     return QW_OK;
+}
+
+/* pos_tables once; where it fails, what it has allocated is given back and no
+ * error of the runtime stays behind (the caller may go on with other kernels). */
+static int pos_build(qw_sim *sim)
+{
+    if (sim->pos_built) return QW_OK;
+    const int64_t bytes = sim->device_bytes;
+    const int64_t rows = 3 * sim->d.total_buckets * (int64_t)(8 + (sim->fp32 ? sizeof(float2) : sizeof(double2)));
+    const int64_t cap = sim->d.cap_row;
+    const int rc = pos_tables(sim);
+    sim->pos_built = rc == QW_OK;
+    if (sim->pos_built) return QW_OK;
+    cudaGetLastError();
+    for (void *p : {(void *)sim->pos_dst, (void *)sim->pos_xptr, (void *)sim->pos_xdst, (void *)sim->pos_rowinst,
+                    (void *)sim->pos_words, sim->pbuf[0], sim->pbuf[1], sim->pbuf[2]})
+        cudaFree(p);
+    sim->pos_dst = sim->pos_xptr = sim->pos_xdst = nullptr;
+    sim->pos_rowinst = nullptr;
+    sim->pos_words = nullptr;
+    for (void *&p : sim->pbuf) p = nullptr;
+    sim->device_bytes = bytes + rows * (sim->d.cap_row - cap); /* grown row buckets stay */
+    return rc;
 }
 
 /* Move the state from the buckets into the positional layout when every

@@ -159,3 +159,22 @@ def test_a_flat_stage_that_gave_up_its_wait_leaves_its_list(fake, variant, nth):
         assert e.value.code == qwalk.QW_ERR_DEVICE_STATUS
         assert fake.fake_map_most() == 1000
         sim.apply_walk_step(1)
+
+
+@pytest.mark.parametrize("after", range(7))
+def test_autotuner_at_s4_without_room_for_the_positional_layout(fake, after):
+    """Device memory that is out while the layout is built, at its first allocation up
+    to its last, leaves the choice among the other kernels, and nothing allocated."""
+    for v in (0, 1, 2, 3):
+        fake.fake_set_step(MODE[v], 20.0 + v)
+    fake.fake_set_times(2.0, 2.0, 0.0, 0.0)
+    with _sim(40, 4) as sim:
+        sim.state_init(_b(40))
+        live = fake.fake_live()
+        for _ in range(2):
+            fake.fake_fail_malloc(after)
+            v, us = sim.autotune(2)
+            assert v == 0 and us[7] == 0.0 and fake.fake_live() == live
+        sim.apply_walk_step(3)
+        fake.fake_fail_malloc(-1)
+        assert sim.autotune(2)[1][7] > 0.0
