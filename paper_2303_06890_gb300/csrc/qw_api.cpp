@@ -1921,6 +1921,9 @@ extern "C" int qw_autotune(qw_sim *sim, int32_t steps, int32_t *choice, double *
        60 at N = 6000 (complex128) 1890 -> 296 */
     const bool slot = qw_slot_supported(sim->d);
     bool pos = qw_pos_supported(sim->d) && sim->d.nparts == 1;
+    /* s = 4: not where a caller's row_capacity has no room for a positional row (4 s at
+       most: a column's unpaired entries come from the s rows before it) */
+    if (sim->d.s < 8 && sim->d.cap_row < 4 * sim->d.s) pos = false;
     if (pos) {
         const int rc = pos_build(sim);
         if (rc != QW_OK && sim->d.s >= 8) return rc;

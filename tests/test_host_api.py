@@ -178,3 +178,13 @@ def test_autotuner_at_s4_without_room_for_the_positional_layout(fake, after):
         sim.apply_walk_step(3)
         fake.fake_fail_malloc(-1)
         assert sim.autotune(2)[1][7] > 0.0
+
+
+def test_autotuner_at_s4_leaves_a_callers_row_capacity_alone(fake):
+    fake.fake_set_times(2.0, 2.0, 0.0, 0.0)
+    for v in (0, 1, 2, 3):
+        fake.fake_set_step(MODE[v], 20.0 + v)
+    with _sim(40, 4, row_capacity=8, overflow_fallback=False) as sim:
+        sim.state_init(_b(40))
+        live = fake.fake_live()
+        assert sim.autotune(2)[0] == 0 and fake.fake_live() == live
