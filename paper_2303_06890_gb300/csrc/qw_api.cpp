@@ -891,23 +891,42 @@ static int grow_rows(qw_sim *sim, int64_t need)
         return fail(sim, QW_ERR_CAPACITY,
                     "row buckets of " + std::to_string(cap) + " branches per row would need " + std::to_string(newb) +
                         " bytes; device memory is short");
-    drop_graphs(sim);
+    /* all of the new arrays before any of the old ones goes (they fit together:
+       newb is at least 2 oldb, so at most two thirds of what is free): a buffer
+       must never be shorter than cap_row says */
     const int cap_old = sim->d.cap_row;
     const size_t slots = (size_t)sim->d.total_buckets * (size_t)cap;
-    sim->d.cap_row = (int)cap;
-    for (auto &b : sim->buf) {
-        uint64_t *key = nullptr;
-        unsigned char *amp = nullptr;
-        QW_CUDA(sim, dalloc(sim, &key, slots));
-        QW_CUDA(sim, dalloc(sim, &amp, slots * amp_bytes));
-        QW_CUDA(sim, qw_launch_regrow(sim->d, b, cap_old, key, amp, sim->fp32, sim->stream));
-        QW_CUDA(sim, cudaStreamSynchronize(sim->stream));
-        cudaFree(b.key);
-        cudaFree(b.amp);
-        sim->device_bytes -= (int64_t)((size_t)sim->d.total_buckets * (size_t)cap_old * per);
-        b.key = key;
-        b.amp = amp;
+    QwSimDev d = sim->d;
+    d.cap_row = (int)cap;
+    uint64_t *key[3] = {nullptr, nullptr, nullptr};
+    unsigned char *amp[3] = {nullptr, nullptr, nullptr};
+    const int64_t bytes = sim->device_bytes;
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < 3 && e == cudaSuccess; ++i) {
+        e = dalloc(sim, &key[i], slots);
+        if (e == cudaSuccess) e = dalloc(sim, &amp[i], slots * amp_bytes);
+        if (e == cudaSuccess) e = qw_launch_regrow(d, sim->buf[i], cap_old, key[i], amp[i], sim->fp32, sim->stream);
     }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(sim->stream);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        cudaStreamSynchronize(sim->stream);
+        for (int i = 0; i < 3; ++i) {
+            cudaFree(key[i]);
+            cudaFree(amp[i]);
+        }
+        sim->device_bytes = bytes;
+        return cuda_fail(sim, e, "row buckets");
+    }
+    drop_graphs(sim);
+    sim->d.cap_row = (int)cap;
+    for (int i = 0; i < 3; ++i) {
+        cudaFree(sim->buf[i].key);
+        cudaFree(sim->buf[i].amp);
+        sim->buf[i].key = key[i];
+        sim->buf[i].amp = amp[i];
+    }
+    sim->device_bytes -= (int64_t)oldb;
     return QW_OK;
 }
 

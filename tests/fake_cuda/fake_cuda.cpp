@@ -35,6 +35,8 @@ struct Fake {
     int capturing = 0;
     unsigned long long words[8] = {0}; /* the barrier words a positional run started on */
     int64_t tinits = 0;
+    std::map<void *, size_t> sizes; /* of the device allocations */
+    int64_t overruns = 0;           /* row buckets shorter than cap_row says, as a clear of them finds */
     int refuse = 0;                 /* the next positional launch is refused */
     unsigned long long epoch = 0;   /* of the last one that was not */
     int64_t run_steps = 0;          /* steps of the runs since the last reset */
@@ -55,6 +57,7 @@ cudaError_t take(void **p, size_t n)
     if (F.fail_malloc == 0) return done(cudaErrorMemoryAllocation);
     if (F.fail_malloc > 0) --F.fail_malloc;
     *p = std::calloc(n ? n : 1, 1);
+    F.sizes[*p] = n;
     ++F.live;
     return cudaSuccess;
 }
@@ -101,6 +104,7 @@ int64_t fake_tinits() { return F.tinits; }
 void fake_refuse(int n) { F.refuse = n; }
 unsigned long long fake_epoch() { return F.epoch; }
 int64_t fake_run_steps() { return F.run_steps; }
+int64_t fake_overruns() { return F.overruns; }
 double fake_target() { return F.target; }
 int fake_launched(int kind) { return F.launched.count(kind) ? F.launched[kind] : 0; }
 unsigned long long fake_word(int i) { return F.words[i]; }
@@ -336,7 +340,11 @@ POS(32)
 POS(64)
 #undef POS
 
-cudaError_t qw_launch_clear(const QwSimDev &, const QwBufDev &, int64_t, int64_t, int, cudaStream_t) { return launch(105, 0.0); }
+cudaError_t qw_launch_clear(const QwSimDev &d, const QwBufDev &buf, int64_t, int64_t, int, cudaStream_t)
+{
+    if (F.sizes[buf.key] < (size_t)d.total_buckets * (size_t)d.cap_row * 8) ++F.overruns;
+    return launch(105, 0.0);
+}
 cudaError_t qw_launch_init_b(const QwSimDev &, const QwBufDev &, int, const double *, const double *, int, int, const double *,
                              cudaStream_t)
 {

@@ -38,7 +38,7 @@ def fake(fake_path, monkeypatch):
     monkeypatch.setattr(native, "LIB", fake_path)
     monkeypatch.setattr(qwalk, "_lib", None)
     lib = qwalk.load(build_if_missing=False)
-    for name in ("fake_live", "fake_sync_copies", "fake_map_most", "fake_tinits", "fake_run_steps"):
+    for name in ("fake_live", "fake_sync_copies", "fake_map_most", "fake_tinits", "fake_run_steps", "fake_overruns"):
         getattr(lib, name).restype = ctypes.c_int64
     lib.fake_word.restype = lib.fake_epoch.restype = ctypes.c_ulonglong
     lib.fake_target.restype = ctypes.c_double
@@ -188,3 +188,20 @@ def test_autotuner_at_s4_leaves_a_callers_row_capacity_alone(fake):
         sim.state_init(_b(40))
         live = fake.fake_live()
         assert sim.autotune(2)[0] == 0 and fake.fake_live() == live
+
+
+@pytest.mark.parametrize("after", range(6))
+def test_row_buckets_that_could_not_grow_stay_as_they_were(fake, after):
+    """T~ needs rows of 16; the device memory is out at one of the six arrays."""
+    with _sim(row_capacity=8) as sim:
+        sim.state_init(_b(64), apply_T=False)
+        live = fake.fake_live()
+        fake.fake_fail_malloc(after)
+        with pytest.raises(qwalk.QwError) as e:
+            sim.state_init(_b(64))
+        assert e.value.code == qwalk.QW_ERR_CUDA and fake.fake_live() == live
+        fake.fake_fail_malloc(-1)
+        sim.state_init(_b(64), apply_T=False)
+        assert fake.fake_overruns() == 0
+        sim.state_init(_b(64))
+        assert fake.fake_overruns() == 0 and fake.fake_live() == live
