@@ -1335,17 +1335,13 @@ static int pos_pack(qw_sim *sim)
     QW_CUDA(sim, cudaMemcpyAsync(sim->h_st, &sim->sc->status, sizeof(StatusView), cudaMemcpyDeviceToHost, st));
     QW_CUDA(sim, cudaStreamSynchronize(st));
     if (sim->h_st->status & QW_ST_POS_UNREP) {
-        const int32_t zero = 0;
-        QW_CUDA(sim, cudaMemcpy(&sim->sc->status, &zero, 4, cudaMemcpyHostToDevice));
+        QW_CUDA(sim, cudaMemsetAsync(&sim->sc->status, 0, 4, st)); /* on this stream: before its next step reads it */
         sim->pos_try = false;
         return QW_OK;
     }
     sim->pos_full = (sim->h_st->status & QW_ST_POS_FULL) != 0;
     if (sim->h_st->status & ~QW_ST_POS_FULL) return check_status(sim, "positional layout");
-    if (sim->pos_full) {
-        const int32_t zero = 0;
-        QW_CUDA(sim, cudaMemcpy(&sim->sc->status, &zero, 4, cudaMemcpyHostToDevice));
-    }
+    if (sim->pos_full) QW_CUDA(sim, cudaMemsetAsync(&sim->sc->status, 0, 4, st));
     sim->pos_live = true;
     return QW_OK;
 }

@@ -18,7 +18,7 @@ from paper_2303_06890_gb300 import workloads as wl
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "..", "paper_2303_06890_gb300", "csrc")
 MODE = {0: 0, 1: 3, 2: 4, 3: 5, 4: 6}  # walk_variant -> kernel mode (qw_internal.h)
-GRID_WAIT, ROW_OVERFLOW, POS_FULL = 512, 1, 256
+ROW_OVERFLOW, POS_UNREP, POS_FULL = 1, 64, 256  # device status bits
 
 
 @pytest.fixture(scope="module")
@@ -205,3 +205,17 @@ def test_row_buckets_that_could_not_grow_stay_as_they_were(fake, after):
         assert fake.fake_overruns() == 0
         sim.state_init(_b(64))
         assert fake.fake_overruns() == 0 and fake.fake_live() == live
+
+
+@pytest.mark.parametrize("bits", [POS_FULL, POS_UNREP])
+def test_the_status_of_a_move_is_cleared_on_the_simulators_stream(fake, bits):
+    """A synchronous copy is ordered on the default stream alone, and may still be
+    under way when it returns: a step on a non-blocking stream would see the bit and
+    do nothing."""
+    with _sim(walk_variant=7) as sim:
+        sim.state_import(sim.pack(np.zeros((1, 8), dtype=np.uint64)), np.ones(1))
+        copies = fake.fake_sync_copies()
+        fake.fake_status(bits)
+        sim.enqueue_walk_steps(2)
+        assert fake.fake_sync_copies() == copies
+        sim.sync()
