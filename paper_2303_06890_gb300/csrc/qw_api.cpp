@@ -1603,6 +1603,9 @@ static int pos_state_init(qw_sim *sim, int32_t inst, const double *b_re, const d
 {
     const bool all = sim->d.ninst == 1;
     const int64_t g0 = pos_row0(sim, inst);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(sim->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
+        return check_status(sim, "qw_state_init"); /* refused, as everywhere, with the state as it was */
     if (sim->h_b_busy[(size_t)inst]) { /* set again before anything synchronised */
         QW_CUDA(sim, cudaStreamSynchronize(sim->stream));
         std::fill(sim->h_b_busy.begin(), sim->h_b_busy.end(), 0);
@@ -1655,9 +1658,6 @@ static int pos_state_init(qw_sim *sim, int32_t inst, const double *b_re, const d
     sim->pos_live = true;
     sim->has_state = true;
     sim->fresh_T = true;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(sim->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
-        return check_status(sim, "qw_state_init"); /* refused, as everywhere (it cannot synchronise) */
     return QW_OK;
 }
 

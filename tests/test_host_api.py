@@ -219,3 +219,17 @@ def test_the_status_of_a_move_is_cleared_on_the_simulators_stream(fake, bits):
         sim.enqueue_walk_steps(2)
         assert fake.fake_sync_copies() == copies
         sim.sync()
+
+
+def test_a_state_refused_under_capture_is_not_there(fake):
+    """T~|b~> straight into the layout cannot be captured; refused, it leaves nothing
+    launched and the simulator without the state it never got."""
+    with _sim(walk_variant=7) as sim:
+        fake.fake_capture(1)
+        with pytest.raises(qwalk.QwError) as e:
+            sim.state_init(_b(64))
+        assert e.value.code == qwalk.QW_ERR_CUDA and fake.fake_tinits() == 0
+        fake.fake_capture(0)
+        with pytest.raises(qwalk.QwError) as e:
+            sim.measure_register("j", 64)
+        assert e.value.code == qwalk.QW_ERR_STATE
