@@ -967,6 +967,7 @@ static const size_t kIoKeep = (size_t)256 << 20;
 struct FlatScratch {
     qw_sim *sim;
     bool io;
+    bool out = false; /* a take that the device had no memory for */
     size_t bytes = 0;
     std::vector<void *> all;
     explicit FlatScratch(qw_sim *s, bool io_ = false) : sim(s), io(io_) {}
@@ -983,8 +984,22 @@ struct FlatScratch {
     cudaError_t take(size_t n, void **p)
     {
         const cudaError_t e = flat_alloc(sim, n, p);
-        if (e == cudaSuccess) all.push_back(*p), bytes += n;
+        if (e == cudaSuccess) {
+            all.push_back(*p);
+            bytes += n;
+        } else if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError(); /* the call goes on with less: not the next launch's error */
+            out = true;
+        }
         return e;
+    }
+    void give_back() /* all of it, by the pool to the device */
+    {
+        for (void *p : all) cudaFreeAsync(p, sim->stream);
+        all.clear();
+        bytes = 0;
+        cudaStreamSynchronize(sim->stream);
+        if (sim->fpool) cudaMemPoolTrimTo(sim->fpool, 0);
     }
 };
 
@@ -2221,6 +2236,29 @@ static uint64_t get_bits(const uint64_t *w, int pos, int width)
     return v;
 }
 
+/* A gathered list of M branches (two-word keys) to the caller's arrays, sorted on the
+ * host: where the device has room for the list, 32 bytes a branch, but not for the sort
+ * there, 57 more and the caller's key words. */
+static int export_by_host(qw_sim *sim, const void *K, const void *A, size_t M, size_t W, uint64_t *keys, double *amps,
+                          size_t nout)
+{
+    std::vector<uint64_t> k(2 * M), order(M);
+    std::vector<double2> a(M);
+    QW_CUDA(sim, cudaMemcpyAsync(k.data(), K, M * 16, cudaMemcpyDeviceToHost, sim->stream));
+    QW_CUDA(sim, cudaMemcpyAsync(a.data(), A, M * 16, cudaMemcpyDeviceToHost, sim->stream));
+    QW_CUDA(sim, cudaStreamSynchronize(sim->stream));
+    for (size_t i = 0; i < M; ++i) order[i] = i;
+    std::sort(order.begin(), order.end(), [&](uint64_t x, uint64_t y) {
+        return k[2 * x + 1] != k[2 * y + 1] ? k[2 * x + 1] < k[2 * y + 1] : k[2 * x] < k[2 * y];
+    });
+    for (size_t i = 0; i < nout; ++i) {
+        for (size_t t = 0; t < W; ++t) keys[i * W + t] = t < 2 ? k[2 * order[i] + t] : 0ull;
+        amps[2 * i] = a[order[i]].x;
+        amps[2 * i + 1] = a[order[i]].y;
+    }
+    return QW_OK;
+}
+
 extern "C" int qw_state_export(qw_sim *sim, int32_t inst, int32_t key_words, uint64_t *keys,
                                double *amps, int64_t cap, int64_t *count)
 {
@@ -2240,16 +2278,23 @@ extern "C" int qw_state_export(qw_sim *sim, int32_t inst, int32_t key_words, uin
     cudaStream_t st = sim->stream;
     FlatScratch scratch(sim, true);
     const size_t M = (size_t)total, W = (size_t)key_words;
+    const int64_t nout = std::min(total, cap);
     void *K = nullptr, *A = nullptr, *tk = nullptr, *ta = nullptr, *work = nullptr, *out = nullptr;
     QW_CUDA(sim, scratch.take(M * 16, &K));
     QW_CUDA(sim, scratch.take(M * 16, &A));
-    QW_CUDA(sim, scratch.take(M * 16, &tk));
-    QW_CUDA(sim, scratch.take(M * 16, &ta));
-    QW_CUDA(sim, scratch.take(qw_flat_sort_bytes(total), &work));
+    cudaError_t e = scratch.take(M * 16, &tk);
+    if (e == cudaSuccess) e = scratch.take(M * 16, &ta);
+    if (e == cudaSuccess) e = scratch.take(qw_flat_sort_bytes(total), &work);
+    if (e == cudaSuccess && W != 2) e = scratch.take((size_t)nout * W * 8, &out);
+    if (e != cudaSuccess && !scratch.out) return cuda_fail(sim, e, "qw_state_export");
     QW_CUDA(sim, cudaMemsetAsync(&sim->sc->counter, 0, 8, st));
     QW_CUDA(sim, qw_flat_gather(sim->d, sim->buf[sim->cur], inst, sim->fp32, pending_scale(sim), K,
                                 static_cast<double2 *>(A), &sim->sc->counter, total, st, 2));
     sim->launches++;
+    if (scratch.out) {
+        rc = check_status(sim, "qw_state_export");
+        return rc == QW_OK ? export_by_host(sim, K, A, M, W, keys, amps, (size_t)nout) : rc;
+    }
     int in_tmp = 0;
     QW_CUDA(sim, qw_flat_sort(sim->d, K, static_cast<double2 *>(A), tk, static_cast<double2 *>(ta), total, 0, QW_SORT_FULL,
                               work, sim->h_flat + kFlatSort,
@@ -2258,10 +2303,9 @@ extern "C" int qw_state_export(qw_sim *sim, int32_t inst, int32_t key_words, uin
         std::swap(K, tk);
         std::swap(A, ta);
     }
-    const int64_t nout = std::min(total, cap);
-    out = K;
-    if (W != 2) {
-        QW_CUDA(sim, scratch.take((size_t)nout * W * 8, &out));
+    if (W == 2) {
+        out = K;
+    } else {
         QW_CUDA(sim, qw_io_store(K, key_words, nout, static_cast<uint64_t *>(out), st));
         sim->launches++;
     }
@@ -2284,13 +2328,13 @@ extern "C" int qw_step_stats(qw_sim *sim, int64_t *out, int32_t len, int32_t res
     return QW_OK;
 }
 
-/* Which rule an imported list breaks: equal keys first, then the first key
- * that the layout does not hold. */
-static int import_refused(qw_sim *sim, int32_t key_words, const uint64_t *keys, int64_t count)
+/* Whether an imported list keeps the rules, by the host: equal keys first, then the
+ * first key that the layout does not hold; order: its keys ascending. */
+static int import_check(qw_sim *sim, int32_t key_words, const uint64_t *keys, int64_t count, std::vector<int64_t> &order)
 {
     const size_t W = (size_t)key_words;
     const int nb = sim->d.nb, layout = 4 * nb + 34;
-    std::vector<int64_t> order((size_t)count);
+    order.resize((size_t)count);
     for (int64_t i = 0; i < count; ++i) order[(size_t)i] = i;
     std::sort(order.begin(), order.end(), [&](int64_t x, int64_t y) {
         const uint64_t *a = keys + (size_t)x * W, *b = keys + (size_t)y * W;
@@ -2309,7 +2353,121 @@ static int import_refused(qw_sim *sim, int32_t key_words, const uint64_t *keys, 
         if ((int64_t)get_bits(w, 18 + 4 * nb, 16) >= sim->d.ninst)
             return fail(sim, QW_ERR_ARG, "qw_state_import: instance out of range");
     }
-    return fail(sim, QW_ERR_DEVICE_STATUS, "qw_state_import: the keys changed while they were read");
+    return QW_OK;
+}
+
+/* An import's list on the device, checked and with room for its rows: two-word keys and
+ * amplitudes, in the simulator's scratch */
+struct ImportList {
+    void *K = nullptr, *A = nullptr;
+    QwIoFlags *flags = nullptr;
+    double norm2 = 0.0;
+};
+
+/* a row longer than row_capacity: grow the buckets */
+static int import_rows(qw_sim *sim, int64_t longest)
+{
+    return sim->opts.overflow_fallback && longest > sim->d.cap_row ? grow_rows(sim, longest) : QW_OK;
+}
+
+static double list_norm2(const double *amps, int64_t count)
+{
+    double v = 0.0;
+    for (int64_t i = 0; i < count; ++i) v += amps[2 * i] * amps[2 * i] + amps[2 * i + 1] * amps[2 * i + 1];
+    return v;
+}
+
+/* Packed, checked and sorted on the device; *room: cleared where its memory, beside
+ * the scratch of it, was too short. */
+static int import_on_device(qw_sim *sim, FlatScratch &scratch, int32_t key_words, const uint64_t *keys, const double *amps,
+                            int64_t count, ImportList &L, bool *room)
+{
+    cudaStream_t st = sim->stream;
+    const size_t M = (size_t)count;
+    void *in = nullptr;
+    auto take = [&](size_t n, void **p) {
+        const cudaError_t e = scratch.take(n, p);
+        if (scratch.out) *room = false;
+        return e;
+    };
+    QW_CUDA(sim, take(M * (size_t)key_words * 8, &in));
+    QW_CUDA(sim, take(M * 16, &L.K));
+    QW_CUDA(sim, take(M * 16, &L.A));
+    QW_CUDA(sim, take(sizeof(QwIoFlags), (void **)&L.flags));
+    QW_CUDA(sim, cudaMemsetAsync(L.flags, 0, sizeof(QwIoFlags), st));
+    QW_CUDA(sim, cudaMemcpyAsync(in, keys, M * (size_t)key_words * 8, cudaMemcpyHostToDevice, st));
+    QW_CUDA(sim, qw_io_load(sim->d, static_cast<uint64_t *>(in), key_words, count, L.K, L.flags, st));
+    QW_CUDA(sim, qw_io_order(sim->d, L.K, count, L.flags, st));
+    sim->launches += 2;
+    QW_CUDA(sim, cudaMemcpyAsync(L.A, amps, M * 16, cudaMemcpyHostToDevice, st));
+    L.norm2 = list_norm2(amps, count);
+    static_assert(sizeof(QwIoFlags) <= 8 * (kFlatSort - kFlatIo), "flags of an import");
+    const QwIoFlags &h = *reinterpret_cast<const QwIoFlags *>(sim->h_flat + kFlatIo);
+    QW_CUDA(sim, cudaMemcpyAsync(sim->h_flat + kFlatIo, L.flags, sizeof h, cudaMemcpyDeviceToHost, st));
+    QW_CUDA(sim, cudaStreamSynchronize(st));
+    if (h.unsorted && !h.bad) { /* an exported list is sorted; any other is sorted here */
+        void *tk = nullptr, *ta = nullptr, *work = nullptr;
+        QW_CUDA(sim, take(M * 16, &tk));
+        QW_CUDA(sim, take(M * 16, &ta));
+        QW_CUDA(sim, take(qw_flat_sort_bytes(count), &work));
+        QW_CUDA(sim, cudaMemsetAsync(L.flags, 0, sizeof(QwIoFlags), st));
+        int in_tmp = 0;
+        QW_CUDA(sim, qw_flat_sort(sim->d, L.K, static_cast<double2 *>(L.A), tk, static_cast<double2 *>(ta), count, 0,
+                                  QW_SORT_FULL, work, sim->h_flat + kFlatSort, &L.flags->status, st, 2, &in_tmp));
+        if (in_tmp) {
+            std::swap(L.K, tk);
+            std::swap(L.A, ta);
+        }
+        QW_CUDA(sim, qw_io_order(sim->d, L.K, count, L.flags, st));
+        sim->launches++;
+        QW_CUDA(sim, cudaMemcpyAsync(sim->h_flat + kFlatIo, L.flags, sizeof h, cudaMemcpyDeviceToHost, st));
+        QW_CUDA(sim, cudaStreamSynchronize(st));
+        if (h.status != 0 || h.unsorted)
+            return fail(sim, QW_ERR_DEVICE_STATUS, "qw_state_import: the sort of the keys gave up waiting for a tile's count");
+    }
+    if (h.bad || h.dup) {
+        std::vector<int64_t> order;
+        const int rc = import_check(sim, key_words, keys, count, order);
+        return rc != QW_OK ? rc : fail(sim, QW_ERR_DEVICE_STATUS, "qw_state_import: the keys changed while they were read");
+    }
+    const int rc = import_rows(sim, (int64_t)h.longest);
+    if (rc != QW_OK) *room = false; /* (row buckets: the memory is short beside the scratch) */
+    return rc;
+}
+
+/* The same by the host, 32 bytes of scratch a branch, and that only after the rows
+ * have grown: where the device has no room for the list's checks. */
+static int import_by_host(qw_sim *sim, FlatScratch &scratch, int32_t key_words, const uint64_t *keys, const double *amps,
+                          int64_t count, ImportList &L)
+{
+    const size_t M = (size_t)count, W = (size_t)key_words;
+    const int pb1 = 1 + 2 * sim->d.nb; /* a row: the bits from here up */
+    std::vector<int64_t> order;
+    int rc = import_check(sim, key_words, keys, count, order);
+    if (rc != QW_OK) return rc;
+    std::vector<uint64_t> k(2 * M, 0ull);
+    std::vector<double2> a(M);
+    int64_t longest = 0, run = 0;
+    for (size_t i = 0; i < M; ++i) {
+        const uint64_t *w = keys + (size_t)order[i] * W;
+        k[2 * i] = w[0];
+        if (W > 1) k[2 * i + 1] = w[1];
+        a[i] = make_double2(amps[2 * order[i]], amps[2 * order[i] + 1]);
+        const bool same = i > 0 && k[2 * i + 1] == k[2 * i - 1] && (k[2 * i] >> pb1) == (k[2 * i - 2] >> pb1);
+        run = same ? run + 1 : 1;
+        longest = std::max(longest, run);
+    }
+    L.norm2 = list_norm2(amps, count);
+    rc = import_rows(sim, longest);
+    if (rc != QW_OK) return rc;
+    QW_CUDA(sim, scratch.take(M * 16, &L.K));
+    QW_CUDA(sim, scratch.take(M * 16, &L.A));
+    QW_CUDA(sim, scratch.take(sizeof(QwIoFlags), (void **)&L.flags));
+    QW_CUDA(sim, cudaMemsetAsync(L.flags, 0, sizeof(QwIoFlags), sim->stream));
+    QW_CUDA(sim, cudaMemcpyAsync(L.K, k.data(), M * 16, cudaMemcpyHostToDevice, sim->stream));
+    QW_CUDA(sim, cudaMemcpyAsync(L.A, a.data(), M * 16, cudaMemcpyHostToDevice, sim->stream));
+    QW_CUDA(sim, cudaStreamSynchronize(sim->stream));
+    return QW_OK;
 }
 
 extern "C" int qw_state_import(qw_sim *sim, int32_t key_words, const uint64_t *keys, const double *amps,
@@ -2326,55 +2484,17 @@ extern "C" int qw_state_import(qw_sim *sim, int32_t key_words, const uint64_t *k
     if (key_words < 1 || key_words > 10 || key_words * 64 < 4 * nb + 34)
         return fail(sim, QW_ERR_ARG, "key_words too small for the packed register layout");
     if (count < 0 || (count > 0 && (!keys || !amps))) return fail(sim, QW_ERR_ARG, "bad arrays");
-    cudaStream_t st = sim->stream;
     FlatScratch scratch(sim, true);
-    void *K = nullptr, *A = nullptr;
-    QwIoFlags *flags = nullptr;
-    double norm2 = 0.0;
+    ImportList L;
     if (count > 0) {
-        const size_t M = (size_t)count;
-        void *in = nullptr;
-        QW_CUDA(sim, scratch.take(M * (size_t)key_words * 8, &in));
-        QW_CUDA(sim, scratch.take(M * 16, &K));
-        QW_CUDA(sim, scratch.take(M * 16, &A));
-        QW_CUDA(sim, scratch.take(sizeof(QwIoFlags), (void **)&flags));
-        QW_CUDA(sim, cudaMemsetAsync(flags, 0, sizeof(QwIoFlags), st));
-        QW_CUDA(sim, cudaMemcpyAsync(in, keys, M * (size_t)key_words * 8, cudaMemcpyHostToDevice, st));
-        QW_CUDA(sim, qw_io_load(sim->d, static_cast<uint64_t *>(in), key_words, count, K, flags, st));
-        QW_CUDA(sim, qw_io_order(sim->d, K, count, flags, st));
-        sim->launches += 2;
-        QW_CUDA(sim, cudaMemcpyAsync(A, amps, M * 16, cudaMemcpyHostToDevice, st));
-        for (int64_t i = 0; i < count; ++i) norm2 += amps[2 * i] * amps[2 * i] + amps[2 * i + 1] * amps[2 * i + 1];
-        static_assert(sizeof(QwIoFlags) <= 8 * (kFlatSort - kFlatIo), "flags of an import");
-        const QwIoFlags &h = *reinterpret_cast<const QwIoFlags *>(sim->h_flat + kFlatIo);
-        QW_CUDA(sim, cudaMemcpyAsync(sim->h_flat + kFlatIo, flags, sizeof h, cudaMemcpyDeviceToHost, st));
-        QW_CUDA(sim, cudaStreamSynchronize(st));
-        if (h.unsorted && !h.bad) { /* an exported list is sorted; any other is sorted here */
-            void *tk = nullptr, *ta = nullptr, *work = nullptr;
-            QW_CUDA(sim, scratch.take(M * 16, &tk));
-            QW_CUDA(sim, scratch.take(M * 16, &ta));
-            QW_CUDA(sim, scratch.take(qw_flat_sort_bytes(count), &work));
-            QW_CUDA(sim, cudaMemsetAsync(flags, 0, sizeof(QwIoFlags), st));
-            int in_tmp = 0;
-            QW_CUDA(sim, qw_flat_sort(sim->d, K, static_cast<double2 *>(A), tk, static_cast<double2 *>(ta), count, 0,
-                                      QW_SORT_FULL, work, sim->h_flat + kFlatSort, &flags->status, st, 2, &in_tmp));
-            if (in_tmp) {
-                std::swap(K, tk);
-                std::swap(A, ta);
-            }
-            QW_CUDA(sim, qw_io_order(sim->d, K, count, flags, st));
-            sim->launches++;
-            QW_CUDA(sim, cudaMemcpyAsync(sim->h_flat + kFlatIo, flags, sizeof h, cudaMemcpyDeviceToHost, st));
-            QW_CUDA(sim, cudaStreamSynchronize(st));
-            if (h.status != 0 || h.unsorted)
-                return fail(sim, QW_ERR_DEVICE_STATUS, "qw_state_import: the sort of the keys gave up waiting for a tile's count");
+        bool room = true;
+        int rc = import_on_device(sim, scratch, key_words, keys, amps, count, L, &room);
+        if (rc != QW_OK && !room) {
+            scratch.give_back();
+            rc = import_by_host(sim, scratch, key_words, keys, amps, count, L);
+            if (rc == QW_OK) sim->err.clear();
         }
-        if (h.bad || h.dup) return import_refused(sim, key_words, keys, count);
-        /* a row longer than row_capacity: grow the buckets */
-        if (sim->opts.overflow_fallback && (int64_t)h.longest > sim->d.cap_row) {
-            const int rc = grow_rows(sim, (int64_t)h.longest);
-            if (rc != QW_OK) return rc;
-        }
+        if (rc != QW_OK) return rc;
     }
     for (int bi = 0; bi < 3; ++bi) {
         QW_CUDA(sim, qw_launch_clear(sim->d, sim->buf[bi], 0, sim->d.total_buckets, 1, sim->stream));
@@ -2382,7 +2502,7 @@ extern "C" int qw_state_import(qw_sim *sim, int32_t key_words, const uint64_t *k
     }
     Scalars z{};
     z.scale[0] = z.scale[1] = 1.0;
-    z.renorm_target = norm2;
+    z.renorm_target = L.norm2;
     QW_CUDA(sim, pos_forget(sim)); /* what comes now is not those steps' error */
     QW_CUDA(sim, cudaMemcpyAsync(sim->sc, &z, sizeof z, cudaMemcpyHostToDevice, sim->stream));
     sim->scale_slot = sim->sync_slot = 0;
@@ -2390,8 +2510,8 @@ extern "C" int qw_state_import(qw_sim *sim, int32_t key_words, const uint64_t *k
     sim->sync_done = 0;
     drop_graphs(sim);
     if (count > 0) {
-        QW_CUDA(sim, qw_flat_scatter(sim->d, sim->buf[sim->cur], sim->fp32, K, static_cast<double2 *>(A), count,
-                                     &sim->sc->status, &flags->maxrow, &flags->norm, st, 2));
+        QW_CUDA(sim, qw_flat_scatter(sim->d, sim->buf[sim->cur], sim->fp32, L.K, static_cast<double2 *>(L.A), count,
+                                     &sim->sc->status, &L.flags->maxrow, &L.flags->norm, sim->stream, 2));
         sim->launches++;
     }
     int rc = check_status(sim, "qw_state_import");
@@ -2400,7 +2520,7 @@ extern "C" int qw_state_import(qw_sim *sim, int32_t key_words, const uint64_t *k
     sim->fresh_T = false;
     /* each instance's share of the target, which setting one of them again replaces */
     for (auto &v : sim->init_norm2) v = 0.0;
-    if (sim->d.ninst == 1) sim->init_norm2[0] = norm2;
+    if (sim->d.ninst == 1) sim->init_norm2[0] = L.norm2;
     else {
         const int at = (18 + 4 * nb) >> 6, off = (18 + 4 * nb) & 63; /* the instance's 16 bits */
         for (int64_t i = 0; i < count; ++i) {

@@ -11,6 +11,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <vector>
 
 #include "qw_internal.h"
 
@@ -25,6 +26,8 @@ struct Fake {
     double first_us = 0.0;      /* what the first launch of each kind takes on top */
     std::map<int, int> launched; /* launches by mode (a positional run: 100) */
     int fail_malloc = -1;       /* device allocations until one fails; -1: none does */
+    int64_t bytes = 0, room = -1; /* of the device allocations; at most (-1: no limit) */
+    std::vector<uint64_t> list; /* keys, then amplitudes' real parts, of the last two-word scatter */
     cudaError_t last = cudaSuccess;
     int give_up = 0;            /* the next positional launch gives up its wait */
     int status_bits = 0;        /* the next bucket step or scatter sets these */
@@ -40,6 +43,7 @@ struct Fake {
     int refuse = 0;                 /* the next positional launch is refused */
     unsigned long long epoch = 0;   /* of the last one that was not */
     int64_t run_steps = 0;          /* steps of the runs since the last reset */
+    unsigned int longest = 0;       /* an imported list's longest row */
     double target = 0.0; /* the renormalisation target of the last step */
 } F;
 
@@ -54,17 +58,21 @@ cudaError_t done(cudaError_t e = cudaSuccess)
 cudaError_t take(void **p, size_t n)
 {
     *p = nullptr;
-    if (F.fail_malloc == 0) return done(cudaErrorMemoryAllocation);
+    if (F.fail_malloc == 0 || (F.room >= 0 && F.bytes + (int64_t)n > F.room)) return done(cudaErrorMemoryAllocation);
     if (F.fail_malloc > 0) --F.fail_malloc;
     *p = std::calloc(n ? n : 1, 1);
     F.sizes[*p] = n;
+    F.bytes += (int64_t)n;
     ++F.live;
     return cudaSuccess;
 }
 
 cudaError_t give(void *p)
 {
-    if (p) --F.live;
+    if (p) {
+        --F.live;
+        F.bytes -= (int64_t)F.sizes[p];
+    }
     std::free(p);
     return cudaSuccess;
 }
@@ -93,6 +101,9 @@ void fake_set_times(double run, double single, double launch_, double first)
     F.first_us = first;
 }
 void fake_fail_malloc(int after) { F.fail_malloc = after; }
+void fake_room(int64_t more) { F.room = more < 0 ? -1 : F.bytes + more; }
+void fake_longest(int n) { F.longest = (unsigned int)n; }
+uint64_t fake_listed(int64_t i) { return F.list.at((size_t)i); }
 void fake_give_up(int n) { F.give_up = n; }
 void fake_status(int bits) { F.status_bits = bits; }
 void fake_flat_wait(int n) { F.flat_wait = n; }
@@ -368,9 +379,17 @@ cudaError_t qw_launch_count(const QwSimDev &, const QwBufDev &, int, unsigned lo
 }
 cudaError_t qw_launch_qls_norm(const double2 *, int, double *, int64_t *, cudaStream_t) { return launch(111, 0.0); }
 cudaError_t qw_launch_regrow(const QwSimDev &, const QwBufDev &, int, uint64_t *, void *, int, cudaStream_t) { return launch(112, 0.0); }
-cudaError_t qw_flat_gather(const QwSimDev &, const QwBufDev &, int, int, const double *, void *, double2 *, unsigned long long *,
-                           int64_t, cudaStream_t, int)
+/* (two-word keys: from the highest down, key i's amplitude i + 2 i times i) */
+cudaError_t qw_flat_gather(const QwSimDev &, const QwBufDev &, int, int, const double *, void *keys, double2 *amps,
+                           unsigned long long *, int64_t cap, cudaStream_t, int kw)
 {
+    uint64_t *k = static_cast<uint64_t *>(keys);
+    for (int64_t i = 0; kw == 2 && i < cap; ++i) {
+        const int64_t v = cap - 1 - i;
+        k[2 * i] = (uint64_t)(v % 7);
+        k[2 * i + 1] = (uint64_t)(v / 7);
+        amps[i] = make_double2((double)v, 2.0 * (double)v);
+    }
     return launch(113, 0.0);
 }
 cudaError_t qw_flat_map(const QwSimDev &, void *, int64_t M, uint32_t, int32_t *, cudaStream_t, int)
@@ -379,7 +398,7 @@ cudaError_t qw_flat_map(const QwSimDev &, void *, int64_t M, uint32_t, int32_t *
     return launch(114, 0.0);
 }
 cudaError_t qw_flat_phase(const QwSimDev &, const void *, double2 *, int64_t, cudaStream_t, int) { return launch(115, 0.0); }
-size_t qw_flat_sort_bytes(int64_t M) { return (size_t)M * 8; }
+size_t qw_flat_sort_bytes(int64_t M) { return (size_t)M * 25; }
 cudaError_t qw_flat_sort(const QwSimDev &, void *, double2 *, void *, double2 *, int64_t, int, int, void *, unsigned long long *,
                          int32_t *, cudaStream_t, int, int *in_tmp)
 {
@@ -419,15 +438,24 @@ cudaError_t qw_flat_readout(const QwSimDev &, const void *, const double2 *, int
 {
     return launch(118, 0.0);
 }
-cudaError_t qw_flat_scatter(const QwSimDev &, const QwBufDev &, int, const void *, const double2 *, int64_t, int32_t *status,
-                            unsigned int *, double *, cudaStream_t, int)
+cudaError_t qw_flat_scatter(const QwSimDev &, const QwBufDev &, int, const void *keys, const double2 *amps, int64_t M,
+                            int32_t *status, unsigned int *, double *, cudaStream_t, int kw)
 {
+    if (kw == 2) {
+        const uint64_t *k = static_cast<const uint64_t *>(keys);
+        F.list.assign(k, k + 2 * M);
+        for (int64_t i = 0; i < M; ++i) F.list.push_back((uint64_t)amps[i].x);
+    }
     *status |= F.status_bits;
     F.status_bits = 0;
     return launch(119, 0.0);
 }
 cudaError_t qw_io_load(const QwSimDev &, const uint64_t *, int, int64_t, void *, QwIoFlags *, cudaStream_t) { return launch(120, 0.0); }
-cudaError_t qw_io_order(const QwSimDev &, const void *, int64_t, QwIoFlags *, cudaStream_t) { return launch(121, 0.0); }
+cudaError_t qw_io_order(const QwSimDev &, const void *, int64_t, QwIoFlags *f, cudaStream_t)
+{
+    f->longest = F.longest;
+    return launch(121, 0.0);
+}
 cudaError_t qw_io_store(const void *, int, int64_t, uint64_t *, cudaStream_t) { return launch(122, 0.0); }
 cudaError_t qw_flat_finish(const QwStepArgs &a, const double *, const int64_t *, cudaStream_t)
 {

@@ -42,6 +42,8 @@ def fake(fake_path, monkeypatch):
         getattr(lib, name).restype = ctypes.c_int64
     lib.fake_word.restype = lib.fake_epoch.restype = ctypes.c_ulonglong
     lib.fake_target.restype = ctypes.c_double
+    lib.fake_room.argtypes = lib.fake_listed.argtypes = [ctypes.c_int64]
+    lib.fake_listed.restype = ctypes.c_uint64
     lib.fake_set_step.argtypes = [ctypes.c_int, ctypes.c_double]
     lib.fake_set_times.argtypes = [ctypes.c_double] * 4
     lib.fake_reset()
@@ -233,3 +235,66 @@ def test_a_state_refused_under_capture_is_not_there(fake):
         with pytest.raises(qwalk.QwError) as e:
             sim.measure_register("j", 64)
         assert e.value.code == qwalk.QW_ERR_STATE
+
+
+@pytest.mark.parametrize("words", [2, 4])
+@pytest.mark.parametrize("room", [32, 48, 64, 72])
+def test_a_list_is_exported_where_only_itself_fits_the_device(fake, room, words):
+    """32 bytes a branch beside the state have always been enough (1000 branches, keys
+    from the highest down as the fake gathers them)."""
+    with _sim() as sim:
+        sim.state_init(_b(64))
+        live = fake.fake_live()
+        fake.fake_room(1000 * room + 64)
+        keys, amps = sim.state_export(key_words=words)
+        assert np.array_equal(keys[:, 1] * 7 + keys[:, 0], np.arange(1000)) and not keys[:, 2:].any()
+        assert np.array_equal(amps, np.arange(1000) * (1.0 + 2.0j))
+        sim.state_init(_b(64))  # no error is left behind
+        assert fake.fake_live() == live
+
+
+@pytest.mark.parametrize("words", [2, 4])
+@pytest.mark.parametrize("room", [32, 40, 47])
+def test_a_list_is_imported_where_only_itself_fits_the_device(fake, room, words):
+    """So too for an import, in any order of its keys; a list that is refused is
+    refused for the same reason, and one that does not fit at all leaves no error."""
+    with _sim() as sim:
+        sim.state_init(_b(64))
+        live = fake.fake_live()
+        regs = np.zeros((1000, 8), dtype=np.uint64)
+        v = np.random.default_rng(3).permutation(1000).astype(np.uint64)
+        regs[:, 0], regs[:, 4], regs[:, 5] = v // 32, v // 2 % 16, v % 2  # jc, k, b2
+        keys, amps = sim.pack(regs, words), v.astype(float)
+        fake.fake_room(1000 * room + 64)
+        sim.state_import(keys, amps)
+        order = np.lexsort(keys.T)
+        for i in (0, 1, 500, 998, 999):
+            assert [fake.fake_listed(2 * i), fake.fake_listed(2 * i + 1)] == [int(x) for x in keys[order[i], :2]]
+            assert fake.fake_listed(2000 + i) == int(v[order[i]])
+        twice, beyond = keys.copy(), keys.copy()
+        twice[7] = twice[600]
+        beyond[9, -1] |= np.uint64(1 << 63)
+        regs[11, 6] = 1  # register A
+        for bad, why in ((twice, "duplicate"), (beyond, "above the layout"), (sim.pack(regs, words), "register A")):
+            with pytest.raises(qwalk.QwError, match=why) as e:
+                sim.state_import(bad, amps)
+            assert e.value.code == qwalk.QW_ERR_ARG
+        fake.fake_room(1000 * 16)
+        with pytest.raises(qwalk.QwError) as e:
+            sim.state_import(keys, amps)
+        assert e.value.code == qwalk.QW_ERR_CUDA
+        sim.state_init(_b(64))
+        assert fake.fake_live() == live
+
+
+def test_an_import_grows_the_rows_before_its_list_takes_the_memory(fake):
+    """Row buckets that fit the device, but not beside the scratch of the checks there."""
+    with _sim(row_capacity=8) as sim:
+        sim.state_init(_b(64), apply_T=False)
+        regs = np.zeros((100, 8), dtype=np.uint64)
+        regs[:, 3], regs[:, 4] = np.arange(100) % 50, np.arange(100) // 50  # kc, k: one row
+        fake.fake_longest(100)
+        rows = 3 * 24 * (128 + 256) * 128  # total_buckets, 128 branches a row
+        fake.fake_room(rows + 4000)  # the scratch there: 4832 bytes
+        sim.state_import(sim.pack(regs), np.ones(100))
+        assert fake.fake_overruns() == 0
