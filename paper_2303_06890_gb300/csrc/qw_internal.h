@@ -70,7 +70,7 @@ struct QwPartEntry {
 #define QW_MODE_WALK_SLOT 6     /* fused step, one lane per QRAM slot (s = 8, 16, 32) */
 #define QW_MODE_WALK_FLAT 7     /* the literal step on one globally sorted branch list (qw_flat.cu) */
 #define QW_MODE_WALK_FAITHFUL 8 /* the flat step with every working register in a 10-word key */
-#define QW_MODE_WALK_POS 9      /* the state held by position, one lane per QRAM slot (s = 8, 16, 32) */
+#define QW_MODE_WALK_POS 9      /* the state held by position, one lane per QRAM slot (s = 4 .. 64) */
 
 struct QwSimDev {
     int nb, s, L, ninst;
@@ -190,7 +190,7 @@ cudaError_t qw_launch_step(const QwSimDev &d, const QwBufDev &in, const QwBufDev
                            cudaStream_t st);
 /* whether the slot kernel (QW_MODE_WALK_SLOT) covers this sparsity */
 int qw_slot_supported(const QwSimDev &d);
-/* whether the positional layout (QW_MODE_WALK_POS) covers this s (8 .. 64) */
+/* whether the positional layout (QW_MODE_WALK_POS) covers this s (4 .. 64) */
 int qw_pos_supported(const QwSimDev &d);
 /* dynamic shared memory per block of the step kernel of `mode` */
 size_t qw_step_smem_bytes(const QwSimDev &d, int fp32, int mode);

@@ -312,118 +312,118 @@ __device__ __forceinline__ void pos_group(const QwSimDev &d, const typename Amp<
     constexpr float kHalfS = 0.5f * S, kErr = Amp<AmpT>::kApproxErr;
     const AmpT zero = Amp<AmpT>::zero();
     const int lane = threadIdx.x & 31, ul = lane / SW, lb = lane % SW;
-                AmpT a0[SPL], a1[SPL], q0[SPL], q1[SPL];
-                float A0[SPL], A1[SPL], Q0[SPL];
-                bool any = false;
-    #pragma unroll
-                for (int q = 0; q < SPL; ++q) {
-                    a0[q] = in[q].a0;
-                    a1[q] = in[q].a1;
-                    q0[q] = in[q].b0;
-                    q1[q] = FULLST ? in[q].b1 : zero;
-                    if (rescale) {
-                        a0[q] = scale.apply(a0[q]);
-                        a1[q] = scale.apply(a1[q]);
-                        q0[q] = scale.apply(q0[q]);
-                        if (FULLST) q1[q] = scale.apply(q1[q]);
-                    }
-                    A0[q] = Amp<AmpT>::inf_norm(a0[q]);
-                    A1[q] = Amp<AmpT>::inf_norm(a1[q]);
-                    Q0[q] = Amp<AmpT>::inf_norm(q0[q]);
-                    const bool n0 = A0[q] != 0.0f, n1 = A1[q] != 0.0f, m0 = Q0[q] != 0.0f, m1 = FULLST && nz(q1[q]) != 0u;
-                    if (n0) cnt += kCntIn;
-                    if (n1) cnt += kCntIn;
-                    if (m0) cnt += kCntIn;
-                    if (m1) cnt += kCntIn;
-                    any = any || n0 || n1 || m0 || m1;
-                }
-                {
-                    const unsigned m = __ballot_sync(FULL, any);
-                    const unsigned um = SW == 32 ? m : (m >> (ul * SW)) & ((1u << (SW & 31)) - 1u);
-                    if (lb == 0 && um != 0) st.rows += 1; /* units holding branches */
-                }
-                /* b1 = 0: R^dag's b2 = 0 output u (its exact value, scaled by 2 / s),
-                   and whether u and v are kept: |v| >= | f |a1| - g |a0| | in the
-                   maximum norm, which the phases leave alone, so the norms decide
-                   unless they nearly cancel */
-                typename Amp<AmpT>::Wide u[SPL];
-                PairState<AmpT> ps[SPL];
-                float f[SPL], g_[SPL], U[SPL];
-    #pragma unroll
-                for (int q = 0; q < SPL; ++q) {
-                    const uint32_t sgn = (dst[q] & 0x40000000u) >> 15; /* the value's sign bit (bit 15) */
-                    const bool sneg = (dst[q] >> 31) != 0u;
-                    f[q] = Amp<AmpT>::rot_f(rv[q]);
-                    g_[q] = Amp<AmpT>::rot_g(rv[q]);
-                    u[q] = Amp<AmpT>::rdag0(Amp<AmpT>::prescale(rv[q], LOG2S - 1), sgn, sneg, a0[q], a1[q]);
-                    U[q] = kHalfS * Amp<AmpT>::inf_norm(Amp<AmpT>::narrow(u[q]));
-                    const float fa = f[q] * A1[q], ga = g_[q] * A0[q];
-                    ps[q].c0 = U[q] > d.thr32;
-                    ps[q].c1 = fabsf(fa - ga) > fmaf(kErr, fa + ga, d.thr32);
-                    ps[q].lossy = false;
-                    if ((!ps[q].c0 && U[q] > 0.0f) || (!ps[q].c1 && fa + ga > 0.0f)) {
-                        const unsigned e = pair_exact<AmpT>(d, rv[q], sgn, sneg, a0[q], a1[q]);
-                        ps[q].c0 = (e & 1u) != 0u;
-                        ps[q].c1 = (e & 2u) != 0u;
-                        ps[q].lossy = (e & 4u) != 0u;
-                        if (!ps[q].c0) {
-                            u[q] = Amp<AmpT>::wide_zero();
-                            U[q] = 0.0f;
-                        }
-                    }
-                    if (ps[q].c0) cnt += kCntRdag;
-                    if (ps[q].c1) cnt += kCntRdag + kCntHph;
-                }
-                __syncwarp();
-                typename Amp<AmpT>::Sum sum;
-                sum.set(u[0]);
-    #pragma unroll
-                for (int q = 1; q < SPL; ++q) sum.add(u[q]);
-                sum.reduce(SW, SW);
-                on_sum(sum);
-                const float Rn = Amp<AmpT>::inf_norm(Amp<AmpT>::sum_amp(sum));
-    #pragma unroll
-                for (int q = 0; q < SPL; ++q) {
-                    const uint32_t sgn = (dst[q] & 0x40000000u) >> 15;
-                    const bool sneg = (dst[q] >> 31) != 0u;
-                    /* the reflected r - u, then R: (f r - a0, g r - a1) */
-                    AmpT rA0, rA1;
-                    bool d0 = fabsf(Rn - U[q]) > fmaf(kErr, Rn + U[q], d.thr32);
-                    Amp<AmpT>::reflect(sum, rv[q], sgn, sneg, a0[q], a1[q], rA0, rA1);
-                    if (ps[q].lossy || (!d0 && Rn + U[q] > 0.0f))
-                        d0 = pair_reflect_exact<AmpT>(d, sum, rv[q], sgn, sneg, a0[q], a1[q], ps[q], rA0, rA1);
-                    if (d0) cnt += kCntHph;
-                    /* b1 = 1: R^dag, -1, R */
-                    AmpT rB0 = Amp<AmpT>::neg(q0[q]), rB1 = Amp<AmpT>::neg(q1[q]);
-                    if (FULLST) {
-                        const unsigned kept = pair_negate<AmpT>(d, rv[q], sgn, sneg, q0[q], q1[q], rB0, rB1);
-                        cnt += kept * (kCntRdag + kCntHph);
-                    } else { /* q1 = 0: |u| = f |q0|, |v| = g |q0| */
-                        const float fq = f[q] * Q0[q], gq = g_[q] * Q0[q], lim = fmaf(kErr, Q0[q], d.thr32);
-                        const bool c0 = fq > lim, c1 = gq > lim;
-                        unsigned kept = (c0 ? 1u : 0u) + (c1 ? 1u : 0u);
-                        if ((!c0 && fq > 0.0f) || (!c1 && gq > 0.0f))
-                            negate_exact<AmpT>(d, rv[q], sgn, sneg, q0[q], zero, rB0, rB1, kept);
-                        cnt += kept * (kCntRdag + kCntHph);
-                    }
-                    const bool eA0 = pos_keep(d, rA0), eA1 = pos_keep(d, rA1);
-                    const bool eB0 = pos_keep(d, rB0), eB1 = FULLST && pos_keep(d, rB1);
-                    if (valid) {
-                        if (renorm) {
-                            if (eA0) norm_add(nrm, rA0);
-                            if (eB0) norm_add(nrm, rB0);
-                            if (eA1) norm_add(nrm, rA1);
-                            if (FULLST && eB1) norm_add(nrm, rB1);
-                        }
-                        /* S: (k, b2) <-> (j, b1) */
-                        const Entry<AmpT> o = {eA0 ? rA0 : zero, eB0 ? rB0 : zero, eA1 ? rA1 : zero, eB1 ? rB1 : zero};
-                        on_out(q, o);
-                    }
-                    if (eA0) cnt += kCntOut;
-                    if (eB0) cnt += kCntOut;
-                    if (eA1) cnt += kCntOut;
-                    if (eB1) cnt += kCntOut;
-                }
+    AmpT a0[SPL], a1[SPL], q0[SPL], q1[SPL];
+    float A0[SPL], A1[SPL], Q0[SPL];
+    bool any = false;
+#pragma unroll
+    for (int q = 0; q < SPL; ++q) {
+        a0[q] = in[q].a0;
+        a1[q] = in[q].a1;
+        q0[q] = in[q].b0;
+        q1[q] = FULLST ? in[q].b1 : zero;
+        if (rescale) {
+            a0[q] = scale.apply(a0[q]);
+            a1[q] = scale.apply(a1[q]);
+            q0[q] = scale.apply(q0[q]);
+            if (FULLST) q1[q] = scale.apply(q1[q]);
+        }
+        A0[q] = Amp<AmpT>::inf_norm(a0[q]);
+        A1[q] = Amp<AmpT>::inf_norm(a1[q]);
+        Q0[q] = Amp<AmpT>::inf_norm(q0[q]);
+        const bool n0 = A0[q] != 0.0f, n1 = A1[q] != 0.0f, m0 = Q0[q] != 0.0f, m1 = FULLST && nz(q1[q]) != 0u;
+        if (n0) cnt += kCntIn;
+        if (n1) cnt += kCntIn;
+        if (m0) cnt += kCntIn;
+        if (m1) cnt += kCntIn;
+        any = any || n0 || n1 || m0 || m1;
+    }
+    {
+        const unsigned m = __ballot_sync(FULL, any);
+        const unsigned um = SW == 32 ? m : (m >> (ul * SW)) & ((1u << (SW & 31)) - 1u);
+        if (lb == 0 && um != 0) st.rows += 1; /* units holding branches */
+    }
+    /* b1 = 0: R^dag's b2 = 0 output u (its exact value, scaled by 2 / s),
+       and whether u and v are kept: |v| >= | f |a1| - g |a0| | in the
+       maximum norm, which the phases leave alone, so the norms decide
+       unless they nearly cancel */
+    typename Amp<AmpT>::Wide u[SPL];
+    PairState<AmpT> ps[SPL];
+    float f[SPL], g_[SPL], U[SPL];
+#pragma unroll
+    for (int q = 0; q < SPL; ++q) {
+        const uint32_t sgn = (dst[q] & 0x40000000u) >> 15; /* the value's sign bit (bit 15) */
+        const bool sneg = (dst[q] >> 31) != 0u;
+        f[q] = Amp<AmpT>::rot_f(rv[q]);
+        g_[q] = Amp<AmpT>::rot_g(rv[q]);
+        u[q] = Amp<AmpT>::rdag0(Amp<AmpT>::prescale(rv[q], LOG2S - 1), sgn, sneg, a0[q], a1[q]);
+        U[q] = kHalfS * Amp<AmpT>::inf_norm(Amp<AmpT>::narrow(u[q]));
+        const float fa = f[q] * A1[q], ga = g_[q] * A0[q];
+        ps[q].c0 = U[q] > d.thr32;
+        ps[q].c1 = fabsf(fa - ga) > fmaf(kErr, fa + ga, d.thr32);
+        ps[q].lossy = false;
+        if ((!ps[q].c0 && U[q] > 0.0f) || (!ps[q].c1 && fa + ga > 0.0f)) {
+            const unsigned e = pair_exact<AmpT>(d, rv[q], sgn, sneg, a0[q], a1[q]);
+            ps[q].c0 = (e & 1u) != 0u;
+            ps[q].c1 = (e & 2u) != 0u;
+            ps[q].lossy = (e & 4u) != 0u;
+            if (!ps[q].c0) {
+                u[q] = Amp<AmpT>::wide_zero();
+                U[q] = 0.0f;
+            }
+        }
+        if (ps[q].c0) cnt += kCntRdag;
+        if (ps[q].c1) cnt += kCntRdag + kCntHph;
+    }
+    __syncwarp();
+    typename Amp<AmpT>::Sum sum;
+    sum.set(u[0]);
+#pragma unroll
+    for (int q = 1; q < SPL; ++q) sum.add(u[q]);
+    sum.reduce(SW, SW);
+    on_sum(sum);
+    const float Rn = Amp<AmpT>::inf_norm(Amp<AmpT>::sum_amp(sum));
+#pragma unroll
+    for (int q = 0; q < SPL; ++q) {
+        const uint32_t sgn = (dst[q] & 0x40000000u) >> 15;
+        const bool sneg = (dst[q] >> 31) != 0u;
+        /* the reflected r - u, then R: (f r - a0, g r - a1) */
+        AmpT rA0, rA1;
+        bool d0 = fabsf(Rn - U[q]) > fmaf(kErr, Rn + U[q], d.thr32);
+        Amp<AmpT>::reflect(sum, rv[q], sgn, sneg, a0[q], a1[q], rA0, rA1);
+        if (ps[q].lossy || (!d0 && Rn + U[q] > 0.0f))
+            d0 = pair_reflect_exact<AmpT>(d, sum, rv[q], sgn, sneg, a0[q], a1[q], ps[q], rA0, rA1);
+        if (d0) cnt += kCntHph;
+        /* b1 = 1: R^dag, -1, R */
+        AmpT rB0 = Amp<AmpT>::neg(q0[q]), rB1 = Amp<AmpT>::neg(q1[q]);
+        if (FULLST) {
+            const unsigned kept = pair_negate<AmpT>(d, rv[q], sgn, sneg, q0[q], q1[q], rB0, rB1);
+            cnt += kept * (kCntRdag + kCntHph);
+        } else { /* q1 = 0: |u| = f |q0|, |v| = g |q0| */
+            const float fq = f[q] * Q0[q], gq = g_[q] * Q0[q], lim = fmaf(kErr, Q0[q], d.thr32);
+            const bool c0 = fq > lim, c1 = gq > lim;
+            unsigned kept = (c0 ? 1u : 0u) + (c1 ? 1u : 0u);
+            if ((!c0 && fq > 0.0f) || (!c1 && gq > 0.0f))
+                negate_exact<AmpT>(d, rv[q], sgn, sneg, q0[q], zero, rB0, rB1, kept);
+            cnt += kept * (kCntRdag + kCntHph);
+        }
+        const bool eA0 = pos_keep(d, rA0), eA1 = pos_keep(d, rA1);
+        const bool eB0 = pos_keep(d, rB0), eB1 = FULLST && pos_keep(d, rB1);
+        if (valid) {
+            if (renorm) {
+                if (eA0) norm_add(nrm, rA0);
+                if (eB0) norm_add(nrm, rB0);
+                if (eA1) norm_add(nrm, rA1);
+                if (FULLST && eB1) norm_add(nrm, rB1);
+            }
+            /* S: (k, b2) <-> (j, b1) */
+            const Entry<AmpT> o = {eA0 ? rA0 : zero, eB0 ? rB0 : zero, eA1 ? rA1 : zero, eB1 ? rB1 : zero};
+            on_out(q, o);
+        }
+        if (eA0) cnt += kCntOut;
+        if (eB0) cnt += kCntOut;
+        if (eA1) cnt += kCntOut;
+        if (eB1) cnt += kCntOut;
+    }
 }
 
 template <typename AmpT, int S, bool FULLST, bool TAB>
