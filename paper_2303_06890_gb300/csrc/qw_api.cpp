@@ -1907,7 +1907,7 @@ static int tune_time(qw_sim *sim, int32_t steps, cudaEvent_t *ev, double *us)
     QW_CUDA(sim, cudaStreamSynchronize(st));
     for (int r = 0; r < (runs ? 3 : 1); ++r) {
         if (r > 0) QW_CUDA(sim, cudaEventRecord(ev[r - 1], st));
-        const int rc = runs ? launch_pos(sim, m, -1, 0) : launch_walk(sim, 0);
+        const int rc = runs ? launch_pos(sim, r == 0 ? 2 : m, -1, 0) : launch_walk(sim, 0);
         sim->cur = cur;
         sim->scale_slot = slot;
         sim->issued = issued;
