@@ -1941,6 +1941,10 @@ extern "C" int qw_autotune(qw_sim *sim, int32_t steps, int32_t *choice, double *
         if (choice) *choice = -1;
         return QW_OK;
     }
+    if (sim->pos_issued) { /* their status read first: the bucket steps to come have errors of their own */
+        const int rc = sync_walk(sim, "qw_autotune");
+        if (rc != QW_OK) return rc;
+    }
     /* candidates: walk_variant -> mode.  A segment holds two rows on chip:
        tried only when the warp buffer fits them; the slot kernel (which falls
        back to segments) also needs s = 8, 16 or 32; the positional layout

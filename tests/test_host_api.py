@@ -109,6 +109,18 @@ def test_an_import_that_overflows_after_positional_steps_is_a_capacity_error(fak
         assert e.value.code == qwalk.QW_ERR_CAPACITY
 
 
+def test_a_bucket_step_that_overflows_in_the_autotuner_is_a_capacity_error(fake):
+    """Nor that of the positional steps issued before the call; the state is kept."""
+    with _sim(walk_variant=7, overflow_fallback=False) as sim:
+        sim.state_init(_b(64))
+        sim.enqueue_walk_steps(2)
+        fake.fake_status(ROW_OVERFLOW)
+        with pytest.raises(qwalk.QwError) as e:
+            sim.autotune(2)
+        assert e.value.code == qwalk.QW_ERR_CAPACITY
+        sim.apply_walk_step(1)
+
+
 @pytest.mark.parametrize("how", ["init", "init without T", "import", "read", "sync"])
 def test_a_run_starts_on_clear_barrier_words_after_one_that_gave_up(fake, how):
     """A launch that gives up its wait leaves words that some blocks arrived at.  They
