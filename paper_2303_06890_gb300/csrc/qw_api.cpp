@@ -186,6 +186,7 @@ static const int kGraphTerms = 3;  /* QLS terms per graph: 2 walk steps each */
    bits (2 x 10) */
 static const int kFlatTotal = 0, kFlatCount = 1, kFlatRow = 2, kFlatIo = 4, kFlatSort = 16, kFlatWords = 40;
 static const int64_t kPosSteps = 1024; /* walk steps of one positional launch: a few milliseconds */
+static const int64_t kPinnedBins = 65536; /* of a marginal in pinned memory: the largest register's, 512 KB */
 static const int64_t kTuneSteps = 32;  /* at least, of one the autotuner times: the launch is a small part */
 
 static void drop_graphs(qw_sim *sim)
@@ -2155,7 +2156,7 @@ extern "C" int qw_measure_register(qw_sim *sim, int32_t inst, int32_t reg, doubl
         QW_CUDA(sim, cudaMalloc((void **)&sim->meas_dev, (size_t)len * sizeof(double)));
         sim->meas_cap = len;
     }
-    if (sim->pos_live && (reg == QW_REG_J || reg == QW_REG_K)) {
+    if (sim->pos_live && (reg == QW_REG_J || reg == QW_REG_K) && len <= kPinnedBins) {
         /* every bin written by one launch, into pinned memory, with the status
            head beside it */
         if (sim->h_probs_cap < len) {

@@ -33,6 +33,7 @@ struct Fake {
     int status_bits = 0;        /* the next bucket step or scatter sets these */
     int flat_wait = 0;          /* the next single-pass launch of the flat path gives up */
     int64_t map_most = 0;       /* entries of the longest list given to qw_flat_map */
+    size_t pinned_most = 0;     /* the largest pinned allocation */
     int64_t live = 0;           /* device allocations not yet freed */
     int64_t sync_copies = 0;    /* cudaMemcpy: ordered on the default stream alone */
     int capturing = 0;
@@ -109,6 +110,7 @@ void fake_status(int bits) { F.status_bits = bits; }
 void fake_flat_wait(int n) { F.flat_wait = n; }
 void fake_capture(int on) { F.capturing = on; }
 int64_t fake_live() { return F.live; }
+int64_t fake_pinned_most() { return (int64_t)F.pinned_most; }
 int64_t fake_sync_copies() { return F.sync_copies; }
 int64_t fake_map_most() { return F.map_most; }
 int64_t fake_tinits() { return F.tinits; }
@@ -129,6 +131,7 @@ cudaError_t cudaFree(void *p) { return give(p); }
 cudaError_t cudaFreeAsync(void *p, cudaStream_t) { return give(p); }
 cudaError_t cudaMallocHost(void **p, size_t n)
 {
+    F.pinned_most = n > F.pinned_most ? n : F.pinned_most;
     *p = std::calloc(n ? n : 1, 1);
     return cudaSuccess;
 }

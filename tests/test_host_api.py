@@ -38,7 +38,8 @@ def fake(fake_path, monkeypatch):
     monkeypatch.setattr(native, "LIB", fake_path)
     monkeypatch.setattr(qwalk, "_lib", None)
     lib = qwalk.load(build_if_missing=False)
-    for name in ("fake_live", "fake_sync_copies", "fake_map_most", "fake_tinits", "fake_run_steps", "fake_overruns"):
+    for name in ("fake_live", "fake_sync_copies", "fake_map_most", "fake_tinits", "fake_run_steps", "fake_overruns",
+                 "fake_pinned_most"):
         getattr(lib, name).restype = ctypes.c_int64
     lib.fake_word.restype = lib.fake_epoch.restype = ctypes.c_ulonglong
     lib.fake_target.restype = ctypes.c_double
@@ -310,3 +311,13 @@ def test_an_import_grows_the_rows_before_its_list_takes_the_memory(fake):
         fake.fake_room(rows + 4000)  # the scratch there: 4832 bytes
         sim.state_import(sim.pack(regs), np.ones(100))
         assert fake.fake_overruns() == 0
+
+
+def test_a_marginal_of_any_length_takes_bounded_pinned_memory(fake):
+    """Bins beyond the register's are zeros that the caller asked for; the pinned memory
+    that a simulator keeps does not grow with them."""
+    with _sim(walk_variant=7) as sim:
+        sim.state_init(_b(64))
+        for length in (65536, 65537, 1 << 20):
+            assert sim.measure_register("j", length).sum() == length  # (the fake writes 1 to each bin)
+        assert fake.fake_pinned_most() == 65536 * 8
