@@ -248,7 +248,8 @@ int qw_sync(qw_sim *sim);
  * 6) are never chosen; variants not tried are reported as 0 us.  s = 4: a
  * simulator is not created with variant 7, so *choice names the fastest of the
  * others, which one can be created with, while this simulator keeps the
- * positional layout if us_per_step[7] is the least.
+ * positional layout if us_per_step[7] is the least (not tried there with a row_capacity
+ * below 4 s, nor where its tables do not fit the device).
  * The state advances by steps_per_candidate walk steps per
  * variant tried (the variants give the same results).  *choice (nullable)
  * receives the variant, *us_per_step (nullable, QW_WALK_VARIANTS doubles) the

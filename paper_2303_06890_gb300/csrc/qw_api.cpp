@@ -1904,8 +1904,7 @@ static int tune_time(qw_sim *sim, int32_t steps, cudaEvent_t *ev, double *us)
     const int cur = sim->cur, slot = sim->scale_slot;
     const int64_t issued = sim->issued;
     const size_t head = offsetof(Scalars, steps_done);
-    QW_CUDA(sim, cudaMemcpyAsync(sim->h_sc, sim->sc, sizeof(Scalars), cudaMemcpyDeviceToHost, st));
-    QW_CUDA(sim, cudaStreamSynchronize(st));
+    QW_CUDA(sim, cudaMemcpyAsync(sim->h_sc, sim->sc, sizeof(Scalars), cudaMemcpyDeviceToHost, st)); /* (pinned) */
     for (int r = 0; r < (runs ? 3 : 1); ++r) {
         if (r > 0) QW_CUDA(sim, cudaEventRecord(ev[r - 1], st));
         const int rc = runs ? launch_pos(sim, r == 0 ? 2 : m, -1, 0) : launch_walk(sim, 0);
