@@ -1310,6 +1310,9 @@ static int pos_tables(qw_sim *sim)
     const size_t words = QW_POS_WORDS + 2 * (size_t)sim->pos_plan.grid;
     QW_CUDA(sim, dalloc(sim, &sim->pos_words, words));
     QW_CUDA(sim, cudaMemset(sim->pos_words, 0, words * sizeof(unsigned long long)));
+    /* all of it before the simulator's stream goes on, which need not wait for the
+       default one: a memset, and a copy from pageable memory, may return before it is done */
+    QW_CUDA(sim, cudaStreamSynchronize(nullptr));
     sim->mode_alt = d.warp_cap < 2 * d.cap_row ? QW_MODE_WALK_FUSED
                     : (qw_slot_supported(d) ? QW_MODE_WALK_SLOT : QW_MODE_WALK_SEG);
     sim->grid_alt = qw_step_grid(d, sim->fp32, sim->mode_alt);

@@ -36,6 +36,8 @@ struct Fake {
     size_t pinned_most = 0;     /* the largest pinned allocation */
     int64_t live = 0;           /* device allocations not yet freed */
     int64_t sync_copies = 0;    /* cudaMemcpy: ordered on the default stream alone */
+    bool pending = false;       /* default-stream work that need not be done when its call returns */
+    int64_t unordered = 0;      /* kernels launched meanwhile (on another stream, as the tests read it) */
     int capturing = 0;
     unsigned long long words[8] = {0}; /* the barrier words a positional run started on */
     int64_t tinits = 0;
@@ -81,6 +83,7 @@ cudaError_t give(void *p)
 /* what every launcher ends with: an error of an earlier call not yet taken shows here */
 cudaError_t launch(int kind, double us)
 {
+    F.unordered += F.pending;
     F.clock_us += us + (F.launched[kind]++ == 0 ? F.first_us : 0.0);
     const cudaError_t e = F.last;
     F.last = cudaSuccess;
@@ -110,6 +113,7 @@ void fake_status(int bits) { F.status_bits = bits; }
 void fake_flat_wait(int n) { F.flat_wait = n; }
 void fake_capture(int on) { F.capturing = on; }
 int64_t fake_live() { return F.live; }
+int64_t fake_unordered() { return F.unordered; }
 int64_t fake_pinned_most() { return (int64_t)F.pinned_most; }
 int64_t fake_sync_copies() { return F.sync_copies; }
 int64_t fake_map_most() { return F.map_most; }
@@ -140,9 +144,10 @@ cudaError_t cudaFreeHost(void *p)
     std::free(p);
     return cudaSuccess;
 }
-cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind)
+cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind kind)
 {
     ++F.sync_copies;
+    F.pending = kind == cudaMemcpyHostToDevice; /* (one to the host is waited for) */
     std::memmove(d, s, n);
     return cudaSuccess;
 }
@@ -154,6 +159,7 @@ cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cu
 }
 cudaError_t cudaMemset(void *d, int v, size_t n)
 {
+    F.pending = true;
     std::memset(d, v, n);
     return cudaSuccess;
 }
@@ -172,9 +178,14 @@ cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr a, int)
     *v = a == cudaDevAttrMaxSharedMemoryPerBlockOptin ? 232448 : 1;
     return cudaSuccess;
 }
-cudaError_t cudaDeviceSynchronize(void) { return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t)
+cudaError_t cudaDeviceSynchronize(void)
 {
+    F.pending = false;
+    return cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t st)
+{
+    if (!st) F.pending = false;
     return F.capturing ? done(cudaErrorStreamCaptureUnsupported) : cudaSuccess;
 }
 cudaError_t cudaGetLastError(void)

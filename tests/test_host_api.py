@@ -39,7 +39,7 @@ def fake(fake_path, monkeypatch):
     monkeypatch.setattr(qwalk, "_lib", None)
     lib = qwalk.load(build_if_missing=False)
     for name in ("fake_live", "fake_sync_copies", "fake_map_most", "fake_tinits", "fake_run_steps", "fake_overruns",
-                 "fake_pinned_most"):
+                 "fake_pinned_most", "fake_unordered"):
         getattr(lib, name).restype = ctypes.c_int64
     lib.fake_word.restype = lib.fake_epoch.restype = ctypes.c_ulonglong
     lib.fake_target.restype = ctypes.c_double
@@ -321,3 +321,16 @@ def test_a_marginal_of_any_length_takes_bounded_pinned_memory(fake):
         for length in (65536, 65537, 1 << 20):
             assert sim.measure_register("j", length).sum() == length  # (the fake writes 1 to each bin)
         assert fake.fake_pinned_most() == 65536 * 8
+
+
+@pytest.mark.parametrize("kw,tune", [(dict(walk_variant=7), False), (dict(), True)])
+def test_the_layouts_tables_are_there_before_the_simulators_stream_goes_on(fake, kw, tune):
+    """They are written through the default stream, which another, non-blocking one does
+    not wait for; the barrier words of a run among them."""
+    with _sim(stream=64, **kw) as sim:
+        sim.state_init(_b(64))
+        if tune:
+            sim.autotune(2)
+        sim.state_init(_b(64))
+        sim.apply_walk_step(3)
+        assert fake.fake_unordered() == 0
