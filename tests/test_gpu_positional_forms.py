@@ -1,8 +1,12 @@
 """Forms of the positional layout's runs beside those of test_gpu_positional_runs.py:
 complex64 entries, batches on the cluster and over the grid, tables that do not
-fit shared memory, and solves, each against the same steps launched one at a time."""
+fit shared memory, and solves, each against the same steps launched one at a time;
+simulators on streams of their own."""
+from concurrent.futures import ThreadPoolExecutor
+
 import numpy as np
 import pytest
+import torch
 
 from paper_2303_06890_gb300 import qwalk
 from paper_2303_06890_gb300 import workloads as wl
@@ -87,3 +91,26 @@ def test_a_complex64_solve(n, s):
     ys = [sim.apply_qls(coeffs)[0] for sim in
           _pair(lambda g: _positional(m, s, b, precision=qwalk.QW_FP32_AMP, renorm=0, graphs=g))]
     assert np.abs(ys[0] - ys[1]).max() <= 16 * 2.0**-53 * np.abs(coeffs).sum()
+
+
+@pytest.mark.parametrize("n,s", [(300, 8), (5000, 16)])
+def test_simulators_on_streams_of_their_own(n, s):
+    """Two simulators on two non-blocking streams, each driven by a thread: the bits of
+    the same walks one after another."""
+    mats, bs = [_matrix(n, s), _matrix(n + 1, s)], [_b(n, 1), _b(n + 1, 2)]
+    streams = [torch.cuda.Stream() for _ in mats]
+
+    def walk(i):
+        sim = qwalk.Sim(mats[i], s_pad=s, walk_variant=7, stream=streams[i].cuda_stream)
+        out = []
+        for steps in (1, 40, 41):
+            sim.state_init(bs[i])
+            sim.enqueue_walk_steps(steps)
+            out += [sim.measure_register(r, mats[i].n) for r in ("j", "k")]
+        sim.close()
+        return out
+
+    with ThreadPoolExecutor(2) as pool:
+        together = list(pool.map(walk, range(2)))
+    for i in range(2):
+        assert all(np.array_equal(x, y) for x, y in zip(together[i], walk(i)))
