@@ -339,7 +339,7 @@ def run_ours(args, rank, world, local_rank):
         return sm, v, us
 
     sim, variant, tune_us = tuned(qwalk.QW_FP32_AMP)
-    sim.apply_walk_step(args.warmup)
+    timed_walk(sim, args.warmup, torch, flush)  # dropped: warm-up steps issued as the timed ones are
     sim.step_stats(reset=True)
     launches0 = sim.launch_count()
     clocks = ClockSampler(local_rank)
@@ -363,7 +363,7 @@ def run_ours(args, rank, world, local_rank):
 
     # --- the plain FP64 path on the same workload ---
     sim64, variant64, tune64 = tuned(qwalk.QW_FP64)
-    sim64.apply_walk_step(args.warmup)
+    timed_walk(sim64, args.warmup, torch, flush)
     sim64.step_stats(reset=True)
     barrier()
     t64, per64 = timed_walk(sim64, args.fp64_steps, torch, flush)
